@@ -189,6 +189,7 @@ static void dag_release(pvt_dag *g)
         release(g->etab[c].p);
     }
     release(g->cframes.p);
+    release(g->cframes1.p);
     release(g->range_roots.p);
     release(g->range_pos.p);
     if (fs) cudaStreamSynchronize(fs);

@@ -26,6 +26,13 @@ extern template pvt_status launch_class<16, MODE_GLOBAL, true>(pvt_dag *, const 
 extern template pvt_status launch_class<16, MODE_VERTEX, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
 extern template pvt_status launch_class<16, MODE_EDGE, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
 extern template pvt_status launch_class<32, MODE_GLOBAL, true>(pvt_dag *, const CountArgs &, int, cudaStream_t);
+extern template pvt_status launch_class<3, MODE_GLOBAL, true>(pvt_dag *, const CountArgs &, int, cudaStream_t);
+extern template pvt_status launch_class<5, MODE_GLOBAL, true>(pvt_dag *, const CountArgs &, int, cudaStream_t);
+extern template pvt_status launch_class<6, MODE_GLOBAL, true>(pvt_dag *, const CountArgs &, int, cudaStream_t);
+extern template pvt_status launch_class<10, MODE_GLOBAL, true>(pvt_dag *, const CountArgs &, int, cudaStream_t);
+extern template pvt_status launch_class<12, MODE_GLOBAL, true>(pvt_dag *, const CountArgs &, int, cudaStream_t);
+extern template pvt_status launch_class<20, MODE_GLOBAL, true>(pvt_dag *, const CountArgs &, int, cudaStream_t);
+extern template pvt_status launch_class<24, MODE_GLOBAL, true>(pvt_dag *, const CountArgs &, int, cudaStream_t);
 extern template pvt_status launch_class<32, MODE_VERTEX, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
 extern template pvt_status launch_class<32, MODE_EDGE, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
 extern template pvt_status launch_batch_class<1, MODE_GLOBAL>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
@@ -229,7 +236,7 @@ static pvt_status launch_frames(pvt_dag *g, const CountArgs &base, cudaStream_t 
     A.qdone = g->qready[0].p + SPLIT_QCAP;
     A.qctl = g->qctl;
     A.qcap = SPLIT_QCAP;
-    constexpr size_t smem = sizeof(WarpWork<1>) * FRAME_WPB + sizeof(unsigned long long) * HIST_H * HIST_P;
+    constexpr size_t smem = sizeof(WarpWork<1>) * FRAME_WPB + sizeof(unsigned) * HIST_H * HIST_P;
     auto kern = k_walk_frames<true>;
     PVT_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
@@ -246,57 +253,133 @@ static pvt_status launch_frames(pvt_dag *g, const CountArgs &base, cudaStream_t 
     return PVT_OK;
 }
 
+// Frames the wide walks may emit: an allowance per root by class (a wider
+// root meets many more small labels), at most 2^26 (9.7 GB).  The frame walk
+// takes 3 to 4 ns of the GPU per frame, the wide kernels' few warps about
+// ten times that for a frame walked in place: on a 12M-edge graph of
+// degeneracy 280 (k <= 4, 34M frames) a buffer of 2^22 frames cost 204 ms
+// in all, one that holds them 55 ms.
+constexpr unsigned FRAME_CAP_SMALL = 1u << 22, FRAME_CAP_MAX = 1u << 26;
+static unsigned frame_cap(const pvt_dag *g)
+{
+    constexpr int64_t per_root[NCLASS] = {0, 0, 16, 64, 1024, 8192, 32768};
+    int64_t want = 1 << 16;
+    for (int c = 2; c < NCLASS; ++c) want += per_root[c] * g->wcnt[c];
+    return (unsigned)(std::min<int64_t>(want, FRAME_CAP_MAX) / EMIT_RESERVE * EMIT_RESERVE);
+}
+
+// The walk of a class above 32 with a warp per root.  Global counts take the
+// narrowest bitset that holds the class's largest out-degree: a narrower
+// row is fewer words per pivot word loop and less shared memory per warp,
+// hence more resident warps.
+template <int MODE>
+static pvt_status launch_wide(pvt_dag *g, const CountArgs &A, int c, cudaStream_t s)
+{
+    constexpr bool SH = MODE == MODE_GLOBAL;
+    if constexpr (MODE == MODE_GLOBAL) {
+        const int words = (std::min(32 << (c - 1), (int)g->alpha) + 31) / 32;
+        if (c == 3 && words <= 3) return launch_class<3, MODE, SH>(g, A, c, s);
+        if (c == 4 && words <= 5) return launch_class<5, MODE, SH>(g, A, c, s);
+        if (c == 4 && words <= 6) return launch_class<6, MODE, SH>(g, A, c, s);
+        if (c == 5 && words <= 10) return launch_class<10, MODE, SH>(g, A, c, s);
+        if (c == 5 && words <= 12) return launch_class<12, MODE, SH>(g, A, c, s);
+        if (c == 6 && words <= 20) return launch_class<20, MODE, SH>(g, A, c, s);
+        if (c == 6 && words <= 24) return launch_class<24, MODE, SH>(g, A, c, s);
+    }
+    switch (c) {
+        case 2: return launch_class<2, MODE, SH>(g, A, c, s);
+        case 3: return launch_class<4, MODE, SH>(g, A, c, s);
+        case 4: return launch_class<8, MODE, SH>(g, A, c, s);
+        case 5: return launch_class<16, MODE, SH>(g, A, c, s);
+        default: return launch_class<32, MODE, SH>(g, A, c, s);
+    }
+}
+
+// The <= 32 class of a global count takes the two-phase form (gather, then
+// the lane walk) from this many roots on; below it the class is one short
+// launch (33 us for 2,000 roots) and a second kernel with its queue set-up
+// (about 25 us) would only add latency.
+constexpr int64_t GATHER1_MIN = 8192;
+// ... and in passes of at most this many roots (600 MB of frames)
+constexpr int64_t GATHER1_MAX = 1 << 22;
+
 template <int MODE>
 static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
 {
     // two-phase global counts: the classes above 32 emit their small labels
     // as frames into cframes (capacity from the number of heavy roots; a
-    // full buffer only sends frames back to in-place walking)
+    // full buffer only sends frames back to in-place walking), the <= 32
+    // class its roots into cframes1
     CountArgs A = A0;
+    pvt_status st = PVT_OK;
     int64_t heavy = 0;
     for (int c = 2; c < NCLASS; ++c) heavy += g->wcnt[c];
-    const bool frames = MODE == MODE_GLOBAL && g->policy.frames && g->policy.persistent && heavy > 0;
+    const bool two_phase = MODE == MODE_GLOBAL && g->policy.frames && g->policy.persistent;
+    const bool frames = two_phase && heavy > 0;
+    const bool gather1 = two_phase && g->policy.lanes && g->wcnt[1] >= GATHER1_MIN;
     if (frames) {
-        const unsigned cap = (unsigned)std::min<int64_t>(std::max<int64_t>(64 * heavy, 1 << 16), 1 << 22);
-        pvt_status st = grow(g->cframes, (size_t)cap * FRAME_WORDS, s);
+        unsigned cap = frame_cap(g);
+        while ((st = grow(g->cframes, (size_t)cap * FRAME_WORDS, s)) == PVT_ENOMEM && cap > FRAME_CAP_SMALL) {
+            (void)cudaGetLastError();  // scratch is short: a smaller buffer only walks more in place
+            cap = std::max(cap / 4, FRAME_CAP_SMALL);
+        }
         if (st != PVT_OK) return st;
         A.emit = g->cframes.p;
         A.emit_count = reinterpret_cast<unsigned long long *>(g->d_q + 8);  // words 8..9
         A.emit_cap = cap;
     }
+    const int64_t pass1 = std::min(g->wcnt[1], GATHER1_MAX);
+    unsigned slots1 = 0;
+    if (gather1) {
+        slots1 = gather1_slots(g, (unsigned)pass1);
+        if ((st = grow(g->cframes1, (size_t)slots1 * FRAME_WORDS, s)) != PVT_OK) return st;
+        A.emit1 = g->cframes1.p;
+        A.emit1_count = g->d_q + 10;
+    }
     // heavy classes on side streams so that they overlap the light ones (or
     // all on s, one after another, when the autotuner times them)
     const bool serial = g->serial || g->policy.serial;
     if (!serial) PVT_CK(cudaEventRecord(g->ev_fork, s));
-    pvt_status st = PVT_OK;
     for (int c = NCLASS - 1; c >= 1 && st == PVT_OK; --c) {
         cudaStream_t cs = serial ? s : g->side[c];
         if (!serial) PVT_CK(cudaStreamWaitEvent(cs, g->ev_fork, 0));
         switch (c) {
-            case 1: st = launch_class<1, MODE, MODE == MODE_GLOBAL>(g, A0, c, cs); break;
-            case 2: st = launch_class<2, MODE, MODE == MODE_GLOBAL>(g, A, c, cs); break;
-            case 4:
-            case 5:
-            case 6:
-                if (MODE == MODE_GLOBAL && g->policy.persistent && g->policy.cta[c]) {
-                    st = launch_cta_class(g, A, c, cs);
-                    break;
+            case 1:
+                if (gather1) {
+                    phase_begin(g, 1 + c, cs);
+                    st = launch_gather1(g, A, g->wroots + g->wstart[1], (unsigned)pass1, slots1, cs);
+                    phase_end(g, 1 + c, cs);
+                } else {
+                    st = launch_class<1, MODE, MODE == MODE_GLOBAL>(g, A0, c, cs);
                 }
-                if (c == 4) st = launch_class<8, MODE, MODE == MODE_GLOBAL>(g, A, c, cs);
-                else if (c == 5) st = launch_class<16, MODE, MODE == MODE_GLOBAL>(g, A, c, cs);
-                else st = launch_class<32, MODE, MODE == MODE_GLOBAL>(g, A, c, cs);
                 break;
-            case 3: st = launch_class<4, MODE, MODE == MODE_GLOBAL>(g, A, c, cs); break;
+            default:
+                if (MODE == MODE_GLOBAL && g->policy.persistent && g->policy.cta[c] && c >= 4)
+                    st = launch_cta_class(g, A, c, cs);
+                else
+                    st = launch_wide<MODE>(g, A, c, cs);
+                break;
         }
         if (!serial) PVT_CK(cudaEventRecord(g->ev_join[c], cs));
     }
     if (st != PVT_OK) return st;
-    if (frames) {
-        // the frame walk follows the heavy classes; the <= 32 class may
-        // still be running beside it
+    if (frames || gather1) {
+        // the frame walk follows the classes that emit; a <= 32 class that
+        // walks its own roots may still be running beside it
         if (!serial)
-            for (int c = NCLASS - 1; c >= 2; --c) PVT_CK(cudaStreamWaitEvent(s, g->ev_join[c], 0));
+            for (int c = NCLASS - 1; c >= (gather1 ? 1 : 2); --c) PVT_CK(cudaStreamWaitEvent(s, g->ev_join[c], 0));
+        A.emit1_cap = slots1;
         if ((st = launch_frames(g, A, s)) != PVT_OK) return st;
+    }
+    // the roots beyond the first pass of the gather
+    for (int64_t at = pass1; gather1 && at < g->wcnt[1]; at += pass1) {
+        const unsigned cnt = (unsigned)std::min(pass1, g->wcnt[1] - at);
+        CountArgs P = A;
+        P.emit = nullptr;
+        PVT_CK(cudaMemsetAsync(g->d_q + 1, 0, sizeof(unsigned), s));
+        PVT_CK(cudaMemsetAsync(g->d_q + 10, 0, sizeof(unsigned), s));
+        if ((st = launch_gather1(g, P, g->wroots + g->wstart[1] + at, cnt, slots1, s)) != PVT_OK) return st;
+        if ((st = launch_frames(g, P, s)) != PVT_OK) return st;
     }
     if (!serial)
         for (int c = NCLASS - 1; c >= 1; --c) PVT_CK(cudaStreamWaitEvent(s, g->ev_join[c], 0));
@@ -906,6 +989,7 @@ __global__ void __launch_bounds__(32 * warps_per_block<NW>()) k_count_noalloc(Co
     WarpWork<NW> *ww = reinterpret_cast<WarpWork<NW> *>(smem);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     WalkCounters wc;
+    Emitter em;
     for (;;) {
         unsigned qi = 0;
         if (lane == 0) qi = atomicAdd(A.qhead, 1u);
@@ -916,8 +1000,7 @@ __global__ void __launch_bounds__(32 * warps_per_block<NW>()) k_count_noalloc(Co
             if (lane == 0) atomicOr(A.err, DERR_RANGE);
             break;
         }
-        walk_root<NW, MODE_GLOBAL, false, false>(ww[wid], nullptr, A, lane, qi, wc);
-        wc.fold();
+        walk_root<NW, MODE_GLOBAL, false, false>(ww[wid], nullptr, A, lane, qi, wc, em);
         if (vload(A.err) & (DERR_STACK | DERR_RANGE)) break;
     }
     (void)WPB;

@@ -76,10 +76,12 @@ struct CtaLayout {
                sizeof(unsigned) * HIST_H * HIST_P + (size_t)dmax * RS * sizeof(uint32_t);
     }
     // per warp in global memory: the DFS stack of the root's level, then
-    // that of the mid level
+    // that of the mid level.  Rounded up to an even number of words: the
+    // blocks' gather scratch follows the stacks of all warps and holds 8-byte
+    // entries, whatever the product of blocks and warps.
     __host__ __device__ static size_t stack_words(int dmax)
     {
-        return (size_t)(dmax + 1) * (NW + 1) + (size_t)(MID_D + 1) * (MID_NW + 1);
+        return ((size_t)(dmax + 1) * (NW + 1) + (size_t)(MID_D + 1) * (MID_NW + 1) + 1) / 2 * 2;
     }
     // global scratch of a block's gather: member ids, prefix offsets (dmax + 2
     // words) and out-list starts (dmax 8-byte words)
@@ -92,35 +94,9 @@ struct LaneState {
     int h = 0, p = 0;
     bool has = false;
     unsigned top = 0, bot = 0;
+    unsigned cls = 0;  // unused here: every subtree is of the launch's class
     __device__ __forceinline__ bool free_() const { return !has && top == bot; }
 };
-
-// The subtree of a label of at most two members in closed form (the cases
-// of close_small in walk.cuh), tallied in the block's 32-bit histogram.
-// UNIFORM: every lane calls with the same arguments, lane 0 tallies.
-template <bool UNIFORM>
-__device__ __forceinline__ void cta_close_small(unsigned *sh32, const CountArgs &A, int lane, int cs, bool adjacent,
-                                                int h, int p, unsigned wpm, WalkCounters &wc)
-{
-    const bool split = cs == 2 && !adjacent;
-    const bool hold = split && h + 1 <= A.kmax;
-    if (UNIFORM) {
-        wc.nodes += 1 + split + hold;
-        wc.leaves += 1 + hold;
-        wc.words += (unsigned long long)cs * wpm;
-    } else {
-        wc.xnodes += 1u + split + hold;
-        wc.xleaves += 1u + hold;
-        wc.xwords += (unsigned)cs * wpm;
-    }
-    if (UNIFORM && lane != 0) return;
-    if (!split) {
-        lane_tally(sh32, A, h, p + cs);
-        return;
-    }
-    lane_tally(sh32, A, h, p + 1);  // the pivot leaf below the pair
-    if (hold) lane_tally(sh32, A, h + 1, p);
-}
 
 // Run the warp's lane batch: at most `budget` node steps, stopping early
 // once `stop_free` lanes are free (0: only when every lane is idle).
@@ -131,7 +107,7 @@ __device__ inline void lane_run(LaneWork &L, unsigned *sh32, const CountArgs &A,
         const unsigned freeM = __ballot_sync(FULL, ls.free_());
         if (freeM == FULL) return;
         if (stop_free && __popc(freeM) >= stop_free) return;
-        if (freeM) lane_steal(L, lane, freeM, ls.S, ls.h, ls.p, ls.has, ls.top, ls.bot);
+        if (freeM) lane_steal(L, lane, freeM, ls.S, ls.h, ls.p, ls.has, ls.top, ls.bot, ls.cls);
         if (!ls.has && ls.top != ls.bot) {
             --ls.top;
             ls.S = L.stkS[ls.top & (LSTK - 1)][lane];
@@ -143,33 +119,6 @@ __device__ inline void lane_run(LaneWork &L, unsigned *sh32, const CountArgs &A,
         if (ls.has) lane_node(L, sh32, A, lane, ls.S, ls.h, ls.p, ls.has, ls.top, ls.bot, lc);
         __syncwarp();
     }
-}
-
-// Relabel the warp's current label (wS: NW-word bitset over the root's
-// members, s <= 32 of them): member k of the label = its k-th member in
-// ascending order; lane k returns row k of the one-word adjacency (the
-// ballot over lanes j of "member k is adjacent to member j").
-template <int NW, int RS>
-__device__ __forceinline__ uint32_t relabel_small(const uint32_t *adj, const uint32_t *wS, uint32_t *wM, int lane,
-                                                  int s)
-{
-    int before = 0;
-    for (int w = 0; w < NW; ++w) {
-        const uint32_t sw = wS[w];
-        if ((sw >> lane) & 1u) wM[before + __popc(sw & ((1u << lane) - 1u))] = (uint32_t)(w * 32 + lane);
-        before += __popc(sw);
-    }
-    __syncwarp();
-    const uint32_t mj = lane < s ? wM[lane] : 0u;
-    uint32_t mine = 0;
-    for (int k = 0; k < s; ++k) {
-        const uint32_t mk = __shfl_sync(FULL, mj, k);
-        const bool bit = lane < s && ((adj[mj * RS + (mk >> 5)] >> (mk & 31)) & 1u);
-        const uint32_t row = __ballot_sync(FULL, bit);
-        if (lane == k) mine = row;
-    }
-    __syncwarp();
-    return mine;
 }
 
 // A relabelled small label into a free lane of the warp's own batch (run
@@ -215,15 +164,25 @@ __device__ __forceinline__ void cta_unlock(int *lk)
     atomicExch(lk, 0);
 }
 
-// A small label (s <= 32 members) found by a wide walk: relabelled into the
-// block's ring, from which any warp with free lanes takes it; into the
-// warp's own batch when the ring is full.
+// A small label (s <= 32 members) found by a wide walk: relabelled and, in
+// the two-phase form, emitted as a frame of the frame walk while its buffer
+// has room; else into the block's ring, from which any warp with free lanes
+// takes it; into the warp's own batch when the ring is full.
 template <int NW, int LNW, int RS>
 __device__ __forceinline__ void cta_push_small(CtaQueue<NW> &Q, LaneWork &L, unsigned *sh32, const CountArgs &A,
                                                int lane, int wid, LaneState &ls, LaneCounters &lc,
-                                               const uint32_t *adj, int s, int h, int p)
+                                               const uint32_t *adj, int s, int h, int p, Emitter &em)
 {
-    const uint32_t row = relabel_small<LNW, RS>(adj, Q.wS[wid], Q.wM[wid], lane, s);
+    const uint32_t row =
+        relabel_rows<LNW, RS>(adj, Q.wM[wid], lane, lane < LNW ? Q.wS[wid][lane] : 0u, s);
+    if (A.emit) {
+        ++em.met;
+        uint32_t *fr = em.next(A, lane);
+        if (fr) {
+            frame_write(fr, A, lane, row, s, h, p);
+            return;
+        }
+    }
     int t = -1;
     if (lane == 0 && *(volatile int *)&Q.ctail - *(volatile int *)&Q.chead < CTA_CQCAP && cta_lock(&Q.lock, A.err)) {
         if (Q.ctail - Q.chead < CTA_CQCAP) t = Q.ctail++;
@@ -303,7 +262,7 @@ template <int NW, int LNW, int RS, bool TOP>
 __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork &L, unsigned *sh32,
                                           const CountArgs &A, int lane, int wid, LaneState &ls, LaneCounters &lc,
                                           WalkCounters &wc, const uint32_t *rows, uint32_t *stk, uint32_t *mstk,
-                                          uint32_t (&S)[LNW], int h, int p, int cap)
+                                          uint32_t (&S)[LNW], int h, int p, int cap, Emitter &em)
 {
     constexpr int FW = LNW + 1;  // stack frame words: S, then (h << 16) | p
     uint32_t *wS = Q.wS[wid], *wR = Q.wR[wid];
@@ -321,7 +280,7 @@ __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork
         __syncwarp();
         bool closed = true;
         if (s <= 32) {
-            cta_push_small<NW, LNW, RS>(Q, L, sh32, A, lane, wid, ls, lc, rows, s, h, p);
+            cta_push_small<NW, LNW, RS>(Q, L, sh32, A, lane, wid, ls, lc, rows, s, h, p, em);
         } else if (TOP && LNW > MID_NW && s <= MID_D && A.kmax - h >= CTA_MID_DEPTH) {
             // relabel the members to 0..s-1 and walk the label over MID_NW-word rows
             int before = 0;
@@ -353,7 +312,7 @@ __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork
                 M[q] = bits >= 32 ? FULL : (bits <= 0 ? 0u : ((1u << bits) - 1u));
             }
             cta_level<NW, MID_NW, MID_RS, false>(Q, CW, L, sh32, A, lane, wid, ls, lc, wc, CW.mid, mstk, nullptr, M,
-                                                 h, p, MID_D);
+                                                 h, p, MID_D, em);
         } else {
             wc.nodes++;
             ++clock;
@@ -375,7 +334,7 @@ __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork
             const int piv = 1023 - (int)(best & 1023u);
             if (dsum == (uint32_t)s * (uint32_t)(s - 1)) {
                 wc.leaves++;
-                if (lane == 0) lane_tally(sh32, A, h, p + s);
+                if (lane == 0) tally_n<true>(sh32, A, h, p + s, 1u);
             } else {
                 const uint32_t *prow = rows + piv * RS;
                 uint32_t R[LNW];
@@ -407,13 +366,15 @@ __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork
                     // hold child of member j*32+lane: N(S, v) minus the earlier
                     // members of R; labels of at most two members close here
                     int before = 0;
+                    SmallCounts small;
                     for (int j = 0; j < LNW; ++j) {
                         const uint32_t Rj = wR[j];
                         const bool inR = (Rj >> lane) & 1u;
                         bool push = inR;
                         const uint32_t *row = rows + (j * 32 + lane) * RS;
+                        int cs = 0;
                         if (inR) {
-                            int cs = 0, a = 0, b = 0;
+                            int a = 0, b = 0;
 #pragma unroll
                             for (int w = 0; w < LNW; ++w) {
                                 const uint32_t bl = w < j ? R[w] : (w == j ? (Rj & low) : 0u);
@@ -426,8 +387,27 @@ __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork
                             }
                             if (cs <= 2) {
                                 const bool adjp = cs == 2 && ((rows[a * RS + (b >> 5)] >> (b & 31)) & 1u);
-                                cta_close_small<false>(sh32, A, lane, cs, adjp, h + 1, p, 1u, wc);
+                                small.add(cs, adjp);
                                 push = false;
+                            }
+                        }
+                        if (A.emit) {
+                            // labels of at most 32 members leave at once, without
+                            // a trip through the stack
+                            for (unsigned eb = __ballot_sync(FULL, push && cs <= 32); eb; eb &= eb - 1) {
+                                uint32_t *fr = em.next(A, lane);
+                                if (!fr) break;  // full: pushed below
+                                const int v = __ffs(eb) - 1;  // member j * 32 + v
+                                uint32_t cw = 0;
+                                if (lane < LNW) {
+                                    const uint32_t bl = lane < j ? wR[lane] : (lane == j ? Rj & ((1u << v) - 1u) : 0u);
+                                    cw = rows[(j * 32 + v) * RS + lane] & wS[lane] & ~bl;
+                                }
+                                int es = 0;
+                                const uint32_t r1 = relabel_rows<LNW, RS>(rows, Q.wM[wid], lane, cw, es);
+                                frame_write(fr, A, lane, r1, es, h + 1, p);
+                                ++em.met;
+                                if (lane == v) push = false;
                             }
                         }
                         const uint32_t pushed = __ballot_sync(FULL, push);
@@ -443,19 +423,24 @@ __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork
                         before += __popc(pushed);
                     }
                     top += before;
+                    small.close<true>(sh32, A, lane, h + 1, p, wc.nodes, wc.leaves, wc.words);
                     __syncwarp();
                     if (TOP && clock >= CTA_DONATE_EVERY) {
                         clock = 0;
-                        // a warp of the block is not walking a wide subtree: hand
-                        // it our oldest pending one (the largest), if there is room
+                        // warps of the block are not walking a wide subtree: hand
+                        // them our oldest pending ones (the largest), two for
+                        // each such warp while there is room.  One at a time
+                        // would leave most of the block waiting while the warp
+                        // that expanded the root deals out its children.
                         int give = 0;
                         if (lane == 0 && top - bot >= 2 && *(volatile int *)&Q.busy < warps &&
                             *(volatile int *)&Q.tail - *(volatile int *)&Q.head < CTA_QCAP) {
                             int sz = 0;
                             for (int w = 0; w < LNW; ++w) sz += __popc(stk[bot * FW + w]);
                             if (sz >= DONATE_MIN_WIDE && cta_lock(&Q.lock, A.err)) {
-                                give = 1;
-                                if (Q.tail - Q.head >= CTA_QCAP) {
+                                give = min(min(top - bot - 1, 2 * (warps - *(volatile int *)&Q.busy)),
+                                           CTA_QCAP - (Q.tail - Q.head));
+                                if (give <= 0) {
                                     cta_unlock(&Q.lock);
                                     give = 0;
                                 }
@@ -463,16 +448,20 @@ __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork
                         }
                         give = __shfl_sync(FULL, give, 0);
                         if (give) {
-                            const int slot = Q.tail % CTA_QCAP;
-                            if (lane < LNW) Q.S[slot][lane] = stk[bot * FW + lane];
-                            if (lane == 0) Q.hp[slot] = stk[bot * FW + LNW];
+                            const int at = *(volatile int *)&Q.tail;
+                            for (int t = lane; t < give * FW; t += 32) {
+                                const int f = t / FW, w = t % FW, slot = (at + f) % CTA_QCAP;
+                                const uint32_t x = stk[(bot + f) * FW + w];
+                                if (w < LNW) Q.S[slot][w] = x;
+                                else Q.hp[slot] = x;
+                            }
                             __syncwarp();
                             if (lane == 0) {
-                                Q.tail += 1;
+                                Q.tail += give;
                                 Q.progress += 1;
                                 cta_unlock(&Q.lock);
                             }
-                            ++bot;
+                            bot += give;
                         }
                     }
                 }
@@ -490,7 +479,7 @@ __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork
                 }
                 if (ps <= 2) {
                     const bool adjp = ps == 2 && ((rows[a * RS + (b >> 5)] >> (b & 31)) & 1u);
-                    cta_close_small<true>(sh32, A, lane, ps, adjp, h, p + 1, 1u, wc);
+                    close_small<true>(sh32, A, lane, ps, adjp, h, p + 1, wc.nodes, wc.leaves, wc.words);
                 } else {
                     closed = false;
 #pragma unroll
@@ -517,7 +506,7 @@ __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork
 template <int NW>
 __device__ __forceinline__ void cta_dfs(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork &L, unsigned *sh32,
                                         const CountArgs &A, int lane, int wid, LaneState &ls, LaneCounters &lc,
-                                        WalkCounters &wc, const uint32_t *adj, uint32_t *gstk, int qs, int d)
+                                        WalkCounters &wc, const uint32_t *adj, uint32_t *gstk, int qs, int d, Emitter &em)
 {
     uint32_t S[NW];
 #pragma unroll
@@ -530,7 +519,7 @@ __device__ __forceinline__ void cta_dfs(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork &
     }
     uint32_t *mstk = gstk + (size_t)(d + 1) * (NW + 1);
     cta_level<NW, NW, CtaLayout<NW>::RS, true>(Q, CW, L, sh32, A, lane, wid, ls, lc, wc, adj, gstk, mstk, S,
-                                               (int)(hp0 >> 16), (int)(hp0 & 0xFFFFu), d);
+                                               (int)(hp0 >> 16), (int)(hp0 & 0xFFFFu), d, em);
 }
 
 // The block's rows for root r (all threads): member ids, their out-list
@@ -647,6 +636,7 @@ __global__ void __launch_bounds__(32 * CTA_MAXW, 1) k_cta(CountArgs A, int dmax)
     LaneState ls;
     LaneCounters lc;
     WalkCounters wc;
+    Emitter em;
     for (int i = threadIdx.x; i < HIST_H * HIST_P; i += blockDim.x) sh32[i] = 0;
     for (int i = threadIdx.x; i < CTA_CQCAP; i += blockDim.x) Q.cseq[i] = 0;
     if (threadIdx.x == 0) {
@@ -706,8 +696,7 @@ __global__ void __launch_bounds__(32 * CTA_MAXW, 1) k_cta(CountArgs A, int dmax)
             took = __shfl_sync(FULL, took, 0);
             if (took < 0) break;
             if (took > 0) {
-                cta_dfs<NW>(Q, cw[wid], L, sh32, A, lane, wid, ls, lc, wc, adj, gstk, took - 1, d);
-                wc.fold();
+                cta_dfs<NW>(Q, cw[wid], L, sh32, A, lane, wid, ls, lc, wc, adj, gstk, took - 1, d, em);
                 __syncwarp();
                 if (lane == 0) {
                     atomicSub(&Q.busy, 1);
@@ -751,8 +740,9 @@ __global__ void __launch_bounds__(32 * CTA_MAXW, 1) k_cta(CountArgs A, int dmax)
         __syncthreads();
     }
     wc.flush(A.stats, A.cls, lane);
+    em.finish(A, lane);
     lc.flush(A.stats, A.cls, lane);
-    lane_hist_flush(sh32, A);
+    hist_flush(sh32, A);
 }
 
 }  // namespace pvt

@@ -41,16 +41,19 @@ struct LaneWork {
 };
 
 // Per-lane walk statistics (each lane its own subtrees; summed at the end).
+// words1: the share of words that belongs to roots of the <= 32 class.
 struct LaneCounters {
-    unsigned long long nodes = 0, leaves = 0, words = 0;
+    unsigned long long nodes = 0, leaves = 0, words = 0, words1 = 0;
     __device__ __forceinline__ void flush(unsigned long long *stats, int slot, int lane)
     {
         const unsigned long long n = warp_sum64(nodes), l = warp_sum64(leaves), w = warp_sum64(words);
+        const unsigned long long w1 = warp_sum64(words1);
         if (lane == 0 && n) {
             atomicAdd(&stats[0], n);
             atomicAdd(&stats[1], l);
             atomicAdd(&stats[2], w);
-            if (slot >= 0) atomicAdd(&stats[3 + slot], w);
+            if (slot >= 0) atomicAdd(&stats[3 + slot], w - w1);
+            if (w1) atomicAdd(&stats[3 + 1], w1);
         }
     }
     __device__ __forceinline__ static unsigned long long warp_sum64(unsigned long long x)
@@ -60,32 +63,6 @@ struct LaneCounters {
         return x;
     }
 };
-
-// Leaf tally of one lane.  Leaves with h < HIST_H and p < HIST_P go to the
-// block's 32-bit histogram in shared memory (native 32-bit shared atomics,
-// which 32 lanes tallying at once need); an increment that wraps a counter
-// adds 2^32 to the 64-bit histogram in global memory, so the sum of the two
-// is exact at any count.  lane_hist_flush adds what is left at the end.
-__device__ __forceinline__ void lane_tally(unsigned *sh32, const CountArgs &A, int h, int p)
-{
-    if (h < HIST_H && p < HIST_P) {
-        const unsigned old = atomicAdd(&sh32[h * HIST_P + p], 1u);
-        if (old == 0xFFFFFFFFu) atomicAdd(&A.hist[(size_t)h * A.hstride + p], 1ull << 32);
-    } else {
-        atomicAdd(&A.hist[(size_t)h * A.hstride + p], 1ull);
-    }
-}
-
-// The block's 32-bit histogram into the global one (all threads of the block,
-// after the last tally).
-__device__ __forceinline__ void lane_hist_flush(unsigned *sh32, const CountArgs &A)
-{
-    __syncthreads();
-    for (int i = threadIdx.x; i < HIST_H * HIST_P; i += blockDim.x) {
-        const unsigned x = sh32[i];
-        if (x) atomicAdd(&A.hist[(size_t)(i / HIST_P) * A.hstride + (i % HIST_P)], (unsigned long long)x);
-    }
-}
 
 // Subtree of a label of at most two members in closed form, by one lane
 // (the cases of close_small in walk.cuh).
@@ -98,11 +75,11 @@ __device__ __forceinline__ void lane_close_small(unsigned *sh32, const CountArgs
     lc.leaves += 1 + hold;
     lc.words += (unsigned)cs;
     if (!split) {
-        lane_tally(sh32, A, h, p + cs);
+        tally_n<true>(sh32, A, h, p + cs, 1u);
         return;
     }
-    lane_tally(sh32, A, h, p + 1);  // the pivot leaf below the pair
-    if (hold) lane_tally(sh32, A, h + 1, p);
+    tally_n<true>(sh32, A, h, p + 1, 1u);  // the pivot leaf below the pair
+    if (hold) tally_n<true>(sh32, A, h + 1, p, 1u);
 }
 
 // One node of the lane's current subtree: label S reached with (h, p).
@@ -116,7 +93,7 @@ __device__ __forceinline__ void lane_node(LaneWork &L, unsigned *sh32, const Cou
     ++lc.nodes;
     if (s == 0) {
         ++lc.leaves;
-        lane_tally(sh32, A, h, p);
+        tally_n<true>(sh32, A, h, p, 1u);
         has = false;
         return;
     }
@@ -141,7 +118,7 @@ __device__ __forceinline__ void lane_node(LaneWork &L, unsigned *sh32, const Cou
     lc.words += (unsigned)s;
     if (dsum == (uint32_t)s * (uint32_t)(s - 1)) {
         ++lc.leaves;
-        lane_tally(sh32, A, h, p + s);
+        tally_n<true>(sh32, A, h, p + s, 1u);
         has = false;
         return;
     }
@@ -184,7 +161,7 @@ __device__ __forceinline__ void lane_node(LaneWork &L, unsigned *sh32, const Cou
 // busy lane (one that keeps work), with that lane's rows.  Returns the
 // lanes that received one.
 __device__ __forceinline__ unsigned lane_steal(LaneWork &L, int lane, unsigned freeM, uint32_t &S, int &h, int &p,
-                                               bool &has, unsigned top, unsigned &bot)
+                                               bool &has, unsigned top, unsigned &bot, unsigned &cls)
 {
     const unsigned pend = top - bot;
     const unsigned donors = __ballot_sync(FULL, pend >= 2 || (pend == 1 && has));
@@ -203,6 +180,7 @@ __device__ __forceinline__ unsigned lane_steal(LaneWork &L, int lane, unsigned f
         }
     }
     const unsigned sbot = __shfl_sync(FULL, bot, src);
+    cls = __shfl_sync(FULL, cls, src);  // src is the lane itself where nothing is received
     if (recv) {
         S = L.stkS[sbot & (LSTK - 1)][src];
         const uint32_t hp = L.stkHP[sbot & (LSTK - 1)][src];
@@ -220,9 +198,10 @@ __device__ __forceinline__ unsigned lane_steal(LaneWork &L, int lane, unsigned f
 
 // Lane j takes frame `item` of the emitted buffer: its 32 rows into column j
 // with eight 16-byte loads (every lane its own frame, so the warp's stores
-// hit 32 distinct banks), its label and (h, p).
-__device__ __forceinline__ void lane_load_frame(LaneWork &L, const uint32_t *fr, int lane, uint32_t &S, int &h,
-                                                int &p)
+// hit 32 distinct banks), its label, (h, p) and root class.  False for a
+// slot that holds no subtree.
+__device__ __forceinline__ bool lane_load_frame(LaneWork &L, const uint32_t *fr, int lane, uint32_t &S, int &h,
+                                                int &p, unsigned &cls)
 {
     const uint4 *v = reinterpret_cast<const uint4 *>(fr + 4);
 #pragma unroll
@@ -237,18 +216,25 @@ __device__ __forceinline__ void lane_load_frame(LaneWork &L, const uint32_t *fr,
     S = head.z;
     h = (int)(head.y >> 16);
     p = (int)(head.y & 0xFFFFu);
+    cls = head.w;
+    return head.x == FRAME_COMPACT;
 }
 
 constexpr unsigned LANE_CLAIM = 32;  // source items a warp claims at once
 
-// The lane walk over the first `nitems` emitted frames (A.emit).  A warp
-// claims LANE_CLAIM frames at a time through qctl[Q_ROOT] and hands them to
+// The lane walk over the first `nwide` frames of A.emit, then those of
+// A.emit1 up to `nitems` in all.  A warp claims LANE_CLAIM frames at a time through qctl[Q_ROOT] and hands them to
 // its free lanes; qctl[Q_OUT] counts items not yet finished (a warp
 // returns its items once every lane is idle), and warps that run dry wait on
 // the ring queue for donated frames until it drops to zero (walk.cuh:
 // queue_take).
-__device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A, int lane, unsigned nitems, int slot)
+__device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A, int lane, unsigned nwide,
+                                 unsigned nitems, int slot)
 {
+    auto frame_of = [&](unsigned i) {
+        return i < nwide ? A.emit + (size_t)i * FRAME_WORDS : A.emit1 + (size_t)(i - nwide) * FRAME_WORDS;
+    };
+    unsigned cls = 0;            // out-degree class of the root whose rows the lane holds
     LaneCounters lc;
     uint32_t S = 0;
     int h = 0, p = 0;
@@ -272,7 +258,7 @@ __device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A
                     end = min(base + LANE_CLAIM, nitems);
                     if (lane < (int)(end - cur)) {
                         // the claimed frames into L2 ahead of their lanes
-                        const char *a = reinterpret_cast<const char *>(A.emit + (size_t)(cur + lane) * FRAME_WORDS);
+                        const char *a = reinterpret_cast<const char *>(frame_of(cur + lane));
                         asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
                         asm volatile("prefetch.global.L2 [%0];" ::"l"(a + 128));
                     }
@@ -283,8 +269,7 @@ __device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A
                 const unsigned got = min((unsigned)__popc(freeM), end - cur);
                 const unsigned rank = (unsigned)__popc(freeM & ((1u << lane) - 1u));
                 if (((freeM >> lane) & 1u) && rank < got) {
-                    lane_load_frame(L, A.emit + (size_t)(cur + rank) * FRAME_WORDS, lane, S, h, p);
-                    has = true;
+                    has = lane_load_frame(L, frame_of(cur + rank), lane, S, h, p, cls);
                 }
                 cur += got;
                 held += got;
@@ -293,7 +278,7 @@ __device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A
             }
         }
         if (freeM && src_done) {
-            lane_steal(L, lane, freeM, S, h, p, has, top, bot);
+            lane_steal(L, lane, freeM, S, h, p, has, top, bot, cls);
             freeM = __ballot_sync(FULL, !has && top == bot);
             if (freeM == FULL) {
                 // every lane idle: return this warp's items, then wait for a
@@ -309,6 +294,7 @@ __device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A
                 if (lane == 0) {
                     const uint32_t hp = __ldcg(fr + 1);
                     S = __ldcg(fr + 2);
+                    cls = __ldcg(fr + 3);
                     h = (int)(hp >> 16);
                     p = (int)(hp & 0xFFFFu);
                     for (int v2 = 0; v2 < 32; ++v2) L.rows[v2][0] = __ldcg(fr + 4 + v2);
@@ -330,7 +316,11 @@ __device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A
             p = (int)(hp & 0xFFFFu);
             has = true;
         }
-        if (has) lane_node(L, sh32, A, lane, S, h, p, has, top, bot, lc);
+        if (has) {
+            const unsigned long long w = lc.words;
+            lane_node(L, sh32, A, lane, S, h, p, has, top, bot, lc);
+            if (cls == 1) lc.words1 += lc.words - w;
+        }
         __syncwarp();
         if (++steps % LANE_DONATE_EVERY == 0) {
             // warps wait on the ring: donate, for up to LANE_DONATE_MAX of
@@ -353,7 +343,7 @@ __device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A
                     fr[0] = FRAME_COMPACT;
                     fr[1] = L.stkHP[bot & (LSTK - 1)][lane];
                     fr[2] = L.stkS[bot & (LSTK - 1)][lane];
-                    fr[3] = (uint32_t)A.cls;
+                    fr[3] = cls;
                     ++bot;
                 }
                 frame_publish(A, lane, t);

@@ -83,6 +83,7 @@ struct pvt_dag {
     bool profiling = false;
     pvt_policy policy = {1, 4, {0, 0, 1, 1, 1, 1, 1}, 0, 1, 0, 1, {0, 0, 0, 0, 0, 1, 1}, 0};
     pvt::DevBuf<uint32_t> cframes;  // compacted frames emitted by the wide walks
+    pvt::DevBuf<uint32_t> cframes1;  // frames of the <= 32 class (its gather)
     bool serial = false;           // launch the classes one after another on the caller's stream
     bool capturing = false;        // recording a CUDA graph: no phase events
     cudaGraphExec_t graph_exec = nullptr;  // recorded global count (policy.graph)

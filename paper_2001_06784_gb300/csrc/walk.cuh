@@ -42,10 +42,10 @@ enum Mode { MODE_GLOBAL = 0, MODE_VERTEX = 1, MODE_EDGE = 2 };
 template <int NW>
 struct WarpWork {
     static constexpr int D = 32 * NW;                // largest out-degree handled
-    static constexpr int RS = NW == 1 ? 1 : NW + 1;  // odd row stride: no bank conflicts
+    static constexpr int RS = (NW & 1) ? NW : NW + 1;  // odd row stride: no bank conflicts
     // wide classes keep their (worst case d+1 frames) DFS stack in per-warp
     // global memory, which leaves room for more resident warps
-    static constexpr bool GSTACK = NW >= 8;
+    static constexpr bool GSTACK = NW > 4;
     int64_t rs[D];               // start of N+(member) in ocol
     uint32_t ids[D];             // member vertex ids (ascending)
     uint32_t off[D + 1];         // prefix sums of |N+(member)|
@@ -54,7 +54,6 @@ struct WarpWork {
     uint32_t *gstk;              // this warp's (D+1)*NW-word stack (GSTACK)
     uint32_t *etab;              // per-edge counts: this warp's D x D edge ids of member pairs
                                  // (written by the gather; null: search the out-lists)
-    uint32_t hp[D + 1];          // DFS stack: (h << 16) | p
     // local counts only (point into a shared-memory region of LOCAL_BYTES):
     uint16_t *lk;                // DFS stack: link into the frame
     uint16_t *path;              // link label at each depth of the current path
@@ -68,13 +67,25 @@ struct WarpWork {
         memH = path + (D + 2);
         memP = memH + (D + 2);
     }
-    uint2 cstk[33];              // one-word walk of a compacted subtree: (S, (h << 16) | p)
+    static constexpr int FILTER_LOG = NW <= 4 ? 12 : 13;  // log2 of the filter's bits
+    union {
+        struct {  // gather: bit filter of the member ids, and entries that passed it
+            uint32_t filter[(1 << FILTER_LOG) / 32];
+            uint2 hits[64];
+        };
+        struct {  // walk
+            uint2 cstk[33];      // one-word walk of a compacted subtree: (S, (h << 16) | p)
+            uint32_t hp[D + 1];  // DFS stack: (h << 16) | p
+        };
+    };
     uint16_t cmap[32];           // compacted index -> member index
     uint32_t fbuf[36];           // copy of a donated frame taken from the queue
     __device__ __forceinline__ uint32_t *stk() { return GSTACK ? gstk : stk_s; }
 };
 
 constexpr uint16_t LINK_PIVOT = 0x8000u;
+// 2^32 / golden ratio: multiplicative (Fibonacci) hashing of vertex ids, Knuth, TAOCP 3, 6.4
+constexpr uint32_t FIB_HASH = 0x9E3779B1u;
 
 // --------------------------------------------------- multi-word atomics
 
@@ -149,9 +160,14 @@ struct CountArgs {
     // two-phase global counts: the wide walk emits every compacted subtree
     // as a frame (layout below) for k_walk_frames; null: walk them in place
     uint32_t *emit;             // [emit_cap][FRAME_WORDS]
-    unsigned long long *emit_count;  // compacted subtrees met so far (passes emit_cap once the
-                                     // buffer is full; 64-bit: long walks meet billions)
-    unsigned emit_cap;
+    unsigned long long *emit_count;  // slots reserved so far (passes emit_cap once the buffer is
+                                     // full; slots without a subtree are marked FRAME_NONE)
+    unsigned emit_cap;               // a multiple of EMIT_RESERVE
+    // two-phase <= 32 class: the frames its gather emits (emit1_count of
+    // emit1_cap slots reserved, empty ones marked kind 0; null: none)
+    uint32_t *emit1;
+    unsigned *emit1_count;
+    unsigned emit1_cap;
     // bounded waits: an idle warp gives up after idle_ns without progress, a
     // donor after slot_ns for a ring slot (policy.wait_limit_us overrides both)
     unsigned long long idle_ns = SPLIT_IDLE_LIMIT_NS, slot_ns = SPLIT_SLOT_LIMIT_NS;
@@ -171,32 +187,20 @@ constexpr int Q_HEAD = 0, Q_TAIL = 32, Q_OUT = 64, Q_ROOT = 96, QCTL_WORDS = 128
 // compacted (2): [1] (h<<16)|p, [2] S, [3] out-degree class of the root,
 // [4..36) the 32 one-word rows.
 constexpr int FRAME_WORDS = 36;
-constexpr uint32_t FRAME_WIDE = 1u, FRAME_COMPACT = 2u;
+// Kind FRAME_NONE marks a reserved slot that holds no subtree.
+constexpr uint32_t FRAME_NONE = 0u, FRAME_WIDE = 1u, FRAME_COMPACT = 2u;
 
 // Block-level (h, p) leaf histogram in shared memory for h < HIST_H, p < HIST_P
 // (where almost every leaf falls); other leaves go straight to the global one.
 constexpr int HIST_H = 32, HIST_P = 48;
 
-// Walk statistics.  nodes / leaves / words advance in step on every lane of
-// the warp; the x* fields count, per lane, the small subtrees that lane
-// closed in closed form (close_small), as the nodes, leaves and pivot words
-// the walk would have spent on them, until fold() adds their warp sums in.
+// Walk statistics, the same on every lane of the warp.
 struct WalkCounters {
     unsigned long long nodes = 0, leaves = 0, words = 0;
-    unsigned xnodes = 0, xleaves = 0, xwords = 0;
-    // after every walk item (all lanes)
-    __device__ __forceinline__ void fold()
-    {
-        nodes += __reduce_add_sync(0xFFFFFFFFu, xnodes);
-        leaves += __reduce_add_sync(0xFFFFFFFFu, xleaves);
-        words += __reduce_add_sync(0xFFFFFFFFu, xwords);
-        xnodes = xleaves = xwords = 0;
-    }
     // add the warp's totals to stats[0..2] and, if cls >= 0, to stats[3 + cls]
     // (all lanes)
     __device__ __forceinline__ void flush(unsigned long long *stats, int cls, int lane)
     {
-        fold();
         if (lane == 0 && nodes) {
             atomicAdd(&stats[0], nodes);
             atomicAdd(&stats[1], leaves);
@@ -206,51 +210,76 @@ struct WalkCounters {
     }
 };
 
+// n leaves (h, p), by one lane.  The block's histogram is 32-bit (native
+// shared atomics); an addition that wraps a counter adds 2^32 to the 64-bit
+// histogram in global memory, so the sum of the two is exact at any count.
 template <bool SHIST>
-__device__ __forceinline__ void tally_leaf(unsigned long long *shist, const CountArgs &A, int lane, int h, int p)
+__device__ __forceinline__ void tally_n(unsigned *shist, const CountArgs &A, int h, int p, unsigned n)
 {
-    if (lane == 0) {
-        if (SHIST && h < HIST_H && p < HIST_P) atomicAdd(&shist[h * HIST_P + p], 1ull);
-        else atomicAdd(&A.hist[(size_t)h * A.hstride + p], 1ull);
-    }
-}
-
-// Leaf tally by the calling lane alone (lanes tally independently).
-template <bool SHIST>
-__device__ __forceinline__ void tally_lane(unsigned long long *shist, const CountArgs &A, int h, int p)
-{
-    if (SHIST && h < HIST_H && p < HIST_P) atomicAdd(&shist[h * HIST_P + p], 1ull);
-    else atomicAdd(&A.hist[(size_t)h * A.hstride + p], 1ull);
-}
-
-// The subtree of a node with label S' of at most two members, reached with
-// (h, p), in closed form (global counts): |S'| = 0 is a leaf (h, p); a
-// single member or an adjacent pair is a clique, one leaf (h, p + |S'|); a
-// non-adjacent pair {a < b} takes a as pivot (a pivot leaf (h, p + 1)) and
-// holds b (a leaf (h + 1, p), cut when h + 1 > kmax).  Counts the nodes,
-// leaves and pivot words (wpm per member: 1, a label of at most two members
-// fits one word) the walk would have spent.
-// UNIFORM: every lane calls with the same arguments, lane 0 tallies.
-template <bool SHIST, bool UNIFORM>
-__device__ __forceinline__ void close_small(unsigned long long *shist, const CountArgs &A, int lane, int cs,
-                                            bool adjacent, int h, int p, unsigned wpm, WalkCounters &wc)
-{
-    if (UNIFORM) {
-        wc.nodes += 1 + (cs == 2 && !adjacent) + (cs == 2 && !adjacent && h + 1 <= A.kmax);
-        wc.leaves += 1 + (cs == 2 && !adjacent && h + 1 <= A.kmax);
-        wc.words += (unsigned long long)cs * wpm;
+    if (SHIST && h < HIST_H && p < HIST_P) {
+        const unsigned old = atomicAdd(&shist[h * HIST_P + p], n);
+        if (old + n < old) atomicAdd(&A.hist[(size_t)h * A.hstride + p], 1ull << 32);
     } else {
-        wc.xnodes += 1u + (cs == 2 && !adjacent) + (cs == 2 && !adjacent && h + 1 <= A.kmax);
-        wc.xleaves += 1u + (cs == 2 && !adjacent && h + 1 <= A.kmax);
-        wc.xwords += (unsigned)cs * wpm;
+        atomicAdd(&A.hist[(size_t)h * A.hstride + p], (unsigned long long)n);
     }
-    if (UNIFORM && lane != 0) return;
-    if (cs <= 1 || adjacent) {
-        tally_lane<SHIST>(shist, A, h, p + cs);
-        return;
+}
+
+// The block's 32-bit histogram into the global one (all threads of the block,
+// after the last tally).
+__device__ __forceinline__ void hist_flush(unsigned *shist, const CountArgs &A)
+{
+    __syncthreads();
+    for (int i = threadIdx.x; i < HIST_H * HIST_P; i += blockDim.x) {
+        const unsigned x = shist[i];
+        if (x) atomicAdd(&A.hist[(size_t)(i / HIST_P) * A.hstride + (i % HIST_P)], (unsigned long long)x);
     }
-    tally_lane<SHIST>(shist, A, h, p + 1);  // the pivot leaf below the pair
-    if (h + 1 <= A.kmax) tally_lane<SHIST>(shist, A, h + 1, p);
+}
+
+// Subtrees of labels S' of at most two members, reached with (h, p), in
+// closed form (global counts): |S'| = 0 is a leaf (h, p); a single member or
+// an adjacent pair is a clique, one leaf (h, p + |S'|); a non-adjacent pair
+// {a < b} takes a as pivot (a pivot leaf (h, p + 1)) and holds b (a leaf
+// (h + 1, p), cut when h + 1 > kmax).  The labels that close below one node
+// are counted by kind and tallied together: one atomic per kind, instead of
+// one per label on the same few counters.  nodes, leaves and words grow by
+// what the walk would have spent (a label of at most two members fits one
+// word).
+struct SmallCounts {
+    unsigned c01 = 0, c2 = 0;  // per lane, 16 bits each: empty | single, adjacent | non-adjacent pair
+    __device__ __forceinline__ void add(int cs, bool adjacent)
+    {
+        if (cs < 2) c01 += cs ? 0x10000u : 1u;
+        else c2 += adjacent ? 1u : 0x10000u;
+    }
+    // all lanes; every lane passes the same (h, p)
+    template <bool SHIST, typename N>
+    __device__ __forceinline__ void close(unsigned *shist, const CountArgs &A, int lane, int h, int p, N &nodes,
+                                          N &leaves, N &words) const
+    {
+        const unsigned a = __reduce_add_sync(0xFFFFFFFFu, c01), b = __reduce_add_sync(0xFFFFFFFFu, c2);
+        if ((a | b) == 0) return;
+        const unsigned n0 = a & 0xFFFFu, n1 = a >> 16, adj = b & 0xFFFFu, non = b >> 16;
+        const unsigned held = h + 1 <= A.kmax ? non : 0u;
+        nodes += n0 + n1 + adj + 2 * non + held;
+        leaves += n0 + n1 + adj + non + held;
+        words += n1 + 2 * (adj + non);
+        const unsigned n = lane == 0 ? n0 : lane == 1 ? n1 + non : lane == 2 ? adj : lane == 3 ? held : 0u;
+        if (n) tally_n<SHIST>(shist, A, lane == 3 ? h + 1 : h, lane == 3 ? p : p + lane, n);
+    }
+};
+
+// The same for one label, every lane with the same arguments.
+template <bool SHIST, typename N>
+__device__ __forceinline__ void close_small(unsigned *shist, const CountArgs &A, int lane, int cs, bool adjacent, int h,
+                                            int p, N &nodes, N &leaves, N &words)
+{
+    const bool split = cs == 2 && !adjacent;
+    const bool held = split && h + 1 <= A.kmax;
+    nodes += 1 + split + held;
+    leaves += 1 + held;
+    words += (unsigned)cs;
+    if (lane == 0) tally_n<SHIST>(shist, A, h, split ? p + 1 : p + cs, 1u);
+    if (lane == 1 && held) tally_n<SHIST>(shist, A, h + 1, p, 1u);
 }
 
 // Donated frames must carry enough work to pay for the queue round trip.
@@ -466,11 +495,13 @@ __device__ __forceinline__ void donate_wide(WarpWork<NW> &Wk, const CountArgs &A
 // (global counts).  In the split form, pending frames are donated to idle
 // warps as self-contained compacted frames (rows travel with the frame).
 template <int NW, bool SHIST, bool SPLIT>
-__device__ void compact_loop(WarpWork<NW> &Wk, unsigned long long *shist, const CountArgs &A, int lane,
+__device__ void compact_loop(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A, int lane,
                              uint32_t r1, uint32_t S1, int h, int p, WalkCounters &wc, const Outer *outer,
                              Clock &clk)
 {
-    auto tally = [&](int hh, int pp) { tally_leaf<SHIST>(shist, A, lane, hh, pp); };
+    auto tally = [&](int hh, int pp) {
+        if (lane == 0) tally_n<SHIST>(shist, A, hh, pp, 1u);
+    };
     // this call's nodes, leaves and pivot words (every lane alike; at most a
     // 32-member label's tree, so 32 bits hold them), added to wc on exit
     unsigned cn = 0, cl = 0, cw = 0;
@@ -509,9 +540,9 @@ __device__ void compact_loop(WarpWork<NW> &Wk, unsigned long long *shist, const 
                     const uint32_t child = inR ? (r1 & S1 & ~(R0 & ((1u << lane) - 1u))) : 0u;
                     const int cs = __popc(child);
                     const uint32_t ra = __shfl_sync(FULL, r1, (__ffs(child) - 1) & 31);
-                    if (inR && cs <= 2)
-                        close_small<SHIST, false>(shist, A, lane, cs, (ra >> ((31 - __clz(child)) & 31)) & 1u, h + 1, p,
-                                                  1u, wc);
+                    SmallCounts small;
+                    if (inR && cs <= 2) small.add(cs, (ra >> ((31 - __clz(child)) & 31)) & 1u);
+                    small.close<SHIST>(shist, A, lane, h + 1, p, cn, cl, cw);
                     R = __ballot_sync(FULL, inR && cs > 2);
                 }
                 const int nR = __popc(R);
@@ -580,7 +611,7 @@ __device__ void compact_loop(WarpWork<NW> &Wk, unsigned long long *shist, const 
                 const int ps = __popc(P1);
                 if (ps <= 2) {
                     const uint32_t ra = __shfl_sync(FULL, r1, (__ffs(P1) - 1) & 31);
-                    close_small<SHIST, true>(shist, A, lane, ps, (ra >> ((31 - __clz(P1)) & 31)) & 1u, h, p + 1, 1u, wc);
+                    close_small<SHIST>(shist, A, lane, ps, (ra >> ((31 - __clz(P1)) & 31)) & 1u, h, p + 1, cn, cl, cw);
                 } else {
                     closed = false;
                     S1 = P1;
@@ -601,55 +632,102 @@ __device__ void compact_loop(WarpWork<NW> &Wk, unsigned long long *shist, const 
     __syncwarp();
 }
 
-// Compact a node whose label S (in NW-word bitsets over the root's members)
-// has s <= 32 members: relabel them 0..s-1 in ascending order; lane k gets
-// row k of the induced adjacency -- by symmetry, the ballot over lanes j of
-// "member k is in my row" is exactly that row.
-template <int NW>
-__device__ __forceinline__ uint32_t compact_rows(WarpWork<NW> &Wk, int lane, const uint32_t *S, int s)
+// Relabel a label of at most 32 members (word w of its bitset in lane w's cw,
+// 0 in the lanes from the word count on; s: their number): member k of the label = its k-th
+// member in ascending order, listed in cmap.  Lane j returns row j of the
+// one-word adjacency: rows are symmetric, so the row of member j itself,
+// compressed to the label's members, word by word from the top.
+template <int NW, int RS, typename M>
+__device__ __forceinline__ uint32_t relabel_rows(const uint32_t *adj, M *cmap, int lane, uint32_t cw, int &s)
 {
-    constexpr int RS = WarpWork<NW>::RS;
-    int before = 0;
+    const int c = __popc(cw);
+    int inc = c;
 #pragma unroll
-    for (int w = 0; w < NW; ++w) {
-        if ((S[w] >> lane) & 1u) Wk.cmap[before + __popc(S[w] & ((1u << lane) - 1u))] = (uint16_t)(w * 32 + lane);
-        before += __popc(S[w]);
+    for (int o = 1; o < NW; o <<= 1) {
+        const int t = __shfl_up_sync(FULL, inc, o);
+        if (lane >= o) inc += t;
+    }
+    s = __shfl_sync(FULL, inc, NW - 1);
+    M *dst = cmap + (inc - c);
+    for (uint32_t x = cw; x; x &= x - 1) *dst++ = (M)(lane * 32 + __ffs(x) - 1);
+    __syncwarp();
+    const uint32_t *mine = adj + (lane < s ? (int)cmap[lane] : 0) * RS;
+    uint32_t r = 0;
+    for (unsigned nz = __ballot_sync(FULL, cw != 0); nz;) {
+        const int w = 31 - __clz(nz);
+        nz ^= 1u << w;
+        const uint32_t a = mine[w];
+        for (uint32_t m = __shfl_sync(FULL, cw, w); m;) {
+            const int z = __clz(m);
+            m ^= 0x80000000u >> z;
+            r = __funnelshift_l(a << z, r, 1);  // r * 2 + bit 31 - z of a
+        }
     }
     __syncwarp();
-    const int mj = lane < s ? Wk.cmap[lane] : 0;
-    uint32_t r1 = 0;
-    for (int k = 0; k < s; ++k) {
-        const int mk = Wk.cmap[k];
-        const bool bit = lane < s && ((Wk.adj[mj * RS + (mk >> 5)] >> (mk & 31)) & 1u);
-        const uint32_t col = __ballot_sync(FULL, bit);
-        if (lane == k) r1 = col;
+    return lane < s ? r : 0u;
+}
+
+// Frame slots a warp reserved in the emit buffer.  Slots are reserved in
+// groups (one atomic round trip per group instead of per frame); the emit
+// buffer's capacity is a multiple of the group.
+constexpr unsigned EMIT_RESERVE = 16;
+struct Emitter {
+    unsigned long long met = 0;     // compacted subtrees met, emitted or walked in place
+    unsigned slot = 0, end = 0;     // reserved slots
+    bool full = false;              // the buffer is full
+    // the next slot, or nullptr once the buffer is full (all lanes)
+    __device__ __forceinline__ uint32_t *next(const CountArgs &A, int lane)
+    {
+        if (slot == end) {
+            if (full) return nullptr;
+            unsigned long long b = 0;
+            if (lane == 0) b = atomicAdd(A.emit_count, (unsigned long long)EMIT_RESERVE);
+            b = __shfl_sync(FULL, b, 0);
+            if (b + EMIT_RESERVE > (unsigned long long)A.emit_cap) {
+                full = true;
+                return nullptr;
+            }
+            slot = (unsigned)b;
+            end = slot + EMIT_RESERVE;
+        }
+        return A.emit + (size_t)(slot++) * FRAME_WORDS;
     }
-    __syncwarp();
-    return r1;
+    // end of the launch: mark the slots left over, count the subtrees met
+    __device__ __forceinline__ void finish(const CountArgs &A, int lane)
+    {
+        if (slot + (unsigned)lane < end) A.emit[(size_t)(slot + lane) * FRAME_WORDS] = FRAME_NONE;
+        if (lane == 0 && met) atomicAdd(&A.stats[3 + NCLASS + 1], met);
+    }
+};
+
+// Write a compacted frame: label of s members reached with (h, p), row r1 of
+// its adjacency in each lane.
+__device__ __forceinline__ void frame_write(uint32_t *fr, const CountArgs &A, int lane, uint32_t r1, int s, int h,
+                                            int p)
+{
+    fr[4 + lane] = r1;
+    if (lane == 0)
+        *reinterpret_cast<uint4 *>(fr) = make_uint4(FRAME_COMPACT, ((uint32_t)h << 16) | (uint32_t)p,
+                                                    s >= 32 ? FULL : ((1u << s) - 1u), (uint32_t)A.cls);
 }
 
 // Walk the compacted subtree in place, or (two-phase global counts) emit it
-// as a frame for k_walk_frames while the buffer has room.
+// as a frame for the frame walk while the buffer has room.
 template <int NW, bool SHIST, bool SPLIT>
-__device__ void walk_compact(WarpWork<NW> &Wk, unsigned long long *shist, const CountArgs &A, int lane,
+__device__ void walk_compact(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A, int lane,
                              const uint32_t *S, int s, int h, int p, WalkCounters &wc, const Outer *outer,
-                             Clock &clk)
+                             Clock &clk, Emitter &em)
 {
-    const uint32_t r1 = compact_rows<NW>(Wk, lane, S, s);
-    const uint32_t S1 = s >= 32 ? FULL : ((1u << s) - 1u);
+    uint32_t cw = 0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w)
+        if (lane == w) cw = S[w];
+    const uint32_t r1 = relabel_rows<NW, WarpWork<NW>::RS>(Wk.adj, Wk.cmap, lane, cw, s);
     if (A.emit) {
-        unsigned long long i = 0;
-        if (lane == 0) i = atomicAdd(A.emit_count, 1ull);
-        i = __shfl_sync(FULL, i, 0);
-        if (i < (unsigned long long)A.emit_cap) {
-            uint32_t *fr = A.emit + (size_t)i * FRAME_WORDS;
-            fr[4 + lane] = r1;
-            if (lane == 0) {
-                fr[0] = FRAME_COMPACT;
-                fr[1] = ((uint32_t)h << 16) | (uint32_t)p;
-                fr[2] = S1;
-                fr[3] = (uint32_t)A.cls;
-            }
+        ++em.met;
+        uint32_t *fr = em.next(A, lane);
+        if (fr) {
+            frame_write(fr, A, lane, r1, s, h, p);
             // an emission is where the wide walk spends its time: let it
             // advance the donation clock, so that a heavy root's pending wide
             // frames move to idle warps
@@ -657,22 +735,26 @@ __device__ void walk_compact(WarpWork<NW> &Wk, unsigned long long *shist, const 
             return;
         }
     }
-    compact_loop<NW, SHIST, SPLIT>(Wk, shist, A, lane, r1, S1, h, p, wc, outer, clk);
+    compact_loop<NW, SHIST, SPLIT>(Wk, shist, A, lane, r1, s >= 32 ? FULL : ((1u << s) - 1u), h, p, wc, outer, clk);
 }
 
 // One walk item: a whole root r (frame == nullptr), or a frame of root qi's
 // subtree that another warp donated (split form).
 template <int NW, int MODE, bool SHIST, bool SPLIT>
-__device__ void walk_root(WarpWork<NW> &Wk, unsigned long long *shist, const CountArgs &A, int lane,
-                          uint32_t r, WalkCounters &wc, unsigned qi = 0, const uint32_t *frame = nullptr)
+__device__ void walk_root(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A, int lane,
+                          uint32_t r, WalkCounters &wc, Emitter &em, unsigned qi = 0, const uint32_t *frame = nullptr)
 {
     Clock clk;
     constexpr int D = WarpWork<NW>::D;
     constexpr int RS = WarpWork<NW>::RS;
     constexpr bool REG = NW <= 4;  // keep this lane's adjacency rows in registers
-    // the member-word loops of the widest classes stay rolled: unrolled they
-    // multiply the code (and its compile time) by NW for a rare class
-    constexpr int UNROLL_J = NW <= 8 ? NW : 1;
+    // the member-word loops (32 members a turn) of the wider rows stay rolled:
+    // unrolled they multiply the code by NW, and the walk then waits for
+    // instructions (24 % of its stalls on 8-word rows)
+    constexpr int UNROLL_J = REG ? NW : 1;
+    auto word_of = [&](const uint32_t *X, uint32_t mine, int j) -> uint32_t {
+        return REG ? X[j % (REG ? NW : 1)] : __shfl_sync(FULL, mine, j);
+    };
     int64_t rbeg = 0;
     int d = 0;
     uint32_t S[NW];
@@ -722,46 +804,92 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned long long *shist, const Cou
     if (lane == 0) Wk.off[0] = 0;
     for (int t = lane; t < d * RS; t += 32) Wk.adj[t] = 0;
     __syncwarp();
-    // entry t of the concatenated out-lists belongs to member lo, the largest
+    // Entry t of the concatenated out-lists belongs to member lo, the largest
     // i with off[i] <= t; a lane's entries rise, so lo only moves forward.
-    // Four entries per lane per round keep four loads of ocol in flight.
+    // Four entries per lane per round keep four loads of ocol in flight.  An
+    // entry is tested against the members' bit filter (one shared load; about
+    // d / 2^FILTER_LOG of the entries that are no members pass), and only
+    // those that pass are searched among the members, 32 at a time from a
+    // queue, so that the search runs with every lane busy (a search per entry
+    // cost 6 to 10 dependent shared loads on all 32 lanes for about 2 hits).
+    // With the narrower rows of launch_wide, the rolled word loops and the
+    // labels emitted where they are formed, the wide walks of the 10.8M-edge
+    // graph went from 0.62 / 1.10 / 2.28 ms (33..64, 65..128, 129..256) to
+    // 0.50 / 0.86 / 1.08 ms.
+    constexpr int FSH = 32 - WarpWork<NW>::FILTER_LOG;
+    for (int t = lane; t < (1 << WarpWork<NW>::FILTER_LOG) / 32; t += 32) Wk.filter[t] = 0;
+    __syncwarp();
+    for (int i = lane; i < d; i += 32) {
+        const uint32_t hb = (Wk.ids[i] * FIB_HASH) >> FSH;
+        atomicOr(&Wk.filter[hb >> 5], 1u << (hb & 31u));
+    }
+    __syncwarp();
     const uint32_t T = base;
     int lo = 0;
-    for (uint32_t t0 = lane; t0 < T; t0 += 128) {
-        uint32_t x[4];
-        int mi[4];
-        int64_t at[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t t = t0 + 32u * q;
-            mi[q] = -1;
-            if (t < T) {
-                while (Wk.off[lo + 1] <= t) ++lo;  // stops by off[d] = T > t
-                mi[q] = lo;
-                at[q] = Wk.rs[lo] + (t - Wk.off[lo]);
-                x[q] = A.ocol[at[q]];
+    unsigned nq = 0;  // queued entries (uniform)
+    auto lookup = [&](unsigned n) {
+        if ((unsigned)lane < n) {
+            const uint2 e = Wk.hits[lane];
+            const int u = (int)e.y;
+            int64_t at = 0;
+            uint32_t x = e.x;
+            if (MODE == MODE_EDGE) {  // queued by position: the edge id is needed too
+                at = Wk.rs[u] + (e.x - Wk.off[u]);
+                x = A.ocol[at];
             }
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (mi[q] < 0) continue;
             int a = 0, b = d;
             while (a < b) {
-                int mid = (a + b) >> 1;
-                if (Wk.ids[mid] < x[q]) a = mid + 1; else b = mid;
+                const int mid = (a + b) >> 1;
+                if (Wk.ids[mid] < x) a = mid + 1; else b = mid;
             }
-            if (a < d && Wk.ids[a] == x[q]) {
-                const int u = mi[q];
+            if (a < d && Wk.ids[a] == x) {
                 atomicOr(&Wk.adj[u * RS + (a >> 5)], 1u << (a & 31));
                 atomicOr(&Wk.adj[a * RS + (u >> 5)], 1u << (u & 31));
                 if (MODE == MODE_EDGE && Wk.etab) {
-                    const uint32_t e = A.oeid[at[q]];
+                    const uint32_t e = A.oeid[at];
                     Wk.etab[u * D + a] = e;
                     Wk.etab[a * D + u] = e;
                 }
             }
         }
+    };
+    for (uint32_t t0 = 0; t0 < T; t0 += 128) {
+        uint32_t x[4];
+        int mi[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t t = t0 + 32u * q + lane;
+            mi[q] = -1;
+            x[q] = 0;
+            if (t < T) {
+                while (Wk.off[lo + 1] <= t) ++lo;  // stops by off[d] = T > t
+                mi[q] = lo;
+                x[q] = A.ocol[Wk.rs[lo] + (t - Wk.off[lo])];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t hb = (x[q] * FIB_HASH) >> FSH;
+            const bool pass = mi[q] >= 0 && ((Wk.filter[hb >> 5] >> (hb & 31u)) & 1u);
+            const unsigned b = __ballot_sync(FULL, pass);
+            if (!b) continue;
+            if (pass)
+                Wk.hits[nq + __popc(b & ((1u << lane) - 1u))] =
+                    make_uint2(MODE == MODE_EDGE ? t0 + 32u * q + lane : x[q], (uint32_t)mi[q]);
+            nq += __popc(b);
+            if (nq >= 32) {
+                __syncwarp();
+                lookup(32u);
+                nq -= 32;
+                const uint2 rest = Wk.hits[32 + lane];
+                __syncwarp();
+                if ((unsigned)lane < nq) Wk.hits[lane] = rest;
+                __syncwarp();
+            }
+        }
     }
+    __syncwarp();
+    lookup(nq);
     __syncwarp();
     if (SPLIT) {
         // publish the adjacency rows so that donated frames can be walked anywhere
@@ -811,21 +939,27 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned long long *shist, const Cou
         if (NW > 1 && MODE == MODE_GLOBAL && s >= 4 && s <= 32) {
             // small label under a wide root: finish this subtree in one-word bitsets
             const Outer outer{&top, &bot, qi, d};
-            walk_compact<NW, SHIST, SPLIT>(Wk, shist, A, lane, S, s, h, p, wc, &outer, clk);
+            walk_compact<NW, SHIST, SPLIT>(Wk, shist, A, lane, S, s, h, p, wc, &outer, clk, em);
         } else if ((wc.nodes++, clk.nodes++, s == 0)) {
             wc.leaves++;
             if (MODE == MODE_GLOBAL) {
-                tally_leaf<SHIST>(shist, A, lane, h, p);
+                if (lane == 0) tally_n<SHIST>(shist, A, h, p, 1u);
             } else {
                 local_leaf<NW, MODE>(Wk, A, lane, r, rbeg, d, h, p, depth, nullptr);
             }
         } else {
             // pivot: most neighbours inside S, ties -> lowest member index; the
             // degree sum tells whether S is a clique (every member has s-1)
+            uint32_t Sl = 0;  // word `lane` of S
+            if (!REG || (MODE == MODE_GLOBAL && NW > 1)) {
+#pragma unroll
+                for (int w = 0; w < NW; ++w)
+                    if (lane == w) Sl = S[w];
+            }
             uint32_t best = 0, dsum = 0;
 #pragma unroll UNROLL_J
             for (int j = 0; j < NW; ++j) {
-                if ((S[j] >> lane) & 1u) {
+                if ((word_of(S, Sl, j) >> lane) & 1u) {
                     uint32_t c = 0;
 #pragma unroll
                     for (int w = 0; w < NW; ++w) c += __popc(row(j, w) & S[w]);
@@ -842,7 +976,7 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned long long *shist, const Cou
                 // S is a clique: one leaf with |S| more pivot links
                 wc.leaves++;
                 if (MODE == MODE_GLOBAL) {
-                    tally_leaf<SHIST>(shist, A, lane, h, p + s);
+                    if (lane == 0) tally_n<SHIST>(shist, A, h, p + s, 1u);
                 } else {
                     local_leaf<NW, MODE>(Wk, A, lane, r, rbeg, d, h, p + s, depth, S);
                 }
@@ -873,46 +1007,94 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned long long *shist, const Cou
                     }
                     __syncwarp();  // every lane is done reading the last popped frame
                     // hold child of member j*32+lane: N(S, v) minus the earlier
-                    // members of R; global counts close labels of at most two
-                    // members here and push the rest
+                    // members of R.  M holds S without the members of R in the
+                    // words before j.  Global counts close labels of at most
+                    // two members here, emit those of at most 32 below
+                    // (two-phase form) and push the rest
                     int before = 0;
                     const uint32_t low = (1u << lane) - 1u;
+                    SmallCounts small;
+                    const bool emits = MODE == MODE_GLOBAL && NW > 1 && A.emit != nullptr;
+                    uint32_t Rl = 0;      // word `lane` of R
+                    uint32_t emitl = 0;   // members of word `lane` whose labels are emitted
+                    uint32_t M[NW];
+#pragma unroll
+                    for (int w = 0; w < NW; ++w) {
+                        M[w] = S[w];
+                        if ((!REG || (MODE == MODE_GLOBAL && NW > 1)) && lane == w) Rl = R[w];
+                    }
 #pragma unroll UNROLL_J
                     for (int j = 0; j < NW; ++j) {
-                        const bool inR = (R[j] >> lane) & 1u;
+                        const uint32_t Rj = word_of(R, Rl, j);
+                        if (Rj == 0) continue;
+                        const bool inR = (Rj >> lane) & 1u;
                         bool push = inR;
+                        int cs = 0;
                         if (MODE == MODE_GLOBAL && inR) {
-                            int cs = 0, a = 0, b = 0;
 #pragma unroll
-                            for (int w = 0; w < NW; ++w) {
-                                const uint32_t below = w < j ? R[w] : (w == j ? (R[j] & low) : 0u);
-                                const uint32_t cw = row(j, w) & S[w] & ~below;
-                                if (cw) {
-                                    if (cs == 0) a = w * 32 + __ffs(cw) - 1;
-                                    b = w * 32 + 31 - __clz(cw);
-                                }
-                                cs += __popc(cw);
-                            }
+                            for (int w = 0; w < NW; ++w) cs += __popc(row(j, w) & M[w] & (w == j ? ~(Rj & low) : FULL));
                             if (cs <= 2) {
-                                const bool adj = cs == 2 && ((Wk.adj[a * RS + (b >> 5)] >> (b & 31)) & 1u);
-                                close_small<SHIST, false>(shist, A, lane, cs, adj, h + 1, p, 1u, wc);
+                                bool adj = false;
+                                if (cs == 2) {
+                                    int a = 0, b = 0;
+#pragma unroll
+                                    for (int w = NW - 1; w >= 0; --w) {
+                                        const uint32_t cw = row(j, w) & M[w] & (w == j ? ~(Rj & low) : FULL);
+                                        if (cw) {
+                                            a = w * 32 + __ffs(cw) - 1;
+                                            b = max(b, w * 32 + 31 - __clz(cw));
+                                        }
+                                    }
+                                    adj = (Wk.adj[a * RS + (b >> 5)] >> (b & 31)) & 1u;
+                                }
+                                small.add(cs, adj);
                                 push = false;
                             }
+                        }
+                        if (emits) {
+                            const unsigned eb = __ballot_sync(FULL, push && cs <= 32);
+                            if (lane == j) emitl = eb;
+                            push = push && cs > 32;
                         }
                         const uint32_t pushed = __ballot_sync(FULL, push);
                         if (push) {
                             const int f = top + before + __popc(pushed & low);
 #pragma unroll
-                            for (int w = 0; w < NW; ++w) {
-                                const uint32_t below = w < j ? R[w] : (w == j ? (R[j] & low) : 0u);
-                                Wk.stk()[f * NW + w] = row(j, w) & S[w] & ~below;
-                            }
+                            for (int w = 0; w < NW; ++w)
+                                Wk.stk()[f * NW + w] = row(j, w) & M[w] & (w == j ? ~(Rj & low) : FULL);
                             Wk.hp[f] = ((uint32_t)(h + 1) << 16) | (uint32_t)p;
                             if (MODE != MODE_GLOBAL) Wk.lk[f] = (uint16_t)(j * 32 + lane);
                         }
                         before += __popc(pushed);
+#pragma unroll
+                        for (int w = 0; w < NW; ++w)
+                            if (w == j) M[w] &= ~Rj;
+                    }
+                    if (emits) {
+                        // one label at a time, word w of it in lane w
+                        for (unsigned ej = __ballot_sync(FULL, emitl != 0); ej; ej &= ej - 1) {
+                            const int j = __ffs(ej) - 1;
+                            for (unsigned eb = __shfl_sync(FULL, emitl, j); eb; eb &= eb - 1) {
+                                const int v = __ffs(eb) - 1;  // member j * 32 + v
+                                const uint32_t below = lane < j ? Rl : (lane == j ? Rl & ((1u << v) - 1u) : 0u);
+                                const uint32_t cw = lane < NW ? Wk.adj[(j * 32 + v) * RS + lane] & Sl & ~below : 0u;
+                                uint32_t *fr = em.next(A, lane);
+                                if (!fr) {  // the buffer is full: to the stack, walked in place
+                                    if (lane < NW) Wk.stk()[(top + before) * NW + lane] = cw;
+                                    if (lane == 0) Wk.hp[top + before] = ((uint32_t)(h + 1) << 16) | (uint32_t)p;
+                                    ++before;
+                                    continue;
+                                }
+                                int es = 0;
+                                const uint32_t r1 = relabel_rows<NW, RS>(Wk.adj, Wk.cmap, lane, cw, es);
+                                frame_write(fr, A, lane, r1, es, h + 1, p);
+                                ++em.met;
+                                clk.nodes += EMIT_CLOCK;
+                            }
+                        }
                     }
                     top += before;
+                    if (MODE == MODE_GLOBAL) small.close<SHIST>(shist, A, lane, h + 1, p, wc.nodes, wc.leaves, wc.words);
                     __syncwarp();  // pushed frames visible to every lane
                     if (SPLIT && (int)(clk.nodes - clk.next) >= 0) {
                         clk.next = clk.nodes + clk.every;
@@ -944,7 +1126,7 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned long long *shist, const Cou
                 }
                 if (MODE == MODE_GLOBAL && ps <= 2) {
                     const bool adj = ps == 2 && ((Wk.adj[a * RS + (b >> 5)] >> (b & 31)) & 1u);
-                    close_small<SHIST, true>(shist, A, lane, ps, adj, h, p + 1, 1u, wc);
+                    close_small<SHIST>(shist, A, lane, ps, adj, h, p + 1, wc.nodes, wc.leaves, wc.words);
                 } else {
                     closed = false;
 #pragma unroll
@@ -977,7 +1159,7 @@ template <int NW, int MODE, bool SHIST>
 constexpr size_t smem_bytes()
 {
     return sizeof(WarpWork<NW>) * warps_per_block<NW>() +
-           (SHIST ? sizeof(unsigned long long) * HIST_H * HIST_P : 0) +
+           (SHIST ? sizeof(unsigned) * HIST_H * HIST_P : 0) +
            (MODE != MODE_GLOBAL ? WarpWork<NW>::LOCAL_BYTES * warps_per_block<NW>() : 0);
 }
 
@@ -1040,12 +1222,13 @@ __global__ void __launch_bounds__(32 * warps_per_block<NW>())
     constexpr int WPB = warps_per_block<NW>();
     extern __shared__ __align__(16) unsigned char smem[];
     WarpWork<NW> *ww = reinterpret_cast<WarpWork<NW> *>(smem);
-    unsigned long long *shist = reinterpret_cast<unsigned long long *>(ww + WPB);
+    unsigned *shist = reinterpret_cast<unsigned *>(ww + WPB);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     bind_warp<NW, MODE>(ww[wid],
-                        reinterpret_cast<unsigned char *>(shist) + (SHIST ? sizeof(unsigned long long) * HIST_H * HIST_P : 0),
+                        reinterpret_cast<unsigned char *>(shist) + (SHIST ? sizeof(unsigned) * HIST_H * HIST_P : 0),
                         wid, A.gstack, blockIdx.x * WPB + wid, A.eidtab);
     WalkCounters wc;
+    Emitter em;
     if (SHIST) {
         for (int i = threadIdx.x; i < HIST_H * HIST_P; i += blockDim.x) shist[i] = 0;
         __syncthreads();
@@ -1071,12 +1254,11 @@ __global__ void __launch_bounds__(32 * warps_per_block<NW>())
                     compact_loop<NW, SHIST, true>(ww[wid], shist, A, lane, fb[4 + lane], fb[2], (int)(hp0 >> 16),
                                                   (int)(hp0 & 0xFFFFu), wc, nullptr, clk);
                 } else {
-                    walk_root<NW, MODE, SHIST, true>(ww[wid], shist, A, lane, 0u, wc, fb[1], fb + 1);
+                    walk_root<NW, MODE, SHIST, true>(ww[wid], shist, A, lane, 0u, wc, em, fb[1], fb + 1);
                 }
             } else {
-                walk_root<NW, MODE, SHIST, true>(ww[wid], shist, A, lane, A.roots[v], wc, v, nullptr);
+                walk_root<NW, MODE, SHIST, true>(ww[wid], shist, A, lane, A.roots[v], wc, em, v, nullptr);
             }
-            wc.fold();
             __syncwarp();
             if (lane == 0) atomicSub(A.qctl + Q_OUT, 1u);
         }
@@ -1092,20 +1274,14 @@ __global__ void __launch_bounds__(32 * warps_per_block<NW>())
             qi = blockIdx.x * WPB + wid;
         }
         if (qi >= A.nroots) break;
-        walk_root<NW, MODE, SHIST, false>(ww[wid], shist, A, lane, A.roots[qi], wc);
-        wc.fold();
+        walk_root<NW, MODE, SHIST, false>(ww[wid], shist, A, lane, A.roots[qi], wc, em);
         ++qi;
         if (!PERSIST) break;
         if (*(volatile unsigned *)A.err & (DERR_STACK | DERR_RANGE)) break;
     }
     wc.flush(A.stats, A.cls, lane);
-    if (SHIST) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < HIST_H * HIST_P; i += blockDim.x) {
-            unsigned long long v = shist[i];
-            if (v) atomicAdd(&A.hist[(size_t)(i / HIST_P) * A.hstride + (i % HIST_P)], v);
-        }
-    }
+    if (MODE == MODE_GLOBAL && NW > 1) em.finish(A, lane);
+    if (SHIST) hist_flush(shist, A);
 }
 
 template <typename T>
@@ -1132,6 +1308,13 @@ constexpr unsigned SPLIT_QCAP = 1u << 17;
 // The lane walk of one-word labels (lanes.cuh, walk_lanes.cu): the frames of
 // the two-phase count.
 pvt_status launch_lanes_frames(pvt_dag *g, const CountArgs &base, cudaStream_t s);
+// The gather of the <= 32 class of a two-phase count (walk_gather.cu) over
+// roots[0..cnt): closes what has a closed form and emits the rest as frames.
+pvt_status launch_gather1(pvt_dag *g, const CountArgs &base, const uint32_t *roots, unsigned cnt, unsigned slots,
+                          cudaStream_t s);
+// Frame slots the gather may reserve for cnt roots (its warps reserve in
+// groups).
+unsigned gather1_slots(const pvt_dag *g, unsigned cnt);
 // The CTA-per-root walk (cta.cuh, walk_cta.cu) of out-degree class cls >= 4.
 pvt_status launch_cta_class(pvt_dag *g, const CountArgs &base, int cls, cudaStream_t s);
 
@@ -1233,11 +1416,10 @@ __global__ void __launch_bounds__(32 * FRAME_WPB) k_walk_frames(CountArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     WarpWork<1> *ww = reinterpret_cast<WarpWork<1> *>(smem);
-    unsigned long long *shist = reinterpret_cast<unsigned long long *>(ww + FRAME_WPB);
+    unsigned *shist = reinterpret_cast<unsigned *>(ww + FRAME_WPB);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned long long emitted = *(volatile unsigned long long *)A.emit_count;
     const unsigned nframes = (unsigned)min(emitted, (unsigned long long)A.emit_cap);
-    if (blockIdx.x == 0 && threadIdx.x == 0) A.stats[3 + FRAMES_SLOT + 1] = emitted;
     WalkCounters wc;
     if (SHIST) {
         for (int i = threadIdx.x; i < HIST_H * HIST_P; i += blockDim.x) shist[i] = 0;
@@ -1277,23 +1459,18 @@ __global__ void __launch_bounds__(32 * FRAME_WPB) k_walk_frames(CountArgs A)
         } else {
             fr = A.emit + (size_t)v * FRAME_WORDS;
         }
-        const uint32_t r1 = fr[4 + lane], S1 = fr[2], hp0 = fr[1];
-        Clock clk;
-        clk.every = 32;
-        compact_loop<1, SHIST, true>(ww[wid], shist, A, lane, r1, S1, (int)(hp0 >> 16), (int)(hp0 & 0xFFFFu), wc,
-                                     nullptr, clk);
-        wc.fold();
+        if (fr[0] == FRAME_COMPACT) {  // else a reserved slot that holds no subtree
+            const uint32_t r1 = fr[4 + lane], S1 = fr[2], hp0 = fr[1];
+            Clock clk;
+            clk.every = 32;
+            compact_loop<1, SHIST, true>(ww[wid], shist, A, lane, r1, S1, (int)(hp0 >> 16), (int)(hp0 & 0xFFFFu), wc,
+                                         nullptr, clk);
+        }
         __syncwarp();
         if (lane == 0) atomicSub(A.qctl + Q_OUT, 1u);
     }
     wc.flush(A.stats, FRAMES_SLOT, lane);
-    if (SHIST) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < HIST_H * HIST_P; i += blockDim.x) {
-            unsigned long long x = shist[i];
-            if (x) atomicAdd(&A.hist[(size_t)(i / HIST_P) * A.hstride + (i % HIST_P)], x);
-        }
-    }
+    if (SHIST) hist_flush(shist, A);
 }
 
 // Queue counters of the frame walk: outstanding items = the emitted frames
@@ -1323,6 +1500,7 @@ __global__ void __launch_bounds__(32 * warps_per_block<NW>())
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     bind_warp<NW, MODE>(ww[wid], reinterpret_cast<unsigned char *>(ww + WPB), wid, gstack, blockIdx.x * WPB + wid);
     WalkCounters wc;
+    Emitter em;
     for (;;) {
         unsigned qi = 0;
         if (lane == 0) qi = atomicAdd(qhead, 1u);
@@ -1343,8 +1521,7 @@ __global__ void __launch_bounds__(32 * warps_per_block<NW>())
         A.kmax = G.kmax;
         A.err = err;
         A.stats = stats;
-        walk_root<NW, MODE, false, false>(ww[wid], nullptr, A, lane, (uint32_t)e, wc);
-        wc.fold();
+        walk_root<NW, MODE, false, false>(ww[wid], nullptr, A, lane, (uint32_t)e, wc, em);
         if (vload(err) & (DERR_STACK | DERR_RANGE)) break;
     }
     (void)WPB;

@@ -12,7 +12,10 @@ static pvt_status launch_cta_nw(pvt_dag *g, CountArgs A, int cls, int dmax, cuda
     auto kern = k_cta<NW>;
     int optin = 0;
     PVT_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device));
-    const size_t fixed = Lay::bytes(0, dmax);
+    // the limit covers the kernel's static shared memory too
+    cudaFuncAttributes fa{};
+    PVT_CK(cudaFuncGetAttributes(&fa, kern));
+    const size_t fixed = Lay::bytes(0, dmax) + fa.sharedSizeBytes;
     int warps = fixed < (size_t)optin ? (int)(((size_t)optin - fixed) / (sizeof(LaneWork) + sizeof(CtaWarp))) : 0;
     warps = std::min(warps, CTA_MAXW);
     if (warps < 1) {
@@ -54,8 +57,13 @@ pvt_status launch_cta_class(pvt_dag *g, const CountArgs &base, int cls, cudaStre
     const int dmax = std::min(cap, (int)g->alpha);
     switch (cls) {
         case 4: return launch_cta_nw<8>(g, A, cls, dmax, s);
-        case 5: return launch_cta_nw<16>(g, A, cls, dmax, s);
-        case 6: return dmax <= 768 ? launch_cta_nw<24>(g, A, cls, dmax, s) : launch_cta_nw<32>(g, A, cls, dmax, s);
+        case 5:
+            return dmax <= 320   ? launch_cta_nw<10>(g, A, cls, dmax, s)
+                   : dmax <= 384 ? launch_cta_nw<12>(g, A, cls, dmax, s)
+                                 : launch_cta_nw<16>(g, A, cls, dmax, s);
+        case 6:
+            if (dmax <= 640) return launch_cta_nw<20>(g, A, cls, dmax, s);
+            return dmax <= 768 ? launch_cta_nw<24>(g, A, cls, dmax, s) : launch_cta_nw<32>(g, A, cls, dmax, s);
         default:
             set_error("CTA walk: only the out-degree classes above 128");
             return PVT_EINVAL;

@@ -4,21 +4,29 @@
 
 namespace pvt {
 
-// Every emitted compacted frame (A.emit, the count in *A.emit_count capped
-// at A.emit_cap); walk statistics to slot FRAMES_SLOT.
+// Frames of a launch: those the wide walks emitted (the count capped at
+// A.emit_cap; null: none) and the slots the <= 32 class's gather reserved.
+__device__ __forceinline__ unsigned wide_frames(const CountArgs &A)
+{
+    return A.emit ? (unsigned)min(*(volatile unsigned long long *)A.emit_count, (unsigned long long)A.emit_cap) : 0u;
+}
+__device__ __forceinline__ unsigned all_frames(const CountArgs &A)
+{
+    return wide_frames(A) + (A.emit1 ? min(vload(A.emit1_count), A.emit1_cap) : 0u);
+}
+
+// Every emitted frame (A.emit, then A.emit1); walk statistics to slot
+// FRAMES_SLOT, those of <= 32 class roots to their own class.
 __global__ void __launch_bounds__(32 * LANE_WPB, 2) k_lanes(CountArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     LaneWork *lw = reinterpret_cast<LaneWork *>(smem);
     unsigned *sh32 = reinterpret_cast<unsigned *>(lw + LANE_WPB);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const unsigned long long emitted = *(volatile unsigned long long *)A.emit_count;
-    const unsigned nitems = (unsigned)min(emitted, (unsigned long long)A.emit_cap);
-    if (blockIdx.x == 0 && threadIdx.x == 0) A.stats[3 + NCLASS + 1] = emitted;
     for (int i = threadIdx.x; i < HIST_H * HIST_P; i += blockDim.x) sh32[i] = 0;
     __syncthreads();
-    lane_walk(lw[wid], sh32, A, lane, nitems, NCLASS);
-    lane_hist_flush(sh32, A);
+    lane_walk(lw[wid], sh32, A, lane, wide_frames(A), all_frames(A), NCLASS);
+    hist_flush(sh32, A);
 }
 
 
@@ -41,11 +49,10 @@ static pvt_status launch_lanes_kernel(pvt_dag *g, const CountArgs &A, int phase,
     return PVT_OK;
 }
 
-// Frame counters of the second phase: the emitted count is final on the device.
-static __global__ void k_lanes_frames_init(uint32_t *qctl, const unsigned long long *emit_count, unsigned cap)
+// Queue counters of the second phase: the frame counts are final on the device.
+static __global__ void k_lanes_frames_init(CountArgs A)
 {
-    for (int i = threadIdx.x; i < QCTL_WORDS; i += blockDim.x)
-        qctl[i] = i == Q_OUT ? (unsigned)min(*emit_count, (unsigned long long)cap) : 0u;
+    for (int i = threadIdx.x; i < QCTL_WORDS; i += blockDim.x) A.qctl[i] = i == Q_OUT ? all_frames(A) : 0u;
 }
 
 // Ring queue of a lane launch in the buffers of slot `q` of the dag.
@@ -69,7 +76,7 @@ pvt_status launch_lanes_frames(pvt_dag *g, const CountArgs &base, cudaStream_t s
     A.cls = NCLASS;
     pvt_status st = lane_ring(g, A, 0, s);
     if (st != PVT_OK) return st;
-    k_lanes_frames_init<<<1, 128, 0, s>>>(A.qctl, A.emit_count, A.emit_cap);
+    k_lanes_frames_init<<<1, 128, 0, s>>>(A);
     PVT_CK(cudaGetLastError());
     g->stats.launches += 2;
     return launch_lanes_kernel(g, A, PH_FRAMES, s);
