@@ -26,6 +26,19 @@ int32_t min_words(int64_t n, int32_t alpha)
     return w < 1 ? 1 : w;
 }
 
+int32_t safe_size(int64_t n, int32_t alpha)
+{
+    // n * C(alpha, k - 1) in floating point, far from the bound by the factor
+    // two between 2^62 and 2^63; C rises up to k - 1 = alpha / 2 and a graph
+    // that passes there keeps every size
+    double c = (double)n;
+    for (int32_t k = 1; k <= alpha + 1; ++k) {
+        if (c >= 4.6e18) return k - 1;
+        c *= (double)(alpha - k + 1) / (double)k;
+    }
+    return 0x7FFFFFFF;
+}
+
 pvt_status check_device(pvt_dag *g, cudaStream_t s, const char *what)
 {
     PVT_CK(cudaMemcpyAsync(g->h_err, g->d_err, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
@@ -187,6 +200,7 @@ static void dag_release(pvt_dag *g)
         release(g->qready[c].p);
         release(g->gstack[c].p);
         release(g->etab[c].p);
+        release(g->lheavy[c].p);
     }
     release(g->cframes.p);
     release(g->cframes1.p);

@@ -11,14 +11,8 @@
 namespace pvt {
 
 extern template pvt_status launch_class<1, MODE_GLOBAL, true>(pvt_dag *, const CountArgs &, int, cudaStream_t);
-extern template pvt_status launch_class<1, MODE_VERTEX, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
-extern template pvt_status launch_class<1, MODE_EDGE, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
 extern template pvt_status launch_class<2, MODE_GLOBAL, true>(pvt_dag *, const CountArgs &, int, cudaStream_t);
-extern template pvt_status launch_class<2, MODE_VERTEX, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
-extern template pvt_status launch_class<2, MODE_EDGE, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
 extern template pvt_status launch_class<4, MODE_GLOBAL, true>(pvt_dag *, const CountArgs &, int, cudaStream_t);
-extern template pvt_status launch_class<4, MODE_VERTEX, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
-extern template pvt_status launch_class<4, MODE_EDGE, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
 extern template pvt_status launch_class<8, MODE_GLOBAL, true>(pvt_dag *, const CountArgs &, int, cudaStream_t);
 extern template pvt_status launch_class<8, MODE_VERTEX, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
 extern template pvt_status launch_class<8, MODE_EDGE, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
@@ -36,20 +30,22 @@ extern template pvt_status launch_class<24, MODE_GLOBAL, true>(pvt_dag *, const 
 extern template pvt_status launch_class<32, MODE_VERTEX, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
 extern template pvt_status launch_class<32, MODE_EDGE, false>(pvt_dag *, const CountArgs &, int, cudaStream_t);
 extern template pvt_status launch_batch_class<1, MODE_GLOBAL>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
-extern template pvt_status launch_batch_class<1, MODE_VERTEX>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
-extern template pvt_status launch_batch_class<1, MODE_EDGE>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
 extern template pvt_status launch_batch_class<2, MODE_GLOBAL>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
-extern template pvt_status launch_batch_class<2, MODE_VERTEX>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
-extern template pvt_status launch_batch_class<2, MODE_EDGE>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
 extern template pvt_status launch_batch_class<4, MODE_GLOBAL>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
-extern template pvt_status launch_batch_class<4, MODE_VERTEX>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
-extern template pvt_status launch_batch_class<4, MODE_EDGE>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
 extern template pvt_status launch_batch_class<8, MODE_GLOBAL>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
 extern template pvt_status launch_batch_class<8, MODE_VERTEX>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
 extern template pvt_status launch_batch_class<8, MODE_EDGE>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
 extern template pvt_status launch_batch_class<16, MODE_GLOBAL>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
 extern template pvt_status launch_batch_class<16, MODE_VERTEX>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
 extern template pvt_status launch_batch_class<16, MODE_EDGE>(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int, unsigned *, unsigned long long *, int, cudaStream_t);
+
+// Per-vertex and per-edge counts of the classes up to 128 (local.cuh,
+// walk_local*.cu).
+template <int NW, int MODE>
+pvt_status launch_local(pvt_dag *g, const CountArgs &base, int cls, cudaStream_t s);
+template <int NW, int MODE>
+pvt_status launch_local_batch(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int,
+                              unsigned *, unsigned long long *, int, cudaStream_t);
 
 // The test-settable limit of the bounded device waits (policy.wait_limit_us).
 static void apply_wait_limit(const pvt_dag *g, CountArgs &A)
@@ -286,9 +282,14 @@ static pvt_status launch_wide(pvt_dag *g, const CountArgs &A, int c, cudaStream_
         if (c == 6 && words <= 20) return launch_class<20, MODE, SH>(g, A, c, s);
         if (c == 6 && words <= 24) return launch_class<24, MODE, SH>(g, A, c, s);
     }
+    if constexpr (MODE == MODE_GLOBAL) {
+        if (c == 2) return launch_class<2, MODE, SH>(g, A, c, s);
+        if (c == 3) return launch_class<4, MODE, SH>(g, A, c, s);
+    } else {
+        if (c == 2) return launch_local<2, MODE>(g, A, c, s);
+        if (c == 3) return g->alpha <= 96 ? launch_local<3, MODE>(g, A, c, s) : launch_local<4, MODE>(g, A, c, s);
+    }
     switch (c) {
-        case 2: return launch_class<2, MODE, SH>(g, A, c, s);
-        case 3: return launch_class<4, MODE, SH>(g, A, c, s);
         case 4: return launch_class<8, MODE, SH>(g, A, c, s);
         case 5: return launch_class<16, MODE, SH>(g, A, c, s);
         default: return launch_class<32, MODE, SH>(g, A, c, s);
@@ -345,7 +346,9 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
         if (!serial) PVT_CK(cudaStreamWaitEvent(cs, g->ev_fork, 0));
         switch (c) {
             case 1:
-                if (gather1) {
+                if constexpr (MODE != MODE_GLOBAL) {
+                    st = launch_local<1, MODE>(g, A0, c, cs);
+                } else if (gather1) {
                     phase_begin(g, 1 + c, cs);
                     st = launch_gather1(g, A, g->wroots + g->wstart[1], (unsigned)pass1, slots1, cs);
                     phase_end(g, 1 + c, cs);
@@ -807,6 +810,7 @@ pvt_status count_local(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *out, bool 
     A.ocol = g->ocol;
     A.oeid = g->oeid;
     A.out = o;
+    A.ksafe = safe_size(g->n, g->alpha);
     A.B = g->binom.p;
     A.Bw = W;
     A.W = W;
@@ -919,9 +923,21 @@ static pvt_status launch_batch_mode(const BatchGraph *gs, const uint64_t *const 
         unsigned long long *stats = reinterpret_cast<unsigned long long *>(ctl + 32);
         switch (c) {
             case 0:
-            case 1: st = launch_batch_class<1, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s); break;
-            case 2: st = launch_batch_class<2, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s); break;
-            case 3: st = launch_batch_class<4, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s); break;
+            case 1:
+                if constexpr (MODE == MODE_GLOBAL)
+                    st = launch_batch_class<1, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s);
+                else st = launch_local_batch<1, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s);
+                break;
+            case 2:
+                if constexpr (MODE == MODE_GLOBAL)
+                    st = launch_batch_class<2, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s);
+                else st = launch_local_batch<2, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s);
+                break;
+            case 3:
+                if constexpr (MODE == MODE_GLOBAL)
+                    st = launch_batch_class<4, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s);
+                else st = launch_local_batch<4, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s);
+                break;
             case 4: st = launch_batch_class<8, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s); break;
             case 5: st = launch_batch_class<16, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s); break;
             default: set_error("batched walk: out-degree above the batched limit"); st = PVT_EINVAL; break;

@@ -94,6 +94,7 @@ struct pvt_dag {
     bool phase_used[pvt::NPHASE] = {};
     pvt::DevBuf<uint32_t> gstack[pvt::NCLASS];  // DFS stacks of the wide classes (global memory)
     pvt::DevBuf<uint32_t> etab[pvt::NCLASS];    // per-warp member-pair edge ids (per-edge counts)
+    pvt::DevBuf<uint32_t> lheavy[pvt::NCLASS];  // dense roots of a local count
     bool hist_valid = false;       // hist holds the leaves of the last completed global count
 };
 
@@ -119,6 +120,7 @@ struct BatchGraph {
     unsigned long long *out = nullptr;   // result: C [K][W], or table [rows][K][W]
     int mode = BATCH_GLOBAL;
     int kmax = 0, W = 1;
+    int ksafe = 0;                       // as CountArgs::ksafe
 };
 
 // Batched orientation: one block per graph (peel, DAG CSR, edge ids for
@@ -140,6 +142,10 @@ pvt_status build_binom(unsigned long long *B, int rows, int W, unsigned *err, cu
 
 // Thread-local error message used by pvt_last_error().
 void set_error(const std::string &msg);
+
+// Largest k for which every count of k-cliques of a graph is below 2^63: there
+// are at most n * C(alpha, k - 1) of them.
+int32_t safe_size(int64_t n, int32_t alpha);
 
 // Words needed so every count fits: each count is at most n * 2^alpha.
 int32_t min_words(int64_t n, int32_t alpha);

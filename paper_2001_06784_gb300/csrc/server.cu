@@ -281,6 +281,7 @@ void run_group(pvt_server *sv, std::vector<ReqPtr> &group)
         G.hstride = r.alpha + 2;
         G.kmax = r.K - 1;
         G.W = r.W;
+        G.ksafe = safe_size(r.n, r.alpha);
         cudaMemsetAsync(G.out, 0, 8 * std::max<size_t>(words, 1), ws);
         if (hwords) cudaMemsetAsync(G.hist, 0, 8 * hwords, ws);
         r.hres = static_cast<uint64_t *>(sv->pinned.get(8 * std::max<size_t>(words, 1), &r.hres_cls));

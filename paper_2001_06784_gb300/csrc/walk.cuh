@@ -144,6 +144,7 @@ struct CountArgs {
     int Bw;                       // words per table entry (>= W)
     int W;
     int kmax;
+    int ksafe;                    // local counts: no count of a size up to this passes 2^64
     unsigned *err;
     unsigned long long *stats;  // [0] nodes, [1] leaves, [2] pivot words, [3 + class] words
     int cls;                    // out-degree class of the launch
@@ -738,47 +739,13 @@ __device__ void walk_compact(WarpWork<NW> &Wk, unsigned *shist, const CountArgs 
     compact_loop<NW, SHIST, SPLIT>(Wk, shist, A, lane, r1, s >= 32 ? FULL : ((1u << s) - 1u), h, p, wc, outer, clk);
 }
 
-// One walk item: a whole root r (frame == nullptr), or a frame of root qi's
-// subtree that another warp donated (split form).
-template <int NW, int MODE, bool SHIST, bool SPLIT>
-__device__ void walk_root(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A, int lane,
-                          uint32_t r, WalkCounters &wc, Emitter &em, unsigned qi = 0, const uint32_t *frame = nullptr)
+// Gather of root r's members N+(r) = ocol[rbeg .. rbeg + d), d <= 32 * NW, by
+// one warp: member ids, their out-list extents, bitset adjacency rows, and
+// (per-edge counts with a table) the edge ids of adjacent members.
+template <int NW, int MODE, typename Work>
+__device__ __forceinline__ void gather_rows(Work &Wk, const CountArgs &A, int lane, int64_t rbeg, int d)
 {
-    Clock clk;
-    constexpr int D = WarpWork<NW>::D;
-    constexpr int RS = WarpWork<NW>::RS;
-    constexpr bool REG = NW <= 4;  // keep this lane's adjacency rows in registers
-    // the member-word loops (32 members a turn) of the wider rows stay rolled:
-    // unrolled they multiply the code by NW, and the walk then waits for
-    // instructions (24 % of its stalls on 8-word rows)
-    constexpr int UNROLL_J = REG ? NW : 1;
-    auto word_of = [&](const uint32_t *X, uint32_t mine, int j) -> uint32_t {
-        return REG ? X[j % (REG ? NW : 1)] : __shfl_sync(FULL, mine, j);
-    };
-    int64_t rbeg = 0;
-    int d = 0;
-    uint32_t S[NW];
-    int h = 1, p = 0;
-    if (SPLIT && frame) {
-        // ---- donated frame: adjacency rows come from the root's published copy
-        d = (int)frame[1];
-        const uint32_t hp0 = frame[2];
-        h = (int)(hp0 >> 16);
-        p = (int)(hp0 & 0xFFFFu);
-#pragma unroll
-        for (int w = 0; w < NW; ++w) S[w] = frame[3 + w];
-        const uint32_t *src = A.rootbuf + (size_t)qi * D * NW;
-        for (int t = lane; t < d * NW; t += 32) Wk.adj[(t / NW) * RS + (t % NW)] = __ldcg(src + t);
-        __syncwarp();
-    } else {
-    rbeg = A.orow[r];
-    d = (int)(A.orow[r + 1] - rbeg);
-    if (d > D) {
-        if (lane == 0) atomicOr(A.err, DERR_RANGE);
-        return;
-    }
-
-    // ---- 1. gather: member ids, their out-list extents, bitset adjacency
+    constexpr int D = Work::D, RS = Work::RS;
     uint32_t base = 0;
 #pragma unroll
     for (int c = 0; c < NW; ++c) {
@@ -816,8 +783,8 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A,
     // labels emitted where they are formed, the wide walks of the 10.8M-edge
     // graph went from 0.62 / 1.10 / 2.28 ms (33..64, 65..128, 129..256) to
     // 0.50 / 0.86 / 1.08 ms.
-    constexpr int FSH = 32 - WarpWork<NW>::FILTER_LOG;
-    for (int t = lane; t < (1 << WarpWork<NW>::FILTER_LOG) / 32; t += 32) Wk.filter[t] = 0;
+    constexpr int FSH = 32 - Work::FILTER_LOG;
+    for (int t = lane; t < (1 << Work::FILTER_LOG) / 32; t += 32) Wk.filter[t] = 0;
     __syncwarp();
     for (int i = lane; i < d; i += 32) {
         const uint32_t hb = (Wk.ids[i] * FIB_HASH) >> FSH;
@@ -891,6 +858,49 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A,
     __syncwarp();
     lookup(nq);
     __syncwarp();
+}
+
+// One walk item: a whole root r (frame == nullptr), or a frame of root qi's
+// subtree that another warp donated (split form).
+template <int NW, int MODE, bool SHIST, bool SPLIT>
+__device__ void walk_root(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A, int lane,
+                          uint32_t r, WalkCounters &wc, Emitter &em, unsigned qi = 0, const uint32_t *frame = nullptr)
+{
+    Clock clk;
+    constexpr int D = WarpWork<NW>::D;
+    constexpr int RS = WarpWork<NW>::RS;
+    constexpr bool REG = NW <= 4;  // keep this lane's adjacency rows in registers
+    // the member-word loops (32 members a turn) of the wider rows stay rolled:
+    // unrolled they multiply the code by NW, and the walk then waits for
+    // instructions (24 % of its stalls on 8-word rows)
+    constexpr int UNROLL_J = REG ? NW : 1;
+    auto word_of = [&](const uint32_t *X, uint32_t mine, int j) -> uint32_t {
+        return REG ? X[j % (REG ? NW : 1)] : __shfl_sync(FULL, mine, j);
+    };
+    int64_t rbeg = 0;
+    int d = 0;
+    uint32_t S[NW];
+    int h = 1, p = 0;
+    if (SPLIT && frame) {
+        // ---- donated frame: adjacency rows come from the root's published copy
+        d = (int)frame[1];
+        const uint32_t hp0 = frame[2];
+        h = (int)(hp0 >> 16);
+        p = (int)(hp0 & 0xFFFFu);
+#pragma unroll
+        for (int w = 0; w < NW; ++w) S[w] = frame[3 + w];
+        const uint32_t *src = A.rootbuf + (size_t)qi * D * NW;
+        for (int t = lane; t < d * NW; t += 32) Wk.adj[(t / NW) * RS + (t % NW)] = __ldcg(src + t);
+        __syncwarp();
+    } else {
+    rbeg = A.orow[r];
+    d = (int)(A.orow[r + 1] - rbeg);
+    if (d > D) {
+        if (lane == 0) atomicOr(A.err, DERR_RANGE);
+        return;
+    }
+
+    gather_rows<NW, MODE>(Wk, A, lane, rbeg, d);
     if (SPLIT) {
         // publish the adjacency rows so that donated frames can be walked anywhere
         uint32_t *dst = A.rootbuf + (size_t)qi * D * NW;

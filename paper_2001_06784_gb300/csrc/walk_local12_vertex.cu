@@ -1,0 +1,15 @@
+// Per-vertex counts with bitsets of 1 and 2 words.
+#include "local.cuh"
+
+namespace pvt {
+
+template pvt_status launch_local<1, MODE_VERTEX>(pvt_dag *, const CountArgs &, int, cudaStream_t);
+template pvt_status launch_local<2, MODE_VERTEX>(pvt_dag *, const CountArgs &, int, cudaStream_t);
+template pvt_status launch_local_batch<1, MODE_VERTEX>(const BatchGraph *, const uint64_t *, unsigned, unsigned *,
+                                                     const unsigned long long *, int, unsigned *,
+                                                     unsigned long long *, int, cudaStream_t);
+template pvt_status launch_local_batch<2, MODE_VERTEX>(const BatchGraph *, const uint64_t *, unsigned, unsigned *,
+                                                     const unsigned long long *, int, unsigned *,
+                                                     unsigned long long *, int, cudaStream_t);
+
+}  // namespace pvt
