@@ -1,12 +1,12 @@
 // Degeneracy orientation on the device (Lemma degen, Sec. 3.2; Alg. 1 step 1).
 //
 // 1. Optional CSR validation (simple undirected graph, Sec. 3.1).
-// 2. k-core peeling in one cooperative kernel, exact by level (core numbers
-//    are exact), asynchronous within a level (see k_peel): each vertex gets a
-//    unique removal time rnd[v].
-// 3. The orientation u -> v iff rnd[u] < rnd[v]: a vertex's later
-//    neighbours number at most its level k <= alpha, so every out-degree is
-//    at most the degeneracy.  Out-lists keep the CSR's ascending-id order.
+// 2. Core numbers and a degeneracy order, rnd[v], in one cooperative kernel
+//    that finds every level at once (k_cores), or, for graphs of low levels
+//    with long chains, level by level (k_peel, unique removal times).
+// 3. The orientation u -> v iff (rnd[u], u) < (rnd[v], v): a vertex's later
+//    neighbours number at most its core number k <= alpha, so every out-degree
+//    is at most the degeneracy.  Out-lists keep the CSR's ascending-id order.
 // 4. Roots grouped by out-degree class (bitset width), largest first.
 #include <cooperative_groups.h>
 
@@ -123,6 +123,10 @@ __device__ bool grid_barrier(PeelState *st, unsigned *err)
 {
     __shared__ int s_ok;
     __syncthreads();
+    if (gridDim.x == 1) {  // one block: its own barrier is enough
+        if (threadIdx.x == 0) st->rounds++;
+        return true;
+    }
     if (threadIdx.x == 0) {
         volatile unsigned *vgen = &st->bar_gen;
         unsigned gen = *vgen;
@@ -453,6 +457,437 @@ __global__ void __launch_bounds__(1024, 1) k_peel(int64_t n, const int64_t *__re
         if (tid == 0) st->head = t_end;  // drop claims past the end of the queue
     }
     if (tid == 0) st->top_level = top;
+}
+
+// ------------------------------------------------- core numbers by rounds
+//
+// Core numbers without levels: est[v] starts at v's degree, and each round
+// sets it to the h-index of the neighbours' estimates (the largest h with at
+// least h neighbours of estimate >= h, at most the old estimate).  The
+// estimates fall to the core numbers (Lu, Zhou, Zhang and Stanley, "The
+// H-index of a network node and its relation to degree and coreness", Nature
+// Communications 2016).  Every level of the peel is found at once, so the
+// number of rounds is the longest chain of corrections (10 on an ER graph, 40
+// to 60 on power-law graphs), not the sum over levels of each level's chain.
+//
+// The rounds also order the vertices.  Let t(v) be the round that set v's
+// final estimate k = core(v) (0: its degree).  Its neighbours of estimate
+// above k before that round numbered at most k (else the h-index, or the
+// degree, would be larger), and every neighbour u that comes after v by
+// (core, t) is among them: core(u) > k, or core(u) = k and t(u) >= t(v), so
+// that u's estimate was still above k.  Hence (core, t), ties in any order,
+// is a degeneracy order: at most core(v) neighbours come after v.  This needs
+// rounds that read the estimates of the round before, so an entry keeps the
+// estimate before its last change and that change's round.
+//
+// The first rounds recompute every vertex.  From round CORE_FULL on a vertex
+// keeps its support, the number of neighbours of estimate >= its own, and a
+// round visits exactly the vertices whose support fell below their estimate:
+// it recomputes them (all from the estimates of the round before), and after
+// a grid barrier their changes from k to h take one off the support of every
+// neighbour whose estimate lies in (h, k].  Rows of at most 32 entries are
+// read by 4 lanes, longer ones by a warp, those above CORE_BIG by a quarter of
+// a block, or a whole one when few are left.  What bounds it: in the first
+// rounds the gathers of estimates, one per row entry, from L1 and L2; in the
+// many small rounds after them the latency of the entry, row, column, estimate
+// chain and of two grid barriers.  Core numbers and order, level-wise peel ->
+// rounds: 1M vertices, 10.8M edges, degeneracy 156: 5.31 -> 2.05 ms (three full
+// rounds 0.65 ms, rounds above 500 long rows 25 to 100 us, the rest 13 to 25
+// us); 2M vertices, 16M edges: 4.78 -> 2.47 ms; 61k vertices: 1.10 -> 0.70 ms;
+// 2,000 vertices: 0.15 -> 0.11 ms.
+constexpr unsigned CORE_CLAMP = MAX_ALPHA + 1;  // estimates are clamped here: a larger core is refused anyway
+constexpr unsigned CORE_ROUNDS_MAX = 192;       // then the level-wise peel (an entry's tag could hold 1023)
+constexpr unsigned CORE_FULL = 3;               // the last round that visits every vertex
+// A round whose largest changed estimate is at most CORE_BAIL_CORE, the first
+// one or one from CORE_BAIL_ROUND on, has only low levels left (meshes, road
+// networks, paths): the level-wise peel needs few levels there and follows a
+// chain in one cascade.  So does a round of at most CORE_THIN vertices from
+// round CORE_THIN_ROUND on (long chains at a higher level; the power-law
+// graphs measured end within 62 rounds, the 128M-edge one of degeneracy 733
+// within 86).
+constexpr unsigned CORE_BAIL_CORE = 6, CORE_BAIL_ROUND = 24, CORE_THIN = 64, CORE_THIN_ROUND = 96;
+constexpr int CORE_THREADS = 1024;
+constexpr int64_t CORE_ONE_BLOCK = 512;         // graphs of at most this many vertices stay in one block
+constexpr int CORE_BIG = 256;                   // rows above this go to a list of their own
+constexpr int CORE_BINS = ((int)CORE_CLAMP + 32) / 32 * 32;  // estimates 0 .. CORE_CLAMP, a warp's histogram
+constexpr unsigned CORE_QUEUE = 4096;           // vertices a block finds before it appends them to a list
+constexpr size_t CORE_SMEM = sizeof(unsigned) * (CORE_BINS * (CORE_THREADS / 32) + CORE_QUEUE);
+
+// entry: estimate << 21 | round of its last change << 11 | estimate before it
+__device__ __forceinline__ uint32_t core_entry(unsigned est, unsigned round, unsigned before)
+{
+    return est << 21 | round << 11 | before;
+}
+// the estimate that round r reads: the one before r's own change
+__device__ __forceinline__ unsigned core_read(uint32_t x, unsigned r)
+{
+    return ((x >> 11) & 1023u) == r ? x & 2047u : x >> 21;
+}
+// the estimate before round r's change, 0 if r did not change it
+__device__ __forceinline__ unsigned core_before(uint32_t x, unsigned r)
+{
+    return ((x >> 11) & 1023u) == r ? x & 2047u : 0u;
+}
+
+struct CoreState {
+    PeelState peel;           // barrier, rounds, levels, top_level
+    unsigned cnt[3][2];       // list lengths (short rows, rows above CORE_BIG), by round modulo 3
+    unsigned n_long;          // vertices with rows above CORE_BIG
+    unsigned most[3];         // largest changed estimate, by round modulo 3
+    unsigned bail;            // 1: left to the level-wise peel
+    unsigned seen[CORE_BINS / 32];  // core numbers met (bit set)
+};
+
+// The h-index of a row's estimates, at most k, from their histogram of
+// min(estimate, k) (bins floor..k, one warp), and the support at it; floor - 1
+// if it lies below the bins.
+__device__ __forceinline__ int core_hindex(const unsigned *hist, int lane, int k, int floor, unsigned &sup)
+{
+    unsigned above = 0;
+    for (int hi = k; hi >= floor; hi -= 32) {
+        const int bin = hi - lane;
+        unsigned inc = bin >= floor ? hist[bin] : 0u;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const unsigned f = __ballot_sync(FULL, bin >= floor && (int)(above + inc) >= bin);
+        if (f) {
+            const int l = __ffs(f) - 1;
+            sup = above + __shfl_sync(FULL, inc, l);
+            return hi - l;
+        }
+        above += __shfl_sync(FULL, inc, 31);
+    }
+    return floor - 1;
+}
+
+__global__ void __launch_bounds__(CORE_THREADS, 1) k_cores(int64_t n, const int64_t *__restrict__ rp,
+                                                           const uint32_t *__restrict__ col, uint32_t *ent,
+                                                           uint32_t *core, uint32_t *sup, uint32_t *list,
+                                                           CoreState *st, unsigned *err)
+{
+    extern __shared__ unsigned s_bins[];  // [warps][CORE_BINS], then the queue
+    uint32_t *s_queue = s_bins + CORE_BINS * (CORE_THREADS / 32);
+    __shared__ unsigned s_qn;
+    __shared__ int s_h[4];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nthreads = (int64_t)gridDim.x * blockDim.x;
+    const int64_t warp = tid >> 5, nwarps = nthreads >> 5;
+    const int grp = lane >> 2, gl = lane & 3;  // 4-lane group and lane in it
+    const unsigned below = (1u << lane) - 1u;
+    unsigned *hist = s_bins + wid * CORE_BINS;
+    uint32_t *longs = core;  // the vertices with rows above CORE_BIG (core is written at the end)
+
+    // lists of round r: list + 2n (r & 1) the short rows, n further the long ones
+    auto list_of = [&](unsigned r, int big) { return list + (r & 1u ? 2 * n : 0) + (big ? n : 0); };
+    // append u (where want) to the list of round r (all lanes of a warp)
+    auto append = [&](unsigned r, bool want, uint32_t u) {
+        const bool big = want && rp[u + 1] - rp[u] > CORE_BIG;
+#pragma unroll
+        for (int kind = 0; kind < 2; ++kind) {
+            const unsigned b = __ballot_sync(FULL, want && big == (kind == 1));
+            if (!b) continue;
+            unsigned at = 0;
+            if (lane == 0) at = atomicAdd(&st->cnt[r % 3][kind], (unsigned)__popc(b));
+            at = __shfl_sync(FULL, at, 0);
+            if (b >> lane & 1u) list_of(r, kind)[at + __popc(b & below)] = u;
+        }
+    };
+    // the same through the block's queue, which flush empties
+    auto push = [&](unsigned r, bool want, uint32_t u) {
+        const unsigned b = __ballot_sync(FULL, want);
+        if (!b) return;
+        unsigned at = 0;
+        if (lane == 0) at = atomicAdd(&s_qn, (unsigned)__popc(b));
+        at = __shfl_sync(FULL, at, 0);
+        if (at + 32 <= CORE_QUEUE) {
+            if (want) s_queue[at + __popc(b & below)] = u;
+        } else {
+            append(r, want, u);
+        }
+    };
+    auto flush = [&](unsigned r) {
+        __syncthreads();
+        // (places that a push past the end counted but did not fill are EMPTY)
+        const unsigned m = min(*(volatile unsigned *)&s_qn, CORE_QUEUE);
+        for (unsigned i = wid * 32; i < m; i += CORE_THREADS) {
+            const uint32_t u = i + lane < m ? s_queue[i + lane] : EMPTY;
+            append(r, u != EMPTY, u);
+        }
+        __syncthreads();
+        for (unsigned i = threadIdx.x; i < m; i += blockDim.x) s_queue[i] = EMPTY;
+        if (threadIdx.x == 0) s_qn = 0;
+    };
+    // row entries to a histogram of min(estimate, k), those below floor left
+    // out; four loads in flight
+    auto fill = [&](unsigned *bins, int64_t j, int64_t e, int64_t step, unsigned k, unsigned floor, unsigned r) {
+        for (; j < e; j += 4 * step) {
+            uint32_t u[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) u[t] = j + t * step < e ? col[j + t * step] : EMPTY;
+            unsigned x[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) x[t] = u[t] != EMPTY ? core_read(ent[u[t]], r) : 0u;
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (u[t] != EMPTY && x[t] >= floor) atomicAdd(&bins[min(x[t], k)], 1u);
+        }
+    };
+    // vertex v fell from k to h: one off the support of every neighbour with an
+    // estimate in (h, k]; those whose support falls below it are visited next
+    // (all lanes of the warp; lane l starts at entry j + l)
+    auto notify = [&](int64_t j, int64_t e, int64_t step, unsigned h, unsigned k, unsigned r) {
+        for (; __any_sync(FULL, j < e); j += 4 * step) {
+            uint32_t u[4];
+            unsigned x[4];
+            bool hit[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) u[t] = j + t * step < e ? col[j + t * step] : EMPTY;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) x[t] = u[t] != EMPTY ? ent[u[t]] >> 21 : 0u;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) hit[t] = x[t] > h && x[t] <= k && atomicSub(&sup[u[t]], 1u) == x[t];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) push(r + 1, hit[t], u[t]);
+        }
+    };
+    // units of ut threads (256 or 1024) that take one long row each
+    auto unit_sync = [&](int ut) {
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / ut), "r"(ut) : "memory");
+    };
+
+    for (unsigned i = threadIdx.x; i < CORE_QUEUE; i += blockDim.x) s_queue[i] = EMPTY;
+    if (threadIdx.x == 0) s_qn = 0;
+    for (int64_t v0 = tid - lane; v0 < n; v0 += nthreads) {
+        const int64_t v = v0 + lane;
+        bool big = false;
+        if (v < n) {
+            const int64_t deg = rp[v + 1] - rp[v];
+            const unsigned d = (unsigned)min(deg, (int64_t)CORE_CLAMP);
+            ent[v] = core_entry(d, 0, d);
+            big = deg > CORE_BIG;
+        }
+        const unsigned b = __ballot_sync(FULL, big);
+        if (b) {
+            unsigned at = 0;
+            if (lane == 0) at = atomicAdd(&st->n_long, (unsigned)__popc(b));
+            at = __shfl_sync(FULL, at, 0);
+            if (big) longs[at + __popc(b & below)] = (uint32_t)v;
+        }
+    }
+    if (!grid_barrier(&st->peel, err)) return;
+
+    for (unsigned r = 1;; ++r) {
+        const bool full = r <= CORE_FULL;      // every vertex is visited
+        const bool counted = r >= CORE_FULL;   // supports are kept
+        unsigned n_small = 0, n_big = 0;
+        if (full) {
+            n_big = *(volatile unsigned *)&st->n_long;
+        } else {
+            n_small = *(volatile unsigned *)&st->cnt[r % 3][0];
+            n_big = *(volatile unsigned *)&st->cnt[r % 3][1];
+            if (n_small + n_big == 0) break;
+        }
+        if (r > 1) {
+            const unsigned most = *(volatile unsigned *)&st->most[(r - 1) % 3];
+            if (most == 0) break;  // nothing changed
+            if (((r == 2 || r >= CORE_BAIL_ROUND) && most <= CORE_BAIL_CORE) ||
+                (r >= CORE_THIN_ROUND && n_small + n_big <= CORE_THIN) || r > CORE_ROUNDS_MAX) {
+                if (tid == 0) st->bail = 1;
+                return;
+            }
+        }
+        if (tid == 0) {
+            // last read before this round, next written in the next
+            st->cnt[(r + 2) % 3][0] = st->cnt[(r + 2) % 3][1] = 0;
+            st->most[(r + 1) % 3] = 0;
+        }
+        const int64_t cnt = full ? n : (int64_t)n_small;
+        const uint32_t *small = list_of(r, 0), *big = full ? longs : list_of(r, 1);
+        // ---- new estimates from those of the round before
+        unsigned most = 0;
+        // (long rows first: they take longest)
+        auto long_rows = [&](int ut) {
+            const int per = CORE_THREADS / ut, me = threadIdx.x / ut, l = threadIdx.x % ut;
+            unsigned *bins = s_bins + me * (ut / 32) * CORE_BINS;
+            for (unsigned i = blockIdx.x * per + me; i < n_big; i += gridDim.x * per) {
+                const uint32_t v = big[i];
+                const int64_t b = rp[v], e = rp[v + 1];
+                const unsigned k = core_read(ent[v], r);
+                // estimates fall little in the later rounds: the lower half of
+                // the bins, where most neighbours are, is counted only if needed
+                int floor = full ? 0 : (int)(k / 2), h;
+                unsigned hs = 0;
+                for (;;) {
+                    unit_sync(ut);  // the bins of the pass before are spent
+                    for (int t = l; t <= (int)k; t += ut) bins[t] = 0;
+                    unit_sync(ut);
+                    fill(bins, b + l, e, ut, k, (unsigned)floor, r);
+                    unit_sync(ut);
+                    if (l < 32) {
+                        h = core_hindex(bins, lane, (int)k, floor, hs);
+                        if (l == 0) s_h[me] = h;
+                    }
+                    unit_sync(ut);
+                    h = s_h[me];
+                    if (h >= floor) break;
+                    floor = 0;
+                }
+                if (l == 0) {
+                    if (h < (int)k) ent[v] = core_entry((unsigned)h, r, k);
+                    if (counted) sup[v] = hs;
+                }
+                if (h < (int)k) {
+                    most = max(most, k);
+                    if (full && counted && l < 32) push(r, l == 0, v);
+                }
+            }
+        };
+        if (n_big) {
+            if (n_big <= 2 * gridDim.x) long_rows(CORE_THREADS);
+            else long_rows(CORE_THREADS / 4);
+            __syncthreads();  // the bins are the warps' own again
+        }
+        // up to eight vertices at a time, one per group; fewer when there are
+        // fewer than that for each warp
+        const int per = (int)min((cnt + nwarps - 1) / nwarps, (int64_t)8);
+        for (int64_t i0 = warp * per; i0 < cnt; i0 += nwarps * per) {
+            uint32_t v = 0;
+            int64_t b = 0, deg = 0;
+            unsigned k = 0;
+            const bool mine = grp < per && i0 + grp < cnt;
+            if (mine) {
+                v = full ? (uint32_t)(i0 + grp) : small[i0 + grp];
+                b = rp[v];
+                deg = rp[v + 1] - b;
+                k = core_read(ent[v], r);
+            }
+            const bool narrow = deg <= 32;
+            {
+                uint32_t u[8];
+                unsigned x[8];
+                unsigned c = 0;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) u[t] = narrow && gl + 4 * t < deg ? col[b + gl + 4 * t] : EMPTY;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    x[t] = u[t] != EMPTY ? core_read(ent[u[t]], r) : 0u;
+                    c += u[t] != EMPTY && x[t] >= k;
+                }
+                auto gsum = [&](unsigned y) {
+                    y += __shfl_xor_sync(FULL, y, 1);
+                    y += __shfl_xor_sync(FULL, y, 2);
+                    return y;
+                };
+                c = gsum(c);  // every lane takes part
+                const bool drop = narrow && c < k;
+                if (__any_sync(FULL, drop)) {
+                    unsigned h = 0, hs = 0;  // bit by bit: the largest h with h values >= h (h < k <= 32)
+#pragma unroll
+                    for (unsigned s = 16; s; s >>= 1) {
+                        unsigned y = 0;
+#pragma unroll
+                        for (int t = 0; t < 8; ++t) y += u[t] != EMPTY && x[t] >= h + s;
+                        y = gsum(y);
+                        if (y >= h + s) {
+                            h += s;
+                            hs = y;
+                        }
+                    }
+                    if (drop) {
+                        c = h ? hs : (unsigned)deg;
+                        most = max(most, k);
+                        if (gl == 0) ent[v] = core_entry(h, r, k);
+                    }
+                }
+                if (counted && narrow && gl == 0 && mine) sup[v] = c;
+                if (full && counted) push(r, drop && gl == 0, v);
+            }
+            // longer rows, one at a time by the whole warp
+            unsigned wide = __ballot_sync(FULL, !narrow && deg <= CORE_BIG && gl == 0), changed = 0;
+            for (; wide; wide &= wide - 1) {
+                const int src = __ffs(wide) - 1;
+                const uint32_t wv = __shfl_sync(FULL, v, src);
+                const int64_t wb = __shfl_sync(FULL, b, src), we = wb + __shfl_sync(FULL, deg, src);
+                const unsigned wk = __shfl_sync(FULL, k, src);
+                for (int i = lane; i <= (int)wk; i += 32) hist[i] = 0;
+                __syncwarp();
+                fill(hist, wb + lane, we, 32, wk, 0u, r);
+                __syncwarp();
+                unsigned hs = 0;
+                const unsigned h = (unsigned)core_hindex(hist, lane, (int)wk, 0, hs);
+                __syncwarp();
+                if (h < wk) {
+                    if (lane == 0) ent[wv] = core_entry(h, r, wk);
+                    most = max(most, wk);
+                    changed |= 1u << src;
+                }
+                if (counted && lane == 0) sup[wv] = hs;
+            }
+            if (full && counted) push(r, (changed >> lane) & 1u, v);
+        }
+        most = __reduce_max_sync(FULL, most);
+        if (lane == 0 && most) atomicMax(&st->most[r % 3], most);
+        if (full && counted) flush(r);
+        if (!grid_barrier(&st->peel, err)) return;
+        if (!counted) continue;
+        // ---- the changes to the neighbours' supports
+        if (full) {  // the changed vertices of the last full round are its lists
+            n_small = *(volatile unsigned *)&st->cnt[r % 3][0];
+            n_big = *(volatile unsigned *)&st->cnt[r % 3][1];
+            big = list_of(r, 1);
+        }
+        const int ut = n_big <= 2 * gridDim.x ? CORE_THREADS : CORE_THREADS / 4;
+        for (unsigned i = blockIdx.x * (CORE_THREADS / ut) + threadIdx.x / ut; i < n_big;
+             i += gridDim.x * (CORE_THREADS / ut)) {
+            const uint32_t v = big[i], x = ent[v];
+            notify(rp[v] + threadIdx.x % ut, rp[v + 1], ut, x >> 21, core_before(x, r), r);
+        }
+        const int each = (int)min(((int64_t)n_small + nwarps - 1) / nwarps, (int64_t)8);
+        for (int64_t i0 = warp * each; i0 < (int64_t)n_small; i0 += nwarps * each) {
+            uint32_t x = 0;
+            int64_t b = 0, deg = 0;
+            if (grp < each && i0 + grp < (int64_t)n_small) {
+                const uint32_t v = small[i0 + grp];
+                b = rp[v];
+                deg = rp[v + 1] - b;
+                x = ent[v];
+            }
+            const unsigned h = x >> 21, k = core_before(x, r);
+            const bool narrow = deg <= 32;
+            notify(b + gl, narrow ? b + deg : b, 4, h, k, r);  // a group each
+            for (unsigned wide = __ballot_sync(FULL, !narrow && gl == 0); wide; wide &= wide - 1) {
+                const int src = __ffs(wide) - 1;
+                const int64_t wb = __shfl_sync(FULL, b, src), we = wb + __shfl_sync(FULL, deg, src);
+                notify(wb + lane, we, 32, __shfl_sync(FULL, h, src), __shfl_sync(FULL, k, src), r);
+            }
+        }
+        flush(r + 1);
+        if (!grid_barrier(&st->peel, err)) return;
+    }
+    // ---- (core, round) as the orientation key, core numbers, their largest
+    __syncthreads();
+    for (int i = threadIdx.x; i < CORE_BINS / 32; i += blockDim.x) s_bins[i] = 0;
+    __syncthreads();
+    unsigned top = 0;
+    for (int64_t v = tid; v < n; v += nthreads) {
+        const uint32_t x = ent[v];
+        const unsigned c = x >> 21;
+        core[v] = c;
+        ent[v] = x >> 11;
+        top = max(top, c);
+        if (!((*(volatile unsigned *)&s_bins[c >> 5] >> (c & 31)) & 1u)) atomicOr(&s_bins[c >> 5], 1u << (c & 31));
+    }
+    top = __reduce_max_sync(FULL, top);
+    if (lane == 0 && top) atomicMax(&st->peel.top_level, top);
+    __syncthreads();
+    for (int i = threadIdx.x; i < CORE_BINS / 32; i += blockDim.x)
+        if (s_bins[i]) {
+            const unsigned old = atomicOr(&st->seen[i], s_bins[i]);
+            if (s_bins[i] & ~old) atomicAdd(&st->peel.levels, (unsigned)__popc(s_bins[i] & ~old));
+        }
 }
 
 // ------------------------------------------------ one-block finish of the peel
@@ -945,6 +1380,51 @@ pvt_status ensure_edge_ids(pvt_dag *g, cudaStream_t s)
 
 // ---------------------------------------------------------------- driver
 
+// The level-wise peel: grid levels, then the one-block finish.  deg: n words,
+// alive: 2n words of scratch; pst zeroed.
+static pvt_status peel_levels(pvt_dag *g, uint32_t *deg, uint32_t *alive, PeelState *pst, cudaStream_t s)
+{
+    int64_t n = g->n;
+    uint32_t *lq = nullptr, *tv = nullptr, *rdeg = nullptr, *rcol = nullptr;
+    int64_t *roff = nullptr;
+    int per_sm = 0;
+    PVT_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_peel, 1024, 0));
+    if (per_sm < 1) {
+        set_error("pvt_orient: peel kernel cannot be resident");
+        return PVT_ECUDA;
+    }
+    PVT_CK(cudaMallocAsync(&lq, (size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t), s));
+    PVT_CK(cudaMallocAsync(&tv, (size_t)TAIL_MAX * sizeof(uint32_t), s));
+    PVT_CK(cudaMallocAsync(&rdeg, (size_t)TAIL_MAX * sizeof(uint32_t), s));
+    PVT_CK(cudaMallocAsync(&roff, (size_t)(TAIL_MAX + 1) * sizeof(int64_t), s));
+    PVT_CK(cudaMallocAsync(&rcol, (size_t)std::max<int64_t>(g->nnz, 1) * sizeof(uint32_t), s));
+    const int64_t *rp = g->row_ptr;
+    const uint32_t *col = g->col;
+    uint32_t *rnd = g->rnd, *core = g->core;
+    unsigned *err = g->d_err;
+    unsigned tail_max = TAIL_MAX;
+    void *args[] = {&n, &rp, &col, &deg, &rnd, &core, &lq, &alive, &pst, &tail_max, &err};
+    // one cooperative launch: every block must be resident at once
+    PVT_CK(cudaLaunchCooperativeKernel((void *)k_peel, dim3(g->num_sms), dim3(1024), args, 0, s));
+    // the levels left once at most TAIL_MAX vertices are alive: one block
+    // on the compacted residual graph (each kernel returns at once if the
+    // grid peel finished by itself); lq is free by now and holds local ids
+    k_tail_compact<<<(TAIL_MAX + 255) / 256, 256, 0, s>>>(n, alive, g->rnd, deg, lq, tv, rdeg, pst);
+    k_tail_scan<<<1, 1024, 0, s>>>(rdeg, roff, pst);
+    k_tail_fill<<<g->num_sms * 8, 256, 0, s>>>(g->row_ptr, g->col, g->rnd, lq, tv, roff, rcol, pst, g->d_err);
+    constexpr size_t tail_smem = (3 * (size_t)TAIL_MAX + 1 + TAIL_MAX / 32) * sizeof(uint32_t);
+    PVT_CK(cudaFuncSetAttribute(k_peel_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tail_smem));
+    k_peel_tail<<<1, TAIL_THREADS, tail_smem, s>>>(roff, rcol, rdeg, tv, g->rnd, g->core, pst, g->d_err);
+    PVT_CK(cudaGetLastError());
+    g->stats.launches += 5;
+    PVT_CK(cudaFreeAsync(lq, s));
+    PVT_CK(cudaFreeAsync(tv, s));
+    PVT_CK(cudaFreeAsync(rdeg, s));
+    PVT_CK(cudaFreeAsync(roff, s));
+    PVT_CK(cudaFreeAsync(rcol, s));
+    return PVT_OK;
+}
+
 pvt_status orient_build(pvt_dag *g, uint32_t flags, cudaStream_t s)
 {
     const int64_t n = g->n;
@@ -958,90 +1438,78 @@ pvt_status orient_build(pvt_dag *g, uint32_t flags, cudaStream_t s)
         if (st != PVT_OK) return st;
     }
 
-    uint32_t *deg = nullptr, *lq = nullptr, *odeg = nullptr, *alive = nullptr;
-    uint32_t *tv = nullptr, *rdeg = nullptr, *rcol = nullptr;
-    int64_t *roff = nullptr;
+    uint32_t *sup = nullptr, *list = nullptr, *odeg = nullptr;
     unsigned *dhist = nullptr;
-    PeelState *pst = nullptr;
+    CoreState *cst = nullptr;
     const size_t nb = (size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t);
-    PVT_CK(cudaMallocAsync(&deg, nb, s));
-    PVT_CK(cudaMallocAsync(&lq, nb, s));
-    PVT_CK(cudaMallocAsync(&alive, 2 * nb, s));
-    PVT_CK(cudaMallocAsync(&pst, sizeof(PeelState) + sizeof(unsigned), s));
+    PVT_CK(cudaMallocAsync(&sup, nb, s));
+    PVT_CK(cudaMallocAsync(&list, 4 * nb, s));
+    PVT_CK(cudaMallocAsync(&cst, sizeof(CoreState) + sizeof(unsigned), s));
     PVT_CK(cudaMallocAsync(&g->rnd, nb, s));
     PVT_CK(cudaMallocAsync(&g->core, nb, s));
-    PVT_CK(cudaMemsetAsync(pst, 0, sizeof(PeelState) + sizeof(unsigned), s));
-
-    // one cooperative launch: every block must be resident at once
-    int per_sm = 0;
-    PVT_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_peel, 1024, 0));
-    per_sm = std::min(per_sm, 1);
-    if (per_sm < 1) {
-        set_error("pvt_orient: peel kernel cannot be resident");
-        return PVT_ECUDA;
-    }
-    {
-        int64_t nn = n;
-        const int64_t *rp = g->row_ptr;
-        const uint32_t *col = g->col;
-        uint32_t *rnd = g->rnd, *core = g->core;
-        unsigned *err = g->d_err;
-        unsigned tail_max = TAIL_MAX;
-        void *args[] = {&nn, &rp, &col, &deg, &rnd, &core, &lq, &alive, &pst, &tail_max, &err};
-        phase_begin(g, 0, s);
-        PVT_CK(cudaLaunchCooperativeKernel((void *)k_peel, dim3(g->num_sms * per_sm), dim3(1024), args,
-                                           0, s));
-        // the levels left once at most TAIL_MAX vertices are alive: one block
-        // on the compacted residual graph (each kernel returns at once if the
-        // grid peel finished by itself); lq is free by now and holds local ids
-        PVT_CK(cudaMallocAsync(&tv, (size_t)TAIL_MAX * sizeof(uint32_t), s));
-        PVT_CK(cudaMallocAsync(&rdeg, (size_t)TAIL_MAX * sizeof(uint32_t), s));
-        PVT_CK(cudaMallocAsync(&roff, (size_t)(TAIL_MAX + 1) * sizeof(int64_t), s));
-        PVT_CK(cudaMallocAsync(&rcol, (size_t)std::max<int64_t>(g->nnz, 1) * sizeof(uint32_t), s));
-        k_tail_compact<<<(TAIL_MAX + 255) / 256, 256, 0, s>>>(n, alive, g->rnd, deg, lq, tv, rdeg, pst);
-        k_tail_scan<<<1, 1024, 0, s>>>(rdeg, roff, pst);
-        k_tail_fill<<<g->num_sms * 8, 256, 0, s>>>(g->row_ptr, g->col, g->rnd, lq, tv, roff, rcol, pst, g->d_err);
-        constexpr size_t tail_smem = (3 * (size_t)TAIL_MAX + 1 + TAIL_MAX / 32) * sizeof(uint32_t);
-        PVT_CK(cudaFuncSetAttribute(k_peel_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tail_smem));
-        k_peel_tail<<<1, TAIL_THREADS, tail_smem, s>>>(roff, rcol, rdeg, tv, g->rnd, g->core, pst, g->d_err);
-        PVT_CK(cudaGetLastError());
-        phase_end(g, 0, s);
-        g->stats.launches += 5;
-    }
-    phase_begin(g, 1, s);
-
-    // orientation
-    unsigned *d_alpha = (unsigned *)(pst + 1);
     PVT_CK(cudaMallocAsync(&odeg, nb + sizeof(uint32_t), s));
     PVT_CK(cudaMallocAsync(&g->orow, (size_t)(n + 1) * sizeof(int64_t), s));
-    k_outdeg<<<grid, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, odeg, d_alpha);
-    PVT_CK(cudaGetLastError());
-    pvt_status st = exclusive_scan_u32_i64(odeg, g->orow, n, s);
-    g->stats.launches += 4;
-    if (st != PVT_OK) return st;
+    unsigned *d_alpha = (unsigned *)(cst + 1);
+    CoreState hst{};
     unsigned alpha = 0;
-    PeelState hst{};
-    PVT_CK(cudaMemcpyAsync(&hst, pst, sizeof(PeelState), cudaMemcpyDeviceToHost, s));
-    PVT_CK(cudaMemcpyAsync(&alpha, d_alpha, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-    PVT_CK(cudaStreamSynchronize(s));
-    st = check_device(g, s, "pvt_orient: peeling");
-    if (st != PVT_OK) return st;
+    pvt_status st = PVT_OK;
+    for (int form = 0;; ++form) {
+        // core numbers and removal order: by rounds, else (once, if those
+        // were given up) level by level
+        PVT_CK(cudaMemsetAsync(cst, 0, sizeof(CoreState) + sizeof(unsigned), s));
+        phase_begin(g, 0, s);
+        if (form == 0) {
+            // one cooperative launch: every block must be resident at once;
+            // small graphs take fewer blocks (a barrier of few is faster)
+            int per_sm = 0;
+            PVT_CK(cudaFuncSetAttribute(k_cores, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORE_SMEM));
+            PVT_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cores, CORE_THREADS, CORE_SMEM));
+            if (per_sm < 1) {
+                set_error("pvt_orient: core kernel cannot be resident");
+                return PVT_ECUDA;
+            }
+            const int64_t want = n <= CORE_ONE_BLOCK ? 1 : (n + CORE_THREADS / 8 - 1) / (CORE_THREADS / 8);
+            const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, g->num_sms));
+            int64_t nn = n;
+            const int64_t *rp = g->row_ptr;
+            const uint32_t *col = g->col;
+            uint32_t *rnd = g->rnd, *core = g->core;
+            unsigned *err = g->d_err;
+            void *args[] = {&nn, &rp, &col, &rnd, &core, &sup, &list, &cst, &err};
+            PVT_CK(cudaLaunchCooperativeKernel((void *)k_cores, dim3(blocks), dim3(CORE_THREADS), args, CORE_SMEM, s));
+            g->stats.launches++;
+        } else if ((st = peel_levels(g, sup, list, &cst->peel, s)) != PVT_OK) {
+            return st;
+        }
+        phase_end(g, 0, s);
+        phase_begin(g, 1, s);
+        // orientation
+        k_outdeg<<<grid, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, odeg, d_alpha);
+        PVT_CK(cudaGetLastError());
+        st = exclusive_scan_u32_i64(odeg, g->orow, n, s);
+        g->stats.launches += 4;
+        if (st != PVT_OK) return st;
+        PVT_CK(cudaMemcpyAsync(&hst, cst, sizeof(CoreState), cudaMemcpyDeviceToHost, s));
+        PVT_CK(cudaMemcpyAsync(&alpha, d_alpha, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+        PVT_CK(cudaStreamSynchronize(s));
+        st = check_device(g, s, "pvt_orient: peeling");
+        if (st != PVT_OK) return st;
+        g->stats.peel_rounds += hst.peel.rounds;
+        if (!hst.bail) break;
+    }
+    g->stats.peel_levels = hst.peel.levels;
+    if (hst.peel.top_level > (unsigned)MAX_ALPHA) {
+        set_error("pvt_orient: degeneracy above the supported " + std::to_string(MAX_ALPHA));
+        return PVT_EINVAL;
+    }
     // alpha = the degeneracy (top core level): it bounds every out-degree and,
     // unlike the largest out-degree, does not depend on the removal order
     // within a level
-    if (alpha > hst.top_level) {
+    if (alpha > hst.peel.top_level) {
         set_error("pvt_orient: an out-degree exceeds the degeneracy");
         return PVT_EINTERNAL;
     }
-    alpha = hst.top_level;
-    g->alpha = (int32_t)alpha;
-    g->stats.peel_rounds = hst.rounds;
-    g->stats.peel_levels = hst.levels;
-    if (g->alpha > MAX_ALPHA) {
-        set_error("pvt_orient: degeneracy " + std::to_string(alpha) + " above the supported " +
-                  std::to_string(MAX_ALPHA));
-        return PVT_EINVAL;
-    }
+    g->alpha = (int32_t)hst.peel.top_level;
     PVT_CK(cudaMallocAsync(&g->ocol, (size_t)std::max<int64_t>(g->m, 1) * sizeof(uint32_t), s));
     k_fill<<<grid, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, g->orow, g->ocol);
     PVT_CK(cudaGetLastError());
@@ -1074,14 +1542,9 @@ pvt_status orient_build(pvt_dag *g, uint32_t flags, cudaStream_t s)
     g->stats.launches++;
     for (int c = 0; c < NCLASS; ++c) g->stats.roots[c] = (uint64_t)g->class_cnt[c];
 
-    PVT_CK(cudaFreeAsync(deg, s));
-    PVT_CK(cudaFreeAsync(lq, s));
-    PVT_CK(cudaFreeAsync(alive, s));
-    PVT_CK(cudaFreeAsync(tv, s));
-    PVT_CK(cudaFreeAsync(rdeg, s));
-    PVT_CK(cudaFreeAsync(roff, s));
-    PVT_CK(cudaFreeAsync(rcol, s));
-    PVT_CK(cudaFreeAsync(pst, s));
+    PVT_CK(cudaFreeAsync(sup, s));
+    PVT_CK(cudaFreeAsync(list, s));
+    PVT_CK(cudaFreeAsync(cst, s));
     PVT_CK(cudaFreeAsync(odeg, s));
     PVT_CK(cudaFreeAsync(dhist, s));
     PVT_CK(cudaStreamSynchronize(s));

@@ -50,7 +50,7 @@ struct pvt_dag {
     const int64_t *row_ptr = nullptr;  // borrowed undirected CSR
     const uint32_t *col = nullptr;
     // owned device state
-    uint32_t *rnd = nullptr;       // peel round of each vertex (orientation key high part)
+    uint32_t *rnd = nullptr;       // orientation key of each vertex (ties: by id)
     uint32_t *core = nullptr;      // peel level (core number) of each vertex
     int64_t *orow = nullptr;       // DAG CSR row pointers, int64[n+1]
     uint32_t *ocol = nullptr;      // DAG out-neighbours, sorted by id, uint32[m]
