@@ -262,7 +262,7 @@ pvt_status pvt_measure_popc_rate(double *pairs_per_s, void *stream);
  *               whose warps take roots from a device work queue (largest
  *               out-degree first); 0: the plain form, one warp per root and
  *               one launch per class.
- *   chunk       roots taken per queue access in the <=32 class (1..32,
+ *   chunk       roots taken at most per queue access in the <=32 class (1..32,
  *               default 4); ignored by the plain form.
  *   split[c]    per out-degree class c (0, <=32, ..., <=1024): 1 lets the
  *               warps of a global count share the subtrees of heavy roots

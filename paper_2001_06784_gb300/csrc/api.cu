@@ -1,6 +1,9 @@
 // C ABI entry points of libpivoter (declared in include/pivoter.h).
+#include <map>
 #include <mutex>
 #include <new>
+#include <tuple>
+#include <utility>
 #include <vector>
 #include <string>
 
@@ -43,7 +46,12 @@ pvt_status check_device(pvt_dag *g, cudaStream_t s, const char *what)
 {
     PVT_CK(cudaMemcpyAsync(g->h_err, g->d_err, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
     PVT_CK(cudaStreamSynchronize(s));
-    unsigned e = *g->h_err;
+    return check_status(g, what);
+}
+
+pvt_status check_status(const pvt_dag *g, const char *what)
+{
+    const unsigned e = *g->h_err;
     if (!e) return PVT_OK;
     std::string w(what);
     if (e & DERR_NOTSIMPLE) { set_error(w + ": CSR is not a simple undirected graph"); return PVT_ENOTSIMPLE; }
@@ -73,6 +81,33 @@ void stats_reset(pvt_dag *g)
     for (int i = 0; i < NPHASE; ++i) g->phase_used[i] = false;
 }
 
+cudaError_t resident_blocks(const void *kern, int threads, size_t smem, int *per_sm)
+{
+    using Key = std::tuple<int, const void *, int, size_t>;
+    static std::mutex mu;
+    static std::map<Key, int> known;
+    static std::map<std::pair<int, const void *>, size_t> allowed;  // dynamic shared memory, only ever raised
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    const Key key(dev, kern, threads, smem);
+    const auto it = known.find(key);
+    if (it != known.end()) {
+        *per_sm = it->second;
+        return cudaSuccess;
+    }
+    size_t &most = allowed[{dev, kern}];
+    if (smem > most) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        most = smem;
+    }
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, threads, smem);
+    if (e == cudaSuccess) known[key] = *per_sm;
+    return e;
+}
+
 // Per-device resources that every dag needs whatever its graph -- status
 // and statistics words, pinned host copies, queue counters, side streams,
 // events, the Pascal table -- outlive their dag: pvt_dag_free hands them
@@ -96,16 +131,23 @@ static std::vector<DagRes> g_res_pool;
 static cudaError_t res_create(int device, DagRes &r)
 {
     r.device = device;
-    cudaError_t e = cudaMalloc(&r.d_err, sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMalloc(&r.d_q, 16 * sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMalloc(&r.d_stats, 16 * sizeof(unsigned long long));
+    char *ctl = nullptr, *pin = nullptr;
+    cudaError_t e = cudaMalloc(&ctl, 256);
+    if (e == cudaSuccess) {
+        r.d_stats = reinterpret_cast<unsigned long long *>(ctl);
+        r.d_q = reinterpret_cast<unsigned *>(ctl + CTL_Q);
+        r.d_err = reinterpret_cast<unsigned *>(ctl + CTL_ERR);
+    }
     if (e == cudaSuccess) e = cudaMalloc(&r.qctl, NCLASS * 128 * sizeof(uint32_t));
     for (int i = 0; i < NPHASE && e == cudaSuccess; ++i) {
         e = cudaEventCreate(&r.ev_t0[i]);
         if (e == cudaSuccess) e = cudaEventCreate(&r.ev_t1[i]);
     }
-    if (e == cudaSuccess) e = cudaMallocHost(&r.h_err, sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMallocHost(&r.h_stats, 16 * sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMallocHost(&pin, PIN_BYTES);
+    if (e == cudaSuccess) {
+        r.h_stats = reinterpret_cast<unsigned long long *>(pin);
+        r.h_err = reinterpret_cast<unsigned *>(pin + CTL_ERR);
+    }
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&r.ev_fork, cudaEventDisableTiming);
     for (int c = 0; c < NCLASS && e == cudaSuccess; ++c) {
         e = cudaStreamCreateWithFlags(&r.side[c], cudaStreamNonBlocking);
@@ -125,13 +167,10 @@ static void res_destroy(DagRes &r)
         if (r.ev_t0[i]) cudaEventDestroy(r.ev_t0[i]);
         if (r.ev_t1[i]) cudaEventDestroy(r.ev_t1[i]);
     }
-    cudaFree(r.d_err);
-    cudaFree(r.d_q);
-    cudaFree(r.d_stats);
+    cudaFree(r.d_stats);  // with d_q and d_err
     cudaFree(r.qctl);
     cudaFree(r.binom.p);
-    if (r.h_err) cudaFreeHost(r.h_err);
-    if (r.h_stats) cudaFreeHost(r.h_stats);
+    if (r.h_stats) cudaFreeHost(r.h_stats);  // with h_err
     r = DagRes{};
 }
 

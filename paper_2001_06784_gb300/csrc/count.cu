@@ -61,6 +61,16 @@ __global__ void k_add_leaf(unsigned long long *cell, unsigned long long count)
     if (threadIdx.x == 0 && blockIdx.x == 0) *cell += count;
 }
 
+// Start of a global count: a dag's control words and its histogram cleared,
+// with the leaves of the roots that have no out-neighbour.
+__global__ void __launch_bounds__(256) k_begin_global(unsigned *ctl, unsigned long long *hist, int hstride,
+                                                      unsigned long long trivial)
+{
+    const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i0 < (int)(CTL_BYTES / 4)) ctl[i0] = 0;
+    for (int i = i0; i < hstride * hstride; i += gridDim.x * blockDim.x) hist[i] = i == hstride ? trivial : 0ull;
+}
+
 // Sum of histogram row 1 (leaves with h = 1) into *out: taken before a
 // range walk adds to a caller's histogram, as the base of k_check_paths.
 __global__ void __launch_bounds__(256) k_row1_sum(const unsigned long long *__restrict__ hist, int hstride,
@@ -84,7 +94,7 @@ __global__ void __launch_bounds__(256) k_row1_sum(const unsigned long long *__re
 // sum_p p * hist[1][p] + sum_p hist[2][p], are the edges of the DAG,
 // orow[n] - orow[0].  A mismatch means walk work was lost or repeated:
 // DERR_CHECK.
-__global__ void __launch_bounds__(256) k_check_paths(const unsigned long long *__restrict__ hist, int hstride,
+__device__ void check_paths(const unsigned long long *__restrict__ hist, int hstride,
                                                      const unsigned long long *base, unsigned long long roots,
                                                      const int64_t *orow, int64_t n, unsigned *err)
 {
@@ -105,6 +115,13 @@ __global__ void __launch_bounds__(256) k_check_paths(const unsigned long long *_
     bool ok = s1 - (base ? *base : 0ull) == roots;
     if (orow) ok = ok && s2 == (unsigned long long)(orow[n] - orow[0]);
     if (!ok) atomicOr(err, DERR_CHECK);
+}
+
+__global__ void __launch_bounds__(256) k_check_paths(const unsigned long long *__restrict__ hist, int hstride,
+                                                     const unsigned long long *base, unsigned long long roots,
+                                                     const int64_t *orow, int64_t n, unsigned *err)
+{
+    check_paths(hist, hstride, base, roots, orow, n, err);
 }
 
 // Local counts of roots with no out-neighbour: c_1(r) += 1.
@@ -143,13 +160,28 @@ __global__ void k_binom(unsigned long long *B, int rows, int W, unsigned *err)
     }
 }
 
-// C_k = sum over (h, p) of hist[h][p] * C(p, k - h), one block per k, exact.
-__global__ void __launch_bounds__(256) k_combine(const unsigned long long *__restrict__ hist,
-                                                 int hstride, const unsigned long long *__restrict__ B,
-                                                 int W, int kmax, unsigned long long *C, unsigned *err)
+// a[0..W) += b[0..W) with carry; true if it left the top word.
+__device__ __forceinline__ bool add_words(unsigned long long *a, const unsigned long long *b, int W)
 {
-    __shared__ unsigned long long red[256][WMAX];
-    const int k = blockIdx.x;
+    unsigned long long c = 0;
+#pragma unroll
+    for (int w = 0; w < WMAX; ++w) {
+        if (w >= W) break;
+        const unsigned long long s1 = a[w] + b[w], c1 = s1 < a[w], s2 = s1 + c;
+        c = c1 + (s2 < s1);
+        a[w] = s2;
+    }
+    return c != 0;
+}
+
+// C_k = sum over (h, p) of hist[h][p] * C(p, k - h) by one block of 256
+// threads, exact: each thread its pairs, then the warps by shuffles, then the
+// eight warps' sums.
+__device__ void combine_size(const unsigned long long *__restrict__ hist, int hstride,
+                             const unsigned long long *__restrict__ B, int Bw, int W, int k, unsigned long long *C,
+                             unsigned *err)
+{
+    __shared__ unsigned long long red[8][WMAX];
     unsigned long long acc[WMAX];
 #pragma unroll
     for (int w = 0; w < WMAX; ++w) acc[w] = 0;
@@ -163,7 +195,7 @@ __global__ void __launch_bounds__(256) k_combine(const unsigned long long *__res
         if (i < 0 || i > p) continue;
         const unsigned long long x = hist[(size_t)h * hstride + p];
         if (!x) continue;
-        const unsigned long long *b = B + ((size_t)p * (p + 1) / 2 + i) * W;
+        const unsigned long long *b = B + ((size_t)p * (p + 1) / 2 + i) * Bw;
         unsigned long long carry = 0;
 #pragma unroll
         for (int w = 0; w < WMAX; ++w) {
@@ -178,24 +210,42 @@ __global__ void __launch_bounds__(256) k_combine(const unsigned long long *__res
         }
         if (carry) ovf = true;
     }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-    for (int w = 0; w < WMAX; ++w) red[threadIdx.x][w] = acc[w];
-    __syncthreads();
-    for (int stride = 128; stride > 0; stride >>= 1) {
-        if (threadIdx.x < stride) {
-            unsigned long long c = 0;
-            for (int w = 0; w < W; ++w) {
-                unsigned long long x = red[threadIdx.x][w], y = red[threadIdx.x + stride][w];
-                unsigned long long s1 = x + y, c1 = s1 < x, s2 = s1 + c;
-                c = c1 + (s2 < s1);
-                red[threadIdx.x][w] = s2;
-            }
-            if (c) ovf = true;
-        }
-        __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) {
+        unsigned long long other[WMAX];
+#pragma unroll
+        for (int w = 0; w < WMAX; ++w) other[w] = w < W ? __shfl_down_sync(FULL, acc[w], o) : 0ull;
+        if (lane < o && add_words(acc, other, W)) ovf = true;
     }
-    if (threadIdx.x < W) C[(size_t)k * W + threadIdx.x] = red[0][threadIdx.x];
+    if (lane == 0) {
+#pragma unroll
+        for (int w = 0; w < WMAX; ++w) red[wid][w] = acc[w];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < 8; ++i)
+            if (add_words(acc, red[i], W)) ovf = true;
+#pragma unroll
+        for (int w = 0; w < WMAX; ++w)
+            if (w < W) C[w] = acc[w];
+    }
     if (ovf) atomicOr(err, DERR_OVERFLOW);
+}
+
+// One block per k, C[k][W]; with `check` one more block for the root paths
+// (check_paths; base is null).
+__global__ void __launch_bounds__(256) k_combine(const unsigned long long *__restrict__ hist,
+                                                 int hstride, const unsigned long long *__restrict__ B,
+                                                 int W, int kmax, unsigned long long *C, bool check,
+                                                 unsigned long long roots, const int64_t *orow, int64_t n, unsigned *err)
+{
+    const int k = blockIdx.x;
+    if (k > kmax) {
+        if (check) check_paths(hist, hstride, nullptr, roots, orow, n, err);
+        return;
+    }
+    combine_size(hist, hstride, B, W, W, k, C + (size_t)k * W, err);
 }
 
 static pvt_status ensure_binom(pvt_dag *g, int W, cudaStream_t s)
@@ -234,9 +284,8 @@ static pvt_status launch_frames(pvt_dag *g, const CountArgs &base, cudaStream_t 
     A.qcap = SPLIT_QCAP;
     constexpr size_t smem = sizeof(WarpWork<1>) * FRAME_WPB + sizeof(unsigned) * HIST_H * HIST_P;
     auto kern = k_walk_frames<true>;
-    PVT_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    PVT_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * FRAME_WPB, smem));
+    PVT_CK(resident_blocks((const void *)kern, 32 * FRAME_WPB, smem, &per_sm));
     if (per_sm < 1) {
         set_error("frame walk kernel cannot be resident");
         return PVT_ECUDA;
@@ -337,12 +386,20 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
         A.emit1 = g->cframes1.p;
         A.emit1_count = g->d_q + 10;
     }
-    // heavy classes on side streams so that they overlap the light ones (or
-    // all on s, one after another, when the autotuner times them)
-    const bool serial = g->serial || g->policy.serial;
+    // classes on side streams (or all on s, one after another, when the
+    // autotuner times them); classes without roots launch nothing, and a
+    // single class needs no stream of its own
+    int used = 0;
+    for (int c = 1; c < NCLASS; ++c) used += g->wcnt[c] > 0;
+    const bool serial = g->serial || g->policy.serial || used <= 1;
     if (!serial) PVT_CK(cudaEventRecord(g->ev_fork, s));
     for (int c = NCLASS - 1; c >= 1 && st == PVT_OK; --c) {
-        cudaStream_t cs = serial ? s : g->side[c];
+        if (g->wcnt[c] == 0) continue;
+        // a global count's wide classes follow one another, widest first: each
+        // fills the GPU, and side by side they only take shared memory from one
+        // another (count of the 10.8M-edge graph 7.0 ms, in one stream 6.2).
+        // The <= 32 class needs none and runs beside them.
+        cudaStream_t cs = serial ? s : g->side[MODE == MODE_GLOBAL && c >= 2 ? NCLASS - 1 : c];
         if (!serial) PVT_CK(cudaStreamWaitEvent(cs, g->ev_fork, 0));
         switch (c) {
             case 1:
@@ -370,7 +427,8 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
         // the frame walk follows the classes that emit; a <= 32 class that
         // walks its own roots may still be running beside it
         if (!serial)
-            for (int c = NCLASS - 1; c >= (gather1 ? 1 : 2); --c) PVT_CK(cudaStreamWaitEvent(s, g->ev_join[c], 0));
+            for (int c = NCLASS - 1; c >= (gather1 ? 1 : 2); --c)
+                if (g->wcnt[c]) PVT_CK(cudaStreamWaitEvent(s, g->ev_join[c], 0));
         A.emit1_cap = slots1;
         if ((st = launch_frames(g, A, s)) != PVT_OK) return st;
     }
@@ -385,7 +443,8 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
         if ((st = launch_frames(g, P, s)) != PVT_OK) return st;
     }
     if (!serial)
-        for (int c = NCLASS - 1; c >= 1; --c) PVT_CK(cudaStreamWaitEvent(s, g->ev_join[c], 0));
+        for (int c = NCLASS - 1; c >= 1; --c)
+            if (g->wcnt[c]) PVT_CK(cudaStreamWaitEvent(s, g->ev_join[c], 0));
     return st;
 }
 
@@ -406,9 +465,9 @@ static void begin_call(pvt_dag *g)
 // when kmax >= 1; they are tallied without a walk, and counted here.
 static pvt_status end_call(pvt_dag *g, cudaStream_t s, const char *fn, int32_t kmax)
 {
-    PVT_CK(cudaMemcpyAsync(g->h_stats, g->d_stats, (3 + NCLASS + 2) * sizeof(unsigned long long),
-                           cudaMemcpyDeviceToHost, s));
-    pvt_status st = check_device(g, s, fn);
+    PVT_CK(cudaMemcpyAsync(g->h_stats, g->d_stats, CTL_BYTES, cudaMemcpyDeviceToHost, s));
+    PVT_CK(cudaStreamSynchronize(s));
+    pvt_status st = check_status(g, fn);
     const uint64_t trivial = kmax >= 1 ? (uint64_t)g->wcnt[0] : 0;
     g->stats.sct_nodes = g->h_stats[0] + trivial;
     g->stats.sct_leaves = g->h_stats[1] + trivial;
@@ -446,15 +505,12 @@ static pvt_status enqueue_global(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *
     const int hstride = g->alpha + 2;
     if ((st = grow(g->hist, (size_t)hstride * hstride, s)) != PVT_OK) return st;
     if ((st = ensure_binom(g, W, s)) != PVT_OK) return st;
-    PVT_CK(cudaMemsetAsync(g->d_err, 0, sizeof(unsigned), s));
-    PVT_CK(cudaMemsetAsync(g->d_q, 0, 16 * sizeof(unsigned), s));
-    PVT_CK(cudaMemsetAsync(g->hist.p, 0, (size_t)hstride * hstride * sizeof(unsigned long long), s));
-    PVT_CK(cudaMemsetAsync(g->d_stats, 0, 16 * sizeof(unsigned long long), s));
-    if (g->class_cnt[0] && kmax >= 1) {
-        k_add_leaf<<<1, 32, 0, s>>>(g->hist.p + hstride, (unsigned long long)g->class_cnt[0]);
-        PVT_CK(cudaGetLastError());
-        g->stats.launches++;
-    }
+    const unsigned cells = (unsigned)(hstride * hstride);
+    k_begin_global<<<std::min((cells + 255u) / 256u, (unsigned)(4 * g->num_sms)), 256, 0, s>>>(
+        reinterpret_cast<unsigned *>(g->d_stats), g->hist.p, hstride,
+        kmax >= 1 ? (unsigned long long)g->class_cnt[0] : 0ull);
+    PVT_CK(cudaGetLastError());
+    g->stats.launches++;
     CountArgs A{};
     A.orow = g->orow;
     A.ocol = g->ocol;
@@ -469,14 +525,10 @@ static pvt_status enqueue_global(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *
     apply_wait_limit(g, A);
     if ((st = launch_all<MODE_GLOBAL>(g, A, s)) != PVT_OK) return st;
     phase_begin(g, PH_FINISH, s);
-    if (kmax >= 1) {
-        k_check_paths<<<1, 256, 0, s>>>(g->hist.p, hstride, nullptr, (unsigned long long)g->n,
-                                        kmax >= 2 ? g->orow : nullptr, g->n, g->d_err);
-        PVT_CK(cudaGetLastError());
-        g->stats.launches++;
-    }
-    k_combine<<<kmax + 1, 256, 0, s>>>(g->hist.p, hstride, g->binom.p, W, kmax,
-                                       reinterpret_cast<unsigned long long *>(C), g->d_err);
+    k_combine<<<kmax + 1 + (kmax >= 1), 256, 0, s>>>(g->hist.p, hstride, g->binom.p, W, kmax,
+                                                     reinterpret_cast<unsigned long long *>(C), kmax >= 1,
+                                                     (unsigned long long)g->n, kmax >= 2 ? g->orow : nullptr, g->n,
+                                                     g->d_err);
     PVT_CK(cudaGetLastError());
     phase_end(g, PH_FINISH, s);
     g->stats.launches++;
@@ -662,9 +714,7 @@ pvt_status count_hist(pvt_dag *g, int64_t begin, int64_t end, int32_t kmax, uint
         g->stats.launches += 7;
     }
     const int hstride = g->alpha + 2;
-    PVT_CK(cudaMemsetAsync(g->d_err, 0, sizeof(unsigned), s));
-    PVT_CK(cudaMemsetAsync(g->d_q, 0, 16 * sizeof(unsigned), s));
-    PVT_CK(cudaMemsetAsync(g->d_stats, 0, 16 * sizeof(unsigned long long), s));
+    PVT_CK(cudaMemsetAsync(g->d_stats, 0, CTL_BYTES, s));
     // row 1 of the caller's histogram before this range adds to it
     unsigned long long *row1_base = g->d_stats + 14;
     if (kmax >= 1) {
@@ -711,10 +761,10 @@ pvt_status combine_hist(pvt_dag *g, const uint64_t *hist, int32_t kmax, int32_t 
     }
     begin_call(g);
     if ((st = ensure_binom(g, W, s)) != PVT_OK) return st;
-    PVT_CK(cudaMemsetAsync(g->d_err, 0, sizeof(unsigned), s));
-    PVT_CK(cudaMemsetAsync(g->d_stats, 0, 16 * sizeof(unsigned long long), s));
+    PVT_CK(cudaMemsetAsync(g->d_stats, 0, CTL_BYTES, s));
     k_combine<<<kmax + 1, 256, 0, s>>>(reinterpret_cast<const unsigned long long *>(hist), g->alpha + 2, g->binom.p,
-                                       W, kmax, reinterpret_cast<unsigned long long *>(C), g->d_err);
+                                       W, kmax, reinterpret_cast<unsigned long long *>(C), false, 0ull, nullptr, 0,
+                                       g->d_err);
     PVT_CK(cudaGetLastError());
     g->stats.launches++;
     return end_call(g, s, "pvt_combine_hist", -1);
@@ -795,10 +845,8 @@ pvt_status count_local(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *out, bool 
     }
     if ((st = ensure_binom(g, W, s)) != PVT_OK) return st;
     const int64_t rows = edge ? g->m : g->n;
-    PVT_CK(cudaMemsetAsync(g->d_err, 0, sizeof(unsigned), s));
-    PVT_CK(cudaMemsetAsync(g->d_q, 0, 16 * sizeof(unsigned), s));
+    PVT_CK(cudaMemsetAsync(g->d_stats, 0, CTL_BYTES, s));
     if (rows > 0) PVT_CK(cudaMemsetAsync(out, 0, (size_t)rows * (kmax + 1) * W * sizeof(uint64_t), s));
-    PVT_CK(cudaMemsetAsync(g->d_stats, 0, 16 * sizeof(unsigned long long), s));
     unsigned long long *o = reinterpret_cast<unsigned long long *>(out);
     if (!edge && g->class_cnt[0] && kmax >= 1) {
         k_vertex_trivial<<<g->num_sms * 4, 256, 0, s>>>(g->roots + g->class_start[0],
@@ -847,57 +895,9 @@ __global__ void __launch_bounds__(256) k_combine_batch(const BatchGraph *gs, con
                                                        const unsigned long long *__restrict__ B, int Bw,
                                                        unsigned *err)
 {
-    __shared__ unsigned long long red[256][WMAX];
     const int2 wk = work[blockIdx.x];
     const BatchGraph &G = gs[wk.x];
-    const int k = wk.y, W = G.W, hstride = G.hstride;
-    const unsigned long long *hist = G.hist;
-    unsigned long long acc[WMAX];
-#pragma unroll
-    for (int w = 0; w < WMAX; ++w) acc[w] = 0;
-    bool ovf = false;
-    const int pmax = hstride - 2;
-    const int hmax = min(k, hstride - 1);
-    const int total = hmax * (pmax + 1);
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        const int h = 1 + t / (pmax + 1), p = t % (pmax + 1);
-        const int i = k - h;
-        if (i < 0 || i > p) continue;
-        const unsigned long long x = hist[(size_t)h * hstride + p];
-        if (!x) continue;
-        const unsigned long long *b = B + ((size_t)p * (p + 1) / 2 + i) * Bw;
-        unsigned long long carry = 0;
-#pragma unroll
-        for (int w = 0; w < WMAX; ++w) {
-            if (w >= W) break;
-            unsigned long long lo = x * b[w], hi = __umul64hi(x, b[w]);
-            unsigned long long s1 = acc[w] + lo;
-            unsigned long long c1 = s1 < lo;
-            unsigned long long s2 = s1 + carry;
-            unsigned long long c2 = s2 < s1;
-            acc[w] = s2;
-            carry = hi + c1 + c2;
-        }
-        if (carry) ovf = true;
-    }
-#pragma unroll
-    for (int w = 0; w < WMAX; ++w) red[threadIdx.x][w] = acc[w];
-    __syncthreads();
-    for (int stride = 128; stride > 0; stride >>= 1) {
-        if (threadIdx.x < stride) {
-            unsigned long long c = 0;
-            for (int w = 0; w < W; ++w) {
-                unsigned long long x = red[threadIdx.x][w], y = red[threadIdx.x + stride][w];
-                unsigned long long s1 = x + y, c1 = s1 < x, s2 = s1 + c;
-                c = c1 + (s2 < s1);
-                red[threadIdx.x][w] = s2;
-            }
-            if (c) ovf = true;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < W) G.out[(size_t)k * W + threadIdx.x] = red[0][threadIdx.x];
-    if (ovf) atomicOr(err, DERR_OVERFLOW);
+    combine_size(G.hist, G.hstride, B, Bw, G.W, wk.y, G.out + (size_t)wk.y * G.W, err);
 }
 
 pvt_status batch_root_entries(BatchGraph *d_graphs, int count, uint64_t *const *d_entries,
@@ -1028,9 +1028,8 @@ static pvt_status launch_noalloc(const CountArgs &A, int alpha, int num_sms, cud
 {
     constexpr size_t smem = sizeof(WarpWork<NW>) * warps_per_block<NW>();
     auto kern = k_count_noalloc<NW>;
-    PVT_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    PVT_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * warps_per_block<NW>(), smem));
+    PVT_CK(resident_blocks((const void *)kern, 32 * warps_per_block<NW>(), smem, &per_sm));
     if (per_sm < 1) {
         set_error("pvt_count_global_noalloc: walk kernel cannot be resident");
         return PVT_ECUDA;
@@ -1124,7 +1123,8 @@ extern "C" pvt_status pvt_count_global_noalloc(int64_t n, const int64_t *orow, c
                                         err);
         PVT_CK(cudaGetLastError());
     }
-    k_combine<<<kmax + 1, 256, 0, s>>>(hist, hstride, binom, W, kmax, reinterpret_cast<unsigned long long *>(C), err);
+    k_combine<<<kmax + 1, 256, 0, s>>>(hist, hstride, binom, W, kmax, reinterpret_cast<unsigned long long *>(C), false, 0ull,
+                                       nullptr, 0, err);
     PVT_CK(cudaGetLastError());
     unsigned herr = 0;
     PVT_CK(cudaMemcpyAsync(&herr, err, sizeof(unsigned), cudaMemcpyDeviceToHost, s));

@@ -62,7 +62,7 @@ struct alignas(16) CtaQueue {
     // each warp's current label S and non-neighbour set R, for reads of word
     // j by a loop index (registers hold them for the unrolled word loops)
     uint32_t wS[CTA_MAXW][NW], wR[CTA_MAXW][NW];
-    uint32_t wM[CTA_MAXW][32];  // the members of a small label being relabelled
+    alignas(8) uint16_t wM[CTA_MAXW][32];  // the members of a small label being relabelled
 };
 
 template <int NW>
@@ -95,6 +95,7 @@ struct LaneState {
     bool has = false;
     unsigned top = 0, bot = 0;
     unsigned cls = 0;  // unused here: every subtree is of the launch's class
+    uint32_t base = 0; // (h, p) at which the subtree was entered
     __device__ __forceinline__ bool free_() const { return !has && top == bot; }
 };
 
@@ -107,16 +108,16 @@ __device__ inline void lane_run(LaneWork &L, unsigned *sh32, const CountArgs &A,
         const unsigned freeM = __ballot_sync(FULL, ls.free_());
         if (freeM == FULL) return;
         if (stop_free && __popc(freeM) >= stop_free) return;
-        if (freeM) lane_steal(L, lane, freeM, ls.S, ls.h, ls.p, ls.has, ls.top, ls.bot, ls.cls);
+        if (freeM) lane_steal(L, lane, freeM, ls.S, ls.h, ls.p, ls.has, ls.top, ls.bot, ls.base, ls.cls);
         if (!ls.has && ls.top != ls.bot) {
             --ls.top;
             ls.S = L.stkS[ls.top & (LSTK - 1)][lane];
-            const uint32_t hp = L.stkHP[ls.top & (LSTK - 1)][lane];
+            const uint32_t hp = lane_unpack(L.stkHP[ls.top & (LSTK - 1)][lane], ls.base);
             ls.h = (int)(hp >> 16);
             ls.p = (int)(hp & 0xFFFFu);
             ls.has = true;
         }
-        if (ls.has) lane_node(L, sh32, A, lane, ls.S, ls.h, ls.p, ls.has, ls.top, ls.bot, lc);
+        if (ls.has) lane_node(L, sh32, A, lane, ls.S, ls.h, ls.p, ls.has, ls.top, ls.bot, ls.base, lc);
         __syncwarp();
     }
 }
@@ -138,6 +139,7 @@ __device__ __forceinline__ void lane_add(LaneWork &L, unsigned *sh32, const Coun
         ls.S = s >= 32 ? FULL : ((1u << s) - 1u);
         ls.h = h;
         ls.p = p;
+        ls.base = (uint32_t)h << 16 | (uint32_t)p;
         ls.has = true;
         ls.top = ls.bot = 0;
     }
@@ -231,6 +233,7 @@ __device__ __forceinline__ int cta_take_small(CtaQueue<NW> &Q, LaneWork &L, int 
         for (int v = 0; v < 32; ++v) L.rows[v][lane] = Q.crow[e][v];
         ls.S = Q.cS[e];
         const uint32_t hp = Q.chp[e];
+        ls.base = hp;
         ls.h = (int)(hp >> 16);
         ls.p = (int)(hp & 0xFFFFu);
         ls.has = true;
@@ -367,26 +370,34 @@ __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork
                     // members of R; labels of at most two members close here
                     int before = 0;
                     SmallCounts small;
+                    uint32_t M[LNW];  // S without the members of R in the words before j
+#pragma unroll
+                    for (int w = 0; w < LNW; ++w) M[w] = S[w];
                     for (int j = 0; j < LNW; ++j) {
                         const uint32_t Rj = wR[j];
+                        if (Rj == 0) continue;
                         const bool inR = (Rj >> lane) & 1u;
                         bool push = inR;
                         const uint32_t *row = rows + (j * 32 + lane) * RS;
                         int cs = 0;
                         if (inR) {
-                            int a = 0, b = 0;
 #pragma unroll
-                            for (int w = 0; w < LNW; ++w) {
-                                const uint32_t bl = w < j ? R[w] : (w == j ? (Rj & low) : 0u);
-                                const uint32_t cw = row[w] & S[w] & ~bl;
-                                if (cw) {
-                                    if (cs == 0) a = w * 32 + __ffs(cw) - 1;
-                                    b = w * 32 + 31 - __clz(cw);
-                                }
-                                cs += __popc(cw);
-                            }
+                            for (int w = 0; w < LNW; ++w) cs += __popc(row[w] & M[w]);
+                            cs -= __popc(row[j] & wS[j] & Rj & low);  // the earlier members of R in word j
                             if (cs <= 2) {
-                                const bool adjp = cs == 2 && ((rows[a * RS + (b >> 5)] >> (b & 31)) & 1u);
+                                bool adjp = false;
+                                if (cs == 2) {
+                                    int a = 0, b = 0;
+#pragma unroll
+                                    for (int w = LNW - 1; w >= 0; --w) {
+                                        const uint32_t cw = row[w] & M[w] & (w == j ? ~(Rj & low) : FULL);
+                                        if (cw) {
+                                            a = w * 32 + __ffs(cw) - 1;
+                                            b = max(b, w * 32 + 31 - __clz(cw));
+                                        }
+                                    }
+                                    adjp = (rows[a * RS + (b >> 5)] >> (b & 31)) & 1u;
+                                }
                                 small.add(cs, adjp);
                                 push = false;
                             }
@@ -414,13 +425,13 @@ __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork
                         if (push) {
                             uint32_t *fr = stk + (size_t)(top + before + __popc(pushed & low)) * FW;
 #pragma unroll
-                            for (int w = 0; w < LNW; ++w) {
-                                const uint32_t bl = w < j ? R[w] : (w == j ? (Rj & low) : 0u);
-                                fr[w] = row[w] & S[w] & ~bl;
-                            }
+                            for (int w = 0; w < LNW; ++w) fr[w] = row[w] & M[w] & (w == j ? ~(Rj & low) : FULL);
                             fr[LNW] = ((uint32_t)(h + 1) << 16) | (uint32_t)p;
                         }
                         before += __popc(pushed);
+#pragma unroll
+                        for (int w = 0; w < LNW; ++w)
+                            if (w == j) M[w] &= ~Rj;
                     }
                     top += before;
                     small.close<true>(sh32, A, lane, h + 1, p, wc.nodes, wc.leaves, wc.words);

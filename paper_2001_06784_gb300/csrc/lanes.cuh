@@ -29,7 +29,7 @@
 
 namespace pvt {
 
-constexpr int LANE_WPB = 8;     // warps per block
+constexpr int LANE_WPB = 10;    // warps per block (two blocks per SM: 217 KB of shared memory)
 constexpr int LSTK = 32;        // per-lane stack slots (a label of s <= 32 keeps at most 31 pending)
 constexpr unsigned LANE_DONATE_EVERY = 16;  // node steps between looks at the ring queue
 constexpr unsigned LANE_DONATE_MAX = 4;     // entries one look may donate
@@ -37,8 +37,21 @@ constexpr unsigned LANE_DONATE_MAX = 4;     // entries one look may donate
 struct LaneWork {
     uint32_t rows[32][32];      // rows[v][lane]: row v of the lane's current subtree
     uint32_t stkS[LSTK][32];    // pending labels, circular per lane
-    uint32_t stkHP[LSTK][32];   // their (h << 16) | p
+    uint16_t stkHP[LSTK][32];   // their (h, p) less the subtree's (lane_pack)
 };
+
+// (h, p) as h << 16 | p, and in 16 bits relative to the `base` at which the
+// lane's subtree was entered: a label of at most 32 members adds at most 32
+// links of either kind.
+__device__ __forceinline__ uint16_t lane_pack(uint32_t hp, uint32_t base)
+{
+    const uint32_t x = hp - base;
+    return (uint16_t)(x >> 8 | (x & 0xFFu));
+}
+__device__ __forceinline__ uint32_t lane_unpack(uint16_t x, uint32_t base)
+{
+    return base + ((uint32_t)(x & 0xFF00u) << 8 | (x & 0xFFu));
+}
 
 // Per-lane walk statistics (each lane its own subtrees; summed at the end).
 // words1: the share of words that belongs to roots of the <= 32 class.
@@ -87,7 +100,7 @@ __device__ __forceinline__ void lane_close_small(unsigned *sh32, const CountArgs
 // more members are pushed and the lane moves to the pivot child.
 __device__ __forceinline__ void lane_node(LaneWork &L, unsigned *sh32, const CountArgs &A, int lane,
                                           uint32_t &S, int &h, int &p, bool &has, unsigned &top, unsigned bot,
-                                          LaneCounters &lc)
+                                          uint32_t base, LaneCounters &lc)
 {
     const int s = __popc(S);
     ++lc.nodes;
@@ -138,7 +151,7 @@ __device__ __forceinline__ void lane_node(LaneWork &L, unsigned *sh32, const Cou
                 lane_close_small(sh32, A, cs, adj, h + 1, p, lc);
             } else {
                 L.stkS[top & (LSTK - 1)][lane] = child;
-                L.stkHP[top & (LSTK - 1)][lane] = ((uint32_t)(h + 1) << 16) | (uint32_t)p;
+                L.stkHP[top & (LSTK - 1)][lane] = lane_pack(((uint32_t)(h + 1) << 16) | (uint32_t)p, base);
                 ++top;
             }
         }
@@ -161,7 +174,7 @@ __device__ __forceinline__ void lane_node(LaneWork &L, unsigned *sh32, const Cou
 // busy lane (one that keeps work), with that lane's rows.  Returns the
 // lanes that received one.
 __device__ __forceinline__ unsigned lane_steal(LaneWork &L, int lane, unsigned freeM, uint32_t &S, int &h, int &p,
-                                               bool &has, unsigned top, unsigned &bot, unsigned &cls)
+                                               bool &has, unsigned top, unsigned &bot, uint32_t &base, unsigned &cls)
 {
     const unsigned pend = top - bot;
     const unsigned donors = __ballot_sync(FULL, pend >= 2 || (pend == 1 && has));
@@ -181,9 +194,10 @@ __device__ __forceinline__ unsigned lane_steal(LaneWork &L, int lane, unsigned f
     }
     const unsigned sbot = __shfl_sync(FULL, bot, src);
     cls = __shfl_sync(FULL, cls, src);  // src is the lane itself where nothing is received
+    base = __shfl_sync(FULL, base, src);
     if (recv) {
         S = L.stkS[sbot & (LSTK - 1)][src];
-        const uint32_t hp = L.stkHP[sbot & (LSTK - 1)][src];
+        const uint32_t hp = lane_unpack(L.stkHP[sbot & (LSTK - 1)][src], base);
         h = (int)(hp >> 16);
         p = (int)(hp & 0xFFFFu);
         for (int v = 0; v < 32; ++v) L.rows[v][lane] = L.rows[v][src];
@@ -201,7 +215,7 @@ __device__ __forceinline__ unsigned lane_steal(LaneWork &L, int lane, unsigned f
 // hit 32 distinct banks), its label, (h, p) and root class.  False for a
 // slot that holds no subtree.
 __device__ __forceinline__ bool lane_load_frame(LaneWork &L, const uint32_t *fr, int lane, uint32_t &S, int &h,
-                                                int &p, unsigned &cls)
+                                                int &p, uint32_t &base, unsigned &cls)
 {
     const uint4 *v = reinterpret_cast<const uint4 *>(fr + 4);
 #pragma unroll
@@ -214,6 +228,7 @@ __device__ __forceinline__ bool lane_load_frame(LaneWork &L, const uint32_t *fr,
     }
     const uint4 head = __ldcs(reinterpret_cast<const uint4 *>(fr));
     S = head.z;
+    base = head.y;
     h = (int)(head.y >> 16);
     p = (int)(head.y & 0xFFFFu);
     cls = head.w;
@@ -234,6 +249,7 @@ __device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A
     auto frame_of = [&](unsigned i) {
         return i < nwide ? A.emit + (size_t)i * FRAME_WORDS : A.emit1 + (size_t)(i - nwide) * FRAME_WORDS;
     };
+    uint32_t hpbase = 0;         // (h, p) at which the lane's subtree was entered
     unsigned cls = 0;            // out-degree class of the root whose rows the lane holds
     LaneCounters lc;
     uint32_t S = 0;
@@ -269,7 +285,7 @@ __device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A
                 const unsigned got = min((unsigned)__popc(freeM), end - cur);
                 const unsigned rank = (unsigned)__popc(freeM & ((1u << lane) - 1u));
                 if (((freeM >> lane) & 1u) && rank < got) {
-                    has = lane_load_frame(L, frame_of(cur + rank), lane, S, h, p, cls);
+                    has = lane_load_frame(L, frame_of(cur + rank), lane, S, h, p, hpbase, cls);
                 }
                 cur += got;
                 held += got;
@@ -278,7 +294,7 @@ __device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A
             }
         }
         if (freeM && src_done) {
-            lane_steal(L, lane, freeM, S, h, p, has, top, bot, cls);
+            lane_steal(L, lane, freeM, S, h, p, has, top, bot, hpbase, cls);
             freeM = __ballot_sync(FULL, !has && top == bot);
             if (freeM == FULL) {
                 // every lane idle: return this warp's items, then wait for a
@@ -294,6 +310,7 @@ __device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A
                 if (lane == 0) {
                     const uint32_t hp = __ldcg(fr + 1);
                     S = __ldcg(fr + 2);
+                    hpbase = hp;
                     cls = __ldcg(fr + 3);
                     h = (int)(hp >> 16);
                     p = (int)(hp & 0xFFFFu);
@@ -311,14 +328,14 @@ __device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A
         if (!has && top != bot) {
             --top;
             S = L.stkS[top & (LSTK - 1)][lane];
-            const uint32_t hp = L.stkHP[top & (LSTK - 1)][lane];
+            const uint32_t hp = lane_unpack(L.stkHP[top & (LSTK - 1)][lane], hpbase);
             h = (int)(hp >> 16);
             p = (int)(hp & 0xFFFFu);
             has = true;
         }
         if (has) {
             const unsigned long long w = lc.words;
-            lane_node(L, sh32, A, lane, S, h, p, has, top, bot, lc);
+            lane_node(L, sh32, A, lane, S, h, p, has, top, bot, hpbase, lc);
             if (cls == 1) lc.words1 += lc.words - w;
         }
         __syncwarp();
@@ -341,7 +358,7 @@ __device__ inline void lane_walk(LaneWork &L, unsigned *sh32, const CountArgs &A
                 fr[4 + lane] = L.rows[lane][dl];
                 if (lane == dl) {
                     fr[0] = FRAME_COMPACT;
-                    fr[1] = L.stkHP[bot & (LSTK - 1)][lane];
+                    fr[1] = lane_unpack(L.stkHP[bot & (LSTK - 1)][lane], hpbase);
                     fr[2] = L.stkS[bot & (LSTK - 1)][lane];
                     fr[3] = cls;
                     ++bot;

@@ -422,9 +422,11 @@ struct LocalWalk {
                             // pairs of the held member and its label
                             const int m = j * 32 + lane;
                             const uint32_t *em = Wk.etab + (size_t)m * D;
-                            add_edge(em[a], h + 2, pair ? p + 1 : p);
-                            if (cs == 2) add_edge(em[b], h + 2, pair ? p + 1 : p);
-                            if (pair) add_edge(Wk.etab[(size_t)a * D + b], h + 3, p);
+                            const uint32_t ea = em[a], eb = cs == 2 ? em[b] : 0u;
+                            const uint32_t eab = pair ? Wk.etab[(size_t)a * D + b] : 0u;
+                            add_edge(ea, h + 2, pair ? p + 1 : p);
+                            if (cs == 2) add_edge(eb, h + 2, pair ? p + 1 : p);
+                            if (pair) add_edge(eab, h + 3, p);
                         }
                     }
                     // the others to the stack (this part's share of them)
@@ -765,8 +767,7 @@ __global__ void __launch_bounds__(32 * local_wpb<NW>(), local_blocks<NW>())
 template <typename K>
 static pvt_status local_occupancy(K kern, int threads, size_t smem, int *per_sm)
 {
-    PVT_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PVT_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, threads, smem));
+    PVT_CK(resident_blocks((const void *)kern, threads, smem, per_sm));
     if (*per_sm < 1) {
         set_error("local count kernel cannot be resident (shared memory)");
         return PVT_ECUDA;
@@ -786,13 +787,13 @@ pvt_status launch_local(pvt_dag *g, const CountArgs &base, int cls, cudaStream_t
     A.nroots = cnt;
     A.qhead = g->d_q + cls;
     A.cls = cls;
-    A.chunk = NW == 1 ? (unsigned)g->policy.chunk : 1u;
     const int kt = std::min(A.kmax, LocalWork<NW>::WINDOW), amax = g->alpha + 2;
     const size_t smem = local_warp_bytes<NW>(kt) * WPB;
     int per_sm = 0;
     pvt_status st;
     if ((st = local_occupancy(k_local<NW, MODE>, 32 * WPB, smem, &per_sm)) != PVT_OK) return st;
     const unsigned full = (unsigned)(g->num_sms * per_sm);
+    A.chunk = NW == 1 ? claim_size(g, cnt, full * WPB) : 1u;
     const unsigned per_block = WPB * A.chunk;
     const unsigned grid = std::max(1u, std::min(full, (cnt + per_block - 1) / per_block));
     if (LocalWork<NW>::GSTACK) {

@@ -11,7 +11,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
-#include <vector>
+#include <cstddef>
 
 #include "pvt_internal.cuh"
 
@@ -536,7 +536,11 @@ struct CoreState {
     unsigned most[3];         // largest changed estimate, by round modulo 3
     unsigned bail;            // 1: left to the level-wise peel
     unsigned seen[CORE_BINS / 32];  // core numbers met (bit set)
+    unsigned most_out;        // largest out-degree
+    unsigned class_cnt[NCLASS];     // roots per out-degree class
+    unsigned deg_cnt[CORE_CLAMP + 1];  // vertices per out-degree (larger ones in the last), then their first positions
 };
+static_assert(offsetof(CoreState, deg_cnt) <= PIN_BYTES - PIN_ORIENT, "the result part fits its pinned copy");
 
 // The h-index of a row's estimates, at most k, from their histogram of
 // min(estimate, k) (bins floor..k, one warp), and the support at it; floor - 1
@@ -1129,10 +1133,16 @@ __device__ __forceinline__ bool key_less(uint32_t ra, uint32_t a, uint32_t rb, u
     return ra < rb || (ra == rb && a < b);
 }
 
-// Out-degree of every vertex (warp per vertex) and the largest one.
-__global__ void k_outdeg(int64_t n, const int64_t *__restrict__ rp, const uint32_t *__restrict__ col,
-                         const uint32_t *__restrict__ rnd, uint32_t *odeg, unsigned *alpha)
+// Out-degree of every vertex (warp per vertex), the largest one, and how many
+// vertices have each (a block-shared count first: out-degrees crowd into a few
+// small values).
+__global__ void __launch_bounds__(256) k_outdeg(int64_t n, const int64_t *__restrict__ rp,
+                                                const uint32_t *__restrict__ col, const uint32_t *__restrict__ rnd,
+                                                uint32_t *odeg, CoreState *st)
 {
+    __shared__ unsigned sh[CORE_CLAMP + 1];
+    for (int i = threadIdx.x; i <= (int)CORE_CLAMP; i += blockDim.x) sh[i] = 0;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1145,10 +1155,16 @@ __global__ void k_outdeg(int64_t n, const int64_t *__restrict__ rp, const uint32
             c += key_less(rv, (uint32_t)v, rnd[u], u);
         }
         c = __reduce_add_sync(FULL, c);
-        if (lane == 0) odeg[v] = c;
+        if (lane == 0) {
+            odeg[v] = c;
+            atomicAdd(&sh[min(c, CORE_CLAMP)], 1u);
+        }
         most = max(most, c);
     }
-    if (lane == 0 && most) atomicMax(alpha, most);
+    if (lane == 0 && most) atomicMax(&st->most_out, most);
+    __syncthreads();
+    for (int i = threadIdx.x; i <= (int)CORE_CLAMP; i += blockDim.x)
+        if (sh[i]) atomicAdd(&st->deg_cnt[i], sh[i]);
 }
 
 // Out-lists in CSR order (ascending id), compacted with a warp ballot.
@@ -1187,18 +1203,47 @@ __host__ __device__ inline int degree_class(uint32_t d)
     return c;
 }
 
-// (a block-shared histogram first: out-degrees crowd into a few small values)
-__global__ void k_deg_hist(int64_t n, const uint32_t *__restrict__ odeg, unsigned *hist, int nd)
+// Counting sort of the roots by descending out-degree, in one block: each
+// out-degree's count becomes its first position (larger ones first), and the
+// classes' sizes are summed.
+__global__ void __launch_bounds__(1024) k_deg_slots(CoreState *st)
 {
-    extern __shared__ unsigned sh[];
-    for (int i = threadIdx.x; i < nd; i += blockDim.x) sh[i] = 0;
+    __shared__ unsigned s_warp[32], s_base;
+    __shared__ unsigned s_cls[NCLASS + 1];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (threadIdx.x <= NCLASS) s_cls[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_base = 0;
     __syncthreads();
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&sh[min(odeg[v], (uint32_t)(nd - 1))], 1u);
-    __syncthreads();
-    for (int i = threadIdx.x; i < nd; i += blockDim.x)
-        if (sh[i]) atomicAdd(&hist[i], sh[i]);
+    for (int top = (int)CORE_CLAMP; top >= 0; top -= 1024) {
+        const int d = top - (int)threadIdx.x;  // descending
+        const unsigned x = d >= 0 ? st->deg_cnt[d] : 0u;
+        unsigned inc = x;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned t = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc += t;
+        }
+        if (lane == 31) s_warp[wid] = inc;
+        __syncthreads();
+        if (wid == 0) {
+            const unsigned w = s_warp[lane];
+            unsigned wi = w;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned t = __shfl_up_sync(FULL, wi, o);
+                if (lane >= o) wi += t;
+            }
+            s_warp[lane] = wi - w;
+        }
+        __syncthreads();
+        const unsigned first = s_base + s_warp[wid] + inc - x;
+        if (d >= 0) {
+            st->deg_cnt[d] = first;
+            if (x) atomicAdd(&s_cls[min(degree_class((uint32_t)d), NCLASS)], x);
+        }
+        __syncthreads();
+        if (threadIdx.x == 1023) s_base = first + x;
+        __syncthreads();
+    }
+    if (threadIdx.x < NCLASS) st->class_cnt[threadIdx.x] = s_cls[threadIdx.x];
 }
 
 // Scatter roots so that out-degrees descend within the array (slot[d] holds
@@ -1214,7 +1259,7 @@ __global__ void k_deg_scatter(int64_t n, const uint32_t *__restrict__ odeg, unsi
         const bool valid = v < n;
         const unsigned act = __ballot_sync(FULL, valid);
         if (!valid) continue;
-        const uint32_t d = odeg[v];
+        const uint32_t d = min(odeg[v], CORE_CLAMP);
         const unsigned peers = __match_any_sync(act, d);
         const int leader = __ffs(peers) - 1;
         unsigned at = 0;
@@ -1295,8 +1340,20 @@ __global__ void k_scan_add(int64_t *out, int64_t n, const unsigned long long *__
     if (i < n) out[i] += (int64_t)bsum[blockIdx.x];
 }
 
+// Small arrays: the whole scan in one block (one launch, no scratch).
+constexpr int64_t SCAN_ONE_BLOCK = 8192;
+__global__ void __launch_bounds__(1024) k_scan_one(const uint32_t *in, int64_t *out, int64_t n)
+{
+    block_scan_u32_i64(in, out, n);
+}
+
 pvt_status exclusive_scan_u32_i64(const uint32_t *in, int64_t *out, int64_t n, cudaStream_t s)
 {
+    if (n <= SCAN_ONE_BLOCK) {
+        k_scan_one<<<1, 1024, 0, s>>>(in, out, n);
+        PVT_CK(cudaGetLastError());
+        return PVT_OK;
+    }
     int64_t nb = (n + 1023) / 1024;
     unsigned long long *bsum = nullptr;
     PVT_CK(cudaMallocAsync(&bsum, (size_t)std::max<int64_t>(nb, 1) * sizeof(unsigned long long), s));
@@ -1439,31 +1496,32 @@ pvt_status orient_build(pvt_dag *g, uint32_t flags, cudaStream_t s)
     }
 
     uint32_t *sup = nullptr, *list = nullptr, *odeg = nullptr;
-    unsigned *dhist = nullptr;
     CoreState *cst = nullptr;
     const size_t nb = (size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t);
     PVT_CK(cudaMallocAsync(&sup, nb, s));
     PVT_CK(cudaMallocAsync(&list, 4 * nb, s));
-    PVT_CK(cudaMallocAsync(&cst, sizeof(CoreState) + sizeof(unsigned), s));
+    PVT_CK(cudaMallocAsync(&cst, sizeof(CoreState), s));
     PVT_CK(cudaMallocAsync(&g->rnd, nb, s));
     PVT_CK(cudaMallocAsync(&g->core, nb, s));
     PVT_CK(cudaMallocAsync(&odeg, nb + sizeof(uint32_t), s));
     PVT_CK(cudaMallocAsync(&g->orow, (size_t)(n + 1) * sizeof(int64_t), s));
-    unsigned *d_alpha = (unsigned *)(cst + 1);
-    CoreState hst{};
-    unsigned alpha = 0;
+    PVT_CK(cudaMallocAsync(&g->ocol, (size_t)std::max<int64_t>(g->m, 1) * sizeof(uint32_t), s));
+    PVT_CK(cudaMallocAsync(&g->roots, nb, s));
+    CoreState *hst = reinterpret_cast<CoreState *>(reinterpret_cast<char *>(g->h_stats) + PIN_ORIENT);
+    // small graphs: no more blocks than warps have vertices
+    const int og = (int)std::max<int64_t>(1, std::min<int64_t>(grid, (n + 7) / 8));
     pvt_status st = PVT_OK;
     for (int form = 0;; ++form) {
         // core numbers and removal order: by rounds, else (once, if those
-        // were given up) level by level
-        PVT_CK(cudaMemsetAsync(cst, 0, sizeof(CoreState) + sizeof(unsigned), s));
+        // were given up) level by level.  Everything after them is enqueued
+        // without waiting to learn which; the result is read once.
+        PVT_CK(cudaMemsetAsync(cst, 0, sizeof(CoreState), s));
         phase_begin(g, 0, s);
         if (form == 0) {
             // one cooperative launch: every block must be resident at once;
             // small graphs take fewer blocks (a barrier of few is faster)
             int per_sm = 0;
-            PVT_CK(cudaFuncSetAttribute(k_cores, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORE_SMEM));
-            PVT_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cores, CORE_THREADS, CORE_SMEM));
+            PVT_CK(resident_blocks((const void *)k_cores, CORE_THREADS, CORE_SMEM, &per_sm));
             if (per_sm < 1) {
                 set_error("pvt_orient: core kernel cannot be resident");
                 return PVT_ECUDA;
@@ -1476,79 +1534,59 @@ pvt_status orient_build(pvt_dag *g, uint32_t flags, cudaStream_t s)
             uint32_t *rnd = g->rnd, *core = g->core;
             unsigned *err = g->d_err;
             void *args[] = {&nn, &rp, &col, &rnd, &core, &sup, &list, &cst, &err};
-            PVT_CK(cudaLaunchCooperativeKernel((void *)k_cores, dim3(blocks), dim3(CORE_THREADS), args, CORE_SMEM, s));
+            if (blocks == 1)
+                PVT_CK(cudaLaunchKernel((void *)k_cores, dim3(1), dim3(CORE_THREADS), args, CORE_SMEM, s));
+            else
+                PVT_CK(cudaLaunchCooperativeKernel((void *)k_cores, dim3(blocks), dim3(CORE_THREADS), args, CORE_SMEM, s));
             g->stats.launches++;
         } else if ((st = peel_levels(g, sup, list, &cst->peel, s)) != PVT_OK) {
             return st;
         }
         phase_end(g, 0, s);
         phase_begin(g, 1, s);
-        // orientation
-        k_outdeg<<<grid, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, odeg, d_alpha);
+        // orientation; roots by descending out-degree, grouped into classes
+        k_outdeg<<<og, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, odeg, cst);
         PVT_CK(cudaGetLastError());
-        st = exclusive_scan_u32_i64(odeg, g->orow, n, s);
-        g->stats.launches += 4;
-        if (st != PVT_OK) return st;
-        PVT_CK(cudaMemcpyAsync(&hst, cst, sizeof(CoreState), cudaMemcpyDeviceToHost, s));
-        PVT_CK(cudaMemcpyAsync(&alpha, d_alpha, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+        if ((st = exclusive_scan_u32_i64(odeg, g->orow, n, s)) != PVT_OK) return st;
+        k_fill<<<og, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, g->orow, g->ocol);
+        k_deg_slots<<<1, 1024, 0, s>>>(cst);
+        k_deg_scatter<<<og, 256, 0, s>>>(n, odeg, cst->deg_cnt, g->roots);
+        PVT_CK(cudaGetLastError());
+        phase_end(g, 1, s);
+        g->stats.launches += n <= SCAN_ONE_BLOCK ? 5 : 7;
+        PVT_CK(cudaMemcpyAsync(g->h_err, g->d_err, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+        PVT_CK(cudaMemcpyAsync(hst, cst, offsetof(CoreState, deg_cnt), cudaMemcpyDeviceToHost, s));
         PVT_CK(cudaStreamSynchronize(s));
-        st = check_device(g, s, "pvt_orient: peeling");
-        if (st != PVT_OK) return st;
-        g->stats.peel_rounds += hst.peel.rounds;
-        if (!hst.bail) break;
+        st = check_status(g, "pvt_orient: peeling");
+        g->stats.peel_rounds += hst->peel.rounds;
+        if (st != PVT_OK || !hst->bail) break;
     }
-    g->stats.peel_levels = hst.peel.levels;
-    if (hst.peel.top_level > (unsigned)MAX_ALPHA) {
+    PVT_CK(cudaFreeAsync(sup, s));
+    PVT_CK(cudaFreeAsync(list, s));
+    PVT_CK(cudaFreeAsync(cst, s));
+    PVT_CK(cudaFreeAsync(odeg, s));
+    if (st != PVT_OK) return st;
+    g->stats.peel_levels = hst->peel.levels;
+    if (hst->peel.top_level > (unsigned)MAX_ALPHA) {
         set_error("pvt_orient: degeneracy above the supported " + std::to_string(MAX_ALPHA));
         return PVT_EINVAL;
     }
     // alpha = the degeneracy (top core level): it bounds every out-degree and,
     // unlike the largest out-degree, does not depend on the removal order
     // within a level
-    if (alpha > hst.peel.top_level) {
+    if (hst->most_out > hst->peel.top_level) {
         set_error("pvt_orient: an out-degree exceeds the degeneracy");
         return PVT_EINTERNAL;
     }
-    g->alpha = (int32_t)hst.peel.top_level;
-    PVT_CK(cudaMallocAsync(&g->ocol, (size_t)std::max<int64_t>(g->m, 1) * sizeof(uint32_t), s));
-    k_fill<<<grid, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, g->orow, g->ocol);
-    PVT_CK(cudaGetLastError());
-    g->stats.launches++;
-
-    // roots by descending out-degree (counting sort), grouped into classes
-    const int nd = g->alpha + 1;
-    PVT_CK(cudaMallocAsync(&dhist, (size_t)nd * sizeof(unsigned), s));
-    PVT_CK(cudaMemsetAsync(dhist, 0, (size_t)nd * sizeof(unsigned), s));
-    k_deg_hist<<<grid, 256, (size_t)nd * sizeof(unsigned), s>>>(n, odeg, dhist, nd);
-    g->stats.launches++;
-    std::vector<unsigned> hh(nd), slot(nd);
-    PVT_CK(cudaMemcpyAsync(hh.data(), dhist, (size_t)nd * sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-    PVT_CK(cudaStreamSynchronize(s));
-    // positions: larger out-degrees first; class c (degree range) is then a
-    // contiguous slice, higher classes first
-    unsigned pos = 0;
-    for (int d = nd - 1; d >= 0; --d) { slot[d] = pos; pos += hh[d]; }
-    for (int c = 0; c < NCLASS; ++c) g->class_cnt[c] = 0;
-    for (int d = 0; d < nd; ++d) g->class_cnt[degree_class((uint32_t)d)] += hh[d];
-    {
-        int64_t off = 0;
-        for (int c = NCLASS - 1; c >= 0; --c) { g->class_start[c] = off; off += g->class_cnt[c]; }
+    g->alpha = (int32_t)hst->peel.top_level;
+    int64_t off = 0;
+    for (int c = NCLASS - 1; c >= 0; --c) {  // higher classes first
+        g->class_cnt[c] = hst->class_cnt[c];
+        g->class_start[c] = off;
+        off += g->class_cnt[c];
+        g->stats.roots[c] = (uint64_t)g->class_cnt[c];
     }
-    PVT_CK(cudaMemcpyAsync(dhist, slot.data(), (size_t)nd * sizeof(unsigned), cudaMemcpyHostToDevice, s));
-    PVT_CK(cudaMallocAsync(&g->roots, nb, s));
-    k_deg_scatter<<<grid, 256, 0, s>>>(n, odeg, dhist, g->roots);
-    PVT_CK(cudaGetLastError());
-    phase_end(g, 1, s);
-    g->stats.launches++;
-    for (int c = 0; c < NCLASS; ++c) g->stats.roots[c] = (uint64_t)g->class_cnt[c];
-
-    PVT_CK(cudaFreeAsync(sup, s));
-    PVT_CK(cudaFreeAsync(list, s));
-    PVT_CK(cudaFreeAsync(cst, s));
-    PVT_CK(cudaFreeAsync(odeg, s));
-    PVT_CK(cudaFreeAsync(dhist, s));
-    PVT_CK(cudaStreamSynchronize(s));
-    return check_device(g, s, "pvt_orient");
+    return PVT_OK;
 }
 
 

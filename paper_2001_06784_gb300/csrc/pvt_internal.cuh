@@ -185,6 +185,20 @@ void stats_reset(pvt_dag *g);
 
 // Read the device status word (synchronises s) and map it to a status.
 pvt_status check_device(pvt_dag *g, cudaStream_t s, const char *what);
+// The same for a status word that is already in *g->h_err.
+pvt_status check_status(const pvt_dag *g, const char *what);
+
+// A dag's small device words in one allocation -- walk statistics, queue
+// heads, status word -- so that one operation clears them and one copy brings
+// them back (pinned copies at the same offsets; PIN_ORIENT: the orientation's
+// result).
+constexpr size_t CTL_Q = 128, CTL_ERR = 192, CTL_BYTES = 196, PIN_ORIENT = 256, PIN_BYTES = 4096;
+
+// Resident blocks per SM of a kernel with `smem` bytes of dynamic shared
+// memory, which it is allowed to have.  Remembered per device, kernel and
+// launch shape: the driver's answer takes about a microsecond, several times
+// per count call.
+cudaError_t resident_blocks(const void *kern, int threads, size_t smem, int *per_sm);
 
 // A named host range around a library call, so that a profiler's timeline
 // shows where each call begins and ends (NVTX; nothing happens without an

@@ -78,7 +78,7 @@ struct WarpWork {
             uint32_t hp[D + 1];  // DFS stack: (h << 16) | p
         };
     };
-    uint16_t cmap[32];           // compacted index -> member index
+    alignas(8) uint16_t cmap[32];  // members of a label being relabelled
     uint32_t fbuf[36];           // copy of a donated frame taken from the queue
     __device__ __forceinline__ uint32_t *stk() { return GSTACK ? gstk : stk_s; }
 };
@@ -634,12 +634,14 @@ __device__ void compact_loop(WarpWork<NW> &Wk, unsigned *shist, const CountArgs 
 }
 
 // Relabel a label of at most 32 members (word w of its bitset in lane w's cw,
-// 0 in the lanes from the word count on; s: their number): member k of the label = its k-th
-// member in ascending order, listed in cmap.  Lane j returns row j of the
+// 0 in the lanes from the word count on; s: their number): member k of the
+// label = its k-th member in ascending order.  cmap lists them as word << 5 |
+// (31 - bit), padded to a multiple of four.  Lane j returns row j of the
 // one-word adjacency: rows are symmetric, so the row of member j itself,
-// compressed to the label's members, word by word from the top.
-template <int NW, int RS, typename M>
-__device__ __forceinline__ uint32_t relabel_rows(const uint32_t *adj, M *cmap, int lane, uint32_t cw, int &s)
+// compressed to the label's members, from the top; the four loads of a step
+// do not wait for one another.
+template <int NW, int RS>
+__device__ __forceinline__ uint32_t relabel_rows(const uint32_t *adj, uint16_t *cmap, int lane, uint32_t cw, int &s)
 {
     const int c = __popc(cw);
     int inc = c;
@@ -649,23 +651,25 @@ __device__ __forceinline__ uint32_t relabel_rows(const uint32_t *adj, M *cmap, i
         if (lane >= o) inc += t;
     }
     s = __shfl_sync(FULL, inc, NW - 1);
-    M *dst = cmap + (inc - c);
-    for (uint32_t x = cw; x; x &= x - 1) *dst++ = (M)(lane * 32 + __ffs(x) - 1);
+    uint16_t *dst = cmap + (inc - c);
+    for (uint32_t x = cw; x; x &= x - 1) *dst++ = (uint16_t)((lane * 32 + __ffs(x) - 1) ^ 31);
+    const int s4 = (s + 3) & ~3;
+    if (lane >= s && lane < s4) cmap[lane] = 0;
     __syncwarp();
-    const uint32_t *mine = adj + (lane < s ? (int)cmap[lane] : 0) * RS;
+    const uint32_t *mine = adj + (lane < s ? (int)(cmap[lane] ^ 31) : 0) * RS;
     uint32_t r = 0;
-    for (unsigned nz = __ballot_sync(FULL, cw != 0); nz;) {
-        const int w = 31 - __clz(nz);
-        nz ^= 1u << w;
-        const uint32_t a = mine[w];
-        for (uint32_t m = __shfl_sync(FULL, cw, w); m;) {
-            const int z = __clz(m);
-            m ^= 0x80000000u >> z;
-            r = __funnelshift_l(a << z, r, 1);  // r * 2 + bit 31 - z of a
-        }
+    for (int k = s4 - 4; k >= 0; k -= 4) {
+        const uint2 q = *reinterpret_cast<const uint2 *>(cmap + k);
+        const uint32_t v0 = q.x & 0xFFFFu, v1 = q.x >> 16, v2 = q.y & 0xFFFFu, v3 = q.y >> 16;
+        const uint32_t a0 = mine[v0 >> 5], a1 = mine[v1 >> 5], a2 = mine[v2 >> 5], a3 = mine[v3 >> 5];
+        // r * 2 + bit, from member k + 3 down
+        r = __funnelshift_l(__funnelshift_l(0u, a3, v3), r, 1);
+        r = __funnelshift_l(__funnelshift_l(0u, a2, v2), r, 1);
+        r = __funnelshift_l(__funnelshift_l(0u, a1, v1), r, 1);
+        r = __funnelshift_l(__funnelshift_l(0u, a0, v0), r, 1);
     }
     __syncwarp();
-    return lane < s ? r : 0u;
+    return lane < s ? r & (s >= 32 ? FULL : (1u << s) - 1u) : 0u;
 }
 
 // Frame slots a warp reserved in the emit buffer.  Slots are reserved in
@@ -1040,9 +1044,12 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A,
                         const bool inR = (Rj >> lane) & 1u;
                         bool push = inR;
                         int cs = 0;
+                        // the earlier members of R in word j itself, taken off at the end
+                        const uint32_t Sj = word_of(S, Sl, j) & Rj & low;
                         if (MODE == MODE_GLOBAL && inR) {
 #pragma unroll
-                            for (int w = 0; w < NW; ++w) cs += __popc(row(j, w) & M[w] & (w == j ? ~(Rj & low) : FULL));
+                            for (int w = 0; w < NW; ++w) cs += __popc(row(j, w) & M[w]);
+                            cs -= __popc((REG ? row(j, j) : Wk.adj[(j * 32 + lane) * RS + j]) & Sj);
                             if (cs <= 2) {
                                 bool adj = false;
                                 if (cs == 2) {
@@ -1187,12 +1194,14 @@ __device__ __forceinline__ void bind_warp(WarpWork<NW> &Wk, unsigned char *local
 // Lane 0 of a split launch: the next item -- 2 with v = a fresh item index
 // below nitems, 1 with v = the ticket of a donated frame, 3 when no work is
 // left (or an error or a timeout ended the launch).
-__device__ __forceinline__ int queue_take(const CountArgs &A, unsigned nitems, unsigned &v)
+// A warp that may not wait leaves when no published frame is without a taker.
+__device__ __forceinline__ int queue_take(const CountArgs &A, unsigned nitems, unsigned &v, bool may_wait = true)
 {
     if (vload(A.qctl + Q_ROOT) < nitems) {
         const unsigned rr = atomicAdd(A.qctl + Q_ROOT, 1u);
         if (rr < nitems) { v = rr; return 2; }
     }
+    if (!may_wait && vload64(A.qctl + Q_HEAD) >= vload64(A.qctl + Q_TAIL)) return 3;
     // a ticket for the next donated frame; wait on its own slot
     int kind = 0;
     const unsigned t = (unsigned)atomicAdd(qword(A.qctl + Q_HEAD), 1ull);
@@ -1247,10 +1256,15 @@ __global__ void __launch_bounds__(32 * warps_per_block<NW>())
     const unsigned CHUNK = NW == 1 ? A.chunk : 1u;
     unsigned qi = 0, qend = 0;
     if (SPLIT) {
-        // heavy roots and donated subtree frames from one device work queue
+        // heavy roots and donated subtree frames from one device work queue.
+        // Once the roots are out, the second half of the blocks leaves instead
+        // of waiting for donations, so that the next class's kernel can start
+        // on the SMs (waiting was 28 % of the warps' time in the 129..256 class
+        // of the 10.8M-edge graph: donations, not takers, are what is scarce)
+        const bool may_wait = blockIdx.x < (gridDim.x + 1) / 2;
         for (;;) {
             unsigned v = 0;
-            int kind = lane == 0 ? queue_take(A, A.nroots, v) : 0;
+            int kind = lane == 0 ? queue_take(A, A.nroots, v, may_wait) : 0;
             kind = __shfl_sync(FULL, kind, 0);
             v = __shfl_sync(FULL, v, 0);
             if (kind == 3) break;
@@ -1315,6 +1329,14 @@ static __global__ void k_split_init(uint32_t *qctl, unsigned nroots)
 
 constexpr unsigned SPLIT_QCAP = 1u << 17;
 
+// Roots of the <= 32 class taken per queue access: the policy's, but no more
+// than leaves work for every resident warp (four at a time, 5,000 roots were
+// walked by 1,250 warps of 4,864).
+inline unsigned claim_size(const pvt_dag *g, unsigned cnt, unsigned warps)
+{
+    return std::max(1u, std::min((unsigned)g->policy.chunk, cnt / std::max(warps, 1u)));
+}
+
 // The lane walk of one-word labels (lanes.cuh, walk_lanes.cu): the frames of
 // the two-phase count.
 pvt_status launch_lanes_frames(pvt_dag *g, const CountArgs &base, cudaStream_t s);
@@ -1338,7 +1360,6 @@ pvt_status launch_class(pvt_dag *g, const CountArgs &base, int cls, cudaStream_t
     A.nroots = cnt;
     A.qhead = g->d_q + cls;
     A.cls = cls;
-    A.chunk = (unsigned)g->policy.chunk;
     constexpr size_t smem = smem_bytes<NW, MODE, SHIST>();
     constexpr int WPB = warps_per_block<NW>();
     // the widest class always runs persistent warps (its stacks are per resident warp)
@@ -1371,27 +1392,20 @@ pvt_status launch_class(pvt_dag *g, const CountArgs &base, int cls, cudaStream_t
         A.qctl = g->qctl + QCTL_WORDS * cls;
         A.qcap = SPLIT_QCAP;
     }
-    PVT_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    PVT_CK(resident_blocks((const void *)kern, 32 * WPB, smem, &per_sm));
+    if (per_sm < 1) {
+        set_error("count kernel cannot be resident (shared memory)");
+        return PVT_ECUDA;
+    }
+    A.chunk = claim_size(g, cnt, (unsigned)(g->num_sms * per_sm * WPB));
     const unsigned need = (cnt + WPB - 1) / WPB;
-    unsigned grid = need;
+    // persistent: sized to the resident warps (per-warp global stacks too)
+    const unsigned grid = persist ? std::min<unsigned>((unsigned)(g->num_sms * per_sm), need) : need;
     if (WarpWork<NW>::GSTACK) {
-        // per-warp global stacks: size the grid to the resident warps (these
-        // classes always walk their roots from the persistent loop)
-        int per_sm = 0;
-        PVT_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * WPB, smem));
-        grid = std::max(1u, std::min<unsigned>((unsigned)(g->num_sms * std::max(per_sm, 1)), need));
         pvt_status st = grow(g->gstack[cls], (size_t)grid * WPB * (32 * NW + 1) * NW, s);
         if (st != PVT_OK) return st;
         A.gstack = g->gstack[cls].p;
-    }
-    if (persist) {
-        int per_sm = 0;
-        PVT_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * WPB, smem));
-        if (per_sm < 1) {
-            set_error("count kernel cannot be resident (shared memory)");
-            return PVT_ECUDA;
-        }
-        grid = std::min<unsigned>((unsigned)(g->num_sms * per_sm), need);
     }
     if (MODE == MODE_EDGE && persist && NW <= 8) {
         // per-warp edge-id tables of member pairs (the gather fills them)
@@ -1545,9 +1559,8 @@ pvt_status launch_batch_class(const BatchGraph *gs, const uint64_t *entries, uns
 {
     constexpr size_t smem = smem_bytes<NW, MODE, false>();
     auto kern = k_count_batch<NW, MODE>;
-    PVT_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    PVT_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * warps_per_block<NW>(), smem));
+    PVT_CK(resident_blocks((const void *)kern, 32 * warps_per_block<NW>(), smem, &per_sm));
     if (per_sm < 1) {
         set_error("batched walk kernel cannot be resident");
         return PVT_ECUDA;

@@ -23,9 +23,8 @@ static pvt_status launch_cta_nw(pvt_dag *g, CountArgs A, int cls, int dmax, cuda
         return PVT_EINVAL;
     }
     const size_t smem = Lay::bytes(warps, dmax);
-    PVT_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    PVT_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * warps, smem));
+    PVT_CK(resident_blocks((const void *)kern, 32 * warps, smem, &per_sm));
     if (per_sm < 1) {
         set_error("CTA walk kernel cannot be resident");
         return PVT_ECUDA;

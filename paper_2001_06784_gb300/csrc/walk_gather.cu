@@ -21,6 +21,8 @@
 // 0.93 ms here plus about 0.3 ms of the lane walk; on a 61k-vertex graph with
 // planted communities, where one warp's dense root was the time, 1.10 ms
 // became 0.17 + 0.22 ms.
+#include <type_traits>
+
 #include "lanes.cuh"
 
 namespace pvt {
@@ -29,8 +31,12 @@ constexpr int G1_WPB = 8;              // warps per block
 constexpr unsigned G1_RESERVE = 16;    // frame slots a warp reserves at once
 constexpr int G1_ROUNDS = 4;           // rounds of 32 entries with loads in flight
 
+// NARROW: the graph has fewer than 2^32 edges, so positions in the out-lists
+// fit 32 bits.
+template <bool NARROW>
 __global__ void __launch_bounds__(32 * G1_WPB) k_gather1(CountArgs A)
 {
+    using Pos = std::conditional_t<NARROW, uint32_t, int64_t>;
     __shared__ unsigned sh32[HIST_H * HIST_P];
     __shared__ uint32_t s_tmp[G1_WPB][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -91,10 +97,13 @@ __global__ void __launch_bounds__(32 * G1_WPB) k_gather1(CountArgs A)
             // k-th member with a nonempty list in lane k: its index, and the
             // distance from a position in the concatenation to its entry
             const unsigned some = __ballot_sync(FULL, od != 0);
-            if (od) tmp[__popc(some & lt)] = (uint32_t)lane;
-            __syncwarp();
-            const uint32_t mk = tmp[lane] & 31u;
-            const int64_t delta = __shfl_sync(FULL, rs - (int64_t)off, (int)mk);
+            uint32_t mk = (uint32_t)lane;
+            if (some & (some + 1u)) {  // an empty list before another
+                if (od) tmp[__popc(some & lt)] = (uint32_t)lane;
+                __syncwarp();
+                mk = tmp[lane] & 31u;
+            }
+            const Pos delta = __shfl_sync(FULL, (Pos)(rs - (int64_t)off), (int)mk);
             __syncwarp();
             uint32_t row = 0;   // this member's row
             int started = -1;   // lists started before the current round, less one
@@ -109,7 +118,7 @@ __global__ void __launch_bounds__(32 * G1_WPB) k_gather1(CountArgs A)
                     own[q] = started + __popc(starts & le);
                     started += __popc(starts);
                     const uint32_t t = w0 + lane;
-                    const int64_t at = __shfl_sync(FULL, delta, own[q]) + t;
+                    const Pos at = __shfl_sync(FULL, delta, own[q]) + (Pos)t;  // (modulo 2^32 in 32 bits)
                     x[q] = t < T ? A.ocol[at] : 0xFFFFFFFFu;
                 }
 #pragma unroll
@@ -178,18 +187,21 @@ __global__ void __launch_bounds__(32 * G1_WPB) k_gather1(CountArgs A)
     hist_flush(sh32, A);
 }
 
-static cudaError_t gather1_grid(int num_sms, unsigned *blocks)
+using Gather1 = void (*)(CountArgs);
+static Gather1 gather1_kernel(const pvt_dag *g) { return g->m < (1ll << 32) ? k_gather1<true> : k_gather1<false>; }
+
+static cudaError_t gather1_grid(const pvt_dag *g, unsigned *blocks)
 {
     int per_sm = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gather1, 32 * G1_WPB, 0);
-    *blocks = (unsigned)(num_sms * std::max(per_sm, 1));
+    const cudaError_t e = resident_blocks((const void *)gather1_kernel(g), 32 * G1_WPB, 0, &per_sm);
+    *blocks = (unsigned)(g->num_sms * std::max(per_sm, 1));
     return e;
 }
 
 unsigned gather1_slots(const pvt_dag *g, unsigned cnt)
 {
     unsigned blocks = 0;
-    gather1_grid(g->num_sms, &blocks);
+    gather1_grid(g, &blocks);
     return cnt + blocks * G1_WPB * G1_RESERVE;
 }
 
@@ -201,13 +213,13 @@ pvt_status launch_gather1(pvt_dag *g, const CountArgs &base, const uint32_t *roo
     A.roots = roots;
     A.nroots = cnt;
     A.qhead = g->d_q + 1;
-    A.chunk = (unsigned)g->policy.chunk;
     A.emit1_cap = slots;
     unsigned blocks = 0;
-    PVT_CK(gather1_grid(g->num_sms, &blocks));
+    PVT_CK(gather1_grid(g, &blocks));
+    A.chunk = claim_size(g, cnt, blocks * G1_WPB);
     const unsigned per_block = G1_WPB * A.chunk;
     blocks = std::max(1u, std::min(blocks, (cnt + per_block - 1) / per_block));
-    k_gather1<<<blocks, 32 * G1_WPB, 0, s>>>(A);
+    gather1_kernel(g)<<<blocks, 32 * G1_WPB, 0, s>>>(A);
     PVT_CK(cudaGetLastError());
     g->stats.launches++;
     return PVT_OK;

@@ -34,9 +34,8 @@ static pvt_status launch_lanes_kernel(pvt_dag *g, const CountArgs &A, int phase,
 {
     constexpr size_t smem = lane_smem_bytes();
     auto kern = k_lanes;
-    PVT_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    PVT_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * LANE_WPB, smem));
+    PVT_CK(resident_blocks((const void *)kern, 32 * LANE_WPB, smem, &per_sm));
     if (per_sm < 1) {
         set_error("lane walk kernel cannot be resident (shared memory)");
         return PVT_ECUDA;
