@@ -226,12 +226,8 @@ static void dag_release(pvt_dag *g)
     auto release = [&](void *p) {
         if (p) cudaFreeAsync(p, fs);
     };
-    release(g->rnd);
-    release(g->core);
-    release(g->orow);
-    release(g->ocol);
+    release(g->graph_mem);
     release(g->oeid);
-    release(g->roots);
     release(g->hist.p);
     for (int c = 0; c < NCLASS; ++c) {
         release(g->rootbuf[c].p);

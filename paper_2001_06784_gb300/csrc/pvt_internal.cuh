@@ -49,7 +49,8 @@ struct pvt_dag {
     int32_t alpha = 0;
     const int64_t *row_ptr = nullptr;  // borrowed undirected CSR
     const uint32_t *col = nullptr;
-    // owned device state
+    // owned device state (the next five in graph_mem)
+    void *graph_mem = nullptr;
     uint32_t *rnd = nullptr;       // orientation key of each vertex (ties: by id)
     uint32_t *core = nullptr;      // peel level (core number) of each vertex
     int64_t *orow = nullptr;       // DAG CSR row pointers, int64[n+1]
