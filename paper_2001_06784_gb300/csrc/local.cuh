@@ -38,7 +38,9 @@ namespace pvt {
 // part for LOCAL_PART_EDGES edges, more when they are dense: the tree grows
 // with the edges of a sparse member graph and far faster in a dense one, and
 // each part walks the root's pivot chain again.
-constexpr unsigned LOCAL_HEAVY_EDGES = 192, LOCAL_PART_EDGES = 128, LOCAL_MAX_PARTS = 64;
+// A near-clique's tree is small: at most LOCAL_FEW_MISSING edges short of one,
+// a root is not split.
+constexpr unsigned LOCAL_HEAVY_EDGES = 48, LOCAL_PART_EDGES = 192, LOCAL_MAX_PARTS = 64, LOCAL_FEW_MISSING = 8;
 __device__ __forceinline__ unsigned local_parts(unsigned edges, int d)
 {
     const float density = 2.0f * (float)edges / ((float)d * (float)(d - 1));
@@ -66,6 +68,11 @@ struct LocalWork {
         uint32_t stk_s[GSTACK ? 1 : (D + 1) * FW];
     };
     uint8_t mem[D];    // members of a clique leaf
+    // walk of a label of at most 32 members below a wider root (NW > 1): its
+    // members (relabel_rows), rows and stack
+    alignas(8) uint16_t cm[NW > 1 ? 32 : 4];
+    uint32_t crow[NW > 1 ? 32 : 1];
+    uint32_t cstk[NW > 1 ? 33 * 3 : 1];
     uint32_t *gstk;
     uint32_t *etab;    // edge ids of member pairs, D x D
     __device__ __forceinline__ uint32_t *stk() { return GSTACK ? gstk : stk_s; }
@@ -197,15 +204,7 @@ struct LocalWalk {
         }
         if (MODE == MODE_VERTEX) {
             if (lane >= h && lane <= kin) acc += coeff(p, lane - h, path);
-            if (kmost > kt) {
-                // the root's larger sizes, one size per lane
-                unsigned long long *row = A.out + (size_t)r * (A.kmax + 1) * A.W;
-                const unsigned n[4] = {path.a0, path.a1, path.a2, path.a3};
-                for (int k = kt + 1 + lane; k <= kmost; k += 32)
-                    for (int i = 0; i < 4; ++i)
-                        if (n[i] && k - h - i >= 0 && k - h - i <= p)
-                            atomic_add_scaled(row + (size_t)k * A.W, binom_at(A.B, p, k - h - i, A.Bw), n[i], A.W, A.err);
-            }
+            if (kmost > kt) high_root(h, p, path);
         }
         __syncwarp();
     }
@@ -292,6 +291,241 @@ struct LocalWalk {
         }
     }
 
+    // The subtree of a label S of s <= 32 members below a wider root, entered
+    // with (h, p) and the path members H, P (the prefix): relabelled to
+    // one-word rows, one member per lane.  A node costs a few one-word
+    // operations instead of NW times as many, and the prefix's share of it is
+    // summed, one size per lane, and credited once at the end.
+    __device__ void run_small(const uint32_t (&S)[NW], const uint32_t (&H)[NW], const uint32_t (&P)[NW], int s, int h,
+                              int p, WalkCounters &wc)
+    {
+        uint32_t cw = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w)
+            if (lane == w) cw = S[w];
+        int sz = 0;
+        const uint32_t r1 = relabel_rows<NW, RS>(Wk.adj, Wk.cm, lane, cw, sz);
+        const int mk = lane < s ? (int)(Wk.cm[lane] ^ 31) : 0;  // this lane's member
+        Wk.crow[lane] = r1;
+        __syncwarp();
+        auto adjacent = [&](int a, int b) { return (Wk.crow[a] >> b) & 1u; };
+        auto member = [&](int a) { return (int)(Wk.cm[a] ^ 31); };
+        const uint32_t low = (1u << lane) - 1u;
+        uint32_t S1 = s >= 32 ? FULL : (1u << s) - 1u, H1 = 0, P1 = 0;
+        int hh = h, pp = p, top = 0;
+        unsigned long long pre = 0;  // lane k: what a hold member of the prefix gains at size k <= kt
+        int kpre = 0;
+        for (;;) {
+            const int s1 = __popc(S1);
+            const bool in = (S1 >> lane) & 1u;
+            const uint32_t c = in ? (uint32_t)__popc(r1 & S1) : 0u;
+            const uint32_t best = __reduce_max_sync(FULL, in ? ((c + 1u) << 5 | (31u - (uint32_t)lane)) : 0u);
+            const uint32_t dsum = __reduce_add_sync(FULL, c);
+            wc.nodes++;
+            wc.words += (unsigned)s1;
+            bool closed = true;
+            Share path, own;
+            uint32_t PX = P1, N = 0;
+            int pc = pp, piv = 0;
+            if (dsum == (uint32_t)s1 * (uint32_t)(s1 - 1)) {
+                wc.leaves++;
+                path.a0 = 1;
+                pc = pp + s1;
+                PX = P1 | S1;
+            } else {
+                piv = 31 - (int)(best & 31u);
+                const uint32_t a0 = __shfl_sync(FULL, r1, piv);
+                N = a0 & S1;
+                const uint32_t R = hh + 1 > A.kmax ? 0u : S1 & ~a0 & ~(1u << piv);
+                const bool inR = (R >> lane) & 1u;
+                const uint32_t child = inR ? r1 & S1 & ~(R & low) : 0u;
+                const int cs = __popc(child);
+                const int a = child ? __ffs(child) - 1 : 0, b = child ? 31 - __clz(child) : 0;
+                const bool pair = inR && cs == 2 && adjacent(a, b);
+                const unsigned b1 = __ballot_sync(FULL, inR && cs == 1), b2 = __ballot_sync(FULL, pair);
+                const unsigned bn = __ballot_sync(FULL, inR && cs == 2 && !pair);
+                const unsigned bp = __ballot_sync(FULL, inR && cs > 2);
+                const unsigned n1 = __popc(b1), n2 = __popc(b2), nn = __popc(bn);
+                const unsigned n0 = __popc(R & ~(b1 | b2 | bn | bp));
+                if (inR && cs <= 2) {
+                    own.a1 = 1;
+                    own.a2 = cs;
+                    own.a3 = pair;
+                    if (MODE == MODE_EDGE && cs) {
+                        const uint32_t *em = Wk.etab + (size_t)mk * D;
+                        const int ma = member(a), mb = member(b);
+                        add_edge(em[ma], hh + 2, pair ? pp + 1 : pp);
+                        if (cs == 2) add_edge(em[mb], hh + 2, pair ? pp + 1 : pp);
+                        if (pair) add_edge(Wk.etab[(size_t)ma * D + mb], hh + 3, pp);
+                    }
+                }
+                if (top + __popc(bp) > 33) {
+                    if (lane == 0) atomicOr(A.err, DERR_STACK);
+                    return;
+                }
+                __syncwarp();
+                if ((bp >> lane) & 1u) {
+                    uint32_t *f = Wk.cstk + (top + __popc(bp & low)) * 3;
+                    f[0] = child;
+                    f[1] = H1 | 1u << lane;
+                    f[2] = P1;
+                }
+                top += __popc(bp);
+                const unsigned held = hh + 2 <= A.kmax ? nn : 0u;
+                wc.nodes += n0 + n1 + n2 + 2 * nn + held;
+                wc.leaves += n0 + n1 + n2 + nn + held;
+                wc.words += n1 + 2 * (n2 + nn);
+                path.a1 = n0 + n1 + n2 + nn;
+                path.a2 = n1 + 2 * (n2 + nn);
+                path.a3 = n2;
+                if (in) {
+                    const uint32_t lim = r1 & (inR ? low : FULL);
+                    const unsigned t1 = __popc(lim & (b1 | bn)), t2 = __popc(lim & b2);
+                    own.a2 += t1 + t2;
+                    own.a3 += t2;
+                }
+                const int ps = __popc(N);
+                if (ps <= 2) {
+                    const int na = N ? __ffs(N) - 1 : 0, nb = N ? 31 - __clz(N) : 0;
+                    const bool adjp = ps == 2 && adjacent(na, nb);
+                    const bool split = ps == 2 && !adjp;
+                    const bool hold = split && hh + 1 <= A.kmax;
+                    wc.nodes += 1 + split + hold;
+                    wc.leaves += 1 + hold;
+                    wc.words += (unsigned)ps;
+                    path.a0 += 1;
+                    path.a1 += 1 + (unsigned)ps;
+                    path.a2 += ps == 0 ? 0u : (ps == 1 ? 1u : (adjp ? 3u : 2u));
+                    path.a3 += adjp;
+                    if (lane == piv) {
+                        own.a1 += 1;
+                        own.a2 += (unsigned)ps;
+                        own.a3 += adjp;
+                    } else if ((ps >= 1 && lane == na) || (ps == 2 && lane == nb)) {
+                        own.a1 += 1;
+                        own.a2 += adjp ? 2u : 1u;
+                        own.a3 += adjp;
+                    }
+                    if (MODE == MODE_EDGE && ps) {
+                        int x = -1, y = 0;
+                        if (lane == 0) { x = piv; y = na; }
+                        if (lane == 1 && ps == 2) { x = piv; y = nb; }
+                        if (lane == 2 && adjp) { x = na; y = nb; }
+                        if (x >= 0) add_edge(Wk.etab[(size_t)member(x) * D + member(y)], hh + 2, adjp ? pp + 1 : pp);
+                    }
+                } else {
+                    closed = false;
+                }
+            }
+            if (path.any()) {
+                const int kmost = min(A.kmax, hh + pc + (path.a3 ? 3 : (path.a2 ? 2 : (path.a1 ? 1 : 0))));
+                const int kin = min(kt, kmost);
+                kpre = max(kpre, kin);
+                // this lane's member
+                const bool inH = (H1 >> lane) & 1u, inP = (PX >> lane) & 1u;
+                const Share sh = inH || inP ? path : own;
+                const bool has = sh.any();
+                const int hl = inP ? hh + 1 : hh, pl = inP ? pc - 1 : pc;
+                if (pc < LOCAL_BINOM) {
+                    const uint32_t *row = bin + pl * (pl + 1) / 2;
+                    uint32_t c1 = 0, c2 = 0, c3 = 0;
+                    for (int e = 0; hh + e <= kin; ++e) {
+                        const uint32_t c0 = e <= pl ? row[e] : 0u;
+                        const uint32_t v = sh.a0 * c0 + sh.a1 * c1 + sh.a2 * c2 + sh.a3 * c3;
+                        if (has && v && hl + e <= kin) tab[(hl + e) * D + mk] += v;
+                        c3 = c2;
+                        c2 = c1;
+                        c1 = c0;
+                    }
+                } else if (has) {
+                    for (int k = hl; k <= min(kin, hl + pl + 3); ++k) tab[k * D + mk] += coeff(pl, k - hl, sh);
+                }
+                if (lane >= hh && lane <= kin) pre += coeff(pc, lane - hh, path);
+                if (kmost > kt) {  // sizes above the table: everyone at once
+                    if (has) add_high(cell(mk), hl, pl, sh, kt + 1);
+                    high_prefix(hh, pc, H, P, path);
+                }
+                if (MODE == MODE_EDGE) {
+                    // pairs of this lane's member with a path member of the label
+                    for (uint32_t us = H1 | PX; us; us &= us - 1) {
+                        const int u = __ffs(us) - 1;
+                        if (has && !((inH || inP) && lane <= u)) {
+                            const int np = (int)((PX >> u) & 1u) + (inP ? 1 : 0);
+                            add_edge(Wk.etab[(size_t)member(u) * D + mk], hh + np, pc - np, sh);
+                        }
+                    }
+                    // pairs with and inside the prefix
+#pragma unroll
+                    for (int w = 0; w < NW; ++w) {
+                        for (uint32_t us = H[w] | P[w]; us; us &= us - 1) {
+                            const int b = __ffs(us) - 1, u = w * 32 + b;
+                            const int up = (P[w] >> b) & 1u;
+                            const uint32_t *eu = Wk.etab + (size_t)u * D;
+                            if (has) add_edge(eu[mk], hh + up + (inP ? 1 : 0), pc - up - (inP ? 1 : 0), sh);
+#pragma unroll
+                            for (int j = 0; j < NW; ++j) {
+                                const int m = j * 32 + lane, mp = (P[j] >> lane) & 1u;
+                                if (m > u && (((H[j] | P[j]) >> lane) & 1u)) add_edge(eu[m], hh + up + mp, pc - up - mp, path);
+                            }
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+            if (!closed) {
+                S1 = N;
+                P1 |= 1u << piv;
+                pp += 1;
+                continue;
+            }
+            if (top == 0) break;
+            --top;
+            S1 = Wk.cstk[top * 3];
+            H1 = Wk.cstk[top * 3 + 1];
+            P1 = Wk.cstk[top * 3 + 2];
+            hh = h + __popc(H1);
+            pp = p + __popc(P1);
+        }
+        // ---- the prefix: hold members gain pre, pivot members x / (1+x) of it
+        // (every leaf here has them as pivots, so the division is exact)
+        unsigned long long div = 0;
+        for (int k = 1; k <= kpre; ++k) {
+            const unsigned long long x = __shfl_sync(FULL, pre, k - 1), y = __shfl_sync(FULL, div, k - 1);
+            if (lane == k) div = x - y;
+        }
+#pragma unroll
+        for (int w = 0; w < NW; ++w)
+            for (uint32_t us = H[w] | P[w]; us; us &= us - 1) {
+                const int b = __ffs(us) - 1;
+                if (lane <= kpre) tab[lane * D + w * 32 + b] += (P[w] >> b) & 1u ? div : pre;
+            }
+        acc += pre;
+        ktop = max(ktop, kpre);
+        __syncwarp();
+    }
+    // A node's share of the sizes above the table for the prefix members and
+    // the root (as credit's).
+    __device__ __noinline__ void high_prefix(int h, int p, const uint32_t *H, const uint32_t *Pm, const Share &path) const
+    {
+#pragma unroll
+        for (int j = 0; j < NW; ++j) {
+            const bool inP = (Pm[j] >> lane) & 1u;
+            if (((H[j] | Pm[j]) >> lane) & 1u) add_high(cell(j * 32 + lane), inP ? h + 1 : h, inP ? p - 1 : p, path, kt + 1);
+        }
+        high_root(h, p, path);
+    }
+    // ... for the root, one size per lane (per-vertex)
+    __device__ __forceinline__ void high_root(int h, int p, const Share &path) const
+    {
+        if (MODE != MODE_VERTEX) return;
+        unsigned long long *row = A.out + (size_t)r * (A.kmax + 1) * A.W;
+        const unsigned n[4] = {path.a0, path.a1, path.a2, path.a3};
+        for (int k = kt + 1 + lane; k <= min(A.kmax, h + p + 3); k += 32)
+            for (int i = 0; i < 4; ++i)
+                if (n[i] && k - h - i >= 0 && k - h - i <= p)
+                    atomic_add_scaled(row + (size_t)k * A.W, binom_at(A.B, p, k - h - i, A.Bw), n[i], A.W, A.err);
+    }
+
     __device__ void run(unsigned q, unsigned Q, WalkCounters &wc)
     {
         uint32_t row[NW][NW];  // this lane's rows
@@ -312,11 +546,32 @@ struct LocalWalk {
         bool chain = true;      // on the root's pivot chain, which every part walks
         unsigned dealt = 0;     // hold children met along it
         uint32_t *stk = Wk.stk();
+        auto pop = [&]() {
+            --top;
+            const uint32_t *f = stk + (size_t)top * FW;
+            h = 1;
+            p = 0;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) {
+                S[w] = f[w];
+                H[w] = f[NW + w];
+                P[w] = f[2 * NW + w];
+                h += __popc(H[w]);
+                p += __popc(P[w]);
+            }
+        };
         for (;;) {
             const bool mine = !chain || q == 0;  // the chain's own leaves are part 0's
             int s = 0;
 #pragma unroll
             for (int w = 0; w < NW; ++w) s += __popc(S[w]);
+            if (NW > 1 && s <= 32 && (!chain || Q == 1)) {
+                run_small(S, H, P, s, h, p, wc);
+                chain = false;
+                if (top == 0) break;
+                pop();
+                continue;
+            }
             uint32_t best = 0, dsum = 0;
 #pragma unroll
             for (int j = 0; j < NW; ++j) {
@@ -536,18 +791,7 @@ struct LocalWalk {
             }
             chain = false;
             if (top == 0) break;
-            --top;
-            const uint32_t *f = stk + (size_t)top * FW;
-            h = 1;
-            p = 0;
-#pragma unroll
-            for (int w = 0; w < NW; ++w) {
-                S[w] = f[w];
-                H[w] = f[NW + w];
-                P[w] = f[2 * NW + w];
-                h += __popc(H[w]);
-                p += __popc(P[w]);
-            }
+            pop();
         }
         __syncwarp();
         // ---- the root's table to the caller's
@@ -637,7 +881,7 @@ __global__ void __launch_bounds__(32 * local_wpb<NW>(), local_blocks<NW>()) k_lo
                 unsigned bits = 0;
                 for (int t = lane; t < d * Work::RS; t += 32) bits += __popc(Wk.adj[t]);
                 const unsigned edges = __reduce_add_sync(FULL, bits) / 2;
-                if (edges >= LOCAL_HEAVY_EDGES) {
+                if (edges >= LOCAL_HEAVY_EDGES && (unsigned)(d * (d - 1) / 2) - edges > LOCAL_FEW_MISSING) {
                     const unsigned parts = local_parts(edges, d);
                     unsigned slot = 0, at = 0;
                     if (lane == 0) {
