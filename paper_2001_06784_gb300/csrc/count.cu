@@ -304,7 +304,7 @@ static pvt_status launch_frames(pvt_dag *g, const CountArgs &base, cudaStream_t 
 // ten times that for a frame walked in place: on a 12M-edge graph of
 // degeneracy 280 (k <= 4, 34M frames) a buffer of 2^22 frames cost 204 ms
 // in all, one that holds them 55 ms.
-constexpr unsigned FRAME_CAP_SMALL = 1u << 22, FRAME_CAP_MAX = 1u << 26;
+constexpr unsigned FRAME_CAP_MIN = 1u << 16, FRAME_CAP_MAX = 1u << 26;
 static unsigned frame_cap(const pvt_dag *g)
 {
     constexpr int64_t per_root[NCLASS] = {0, 0, 16, 64, 1024, 8192, 32768};
@@ -366,24 +366,30 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
     for (int c = 2; c < NCLASS; ++c) heavy += g->wcnt[c];
     const bool two_phase = MODE == MODE_GLOBAL && g->policy.frames && g->policy.persistent;
     const bool frames = two_phase && heavy > 0;
-    const bool gather1 = two_phase && g->policy.lanes && g->wcnt[1] >= GATHER1_MIN;
     if (frames) {
-        unsigned cap = frame_cap(g);
-        while ((st = grow(g->cframes, (size_t)cap * FRAME_WORDS, s)) == PVT_ENOMEM && cap > FRAME_CAP_SMALL) {
-            (void)cudaGetLastError();  // scratch is short: a smaller buffer only walks more in place
-            cap = std::max(cap / 4, FRAME_CAP_SMALL);
-        }
-        if (st != PVT_OK) return st;
+        // a sequence being recorded takes the buffer its direct call had
+        unsigned cap = g->capturing ? (unsigned)(g->cframes.n / FRAME_WORDS) : frame_cap(g);
+        if ((st = grow_least(g->cframes, cap, FRAME_CAP_MIN, FRAME_WORDS, g->buffer_limit, s)) != PVT_OK) return st;
+        cap = cap / EMIT_RESERVE * EMIT_RESERVE;
         A.emit = g->cframes.p;
         A.emit_count = reinterpret_cast<unsigned long long *>(g->d_q + 8);  // words 8..9
         A.emit_cap = cap;
     }
-    const int64_t pass1 = std::min(g->wcnt[1], GATHER1_MAX);
+    int64_t pass1 = std::min(g->wcnt[1], GATHER1_MAX);
     unsigned slots1 = 0;
+    bool gather1 = two_phase && g->policy.lanes && g->wcnt[1] >= GATHER1_MIN;
     if (gather1) {
         slots1 = gather1_slots(g, (unsigned)pass1);
-        if ((st = grow(g->cframes1, (size_t)slots1 * FRAME_WORDS, s)) != PVT_OK) return st;
-        A.emit1 = g->cframes1.p;
+        const size_t words = (size_t)slots1 * FRAME_WORDS;
+        const bool fixed = words > g->buffer_limit || g->capturing;
+        st = fixed && g->cframes1.n < words ? PVT_ENOMEM : grow(g->cframes1, words, s);
+        if (st != PVT_OK && st != PVT_ENOMEM) return st;
+        if (st == PVT_ENOMEM) {
+            (void)cudaGetLastError();
+            gather1 = false;  // no room for its frames: the class walks its own roots
+            st = PVT_OK;
+        }
+        A.emit1 = gather1 ? g->cframes1.p : nullptr;
         A.emit1_count = g->d_q + 10;
     }
     // classes on side streams (or all on s, one after another, when the
@@ -535,6 +541,27 @@ static pvt_status enqueue_global(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *
     return PVT_OK;
 }
 
+// What a recorded count depends on beside its arguments: every buffer that a
+// later call could have moved, and the table's layout.  ids has
+// 6 + NCLASS entries.
+static void graph_buffers(const pvt_dag *g, const void **ids)
+{
+    *ids++ = g->hist.p;
+    *ids++ = g->binom.p;
+    *ids++ = reinterpret_cast<const void *>((uintptr_t)g->binom_W);
+    *ids++ = g->cframes.p;
+    *ids++ = g->cframes1.p;
+    *ids++ = g->qframes[0].p;
+    for (int c = 0; c < NCLASS; ++c) *ids++ = g->gstack[c].p;
+}
+
+static bool graph_current(const pvt_dag *g)
+{
+    const void *now[6 + NCLASS];
+    graph_buffers(g, now);
+    return std::equal(now, now + 6 + NCLASS, g->graph_scratch);
+}
+
 void drop_graph(pvt_dag *g)
 {
     if (g->graph_exec) cudaGraphExecDestroy(g->graph_exec);
@@ -582,6 +609,7 @@ static pvt_status record_graph(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *C)
     g->graph_W = W;
     g->graph_out = C;
     g->graph_launches = launches;
+    graph_buffers(g, g->graph_scratch);
     return PVT_OK;
 }
 
@@ -592,7 +620,8 @@ pvt_status count_global(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *C, cudaSt
     begin_call(g);
     const bool use_graph = g->policy.graph != 0 && !g->serial && !g->policy.serial;
     g->hist_valid = false;
-    if (use_graph && g->graph_exec && g->graph_kmax == kmax && g->graph_W == W && g->graph_out == C) {
+    if (use_graph && g->graph_exec && g->graph_kmax == kmax && g->graph_W == W && g->graph_out == C &&
+        graph_current(g)) {
         PVT_CK(cudaGraphLaunch(g->graph_exec, s));
         g->stats.launches = g->graph_launches;
         st = end_call(g, s, "pvt_count_global", kmax);

@@ -1048,21 +1048,28 @@ pvt_status launch_local(pvt_dag *g, const CountArgs &base, int cls, cudaStream_t
         if ((st = grow(g->etab[cls], (size_t)grid * WPB * D * D, s)) != PVT_OK) return st;
         A.eidtab = g->etab[cls].p;
     }
-    // dense roots: at most 2^16, and 1 GB of edge-id tables
-    const bool split = g->policy.persistent != 0;
+    // dense roots: at most 2^16, and 1 GB of edge-id tables; those that find no
+    // room are walked by the warp that took them
+    bool split = g->policy.persistent != 0;
     LocalHeavy hv{};
     if (split) {
-        size_t cap = std::min<size_t>(cnt, 1u << 16);
-        if (MODE == MODE_EDGE) cap = std::min<size_t>(cap, ((size_t)1 << 28) / (D * D));
-        const size_t words = cap * (2 * LOCAL_MAX_PARTS + D * NW + 1 + (MODE == MODE_EDGE ? D * D : 0));
-        if ((st = grow(g->lheavy[cls], words, s)) != PVT_OK) return st;
+        unsigned cap = std::min(cnt, 1u << 16);
+        if (MODE == MODE_EDGE) cap = std::min(cap, (unsigned)(((size_t)1 << 28) / (D * D)));
+        const size_t words = 2 * LOCAL_MAX_PARTS + D * NW + 1 + (MODE == MODE_EDGE ? D * D : 0);
+        st = grow_least(g->lheavy[cls], cap, std::min(cap, 64u), words, g->buffer_limit, s);
+        if (st != PVT_OK && st != PVT_ENOMEM) return st;
+        if (st == PVT_ENOMEM) (void)cudaGetLastError();
+        split = st == PVT_OK;
+        hv.cap = cap;
+    }
+    if (split) {
+        const size_t cap = hv.cap;
         uint32_t *w = g->lheavy[cls].p;
         hv.items = reinterpret_cast<uint2 *>(w);
         hv.rows = w + cap * 2 * LOCAL_MAX_PARTS;
         hv.root = hv.rows + cap * D * NW;
         hv.etab = hv.root + cap;
         hv.count = g->qctl + QCTL_WORDS * cls;
-        hv.cap = (unsigned)cap;
         PVT_CK(cudaMemsetAsync(hv.count, 0, 3 * sizeof(unsigned), s));
     }
     phase_begin(g, 1 + cls, s);

@@ -91,6 +91,11 @@ struct pvt_dag {
     int graph_kmax = -1, graph_W = 0;
     void *graph_out = nullptr;
     uint64_t graph_launches = 0;
+    const void *graph_scratch[6 + pvt::NCLASS] = {};  // the buffers it was recorded with
+    // Words an optional buffer may take (frames, dense roots of a local
+    // count): with less of it more is walked in place.  A server, whose
+    // requests share a memory budget, sets it.
+    size_t buffer_limit = ~(size_t)0;
     cudaEvent_t ev_t0[pvt::NPHASE] = {}, ev_t1[pvt::NPHASE] = {};
     bool phase_used[pvt::NPHASE] = {};
     pvt::DevBuf<uint32_t> gstack[pvt::NCLASS];  // DFS stacks of the wide classes (global memory)

@@ -1320,6 +1320,21 @@ inline pvt_status grow(DevBuf<T> &b, size_t n, cudaStream_t s)
     return PVT_OK;
 }
 
+// As grow, for a buffer of `cap` entries of `words` words that a walk can do
+// with less of: cap is cut to the dag's limit and, where scratch is short, by
+// four at a time down to `least` entries.
+inline pvt_status grow_least(DevBuf<uint32_t> &b, unsigned &cap, unsigned least, size_t words, size_t limit, cudaStream_t s)
+{
+    if ((size_t)cap * words <= b.n) return PVT_OK;
+    cap = std::min(cap, std::max(least, (unsigned)std::min<size_t>(limit / words, cap)));
+    pvt_status st;
+    while ((st = grow(b, (size_t)cap * words, s)) == PVT_ENOMEM && cap > least) {
+        (void)cudaGetLastError();
+        cap = std::max(cap / 4, least);
+    }
+    return st;
+}
+
 // Queue counters of a split launch: head, tail, outstanding items (= roots),
 // next root, idle warps.
 static __global__ void k_split_init(uint32_t *qctl, unsigned nroots)
