@@ -650,8 +650,8 @@ def run_profile_case(args, dev):
     cta    orient the bench graph, global count k <= 4 with the 129..256
            out-degree class on the block-per-root kernel (k_cta<8>)
     local  per-vertex and per-edge tables of the 500k-vertex graph, k <= 12
-           (k_count in MODE_VERTEX / MODE_EDGE)
-    peel   orient the bench graph (k_peel, k_peel_tail)"""
+           (k_local, k_local_parts)
+    peel   orient the bench graph (core numbers and order, k_cores)"""
     import torch
     import paper_2001_06784_gb300 as pvt
     from paper_2001_06784_gb300 import graphgen

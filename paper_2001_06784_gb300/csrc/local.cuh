@@ -25,9 +25,9 @@
 // warp after all others have finished.
 // What bounds it: issue slots and load latency at 16 to 32 warps per SM (the
 // table takes 2 to 8 KB of shared memory per warp).  Start -> now, whole
-// calls: per-vertex, 500k vertices, 8.25M edges, k <= 40: 23.6 -> 4.5 ms;
-// 90k vertices, k <= 5: 4.3 -> 1.1 ms; per-edge, 2M edges, k <= 12: 5.3 -> 2.7
-// ms; 56k edges, k <= 22: 0.56 -> 0.39 ms.
+// calls: per-vertex, 500k vertices, 8.25M edges, k <= 40: 23.6 -> 3.9 ms;
+// 90k vertices, k <= 5: 4.3 -> 0.85 ms; per-edge, 2M edges, k <= 12: 5.3 ->
+// 2.4 ms; 56k edges, k <= 22: 0.56 -> 0.39 ms.
 #pragma once
 
 #include "walk.cuh"
