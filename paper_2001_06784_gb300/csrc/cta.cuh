@@ -10,7 +10,7 @@
 // subtree is done takes the next pending one, and busy warps hand over
 // their oldest pending subtree (the largest) while a warp of the block has
 // none.  Labels of at most 32 members leave the wide walk: they are
-// relabelled to one-word rows (the ballots of compact_rows in walk.cuh) into
+// relabelled to one-word rows (relabel_rows in walk.cuh) into
 // a free lane of the warp's lane batch and walked one subtree per lane
 // (lanes.cuh), so the many small subtrees below a dense root never leave the
 // SM.  A warp runs its lanes whenever it has no wide work or no free lane.
