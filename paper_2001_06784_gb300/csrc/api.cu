@@ -119,7 +119,7 @@ struct DagRes {
     unsigned *d_err = nullptr, *d_q = nullptr, *h_err = nullptr;
     unsigned long long *d_stats = nullptr, *h_stats = nullptr;
     uint32_t *qctl = nullptr;
-    cudaEvent_t ev_t0[NPHASE] = {}, ev_t1[NPHASE] = {}, ev_fork = nullptr, ev_join[NCLASS] = {};
+    cudaEvent_t ev_t0[NPHASE] = {}, ev_t1[NPHASE] = {}, ev_fork = nullptr, ev_out = nullptr, ev_join[NCLASS] = {};
     cudaStream_t side[NCLASS] = {};
     DevBuf<unsigned long long> binom;
     int binom_rows = 0, binom_W = 0;
@@ -149,6 +149,7 @@ static cudaError_t res_create(int device, DagRes &r)
         r.h_err = reinterpret_cast<unsigned *>(pin + CTL_ERR);
     }
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&r.ev_fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&r.ev_out, cudaEventDisableTiming);
     for (int c = 0; c < NCLASS && e == cudaSuccess; ++c) {
         e = cudaStreamCreateWithFlags(&r.side[c], cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&r.ev_join[c], cudaEventDisableTiming);
@@ -163,6 +164,7 @@ static void res_destroy(DagRes &r)
         if (r.ev_join[c]) cudaEventDestroy(r.ev_join[c]);
     }
     if (r.ev_fork) cudaEventDestroy(r.ev_fork);
+    if (r.ev_out) cudaEventDestroy(r.ev_out);
     for (int i = 0; i < NPHASE; ++i) {
         if (r.ev_t0[i]) cudaEventDestroy(r.ev_t0[i]);
         if (r.ev_t1[i]) cudaEventDestroy(r.ev_t1[i]);
@@ -205,6 +207,7 @@ static void res_to_dag(const DagRes &r, pvt_dag *g)
         g->ev_t1[i] = r.ev_t1[i];
     }
     g->ev_fork = r.ev_fork;
+    g->ev_out = r.ev_out;
     for (int c = 0; c < NCLASS; ++c) {
         g->ev_join[c] = r.ev_join[c];
         g->side[c] = r.side[c];
@@ -218,11 +221,13 @@ static void dag_release(pvt_dag *g)
 {
     if (!g) return;
     drop_graph(g);
-    // nothing of this dag is in flight once its side streams are idle: every
-    // entry point synchronises the caller's stream before it returns
+    // nothing of this dag is in flight once its side streams are idle and the
+    // copies of its core numbers are made: every other entry point
+    // synchronises the caller's stream before it returns
     for (int c = 0; c < NCLASS; ++c)
         if (g->side[c]) cudaStreamSynchronize(g->side[c]);
     cudaStream_t fs = g->side[0];
+    if (g->out_pending) cudaStreamWaitEvent(fs, g->ev_out);
     auto release = [&](void *p) {
         if (p) cudaFreeAsync(p, fs);
     };
@@ -255,6 +260,7 @@ static void dag_release(pvt_dag *g)
         r.ev_t1[i] = g->ev_t1[i];
     }
     r.ev_fork = g->ev_fork;
+    r.ev_out = g->ev_out;
     for (int c = 0; c < NCLASS; ++c) {
         r.ev_join[c] = g->ev_join[c];
         r.side[c] = g->side[c];
@@ -344,9 +350,15 @@ pvt_status pvt_dag_cores(const pvt_dag *dag, uint32_t *core, void *stream)
         set_error("pvt_dag_cores: invalid argument");
         return PVT_EINVAL;
     }
-    if (dag->n > 0)
-        PVT_CK(cudaMemcpyAsync(core, dag->core, (size_t)dag->n * sizeof(uint32_t), cudaMemcpyDeviceToDevice,
-                               (cudaStream_t)stream));
+    if (dag->n == 0) return PVT_OK;
+    // the copy is only enqueued: pvt_dag_free, which releases its source on a
+    // stream of the dag's own, waits for ev_out.  One event covers copies on
+    // several streams, since each follows the one before.
+    cudaStream_t s = (cudaStream_t)stream;
+    if (dag->out_pending) PVT_CK(cudaStreamWaitEvent(s, dag->ev_out));
+    PVT_CK(cudaMemcpyAsync(core, dag->core, (size_t)dag->n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
+    PVT_CK(cudaEventRecord(dag->ev_out, s));
+    dag->out_pending = true;
     return PVT_OK;
 }
 

@@ -77,6 +77,8 @@ struct pvt_dag {
     int binom_rows = 0, binom_W = 0;
     cudaStream_t side[pvt::NCLASS] = {};    // per-class streams for concurrent launches
     cudaEvent_t ev_fork = nullptr, ev_join[pvt::NCLASS] = {};
+    cudaEvent_t ev_out = nullptr;           // after the last copy of the core numbers to a caller
+    mutable bool out_pending = false;       // ... which nothing has waited for
     // statistics and phase timing of the last call
     unsigned long long *d_stats = nullptr;  // [0] nodes, [1] leaves, [2] pivot words
     unsigned long long *h_stats = nullptr;  // pinned host copy
