@@ -325,7 +325,10 @@ pvt_status pvt_orient(int64_t n, int64_t nnz, const int64_t *row_ptr, const uint
     g->profiling = (flags & PVT_PROFILE) != 0;
     stats_reset(g);
     st = orient_build(g, flags, s);
-    if (st != PVT_OK) return fail(st);
+    if (st != PVT_OK) {
+        cudaStreamSynchronize(s);  // what was enqueued before the failure reads the dag's memory
+        return fail(st);
+    }
     if (alpha_out) *alpha_out = g->alpha;
     *dag_out = g;
     return PVT_OK;

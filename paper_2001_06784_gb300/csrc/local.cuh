@@ -1098,14 +1098,14 @@ pvt_status launch_local_batch(const BatchGraph *gs, const uint64_t *entries, uns
     pvt_status st = local_occupancy(k_local_batch<NW, MODE>, 32 * WPB, smem, &per_sm);
     if (st != PVT_OK) return st;
     const unsigned grid = std::max(1u, std::min<unsigned>((unsigned)(num_sms * per_sm), (cnt + WPB - 1) / WPB));
-    uint32_t *scratch = nullptr;
+    Scratch mem(s);
     const size_t stack = LocalWork<NW>::GSTACK ? (size_t)grid * WPB * (D + 1) * LocalWork<NW>::FW : 0;
     const size_t etab = MODE == MODE_EDGE ? (size_t)grid * WPB * D * D : 0;
-    if (stack + etab) PVT_CK(cudaMallocAsync(&scratch, (stack + etab) * sizeof(uint32_t), s));
+    if (stack + etab) PVT_CK(mem.take((stack + etab) * sizeof(uint32_t)));
+    uint32_t *scratch = mem.as<uint32_t>();
     k_local_batch<NW, MODE><<<grid, 32 * WPB, smem, s>>>(gs, entries, cnt, qhead, B, Bw, BATCH_MAX_ALPHA + 2, err, stats,
                                                        scratch, scratch ? scratch + stack : nullptr);
     PVT_CK(cudaGetLastError());
-    if (scratch) PVT_CK(cudaFreeAsync(scratch, s));
     return PVT_OK;
 }
 

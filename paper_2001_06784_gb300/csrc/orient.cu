@@ -1383,13 +1383,13 @@ pvt_status exclusive_scan_u32_i64(const uint32_t *in, int64_t *out, int64_t n, c
         return PVT_OK;
     }
     int64_t nb = (n + 1023) / 1024;
-    unsigned long long *bsum = nullptr;
-    PVT_CK(cudaMallocAsync(&bsum, (size_t)std::max<int64_t>(nb, 1) * sizeof(unsigned long long), s));
+    Scratch sums(s);
+    PVT_CK(sums.take((size_t)std::max<int64_t>(nb, 1) * sizeof(unsigned long long)));
+    unsigned long long *bsum = sums.as<unsigned long long>();
     if (nb > 0) k_scan_blocks<<<(unsigned)nb, 1024, 0, s>>>(in, out, n, bsum);
     k_scan_sums<<<1, 1024, 0, s>>>(bsum, nb, out + n);
     if (nb > 0) k_scan_add<<<(unsigned)nb, 1024, 0, s>>>(out, n, bsum);
     PVT_CK(cudaGetLastError());
-    PVT_CK(cudaFreeAsync(bsum, s));
     return PVT_OK;
 }
 
@@ -1447,10 +1447,11 @@ pvt_status ensure_edge_ids(pvt_dag *g, cudaStream_t s)
         set_error("pvt_count_local_edge: more than 2^32 edges");
         return PVT_EINVAL;
     }
-    uint32_t *cnt = nullptr;
-    int64_t *up = nullptr;
-    PVT_CK(cudaMallocAsync(&cnt, (size_t)g->n * sizeof(uint32_t) + 4, s));
-    PVT_CK(cudaMallocAsync(&up, (size_t)(g->n + 1) * sizeof(int64_t), s));
+    Scratch cnt_(s), up_(s);
+    PVT_CK(cnt_.take((size_t)g->n * sizeof(uint32_t) + 4));
+    PVT_CK(up_.take((size_t)(g->n + 1) * sizeof(int64_t)));
+    uint32_t *cnt = cnt_.as<uint32_t>();
+    int64_t *up = up_.as<int64_t>();
     PVT_CK(cudaMallocAsync(&g->oeid, (size_t)g->m * sizeof(uint32_t), s));
     int grid = g->num_sms * 8;
     k_upper_count<<<grid, 256, 0, s>>>(g->n, g->row_ptr, g->col, cnt);
@@ -1458,8 +1459,6 @@ pvt_status ensure_edge_ids(pvt_dag *g, cudaStream_t s)
     if (st != PVT_OK) return st;
     k_edge_ids<<<grid, 256, 0, s>>>(g->n, g->row_ptr, g->col, up, g->orow, g->ocol, g->oeid);
     PVT_CK(cudaGetLastError());
-    PVT_CK(cudaFreeAsync(cnt, s));
-    PVT_CK(cudaFreeAsync(up, s));
     return PVT_OK;
 }
 
@@ -1470,19 +1469,21 @@ pvt_status ensure_edge_ids(pvt_dag *g, cudaStream_t s)
 static pvt_status peel_levels(pvt_dag *g, uint32_t *deg, uint32_t *alive, PeelState *pst, cudaStream_t s)
 {
     int64_t n = g->n;
-    uint32_t *lq = nullptr, *tv = nullptr, *rdeg = nullptr, *rcol = nullptr;
-    int64_t *roff = nullptr;
+    Scratch lq_(s), tv_(s), rdeg_(s), roff_(s), rcol_(s);
     int per_sm = 0;
     PVT_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_peel, 1024, 0));
     if (per_sm < 1) {
         set_error("pvt_orient: peel kernel cannot be resident");
         return PVT_ECUDA;
     }
-    PVT_CK(cudaMallocAsync(&lq, (size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t), s));
-    PVT_CK(cudaMallocAsync(&tv, (size_t)TAIL_MAX * sizeof(uint32_t), s));
-    PVT_CK(cudaMallocAsync(&rdeg, (size_t)TAIL_MAX * sizeof(uint32_t), s));
-    PVT_CK(cudaMallocAsync(&roff, (size_t)(TAIL_MAX + 1) * sizeof(int64_t), s));
-    PVT_CK(cudaMallocAsync(&rcol, (size_t)std::max<int64_t>(g->nnz, 1) * sizeof(uint32_t), s));
+    PVT_CK(lq_.take((size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t)));
+    PVT_CK(tv_.take((size_t)TAIL_MAX * sizeof(uint32_t)));
+    PVT_CK(rdeg_.take((size_t)TAIL_MAX * sizeof(uint32_t)));
+    PVT_CK(roff_.take((size_t)(TAIL_MAX + 1) * sizeof(int64_t)));
+    PVT_CK(rcol_.take((size_t)std::max<int64_t>(g->nnz, 1) * sizeof(uint32_t)));
+    uint32_t *lq = lq_.as<uint32_t>(), *tv = tv_.as<uint32_t>(), *rdeg = rdeg_.as<uint32_t>();
+    uint32_t *rcol = rcol_.as<uint32_t>();
+    int64_t *roff = roff_.as<int64_t>();
     const int64_t *rp = g->row_ptr;
     const uint32_t *col = g->col;
     uint32_t *rnd = g->rnd, *core = g->core;
@@ -1502,11 +1503,6 @@ static pvt_status peel_levels(pvt_dag *g, uint32_t *deg, uint32_t *alive, PeelSt
     k_peel_tail<<<1, TAIL_THREADS, tail_smem, s>>>(roff, rcol, rdeg, tv, g->rnd, g->core, pst, g->d_err);
     PVT_CK(cudaGetLastError());
     g->stats.launches += 5;
-    PVT_CK(cudaFreeAsync(lq, s));
-    PVT_CK(cudaFreeAsync(tv, s));
-    PVT_CK(cudaFreeAsync(rdeg, s));
-    PVT_CK(cudaFreeAsync(roff, s));
-    PVT_CK(cudaFreeAsync(rcol, s));
     return PVT_OK;
 }
 
@@ -1544,8 +1540,9 @@ pvt_status orient_build(pvt_dag *g, uint32_t flags, cudaStream_t s)
     at = 0;
     const size_t o_cst = carve(sizeof(CoreState)), o_sup = carve(nv * sizeof(uint32_t));
     const size_t o_list = carve(4 * nv * sizeof(uint32_t)), o_odeg = carve((nv + 1) * sizeof(uint32_t));
-    char *scratch = nullptr;
-    PVT_CK(cudaMallocAsync(&scratch, at, s));
+    Scratch mem(s);
+    PVT_CK(mem.take(at));
+    char *scratch = mem.as<char>();
     CoreState *cst = reinterpret_cast<CoreState *>(scratch + o_cst);
     uint32_t *sup = reinterpret_cast<uint32_t *>(scratch + o_sup), *list = reinterpret_cast<uint32_t *>(scratch + o_list);
     uint32_t *odeg = reinterpret_cast<uint32_t *>(scratch + o_odeg);
@@ -1607,7 +1604,6 @@ pvt_status orient_build(pvt_dag *g, uint32_t flags, cudaStream_t s)
         g->stats.peel_rounds += hst->peel.rounds;
         if (st != PVT_OK || !hst->bail) break;
     }
-    PVT_CK(cudaFreeAsync(scratch, s));
     if (st != PVT_OK) return st;
     g->stats.peel_levels = hst->peel.levels;
     if (hst->peel.top_level > (unsigned)MAX_ALPHA) {

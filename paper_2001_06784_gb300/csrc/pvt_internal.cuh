@@ -167,6 +167,30 @@ pvt_status cuda_fail(cudaError_t e, const char *what);
         if (_e != cudaSuccess) return pvt::cuda_fail(_e, #call); \
     } while (0)
 
+// Stream-ordered scratch of one call, released on every way out of it.
+struct Scratch {
+    void *p = nullptr;
+    cudaStream_t s;
+    explicit Scratch(cudaStream_t stream) : s(stream) {}
+    ~Scratch()
+    {
+        if (p) cudaFreeAsync(p, s);
+    }
+    Scratch(const Scratch &) = delete;
+    Scratch &operator=(const Scratch &) = delete;
+    cudaError_t take(size_t bytes)
+    {
+        const cudaError_t e = cudaMallocAsync(&p, bytes, s);
+        if (e != cudaSuccess) p = nullptr;
+        return e;
+    }
+    template <typename T>
+    T *as() const
+    {
+        return static_cast<T *>(p);
+    }
+};
+
 // Orientation (orient.cu).
 pvt_status orient_build(pvt_dag *g, uint32_t flags, cudaStream_t s);
 pvt_status ensure_edge_ids(pvt_dag *g, cudaStream_t s);

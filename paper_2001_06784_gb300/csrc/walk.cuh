@@ -1582,12 +1582,11 @@ pvt_status launch_batch_class(const BatchGraph *gs, const uint64_t *entries, uns
     }
     const unsigned need = (cnt + warps_per_block<NW>() - 1) / warps_per_block<NW>();
     const unsigned grid = std::max(1u, std::min<unsigned>((unsigned)(num_sms * per_sm), need));
-    uint32_t *gstack = nullptr;
+    Scratch gstack(s);
     if (WarpWork<NW>::GSTACK)
-        PVT_CK(cudaMallocAsync(&gstack, (size_t)grid * warps_per_block<NW>() * (32 * NW + 1) * NW * sizeof(uint32_t), s));
-    kern<<<grid, 32 * warps_per_block<NW>(), smem, s>>>(gs, entries, cnt, qhead, B, Bw, err, stats, gstack);
+        PVT_CK(gstack.take((size_t)grid * warps_per_block<NW>() * (32 * NW + 1) * NW * sizeof(uint32_t)));
+    kern<<<grid, 32 * warps_per_block<NW>(), smem, s>>>(gs, entries, cnt, qhead, B, Bw, err, stats, gstack.as<uint32_t>());
     PVT_CK(cudaGetLastError());
-    if (gstack) PVT_CK(cudaFreeAsync(gstack, s));
     return PVT_OK;
 }
 

@@ -3,12 +3,16 @@ it returns, and what a dag's release has to wait for (integer results:
 tolerance 0)."""
 from __future__ import annotations
 
+import contextlib
+import ctypes
+
 import numpy as np
 import pytest
 
 import oracle
 from paper_2001_06784_gb300 import graphgen
 from tests.test_gpu_parity import gpu_dag
+from tests.test_gpu_paths import mesh
 
 pytestmark = pytest.mark.gpu
 
@@ -17,6 +21,66 @@ pytestmark = pytest.mark.gpu
 def pvt():
     import paper_2001_06784_gb300 as p
     return p
+
+
+class PoolProps(ctypes.Structure):
+    """CUmemPoolProps: pinned memory of one device, at most maxSize bytes."""
+    _fields_ = [("allocType", ctypes.c_int), ("handleTypes", ctypes.c_int), ("locationType", ctypes.c_int),
+                ("locationId", ctypes.c_int), ("security", ctypes.c_void_p), ("maxSize", ctypes.c_size_t),
+                ("usage", ctypes.c_ushort), ("reserved", ctypes.c_ubyte * 54)]
+
+
+USED_MEM_CURRENT = 7  # CU_MEMPOOL_ATTR_USED_MEM_CURRENT
+
+
+@contextlib.contextmanager
+def limited_pool(limit):
+    """Stream-ordered allocations come from a pool of at most `limit` bytes:
+    beyond it they fail as on a full device.  Yields a function that gives the
+    bytes in use."""
+    import torch
+    cu = ctypes.CDLL("libcuda.so.1")
+    torch.cuda.synchronize()
+    pool, usual = ctypes.c_void_p(), ctypes.c_void_p()
+    props = PoolProps(allocType=1, locationType=1, locationId=0, maxSize=limit)
+    assert cu.cuMemPoolCreate(ctypes.byref(pool), ctypes.byref(props)) == 0
+    assert cu.cuDeviceGetMemPool(ctypes.byref(usual), 0) == 0
+    assert cu.cuDeviceSetMemPool(0, pool) == 0
+
+    def used():
+        torch.cuda.synchronize()
+        x = ctypes.c_uint64()
+        assert cu.cuMemPoolGetAttribute(pool, USED_MEM_CURRENT, ctypes.byref(x)) == 0
+        return x.value
+
+    try:
+        yield used
+    finally:
+        torch.cuda.synchronize()
+        assert cu.cuDeviceSetMemPool(0, usual) == 0
+        assert cu.cuMemPoolDestroy(pool) == 0
+
+
+def test_an_orientation_that_finds_no_room_leaves_nothing_behind(pvt):
+    """A mesh, which takes the core rounds and then the level-wise peel, with
+    ever more room: each orientation is refused or right, and none keeps memory."""
+    rp, col = mesh(1400, 1400)
+    ends = set()
+    for limit in range(32 << 20, 400 << 20, 16 << 20):
+        with limited_pool(limit) as used:
+            try:
+                dag = gpu_dag(pvt, rp, col, validate=False)
+            except pvt.PivoterError as e:
+                assert e.status == 3
+                ends.add("refused")
+            else:
+                assert dag.alpha == 2 and int((dag.cores() != 2).sum()) == 0
+                dag.free()
+                ends.add("oriented")
+            assert used() == 0
+        if "oriented" in ends:
+            break
+    assert ends == {"refused", "oriented"}
 
 
 @pytest.mark.parametrize("streams", [1, 2])
