@@ -466,6 +466,16 @@ static void begin_call(pvt_dag *g)
     for (int c = 0; c < NCLASS; ++c) g->stats.roots[c] = (uint64_t)g->class_cnt[c];
 }
 
+// A count that fails half way returns with nothing in flight: classes already
+// launched still add to the caller's table and read the dag's scratch.
+static pvt_status drained(pvt_dag *g, cudaStream_t s, pvt_status st)
+{
+    if (st == PVT_OK) return st;
+    for (int c = 0; c < NCLASS; ++c) cudaStreamSynchronize(g->side[c]);
+    cudaStreamSynchronize(s);
+    return st;
+}
+
 // Copy the walk statistics back, synchronise and check the device status.
 // Roots with no out-neighbour are one node and one leaf each (h = 1, p = 0)
 // when kmax >= 1; they are tallied without a walk, and counted here.
@@ -628,7 +638,7 @@ pvt_status count_global(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *C, cudaSt
         g->hist_valid = st == PVT_OK;
         return st;
     }
-    if ((st = enqueue_global(g, kmax, W, C, s)) != PVT_OK) return st;
+    if ((st = enqueue_global(g, kmax, W, C, s)) != PVT_OK) return drained(g, s, st);
     if ((st = end_call(g, s, "pvt_count_global", kmax)) != PVT_OK) return st;
     g->hist_valid = true;
     return use_graph ? record_graph(g, kmax, W, C) : PVT_OK;
@@ -702,13 +712,8 @@ __global__ void k_range_bounds(const int64_t *__restrict__ pos, ClassBounds full
     }
 }
 
-pvt_status count_hist(pvt_dag *g, int64_t begin, int64_t end, int32_t kmax, uint64_t *hist, cudaStream_t s)
+static pvt_status enqueue_hist(pvt_dag *g, int64_t begin, int64_t end, int32_t kmax, uint64_t *hist, cudaStream_t s)
 {
-    if (!g || !hist || kmax < 0 || begin < 0 || end < begin) {
-        set_error("pvt_count_hist: invalid argument");
-        return PVT_EINVAL;
-    }
-    begin_call(g);
     const int64_t n = g->n;
     end = std::min(end, n);
     begin = std::min(begin, end);
@@ -777,7 +782,31 @@ pvt_status count_hist(pvt_dag *g, int64_t begin, int64_t end, int32_t kmax, uint
         PVT_CK(cudaGetLastError());
         g->stats.launches++;
     }
-    return end_call(g, s, "pvt_count_hist", kmax);
+    return PVT_OK;
+}
+
+pvt_status count_hist(pvt_dag *g, int64_t begin, int64_t end, int32_t kmax, uint64_t *hist, cudaStream_t s)
+{
+    if (!g || !hist || kmax < 0 || begin < 0 || end < begin) {
+        set_error("pvt_count_hist: invalid argument");
+        return PVT_EINVAL;
+    }
+    begin_call(g);
+    const pvt_status st = enqueue_hist(g, begin, end, kmax, hist, s);
+    return st == PVT_OK ? end_call(g, s, "pvt_count_hist", kmax) : drained(g, s, st);
+}
+
+static pvt_status enqueue_combine(pvt_dag *g, const uint64_t *hist, int32_t kmax, int32_t W, uint64_t *C, cudaStream_t s)
+{
+    pvt_status st;
+    if ((st = ensure_binom(g, W, s)) != PVT_OK) return st;
+    PVT_CK(cudaMemsetAsync(g->d_stats, 0, CTL_BYTES, s));
+    k_combine<<<kmax + 1, 256, 0, s>>>(reinterpret_cast<const unsigned long long *>(hist), g->alpha + 2, g->binom.p,
+                                       W, kmax, reinterpret_cast<unsigned long long *>(C), false, 0ull, nullptr, 0,
+                                       g->d_err);
+    PVT_CK(cudaGetLastError());
+    g->stats.launches++;
+    return PVT_OK;
 }
 
 pvt_status combine_hist(pvt_dag *g, const uint64_t *hist, int32_t kmax, int32_t W, uint64_t *C, cudaStream_t s)
@@ -789,14 +818,8 @@ pvt_status combine_hist(pvt_dag *g, const uint64_t *hist, int32_t kmax, int32_t 
         return PVT_EINVAL;
     }
     begin_call(g);
-    if ((st = ensure_binom(g, W, s)) != PVT_OK) return st;
-    PVT_CK(cudaMemsetAsync(g->d_stats, 0, CTL_BYTES, s));
-    k_combine<<<kmax + 1, 256, 0, s>>>(reinterpret_cast<const unsigned long long *>(hist), g->alpha + 2, g->binom.p,
-                                       W, kmax, reinterpret_cast<unsigned long long *>(C), false, 0ull, nullptr, 0,
-                                       g->d_err);
-    PVT_CK(cudaGetLastError());
-    g->stats.launches++;
-    return end_call(g, s, "pvt_combine_hist", -1);
+    st = enqueue_combine(g, hist, kmax, W, C, s);
+    return st == PVT_OK ? end_call(g, s, "pvt_combine_hist", -1) : drained(g, s, st);
 }
 
 // Per-class minimum over three candidate policies, classes timed one at a time.
@@ -862,12 +885,9 @@ pvt_status autotune(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *C, cudaStream
     return PVT_OK;
 }
 
-pvt_status count_local(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *out, bool edge, cudaStream_t s)
+static pvt_status enqueue_local(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *out, bool edge, cudaStream_t s)
 {
-    const char *fn = edge ? "pvt_count_local_edge" : "pvt_count_local_vertex";
-    pvt_status st = check_args(g, kmax, W, out, g ? (edge ? g->m : g->n) : 0, fn);
-    if (st != PVT_OK) return st;
-    begin_call(g);
+    pvt_status st;
     if (edge && !g->oeid) {
         if ((st = ensure_edge_ids(g, s)) != PVT_OK) return st;
         g->stats.launches += 5;
@@ -895,9 +915,17 @@ pvt_status count_local(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *out, bool 
     A.err = g->d_err;
     A.stats = g->d_stats;
     apply_wait_limit(g, A);
-    st = edge ? launch_all<MODE_EDGE>(g, A, s) : launch_all<MODE_VERTEX>(g, A, s);
+    return edge ? launch_all<MODE_EDGE>(g, A, s) : launch_all<MODE_VERTEX>(g, A, s);
+}
+
+pvt_status count_local(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *out, bool edge, cudaStream_t s)
+{
+    const char *fn = edge ? "pvt_count_local_edge" : "pvt_count_local_vertex";
+    pvt_status st = check_args(g, kmax, W, out, g ? (edge ? g->m : g->n) : 0, fn);
     if (st != PVT_OK) return st;
-    return end_call(g, s, fn, kmax);
+    begin_call(g);
+    st = enqueue_local(g, kmax, W, out, edge, s);
+    return st == PVT_OK ? end_call(g, s, fn, kmax) : drained(g, s, st);
 }
 
 

@@ -83,6 +83,41 @@ def test_an_orientation_that_finds_no_room_leaves_nothing_behind(pvt):
     assert ends == {"refused", "oriented"}
 
 
+def test_a_refused_count_leaves_nothing_in_flight(pvt):
+    """Per-edge counts launch the widest class first.  Where a narrower one then
+    finds no room, the call returns with every launched class finished: the
+    table it was given does not change any more."""
+    import torch
+    rp, col = graphgen.generate(4000, er_avg_deg=8.0, planted=[(12, 100, 120, 0.75), (8, 40, 60, 0.8)], seed=53)
+    dag = gpu_dag(pvt, rp, col)
+    want = dag.count_local_edge(kmax=4)
+    dag.free()
+    peek = torch.cuda.Stream()
+    refused = 0
+    for limit in range(32 << 20, 640 << 20, 32 << 20):
+        dag = gpu_dag(pvt, rp, col)
+        out = torch.empty_like(want)
+        torch.cuda.synchronize()
+        with limited_pool(limit):
+            try:
+                dag.count_local_edge(kmax=4, out=out)
+            except pvt.PivoterError as e:
+                assert e.status == 3
+                refused += 1
+                with torch.cuda.stream(peek):
+                    now = out.clone()
+                torch.cuda.synchronize()
+                assert torch.equal(now, out)
+                done = False
+            else:
+                assert torch.equal(out, want)
+                done = True
+        dag.free()
+        if done:
+            break
+    assert refused > 0 and done
+
+
 @pytest.mark.parametrize("streams", [1, 2])
 def test_free_waits_for_the_copies_of_the_core_numbers(pvt, streams):
     """pvt_dag_cores only enqueues its copy.  A dag freed while such copies wait
