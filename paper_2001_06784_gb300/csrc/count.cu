@@ -254,6 +254,7 @@ static pvt_status ensure_binom(pvt_dag *g, int W, cudaStream_t s)
     // at (a(a+1)/2 + b) W whatever the row count), so a pooled table is reused
     const int rows = g->alpha + 3;
     if (g->binom_rows >= rows && g->binom_W == W) return PVT_OK;
+    g->binom_rows = g->binom_W = 0;  // no table until the new one is enqueued
     pvt_status st = grow(g->binom, (size_t)rows * (rows + 1) / 2 * W, s);
     if (st != PVT_OK) return st;
     k_binom<<<1, 1024, 0, s>>>(g->binom.p, rows, W, g->d_err);

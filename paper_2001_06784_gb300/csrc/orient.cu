@@ -1447,18 +1447,20 @@ pvt_status ensure_edge_ids(pvt_dag *g, cudaStream_t s)
         set_error("pvt_count_local_edge: more than 2^32 edges");
         return PVT_EINVAL;
     }
-    Scratch cnt_(s), up_(s);
+    // handed to the dag once everything that fills them is enqueued
+    Scratch cnt_(s), up_(s), ids(s);
     PVT_CK(cnt_.take((size_t)g->n * sizeof(uint32_t) + 4));
     PVT_CK(up_.take((size_t)(g->n + 1) * sizeof(int64_t)));
     uint32_t *cnt = cnt_.as<uint32_t>();
     int64_t *up = up_.as<int64_t>();
-    PVT_CK(cudaMallocAsync(&g->oeid, (size_t)g->m * sizeof(uint32_t), s));
+    PVT_CK(ids.take((size_t)g->m * sizeof(uint32_t)));
     int grid = g->num_sms * 8;
     k_upper_count<<<grid, 256, 0, s>>>(g->n, g->row_ptr, g->col, cnt);
     pvt_status st = exclusive_scan_u32_i64(cnt, up, g->n, s);
     if (st != PVT_OK) return st;
-    k_edge_ids<<<grid, 256, 0, s>>>(g->n, g->row_ptr, g->col, up, g->orow, g->ocol, g->oeid);
+    k_edge_ids<<<grid, 256, 0, s>>>(g->n, g->row_ptr, g->col, up, g->orow, g->ocol, ids.as<uint32_t>());
     PVT_CK(cudaGetLastError());
+    g->oeid = ids.give<uint32_t>();
     return PVT_OK;
 }
 

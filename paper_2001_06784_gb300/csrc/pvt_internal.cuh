@@ -189,6 +189,14 @@ struct Scratch {
     {
         return static_cast<T *>(p);
     }
+    // the caller's from here on
+    template <typename T>
+    T *give()
+    {
+        T *q = static_cast<T *>(p);
+        p = nullptr;
+        return q;
+    }
 };
 
 // Orientation (orient.cu).

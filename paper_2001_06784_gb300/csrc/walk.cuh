@@ -1315,7 +1315,9 @@ inline pvt_status grow(DevBuf<T> &b, size_t n, cudaStream_t s)
     if (b.p) PVT_CK(cudaFreeAsync(b.p, s));
     b.p = nullptr;
     b.n = 0;
-    PVT_CK(cudaMallocAsync(&b.p, n * sizeof(T), s));
+    T *p = nullptr;
+    PVT_CK(cudaMallocAsync(&p, n * sizeof(T), s));
+    b.p = p;
     b.n = n;
     return PVT_OK;
 }

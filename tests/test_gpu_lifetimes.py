@@ -118,6 +118,34 @@ def test_a_refused_count_leaves_nothing_in_flight(pvt):
     assert refused > 0 and done
 
 
+def test_tables_of_a_refused_count_are_built_anew(pvt):
+    """A count that finds no room for its edge ids or its Pascal table is
+    refused, and the next one, with room, does not take them for built."""
+    import torch
+    rp, col = graphgen.generate(300_000, er_avg_deg=6.0, planted=[(2, 20, 40, 0.9)], seed=52)
+    ref = oracle.count(rp, col)
+    K = ref["kmax"]
+    dag = gpu_dag(pvt, rp, col)
+    want = [dag.count_local_edge(kmax=4), dag.count_global(kmax=K)]
+    assert pvt.to_ints(want[1]) == ref["C"]
+    dag.free()
+    refused = 0
+    for limit in [2 << 20, 4 << 20, 8 << 20, 12 << 20, 16 << 20]:
+        dag = gpu_dag(pvt, rp, col)
+        out = torch.empty_like(want[0])
+        with limited_pool(limit):
+            for call in (lambda: dag.count_local_edge(kmax=4, out=out), lambda: dag.count_global(kmax=K, W=18)):
+                try:
+                    call()
+                except pvt.PivoterError as e:
+                    assert e.status == 3
+                    refused += 1
+        assert torch.equal(dag.count_local_edge(kmax=4, out=out), want[0])
+        assert torch.equal(dag.count_global(kmax=K), want[1])
+        dag.free()
+    assert refused > 0
+
+
 @pytest.mark.parametrize("streams", [1, 2])
 def test_free_waits_for_the_copies_of_the_core_numbers(pvt, streams):
     """pvt_dag_cores only enqueues its copy.  A dag freed while such copies wait
