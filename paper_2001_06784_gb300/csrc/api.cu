@@ -18,6 +18,7 @@ void set_error(const std::string &msg) { t_error = msg; }
 pvt_status cuda_fail(cudaError_t e, const char *what)
 {
     set_error(std::string(what) + ": " + cudaGetErrorString(e));
+    (void)cudaGetLastError();  // reported here: the thread's next call must not find it again
     return e == cudaErrorMemoryAllocation ? PVT_ENOMEM : PVT_ECUDA;
 }
 

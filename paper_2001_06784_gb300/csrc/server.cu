@@ -59,7 +59,10 @@ public:
             return p;
         }
         void *p = nullptr;
-        if (cudaMallocHost(&p, cls) != cudaSuccess) return nullptr;
+        if (cudaMallocHost(&p, cls) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return nullptr;
+        }
         return p;
     }
     void put(void *p, size_t cls)
@@ -169,6 +172,7 @@ bool can_admit(pvt_server *sv, const Request &r)
 
 void fail_request(pvt_server *sv, const ReqPtr &r, pvt_status st, const std::string &msg)
 {
+    (void)cudaGetLastError();  // reported with the request: the worker's next one must not find it again
     for (void *p : r->dallocs) cudaFree(p);
     r->dallocs.clear();
     std::lock_guard<std::mutex> lk(sv->mu);

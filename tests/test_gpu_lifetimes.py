@@ -37,7 +37,8 @@ USED_MEM_CURRENT = 7  # CU_MEMPOOL_ATTR_USED_MEM_CURRENT
 def limited_pool(limit):
     """Stream-ordered allocations come from a pool of at most `limit` bytes:
     beyond it they fail as on a full device.  Yields a function that gives the
-    bytes in use."""
+    bytes in use.  The pool itself stays: what was allocated from it may live
+    on."""
     import torch
     cu = ctypes.CDLL("libcuda.so.1")
     torch.cuda.synchronize()
@@ -58,7 +59,21 @@ def limited_pool(limit):
     finally:
         torch.cuda.synchronize()
         assert cu.cuDeviceSetMemPool(0, usual) == 0
-        assert cu.cuMemPoolDestroy(pool) == 0
+
+
+def test_a_reported_failure_is_not_reported_again(pvt):
+    """A call refused for want of memory leaves no error behind: the thread's
+    next call, of this library or of torch, does not fail with it."""
+    import torch
+    rp, col = mesh(1400, 1400)
+    with limited_pool(32 << 20):
+        with pytest.raises(pvt.PivoterError) as e:
+            gpu_dag(pvt, rp, col, validate=False)
+        assert e.value.status == 3
+        assert int(torch.zeros(4, device="cuda").sum()) == 0
+    dag = gpu_dag(pvt, rp, col, validate=False)
+    assert pvt.to_ints(dag.count_global(kmax=4)) == [0, 1400 * 1400, len(col) // 2, 0, 0]
+    dag.free()
 
 
 def test_an_orientation_that_finds_no_room_leaves_nothing_behind(pvt):
@@ -122,15 +137,15 @@ def test_tables_of_a_refused_count_are_built_anew(pvt):
     """A count that finds no room for its edge ids or its Pascal table is
     refused, and the next one, with room, does not take them for built."""
     import torch
-    rp, col = graphgen.generate(300_000, er_avg_deg=6.0, planted=[(2, 20, 40, 0.9)], seed=52)
-    ref = oracle.count(rp, col)
-    K = ref["kmax"]
+    rp, col = graphgen.generate(2_000_000, er_avg_deg=6.0, planted=[(2, 20, 40, 0.9)], seed=52)
+    ref = oracle.count(rp, col, kmax=6)
+    K = 6
     dag = gpu_dag(pvt, rp, col)
     want = [dag.count_local_edge(kmax=4), dag.count_global(kmax=K)]
     assert pvt.to_ints(want[1]) == ref["C"]
     dag.free()
     refused = 0
-    for limit in [2 << 20, 4 << 20, 8 << 20, 12 << 20, 16 << 20]:
+    for limit in range(32 << 20, 160 << 20, 32 << 20):
         dag = gpu_dag(pvt, rp, col)
         out = torch.empty_like(want[0])
         with limited_pool(limit):
