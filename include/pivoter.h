@@ -326,6 +326,21 @@ pvt_status pvt_dag_set_policy(pvt_dag *dag, const pvt_policy *policy);
 pvt_status pvt_dag_get_policy(const pvt_dag *dag, pvt_policy *out);
 
 /*
+ * Limit of the device scratch that later count calls on this dag hold, in
+ * bytes (0: none, the default).  Beside what a count cannot do without (leaf
+ * histogram, work queues, depth-first stacks, published rows) it has optional
+ * buffers: frames of small labels (up to 9.7 GB, by the number of roots in
+ * the classes above 32), frames of the <= 32 class (up to 0.6 GB) and, for
+ * local counts, dense roots kept for a second launch (up to 1 GB per class).
+ * They take at most what the required scratch leaves of the limit, and less
+ * where the device has no room; then more is walked in place, with the same
+ * results.  The required scratch is not refused because of the limit.  The
+ * call gives the optional buffers back and drops a recorded graph.
+ * Errors: PVT_EINVAL (NULL dag).
+ */
+pvt_status pvt_dag_set_scratch_limit(pvt_dag *dag, size_t bytes);
+
+/*
  * Autotuner of the launch policy (no counterpart in the paper).  Runs
  * pvt_count_global(dag, kmax, W, C, stream) under three candidate policies
  * -- {chunk 4, split}, {chunk 1, no split}, {chunk 16, split} -- twice each,

@@ -175,6 +175,11 @@ class Dag:
                           1 if serial else 0)
         _lib.check(_lib.lib().pvt_dag_set_policy(self._h, ctypes.byref(pol)))
 
+    def set_scratch_limit(self, nbytes: int):
+        """Bytes of device scratch that the optional buffers of later counts may
+        bring the dag to (0: no limit; pvt_dag_set_scratch_limit)."""
+        _lib.check(_lib.lib().pvt_dag_set_scratch_limit(self._h, int(nbytes)))
+
     def autotune(self, kmax=None, W=None, out=None, stream=None):
         """Pick the launch policy per out-degree class by timing three
         candidates (pvt_dag_autotune); sets it on the dag and returns

@@ -45,7 +45,7 @@ QUERY_GLOBAL, QUERY_VERTEX, QUERY_EDGE = 0, 1, 2
 # every symbol include/pivoter.h declares
 EXPORTS = ("pvt_orient", "pvt_dag_info", "pvt_dag_cores", "pvt_local_distribution", "pvt_count_hist", "pvt_combine_hist", "pvt_count_global", "pvt_count_local_vertex",
            "pvt_count_local_edge", "pvt_dag_stats", "pvt_dag_set_profiling", "pvt_dag_set_policy",
-           "pvt_dag_get_policy", "pvt_dag_autotune",
+           "pvt_dag_get_policy", "pvt_dag_set_scratch_limit", "pvt_dag_autotune",
            "pvt_count_global_noalloc", "pvt_server_create", "pvt_server_submit", "pvt_server_wait",
            "pvt_server_result", "pvt_server_destroy", "pvt_dag_free",
            "pvt_last_error", "pvt_measure_popc_rate", "pvt_dag_leaf_depths", "pvt_dag_out_lists")
@@ -93,6 +93,8 @@ def load(path: str = LIB_PATH):
     lib.pvt_dag_set_policy.argtypes = [vp, ctypes.POINTER(Policy)]
     lib.pvt_dag_get_policy.restype = i32
     lib.pvt_dag_get_policy.argtypes = [vp, ctypes.POINTER(Policy)]
+    lib.pvt_dag_set_scratch_limit.restype = i32
+    lib.pvt_dag_set_scratch_limit.argtypes = [vp, ctypes.c_size_t]
     lib.pvt_dag_autotune.restype = i32
     lib.pvt_dag_autotune.argtypes = [vp, i32, i32, vp, vp, ctypes.POINTER(Policy), vp]
     lib.pvt_count_global_noalloc.restype = i32

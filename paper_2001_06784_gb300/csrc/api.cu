@@ -462,6 +462,17 @@ pvt_status pvt_dag_set_policy(pvt_dag *dag, const pvt_policy *policy)
     return PVT_OK;
 }
 
+pvt_status pvt_dag_set_scratch_limit(pvt_dag *dag, size_t bytes)
+{
+    if (!dag) {
+        set_error("pvt_dag_set_scratch_limit: NULL dag");
+        return PVT_EINVAL;
+    }
+    dag->scratch_limit = bytes ? bytes : ~(size_t)0;
+    drop_optional(dag, dag->side[0]);
+    return PVT_OK;
+}
+
 pvt_status pvt_dag_get_policy(const pvt_dag *dag, pvt_policy *out)
 {
     if (!dag || !out) {

@@ -255,7 +255,7 @@ static pvt_status ensure_binom(pvt_dag *g, int W, cudaStream_t s)
     const int rows = g->alpha + 3;
     if (g->binom_rows >= rows && g->binom_W == W) return PVT_OK;
     g->binom_rows = g->binom_W = 0;  // no table until the new one is enqueued
-    pvt_status st = grow(g->binom, (size_t)rows * (rows + 1) / 2 * W, s);
+    pvt_status st = grow_buffer(g->binom, (size_t)rows * (rows + 1) / 2 * W, s);
     if (st != PVT_OK) return st;
     k_binom<<<1, 1024, 0, s>>>(g->binom.p, rows, W, g->d_err);
     PVT_CK(cudaGetLastError());
@@ -273,8 +273,8 @@ static pvt_status launch_frames(pvt_dag *g, const CountArgs &base, cudaStream_t 
     CountArgs A = base;
     A.cls = FRAMES_SLOT;
     pvt_status st;
-    if ((st = grow(g->qframes[0], (size_t)SPLIT_QCAP * FRAME_WORDS, s)) != PVT_OK) return st;
-    if ((st = grow(g->qready[0], (size_t)SPLIT_QCAP * 2, s)) != PVT_OK) return st;
+    if ((st = grow(g, g->qframes[0], (size_t)SPLIT_QCAP * FRAME_WORDS, s)) != PVT_OK) return st;
+    if ((st = grow(g, g->qready[0], (size_t)SPLIT_QCAP * 2, s)) != PVT_OK || g->sizing) return st;
     PVT_CK(cudaMemsetAsync(g->qready[0].p, 0, (size_t)SPLIT_QCAP * 2 * sizeof(uint32_t), s));
     k_frames_init<<<1, 128, 0, s>>>(g->qctl, A.emit_count, A.emit_cap);
     PVT_CK(cudaGetLastError());
@@ -354,45 +354,104 @@ constexpr int64_t GATHER1_MIN = 8192;
 // ... and in passes of at most this many roots (600 MB of frames)
 constexpr int64_t GATHER1_MAX = 1 << 22;
 
+// The walk of class c on stream s.  roots1, slots1: the pass of the <= 32
+// class's gather (slots1 = 0: that class walks its own roots).
+template <int MODE>
+static pvt_status launch_one(pvt_dag *g, const CountArgs &A, int c, unsigned roots1, unsigned slots1, cudaStream_t s)
+{
+    if (c == 1) {
+        if constexpr (MODE != MODE_GLOBAL) return launch_local<1, MODE>(g, A, c, s);
+        CountArgs L = A;
+        L.emit = nullptr;
+        if (!slots1) return launch_class<1, MODE_GLOBAL, true>(g, L, c, s);
+        phase_begin(g, 1 + c, s);
+        const pvt_status st = launch_gather1(g, A, g->wroots + g->wstart[1], roots1, slots1, s);
+        phase_end(g, 1 + c, s);
+        return st;
+    }
+    if (MODE == MODE_GLOBAL && g->policy.persistent && g->policy.cta[c] && c >= 4) return launch_cta_class(g, A, c, s);
+    return launch_wide<MODE>(g, A, c, s);
+}
+
+// Every buffer that the classes cannot do without, before the optional ones
+// take what is left.
+template <int MODE>
+static pvt_status size_all(pvt_dag *g, const CountArgs &A, bool two_phase, cudaStream_t s)
+{
+    pvt_status st = PVT_OK;
+    g->sizing = true;
+    for (int c = NCLASS - 1; c >= 1 && st == PVT_OK; --c)
+        if (g->wcnt[c]) st = launch_one<MODE>(g, A, c, 0, 0, s);
+    if (st == PVT_OK && two_phase) st = launch_frames(g, A, s);
+    g->sizing = false;
+    return st;
+}
+
+// Give back the optional buffers (a recorded count that uses them with them);
+// false if there were none.
+bool drop_optional(pvt_dag *g, cudaStream_t s)
+{
+    bool any = false;
+    auto drop = [&](DevBuf<uint32_t> &b) {
+        if (!b.p) return;
+        any = true;
+        cudaFreeAsync(b.p, s);
+        g->scratch -= b.n * sizeof(uint32_t);
+        b.p = nullptr;
+        b.n = 0;
+    };
+    drop(g->cframes);
+    drop(g->cframes1);
+    for (int c = 0; c < NCLASS; ++c) drop(g->lheavy[c]);
+    if (any) drop_graph(g);
+    return any;
+}
+
 template <int MODE>
 static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
 {
     // two-phase global counts: the classes above 32 emit their small labels
     // as frames into cframes (capacity from the number of heavy roots; a
-    // full buffer only sends frames back to in-place walking), the <= 32
-    // class its roots into cframes1
+    // full buffer, or none, only sends frames back to in-place walking), the
+    // <= 32 class its roots into cframes1
     CountArgs A = A0;
     pvt_status st = PVT_OK;
     int64_t heavy = 0;
     for (int c = 2; c < NCLASS; ++c) heavy += g->wcnt[c];
     const bool two_phase = MODE == MODE_GLOBAL && g->policy.frames && g->policy.persistent;
-    const bool frames = two_phase && heavy > 0;
+    bool frames = two_phase && heavy > 0;
+    bool gather1 = two_phase && g->policy.lanes && g->wcnt[1] >= GATHER1_MIN;
+    // (a sequence being recorded finds every buffer as its direct call left it)
+    if ((st = size_all<MODE>(g, A0, frames || gather1, s)) != PVT_OK) return st;
     if (frames) {
-        // a sequence being recorded takes the buffer its direct call had
         unsigned cap = g->capturing ? (unsigned)(g->cframes.n / FRAME_WORDS) : frame_cap(g);
-        if ((st = grow_least(g->cframes, cap, FRAME_CAP_MIN, FRAME_WORDS, g->buffer_limit, s)) != PVT_OK) return st;
+        if (!g->capturing) st = grow_least(g, g->cframes, cap, FRAME_CAP_MIN, FRAME_WORDS, s);
+        if (st != PVT_OK && st != PVT_ENOMEM) return st;
         cap = cap / EMIT_RESERVE * EMIT_RESERVE;
-        A.emit = g->cframes.p;
+        frames = st == PVT_OK && cap > 0;
+        A.emit = frames ? g->cframes.p : nullptr;
         A.emit_count = reinterpret_cast<unsigned long long *>(g->d_q + 8);  // words 8..9
-        A.emit_cap = cap;
+        A.emit_cap = frames ? cap : 0;
     }
+    // the gather's pass: as many roots as its frames find room for
     int64_t pass1 = std::min(g->wcnt[1], GATHER1_MAX);
     unsigned slots1 = 0;
-    bool gather1 = two_phase && g->policy.lanes && g->wcnt[1] >= GATHER1_MIN;
-    if (gather1) {
-        slots1 = gather1_slots(g, (unsigned)pass1);
-        const size_t words = (size_t)slots1 * FRAME_WORDS;
-        const bool fixed = words > g->buffer_limit || g->capturing;
-        st = fixed && g->cframes1.n < words ? PVT_ENOMEM : grow(g->cframes1, words, s);
-        if (st != PVT_OK && st != PVT_ENOMEM) return st;
-        if (st == PVT_ENOMEM) {
-            (void)cudaGetLastError();
-            gather1 = false;  // no room for its frames: the class walks its own roots
-            st = PVT_OK;
+    for (; gather1; pass1 /= 4) {
+        if (pass1 < GATHER1_MIN) gather1 = false;  // no room: the class walks its own roots
+        else {
+            slots1 = gather1_slots(g, (unsigned)pass1);
+            const size_t words = (size_t)slots1 * FRAME_WORDS;
+            if (words <= g->cframes1.n) break;
+            if (g->capturing || words > optional_words(g, g->cframes1)) continue;
+            st = grow_own(g, g->cframes1, words, s);
+            if (st == PVT_OK) break;
+            if (st != PVT_ENOMEM) return st;
         }
-        A.emit1 = gather1 ? g->cframes1.p : nullptr;
-        A.emit1_count = g->d_q + 10;
     }
+    st = PVT_OK;
+    if (!gather1) slots1 = 0;
+    A.emit1 = gather1 ? g->cframes1.p : nullptr;
+    A.emit1_count = g->d_q + 10;
     // classes on side streams (or all on s, one after another, when the
     // autotuner times them); classes without roots launch nothing, and a
     // single class needs no stream of its own
@@ -408,25 +467,7 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
         // The <= 32 class needs none and runs beside them.
         cudaStream_t cs = serial ? s : g->side[MODE == MODE_GLOBAL && c >= 2 ? NCLASS - 1 : c];
         if (!serial) PVT_CK(cudaStreamWaitEvent(cs, g->ev_fork, 0));
-        switch (c) {
-            case 1:
-                if constexpr (MODE != MODE_GLOBAL) {
-                    st = launch_local<1, MODE>(g, A0, c, cs);
-                } else if (gather1) {
-                    phase_begin(g, 1 + c, cs);
-                    st = launch_gather1(g, A, g->wroots + g->wstart[1], (unsigned)pass1, slots1, cs);
-                    phase_end(g, 1 + c, cs);
-                } else {
-                    st = launch_class<1, MODE, MODE == MODE_GLOBAL>(g, A0, c, cs);
-                }
-                break;
-            default:
-                if (MODE == MODE_GLOBAL && g->policy.persistent && g->policy.cta[c] && c >= 4)
-                    st = launch_cta_class(g, A, c, cs);
-                else
-                    st = launch_wide<MODE>(g, A, c, cs);
-                break;
-        }
+        st = launch_one<MODE>(g, A, c, (unsigned)pass1, slots1, cs);
         if (!serial) PVT_CK(cudaEventRecord(g->ev_join[c], cs));
     }
     if (st != PVT_OK) return st;
@@ -520,7 +561,7 @@ static pvt_status enqueue_global(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *
 {
     pvt_status st;
     const int hstride = g->alpha + 2;
-    if ((st = grow(g->hist, (size_t)hstride * hstride, s)) != PVT_OK) return st;
+    if ((st = grow(g, g->hist, (size_t)hstride * hstride, s)) != PVT_OK) return st;
     if ((st = ensure_binom(g, W, s)) != PVT_OK) return st;
     const unsigned cells = (unsigned)(hstride * hstride);
     k_begin_global<<<std::min((cells + 255u) / 256u, (unsigned)(4 * g->num_sms)), 256, 0, s>>>(
@@ -721,8 +762,8 @@ static pvt_status enqueue_hist(pvt_dag *g, int64_t begin, int64_t end, int32_t k
     pvt_status st;
     if (n > 0) {
         // the range's roots, class by class in the order of g->roots
-        if ((st = grow(g->range_roots, (size_t)2 * n, s)) != PVT_OK) return st;
-        if ((st = grow(g->range_pos, (size_t)n + 1, s)) != PVT_OK) return st;
+        if ((st = grow(g, g->range_roots, (size_t)2 * n, s)) != PVT_OK) return st;
+        if ((st = grow(g, g->range_pos, (size_t)n + 1, s)) != PVT_OK) return st;
         uint32_t *flag = g->range_roots.p, *out = g->range_roots.p + n;
         const int grid = g->num_sms * 4;
         k_range_flags<<<grid, 256, 0, s>>>(g->roots, n, begin, end, flag);

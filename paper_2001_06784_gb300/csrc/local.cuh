@@ -1041,13 +1041,14 @@ pvt_status launch_local(pvt_dag *g, const CountArgs &base, int cls, cudaStream_t
     const unsigned per_block = WPB * A.chunk;
     const unsigned grid = std::max(1u, std::min(full, (cnt + per_block - 1) / per_block));
     if (LocalWork<NW>::GSTACK) {
-        if ((st = grow(g->gstack[cls], (size_t)full * WPB * (D + 1) * LocalWork<NW>::FW, s)) != PVT_OK) return st;
+        if ((st = grow(g, g->gstack[cls], (size_t)full * WPB * (D + 1) * LocalWork<NW>::FW, s)) != PVT_OK) return st;
         A.gstack = g->gstack[cls].p;
     }
     if (MODE == MODE_EDGE) {
-        if ((st = grow(g->etab[cls], (size_t)grid * WPB * D * D, s)) != PVT_OK) return st;
+        if ((st = grow(g, g->etab[cls], (size_t)grid * WPB * D * D, s)) != PVT_OK) return st;
         A.eidtab = g->etab[cls].p;
     }
+    if (g->sizing) return PVT_OK;
     // dense roots: at most 2^16, and 1 GB of edge-id tables; those that find no
     // room are walked by the warp that took them
     bool split = g->policy.persistent != 0;
@@ -1056,9 +1057,8 @@ pvt_status launch_local(pvt_dag *g, const CountArgs &base, int cls, cudaStream_t
         unsigned cap = std::min(cnt, 1u << 16);
         if (MODE == MODE_EDGE) cap = std::min(cap, (unsigned)(((size_t)1 << 28) / (D * D)));
         const size_t words = 2 * LOCAL_MAX_PARTS + D * NW + 1 + (MODE == MODE_EDGE ? D * D : 0);
-        st = grow_least(g->lheavy[cls], cap, std::min(cap, 64u), words, g->buffer_limit, s);
+        st = grow_least(g, g->lheavy[cls], cap, std::min(cap, 64u), words, s);
         if (st != PVT_OK && st != PVT_ENOMEM) return st;
-        if (st == PVT_ENOMEM) (void)cudaGetLastError();
         split = st == PVT_OK;
         hv.cap = cap;
     }

@@ -94,10 +94,11 @@ struct pvt_dag {
     void *graph_out = nullptr;
     uint64_t graph_launches = 0;
     const void *graph_scratch[6 + pvt::NCLASS] = {};  // the buffers it was recorded with
-    // Words an optional buffer may take (frames, dense roots of a local
-    // count): with less of it more is walked in place.  A server, whose
-    // requests share a memory budget, sets it.
-    size_t buffer_limit = ~(size_t)0;
+    // Bytes that the count calls' buffers hold, and the most that the optional
+    // ones among them (frames, dense roots of a local count) may bring that to:
+    // with less of them more is walked in place (pvt_dag_set_scratch_limit).
+    size_t scratch = 0, scratch_limit = ~(size_t)0;
+    bool sizing = false;           // the launch functions only size their buffers
     cudaEvent_t ev_t0[pvt::NPHASE] = {}, ev_t1[pvt::NPHASE] = {};
     bool phase_used[pvt::NPHASE] = {};
     pvt::DevBuf<uint32_t> gstack[pvt::NCLASS];  // DFS stacks of the wide classes (global memory)
@@ -213,6 +214,7 @@ pvt_status count_hist(pvt_dag *g, int64_t begin, int64_t end, int32_t kmax, uint
 pvt_status combine_hist(pvt_dag *g, const uint64_t *hist, int32_t kmax, int32_t W, uint64_t *C, cudaStream_t s);
 pvt_status leaf_depths(pvt_dag *g, uint64_t *depth, cudaStream_t s);
 void drop_graph(pvt_dag *g);
+bool drop_optional(pvt_dag *g, cudaStream_t s);
 
 // Exclusive prefix sum of uint32 counts into int64 offsets (out has n+1 entries).
 pvt_status exclusive_scan_u32_i64(const uint32_t *in, int64_t *out, int64_t n, cudaStream_t s);

@@ -423,8 +423,7 @@ void run_direct(pvt_server *sv, const ReqPtr &rp)
         fail_request(sv, rp, st, "server: " + std::string(pvt_last_error()));
         return;
     }
-    // each buffer that a count can do with less of: 576 MiB (2^22 frames)
-    dag->buffer_limit = ((size_t)576 << 20) / sizeof(uint32_t);
+    dag->scratch_limit = (size_t)1152 << 20;  // what a count can do with less of: 2^23 frames
     r.alpha = alpha;
     r.W = min_words(r.n, alpha);
     r.K = (r.kmax_req >= 0 ? r.kmax_req : alpha + 1) + 1;

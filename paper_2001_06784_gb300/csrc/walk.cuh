@@ -1309,7 +1309,7 @@ __global__ void __launch_bounds__(32 * warps_per_block<NW>())
 }
 
 template <typename T>
-inline pvt_status grow(DevBuf<T> &b, size_t n, cudaStream_t s)
+inline pvt_status grow_buffer(DevBuf<T> &b, size_t n, cudaStream_t s)
 {
     if (b.n >= n) return PVT_OK;
     if (b.p) PVT_CK(cudaFreeAsync(b.p, s));
@@ -1322,18 +1322,43 @@ inline pvt_status grow(DevBuf<T> &b, size_t n, cudaStream_t s)
     return PVT_OK;
 }
 
+// The same for a buffer of the dag's own, whose bytes are its scratch.
+template <typename T>
+inline pvt_status grow_own(pvt_dag *g, DevBuf<T> &b, size_t n, cudaStream_t s)
+{
+    g->scratch -= b.n * sizeof(T);
+    const pvt_status st = grow_buffer(b, n, s);
+    g->scratch += b.n * sizeof(T);
+    return st;
+}
+
+// ... that a count cannot do without: where memory is short, the optional
+// buffers of earlier calls make room.
+template <typename T>
+inline pvt_status grow(pvt_dag *g, DevBuf<T> &b, size_t n, cudaStream_t s)
+{
+    pvt_status st = grow_own(g, b, n, s);
+    if (st == PVT_ENOMEM && drop_optional(g, s)) st = grow_own(g, b, n, s);
+    return st;
+}
+
+// 32-bit words that an optional buffer may have beside the dag's others.
+inline size_t optional_words(const pvt_dag *g, const DevBuf<uint32_t> &b)
+{
+    const size_t others = g->scratch - b.n * sizeof(uint32_t);
+    return (g->scratch_limit - std::min(g->scratch_limit, others)) / sizeof(uint32_t);
+}
+
 // As grow, for a buffer of `cap` entries of `words` words that a walk can do
-// with less of: cap is cut to the dag's limit and, where scratch is short, by
-// four at a time down to `least` entries.
-inline pvt_status grow_least(DevBuf<uint32_t> &b, unsigned &cap, unsigned least, size_t words, size_t limit, cudaStream_t s)
+// with less of: cap is cut to the dag's limit and, where memory is short, by
+// four at a time down to `least` entries; PVT_ENOMEM if those find no room.
+inline pvt_status grow_least(pvt_dag *g, DevBuf<uint32_t> &b, unsigned &cap, unsigned least, size_t words, cudaStream_t s)
 {
     if ((size_t)cap * words <= b.n) return PVT_OK;
-    cap = std::min(cap, std::max(least, (unsigned)std::min<size_t>(limit / words, cap)));
+    cap = (unsigned)std::min<size_t>(optional_words(g, b) / words, cap);
+    if (cap < least) return PVT_ENOMEM;
     pvt_status st;
-    while ((st = grow(b, (size_t)cap * words, s)) == PVT_ENOMEM && cap > least) {
-        (void)cudaGetLastError();
-        cap = std::max(cap / 4, least);
-    }
+    while ((st = grow_own(g, b, (size_t)cap * words, s)) == PVT_ENOMEM && cap > least) cap = std::max(cap / 4, least);
     return st;
 }
 
@@ -1393,22 +1418,6 @@ pvt_status launch_class(pvt_dag *g, const CountArgs &base, int cls, cudaStream_t
         if constexpr (WarpWork<NW>::GSTACK) kern = k_count<NW, MODE, SHIST, true, false>;
         else kern = persist ? k_count<NW, MODE, SHIST, true, false> : k_count<NW, MODE, SHIST, false, false>;
     }
-    if (split) {
-        pvt_status st;
-        if ((st = grow(g->rootbuf[cls], (size_t)cnt * 32 * NW * NW, s)) != PVT_OK) return st;
-        if ((st = grow(g->qframes[cls], (size_t)SPLIT_QCAP * FRAME_WORDS, s)) != PVT_OK) return st;
-        if ((st = grow(g->qready[cls], (size_t)SPLIT_QCAP * 2, s)) != PVT_OK) return st;
-        PVT_CK(cudaMemsetAsync(g->qready[cls].p, 0, (size_t)SPLIT_QCAP * 2 * sizeof(uint32_t), s));
-        k_split_init<<<1, 128, 0, s>>>(g->qctl + QCTL_WORDS * cls, cnt);
-        PVT_CK(cudaGetLastError());
-        g->stats.launches++;
-        A.rootbuf = g->rootbuf[cls].p;
-        A.qframes = g->qframes[cls].p;
-        A.qready = g->qready[cls].p;
-        A.qdone = g->qready[cls].p + SPLIT_QCAP;
-        A.qctl = g->qctl + QCTL_WORDS * cls;
-        A.qcap = SPLIT_QCAP;
-    }
     int per_sm = 0;
     PVT_CK(resident_blocks((const void *)kern, 32 * WPB, smem, &per_sm));
     if (per_sm < 1) {
@@ -1419,17 +1428,34 @@ pvt_status launch_class(pvt_dag *g, const CountArgs &base, int cls, cudaStream_t
     const unsigned need = (cnt + WPB - 1) / WPB;
     // persistent: sized to the resident warps (per-warp global stacks too)
     const unsigned grid = persist ? std::min<unsigned>((unsigned)(g->num_sms * per_sm), need) : need;
+    pvt_status st = PVT_OK;
+    if (split) {
+        if ((st = grow(g, g->rootbuf[cls], (size_t)cnt * 32 * NW * NW, s)) != PVT_OK) return st;
+        if ((st = grow(g, g->qframes[cls], (size_t)SPLIT_QCAP * FRAME_WORDS, s)) != PVT_OK) return st;
+        if ((st = grow(g, g->qready[cls], (size_t)SPLIT_QCAP * 2, s)) != PVT_OK) return st;
+    }
     if (WarpWork<NW>::GSTACK) {
-        pvt_status st = grow(g->gstack[cls], (size_t)grid * WPB * (32 * NW + 1) * NW, s);
-        if (st != PVT_OK) return st;
+        if ((st = grow(g, g->gstack[cls], (size_t)grid * WPB * (32 * NW + 1) * NW, s)) != PVT_OK) return st;
         A.gstack = g->gstack[cls].p;
     }
     if (MODE == MODE_EDGE && persist && NW <= 8) {
         // per-warp edge-id tables of member pairs (the gather fills them)
         constexpr size_t D = WarpWork<NW>::D;
-        pvt_status st = grow(g->etab[cls], (size_t)grid * WPB * D * D, s);
-        if (st != PVT_OK) return st;
+        if ((st = grow(g, g->etab[cls], (size_t)grid * WPB * D * D, s)) != PVT_OK) return st;
         A.eidtab = g->etab[cls].p;
+    }
+    if (g->sizing) return PVT_OK;
+    if (split) {
+        PVT_CK(cudaMemsetAsync(g->qready[cls].p, 0, (size_t)SPLIT_QCAP * 2 * sizeof(uint32_t), s));
+        k_split_init<<<1, 128, 0, s>>>(g->qctl + QCTL_WORDS * cls, cnt);
+        PVT_CK(cudaGetLastError());
+        g->stats.launches++;
+        A.rootbuf = g->rootbuf[cls].p;
+        A.qframes = g->qframes[cls].p;
+        A.qready = g->qready[cls].p;
+        A.qdone = g->qready[cls].p + SPLIT_QCAP;
+        A.qctl = g->qctl + QCTL_WORDS * cls;
+        A.qcap = SPLIT_QCAP;
     }
     phase_begin(g, 1 + cls, s);
     kern<<<grid, 32 * WPB, smem, s>>>(A);

@@ -31,8 +31,8 @@ static pvt_status launch_cta_nw(pvt_dag *g, CountArgs A, int cls, int dmax, cuda
     }
     const unsigned blocks = std::max(1u, std::min<unsigned>((unsigned)(g->num_sms * per_sm), A.nroots));
     pvt_status st =
-        grow(g->gstack[cls], (size_t)blocks * warps * Lay::stack_words(dmax) + (size_t)blocks * Lay::gather_words(dmax), s);
-    if (st != PVT_OK) return st;
+        grow(g, g->gstack[cls], (size_t)blocks * warps * Lay::stack_words(dmax) + (size_t)blocks * Lay::gather_words(dmax), s);
+    if (st != PVT_OK || g->sizing) return st;
     A.gstack = g->gstack[cls].p;
     phase_begin(g, 1 + cls, s);
     kern<<<blocks, 32 * warps, smem, s>>>(A, dmax);

@@ -58,8 +58,8 @@ static __global__ void k_lanes_frames_init(CountArgs A)
 static pvt_status lane_ring(pvt_dag *g, CountArgs &A, int q, cudaStream_t s)
 {
     pvt_status st;
-    if ((st = grow(g->qframes[q], (size_t)SPLIT_QCAP * FRAME_WORDS, s)) != PVT_OK) return st;
-    if ((st = grow(g->qready[q], (size_t)SPLIT_QCAP * 2, s)) != PVT_OK) return st;
+    if ((st = grow(g, g->qframes[q], (size_t)SPLIT_QCAP * FRAME_WORDS, s)) != PVT_OK) return st;
+    if ((st = grow(g, g->qready[q], (size_t)SPLIT_QCAP * 2, s)) != PVT_OK || g->sizing) return st;
     PVT_CK(cudaMemsetAsync(g->qready[q].p, 0, (size_t)SPLIT_QCAP * 2 * sizeof(uint32_t), s));
     A.qframes = g->qframes[q].p;
     A.qready = g->qready[q].p;
@@ -74,7 +74,7 @@ pvt_status launch_lanes_frames(pvt_dag *g, const CountArgs &base, cudaStream_t s
     CountArgs A = base;
     A.cls = NCLASS;
     pvt_status st = lane_ring(g, A, 0, s);
-    if (st != PVT_OK) return st;
+    if (st != PVT_OK || g->sizing) return st;
     k_lanes_frames_init<<<1, 128, 0, s>>>(A);
     PVT_CK(cudaGetLastError());
     g->stats.launches += 2;

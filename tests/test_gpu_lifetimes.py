@@ -11,8 +11,9 @@ import pytest
 
 import oracle
 from paper_2001_06784_gb300 import graphgen
+from tests import graphs
 from tests.test_gpu_parity import gpu_dag
-from tests.test_gpu_paths import mesh
+from tests.test_gpu_paths import disjoint, mesh
 
 pytestmark = pytest.mark.gpu
 
@@ -30,14 +31,14 @@ class PoolProps(ctypes.Structure):
                 ("usage", ctypes.c_ushort), ("reserved", ctypes.c_ubyte * 54)]
 
 
-USED_MEM_CURRENT = 7  # CU_MEMPOOL_ATTR_USED_MEM_CURRENT
+RESERVED_MEM_HIGH, USED_MEM_CURRENT = 6, 7  # CU_MEMPOOL_ATTR_*
 
 
 @contextlib.contextmanager
 def limited_pool(limit):
     """Stream-ordered allocations come from a pool of at most `limit` bytes:
-    beyond it they fail as on a full device.  Yields a function that gives the
-    bytes in use.  The pool itself stays: what was allocated from it may live
+    beyond it they fail as on a full device.  Yields a function that gives one
+    of its figures (the bytes in use).  The pool itself stays: what was allocated from it may live
     on."""
     import torch
     cu = ctypes.CDLL("libcuda.so.1")
@@ -48,10 +49,10 @@ def limited_pool(limit):
     assert cu.cuDeviceGetMemPool(ctypes.byref(usual), 0) == 0
     assert cu.cuDeviceSetMemPool(0, pool) == 0
 
-    def used():
+    def used(attr=USED_MEM_CURRENT):
         torch.cuda.synchronize()
         x = ctypes.c_uint64()
-        assert cu.cuMemPoolGetAttribute(pool, USED_MEM_CURRENT, ctypes.byref(x)) == 0
+        assert cu.cuMemPoolGetAttribute(pool, attr, ctypes.byref(x)) == 0
         return x.value
 
     try:
@@ -159,6 +160,76 @@ def test_tables_of_a_refused_count_are_built_anew(pvt):
         assert torch.equal(dag.count_global(kmax=K), want[1])
         dag.free()
     assert refused > 0
+
+
+def classes_graph():
+    """Roots of every class up to 512: 40,000 of at most 32 out-neighbours, and
+    dense groups whose roots are split, walked by blocks and walked in parts."""
+    return disjoint(graphgen.generate(40_000, er_avg_deg=9.0, planted=[(30, 24, 30, 0.8), (12, 40, 60, 0.7),
+                                                                       (4, 90, 120, 0.5)], seed=54),
+                    graphs.clique_minus_random(180, 9, 55), graphs.clique_minus_random(300, 9, 56))
+
+
+COUNTS = {
+    "global": lambda dag, K: dag.count_global(kmax=K),
+    "range": lambda dag, K: dag.combine_hist(dag.count_hist(0, dag.n, kmax=K), kmax=K),
+    "vertex": lambda dag, K: dag.count_local_vertex(kmax=3),
+    "edge": lambda dag, K: dag.count_local_edge(kmax=3),
+}
+
+
+@pytest.mark.parametrize("what", sorted(COUNTS))
+def test_counts_within_a_scratch_limit(pvt, what):
+    """Under any limit the counts, and the tree that is walked, are those of the
+    call without one: with frames for some of the roots, the gather in passes,
+    dense roots walked where they are met, and nothing optional at all."""
+    import torch
+    rp, col = classes_graph()
+    dag = gpu_dag(pvt, rp, col)
+    assert dag.alpha > 256
+    want = COUNTS[what](dag, 4)
+    ref = oracle.count(rp, col, kmax=4)
+    if want.dim() == 2:
+        assert pvt.to_ints(want) == ref["C"]
+    tree = [dag.stats()[k] for k in ("sct_nodes", "sct_leaves", "pivot_words", "roots")]
+    launches = set()
+    for mb in (1, 48, 64, 72, 80, 88, 96, 104, 112, 120, 128, 160, 256, 0):
+        dag.set_scratch_limit(mb << 20)
+        assert torch.equal(COUNTS[what](dag, 4), want), mb
+        st = dag.stats()
+        if what in ("global", "vertex", "edge"):
+            assert [st[k] for k in ("sct_nodes", "sct_leaves", "pivot_words", "roots")] == tree, mb
+        launches.add(st["launches"])
+    assert what == "range" or len(launches) >= 2  # more than one route was taken
+    dag.free()
+
+
+@pytest.mark.parametrize("what", sorted(COUNTS))
+def test_a_count_fits_where_its_required_scratch_does(pvt, what):
+    """Optional buffers take what the required ones leave: in the memory that a
+    count needs without any, it is not refused."""
+    import torch
+    rp, col = classes_graph()
+    dag = gpu_dag(pvt, rp, col)
+    want = COUNTS[what](dag, 4)
+    dag.free()
+    dag = gpu_dag(pvt, rp, col)
+    dag.set_scratch_limit(1)
+    with limited_pool(1 << 40) as used:
+        assert torch.equal(COUNTS[what](dag, 4), want)
+        need = used(RESERVED_MEM_HIGH)
+    dag.free()
+    dag = gpu_dag(pvt, rp, col)
+    with limited_pool(need):
+        assert torch.equal(COUNTS[what](dag, 4), want)
+        # ... nor is another count on the dag, whose optional buffers the first one's are
+        for other in sorted(COUNTS):
+            try:
+                COUNTS[other](dag, 4)
+            except pvt.PivoterError as e:
+                assert e.status == 3
+        assert torch.equal(COUNTS[what](dag, 4), want)
+    dag.free()
 
 
 @pytest.mark.parametrize("streams", [1, 2])
