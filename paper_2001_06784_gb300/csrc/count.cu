@@ -594,24 +594,27 @@ static pvt_status enqueue_global(pvt_dag *g, int32_t kmax, int32_t W, uint64_t *
 }
 
 // What a recorded count depends on beside its arguments: every buffer that a
-// later call could have moved, and the table's layout.  ids has
-// 6 + NCLASS entries.
+// later call could have moved, the sizes of those that one could have moved to
+// less room at the same place, and the table's layout.  ids has 8 + NCLASS
+// entries.
 static void graph_buffers(const pvt_dag *g, const void **ids)
 {
     *ids++ = g->hist.p;
     *ids++ = g->binom.p;
     *ids++ = reinterpret_cast<const void *>((uintptr_t)g->binom_W);
     *ids++ = g->cframes.p;
+    *ids++ = reinterpret_cast<const void *>(g->cframes.n);
     *ids++ = g->cframes1.p;
+    *ids++ = reinterpret_cast<const void *>(g->cframes1.n);
     *ids++ = g->qframes[0].p;
     for (int c = 0; c < NCLASS; ++c) *ids++ = g->gstack[c].p;
 }
 
 static bool graph_current(const pvt_dag *g)
 {
-    const void *now[6 + NCLASS];
+    const void *now[8 + NCLASS];
     graph_buffers(g, now);
-    return std::equal(now, now + 6 + NCLASS, g->graph_scratch);
+    return std::equal(now, now + 8 + NCLASS, g->graph_scratch);
 }
 
 void drop_graph(pvt_dag *g)

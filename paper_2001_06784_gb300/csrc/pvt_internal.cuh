@@ -93,7 +93,7 @@ struct pvt_dag {
     int graph_kmax = -1, graph_W = 0;
     void *graph_out = nullptr;
     uint64_t graph_launches = 0;
-    const void *graph_scratch[6 + pvt::NCLASS] = {};  // the buffers it was recorded with
+    const void *graph_scratch[8 + pvt::NCLASS] = {};  // the buffers it was recorded with
     // Bytes that the count calls' buffers hold, and the most that the optional
     // ones among them (frames, dense roots of a local count) may bring that to:
     // with less of them more is walked in place (pvt_dag_set_scratch_limit).

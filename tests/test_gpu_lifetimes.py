@@ -232,6 +232,25 @@ def test_a_count_fits_where_its_required_scratch_does(pvt, what):
     dag.free()
 
 
+def test_a_recorded_count_after_its_frames_moved(pvt):
+    """A recorded count whose frames another call has since moved to less room is
+    recorded anew, whatever the address."""
+    import torch
+    rp, col = classes_graph()
+    dag = gpu_dag(pvt, rp, col)
+    want = dag.count_global(kmax=5)
+    dag.set_policy(graph=True)
+    out = torch.empty_like(want)
+    for limit in (1 << 40, 256 << 20, 224 << 20, 192 << 20, 1 << 40):
+        with limited_pool(limit):
+            for _ in range(3):
+                assert torch.equal(dag.count_global(kmax=5, out=out.zero_()), want)
+            dag.set_scratch_limit(0)  # the frames move
+            dag.count_hist(0, dag.n, kmax=5)
+            assert torch.equal(dag.count_global(kmax=5, out=out.zero_()), want)
+    dag.free()
+
+
 @pytest.mark.parametrize("streams", [1, 2])
 def test_free_waits_for_the_copies_of_the_core_numbers(pvt, streams):
     """pvt_dag_cores only enqueues its copy.  A dag freed while such copies wait
