@@ -402,7 +402,9 @@ pvt_status pvt_count_global_noalloc(int64_t n, const int64_t *orow, const uint32
  * earlier groups still run, and groups run on separate streams so their work
  * overlaps.  Queries of at least direct_edges edges bypass the batches: a
  * second worker runs them one at a time through pvt_orient and the count
- * entry points on a stream of its own, whole-GPU kernels beside the batches.
+ * entry points on a stream of its own, whole-GPU kernels beside the batches;
+ * their scratch (pvt_dag_set_scratch_limit) is held from the budget too, a
+ * quarter of it between 256 MiB and 1.25 GiB.
  * Results are exact and equal to the single-graph entry points.
  */
 typedef struct pvt_server pvt_server;

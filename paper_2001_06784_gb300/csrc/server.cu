@@ -85,6 +85,7 @@ struct Request {
     std::vector<int64_t> rp;
     std::vector<uint32_t> col;
     size_t reserve = 0;              // budget bytes held
+    size_t scratch = 0;              // ... of them for the scratch of a direct count
     std::vector<void *> dallocs;     // device memory of this query
     BatchGraph desc;
     int alpha = 0, K = 0, W = 0;
@@ -123,6 +124,9 @@ size_t estimate_bytes(const Request &r, int alpha_bound)
     b += align_up(8 * n);                                                   // root entries
     return b;
 }
+
+// Budget bytes a direct query holds for its dag's scratch.
+constexpr size_t DIRECT_SCRATCH_MIN = (size_t)256 << 20, DIRECT_SCRATCH_MAX = (size_t)1280 << 20;
 
 int alpha_bound(const Request &r)
 {
@@ -423,7 +427,7 @@ void run_direct(pvt_server *sv, const ReqPtr &rp)
         fail_request(sv, rp, st, "server: " + std::string(pvt_last_error()));
         return;
     }
-    dag->scratch_limit = (size_t)1152 << 20;  // what a count can do with less of: 2^23 frames
+    dag->scratch_limit = r.scratch;
     r.alpha = alpha;
     r.W = min_words(r.n, alpha);
     r.K = (r.kmax_req >= 0 ? r.kmax_req : alpha + 1) + 1;
@@ -637,8 +641,16 @@ pvt_status pvt_server_submit(pvt_server *sv, int64_t n, int64_t nnz, const int64
     r->col.assign(col, col + nnz);
     r->direct = sv->cfg.direct_edges > 0 && r->m >= sv->cfg.direct_edges;
     const int ab = alpha_bound(*r);
-    // the direct path's dag also holds its own scratch (frame buffer, queues)
-    r->reserve = estimate_bytes(*r, ab) + (r->direct ? ((size_t)256 << 20) : 0);
+    r->reserve = estimate_bytes(*r, ab);
+    if (r->direct) {
+        // the direct path's dag also holds scratch of its own (queues, stacks,
+        // frames): a quarter of the budget, within these bounds; its count does
+        // with less where the rest of the budget is less
+        const size_t most = std::min(std::max(sv->cfg.mem_budget / 4, DIRECT_SCRATCH_MIN), DIRECT_SCRATCH_MAX);
+        const size_t room = sv->cfg.mem_budget - std::min(sv->cfg.mem_budget, r->reserve);
+        r->scratch = std::max(std::min(most, room), DIRECT_SCRATCH_MIN);
+        r->reserve += r->scratch;
+    }
     if (r->reserve > sv->cfg.mem_budget) {
         set_error("pvt_server_submit: query needs more device memory than the server's budget");
         return PVT_ENOMEM;

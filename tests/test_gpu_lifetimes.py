@@ -251,6 +251,24 @@ def test_a_recorded_count_after_its_frames_moved(pvt):
     dag.free()
 
 
+@pytest.mark.parametrize("kind", ["global", "vertex", "edge"])
+def test_a_direct_query_keeps_to_the_budget(pvt, kind):
+    """A server's direct query takes no more device memory than the budget holds
+    for it: optional buffers come out of what was reserved."""
+    rp, col = classes_graph()
+    dag = gpu_dag(pvt, rp, col)
+    want = {"global": dag.count_global, "vertex": dag.count_local_vertex, "edge": dag.count_local_edge}[kind](kmax=3)
+    dag.free()
+    budget = 512 << 20
+    with limited_pool(1 << 40) as used:
+        with pvt.Server(mem_budget=budget, direct_edges=1) as sv:
+            t = sv.submit(rp, col, kind, kmax=3)
+            assert sv.wait(t, 60000)
+            got = sv.result(t)[0].view(np.int64)
+        assert used(RESERVED_MEM_HIGH) <= budget
+    assert np.array_equal(got.reshape(-1), want.cpu().numpy().reshape(-1))
+
+
 @pytest.mark.parametrize("streams", [1, 2])
 def test_free_waits_for_the_copies_of_the_core_numbers(pvt, streams):
     """pvt_dag_cores only enqueues its copy.  A dag freed while such copies wait
