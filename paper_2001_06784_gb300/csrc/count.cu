@@ -45,7 +45,7 @@ template <int NW, int MODE>
 pvt_status launch_local(pvt_dag *g, const CountArgs &base, int cls, cudaStream_t s);
 template <int NW, int MODE>
 pvt_status launch_local_batch(const BatchGraph *, const uint64_t *, unsigned, unsigned *, const unsigned long long *, int,
-                              unsigned *, unsigned long long *, int, cudaStream_t);
+                              unsigned *, unsigned long long *, int, size_t, cudaStream_t);
 
 // The test-settable limit of the bounded device waits (policy.wait_limit_us).
 static void apply_wait_limit(const pvt_dag *g, CountArgs &A)
@@ -1013,7 +1013,8 @@ pvt_status batch_root_entries(BatchGraph *d_graphs, int count, uint64_t *const *
 
 template <int MODE>
 static pvt_status launch_batch_mode(const BatchGraph *gs, const uint64_t *const *h_entries, const unsigned *n_entries,
-                                    const unsigned long long *B, int Bw, unsigned *ctl, int num_sms, cudaStream_t s)
+                                    const unsigned long long *B, int Bw, unsigned *ctl, int num_sms, size_t scratch_room,
+                                    cudaStream_t s)
 {
     pvt_status st = PVT_OK;
     for (int c = NCLASS - 1; c >= 0 && st == PVT_OK; --c) {
@@ -1028,17 +1029,17 @@ static pvt_status launch_batch_mode(const BatchGraph *gs, const uint64_t *const 
             case 1:
                 if constexpr (MODE == MODE_GLOBAL)
                     st = launch_batch_class<1, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s);
-                else st = launch_local_batch<1, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s);
+                else st = launch_local_batch<1, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, scratch_room, s);
                 break;
             case 2:
                 if constexpr (MODE == MODE_GLOBAL)
                     st = launch_batch_class<2, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s);
-                else st = launch_local_batch<2, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s);
+                else st = launch_local_batch<2, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, scratch_room, s);
                 break;
             case 3:
                 if constexpr (MODE == MODE_GLOBAL)
                     st = launch_batch_class<4, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s);
-                else st = launch_local_batch<4, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s);
+                else st = launch_local_batch<4, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, scratch_room, s);
                 break;
             case 4: st = launch_batch_class<8, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s); break;
             case 5: st = launch_batch_class<16, MODE>(gs, e, cnt, qhead, B, Bw, err, stats, num_sms, s); break;
@@ -1052,14 +1053,14 @@ static pvt_status launch_batch_mode(const BatchGraph *gs, const uint64_t *const 
 // [32..] 64-bit walk statistics; zeroed by the caller.
 pvt_status batch_count(BatchGraph *d_graphs, int count, const int2 *d_combine_work, int n_combine,
                        const uint64_t *const *h_entries, const unsigned *n_entries,
-                       const unsigned long long *d_binom, int binom_stride, int num_sms, unsigned *d_ctl,
-                       cudaStream_t s)
+                       const unsigned long long *d_binom, int binom_stride, int num_sms, size_t scratch_room,
+                       unsigned *d_ctl, cudaStream_t s)
 {
     if (count <= 0) return PVT_OK;
     pvt_status st;
-    if ((st = launch_batch_mode<MODE_GLOBAL>(d_graphs, h_entries, n_entries, d_binom, binom_stride, d_ctl, num_sms, s)) != PVT_OK) return st;
-    if ((st = launch_batch_mode<MODE_VERTEX>(d_graphs, h_entries, n_entries, d_binom, binom_stride, d_ctl, num_sms, s)) != PVT_OK) return st;
-    if ((st = launch_batch_mode<MODE_EDGE>(d_graphs, h_entries, n_entries, d_binom, binom_stride, d_ctl, num_sms, s)) != PVT_OK) return st;
+    if ((st = launch_batch_mode<MODE_GLOBAL>(d_graphs, h_entries, n_entries, d_binom, binom_stride, d_ctl, num_sms, scratch_room, s)) != PVT_OK) return st;
+    if ((st = launch_batch_mode<MODE_VERTEX>(d_graphs, h_entries, n_entries, d_binom, binom_stride, d_ctl, num_sms, scratch_room, s)) != PVT_OK) return st;
+    if ((st = launch_batch_mode<MODE_EDGE>(d_graphs, h_entries, n_entries, d_binom, binom_stride, d_ctl, num_sms, scratch_room, s)) != PVT_OK) return st;
     if (n_combine > 0) {
         k_combine_batch<<<n_combine, 256, 0, s>>>(d_graphs, d_combine_work, d_binom, binom_stride, d_ctl);
         PVT_CK(cudaGetLastError());

@@ -1086,10 +1086,12 @@ pvt_status launch_local(pvt_dag *g, const CountArgs &base, int cls, cudaStream_t
     return PVT_OK;
 }
 
+// scratch_room: bytes its stacks and edge tables may take.  Any number of warps
+// walks the entries, so it makes do with less, down to a block's.
 template <int NW, int MODE>
 pvt_status launch_local_batch(const BatchGraph *gs, const uint64_t *entries, unsigned cnt, unsigned *qhead,
                               const unsigned long long *B, int Bw, unsigned *err, unsigned long long *stats, int num_sms,
-                              cudaStream_t s)
+                              size_t scratch_room, cudaStream_t s)
 {
     constexpr int WPB = local_wpb<NW>();
     constexpr size_t D = 32 * NW;
@@ -1097,14 +1099,23 @@ pvt_status launch_local_batch(const BatchGraph *gs, const uint64_t *entries, uns
     int per_sm = 0;
     pvt_status st = local_occupancy(k_local_batch<NW, MODE>, 32 * WPB, smem, &per_sm);
     if (st != PVT_OK) return st;
-    const unsigned grid = std::max(1u, std::min<unsigned>((unsigned)(num_sms * per_sm), (cnt + WPB - 1) / WPB));
+    unsigned grid = std::max(1u, std::min<unsigned>((unsigned)(num_sms * per_sm), (cnt + WPB - 1) / WPB));
+    constexpr size_t stack = LocalWork<NW>::GSTACK ? (size_t)WPB * (D + 1) * LocalWork<NW>::FW : 0;  // words of a block
+    constexpr size_t etab = MODE == MODE_EDGE ? (size_t)WPB * D * D : 0;
+    constexpr size_t block_bytes = (stack + etab) * sizeof(uint32_t);
     Scratch mem(s);
-    const size_t stack = LocalWork<NW>::GSTACK ? (size_t)grid * WPB * (D + 1) * LocalWork<NW>::FW : 0;
-    const size_t etab = MODE == MODE_EDGE ? (size_t)grid * WPB * D * D : 0;
-    if (stack + etab) PVT_CK(mem.take((stack + etab) * sizeof(uint32_t)));
+    if constexpr (block_bytes > 0) {
+        grid = (unsigned)std::max<size_t>(1, std::min<size_t>(grid, scratch_room / block_bytes));
+        cudaError_t e;
+        while ((e = mem.take(grid * block_bytes)) == cudaErrorMemoryAllocation && grid > 1) {
+            (void)cudaGetLastError();
+            grid = std::max(1u, grid / 4);
+        }
+        PVT_CK(e);
+    }
     uint32_t *scratch = mem.as<uint32_t>();
     k_local_batch<NW, MODE><<<grid, 32 * WPB, smem, s>>>(gs, entries, cnt, qhead, B, Bw, BATCH_MAX_ALPHA + 2, err, stats,
-                                                       scratch, scratch ? scratch + stack : nullptr);
+                                                       scratch, scratch ? scratch + stack * grid : nullptr);
     PVT_CK(cudaGetLastError());
     return PVT_OK;
 }

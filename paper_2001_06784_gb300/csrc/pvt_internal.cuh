@@ -138,11 +138,12 @@ pvt_status batch_orient(BatchGraph *d_graphs, int count, cudaStream_t s);
 // Batched walk of the root entries h_entries[mode * NCLASS + class] (device
 // arrays of (graph << 32 | root), n_entries each) and the combine of the
 // global queries (d_combine_work: (graph, k) per block).  d_ctl: zeroed
-// status word, queue heads and statistics (see count.cu).
+// status word, queue heads and statistics (see count.cu).  scratch_room: bytes
+// that a launch's stacks and edge tables should keep to.
 pvt_status batch_count(BatchGraph *d_graphs, int count, const int2 *d_combine_work, int n_combine,
                        const uint64_t *const *h_entries, const unsigned *n_entries,
-                       const unsigned long long *d_binom, int binom_stride, int num_sms, unsigned *d_ctl,
-                       cudaStream_t s);
+                       const unsigned long long *d_binom, int binom_stride, int num_sms, size_t scratch_room,
+                       unsigned *d_ctl, cudaStream_t s);
 // Fill the per-(mode, class) root entry lists of a batch from the descriptors.
 pvt_status batch_root_entries(BatchGraph *d_graphs, int count, uint64_t *const *d_entries,
                               const unsigned *d_class_offsets /*[count][NCLASS]*/, cudaStream_t s);

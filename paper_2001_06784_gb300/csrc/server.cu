@@ -104,6 +104,7 @@ struct Batch {
     cudaStream_t stream = nullptr;
     cudaEvent_t done = nullptr;
     std::vector<void *> dallocs;
+    size_t reserve = 0;              // budget bytes held for the walks' scratch
     unsigned *hctl = nullptr;        // pinned copy of the batch status word
     size_t hctl_cls = 0;
 };
@@ -125,6 +126,9 @@ size_t estimate_bytes(const Request &r, int alpha_bound)
     return b;
 }
 
+// Budget bytes a batch may hold for the scratch of its local counts (per-edge
+// tables of the 65..128 class on every resident warp: 218 MB).
+constexpr size_t BATCH_SCRATCH_MAX = (size_t)224 << 20;
 // Budget bytes a direct query holds for its dag's scratch.
 constexpr size_t DIRECT_SCRATCH_MIN = (size_t)256 << 20, DIRECT_SCRATCH_MAX = (size_t)1280 << 20;
 
@@ -374,10 +378,20 @@ void run_group(pvt_server *sv, std::vector<ReqPtr> &group)
     cudaMemcpyAsync(d_off, off.data(), 4 * off.size(), cudaMemcpyHostToDevice, ws);
     if (!work.empty()) cudaMemcpyAsync(d_work, work.data(), sizeof(int2) * work.size(), cudaMemcpyHostToDevice, ws);
     cudaMemsetAsync(d_ctl, 0, 4 * 64, ws);
+    // local counts keep stacks and edge tables per resident warp, one class
+    // after another on ws: half of what the budget has left, up to what the
+    // largest class can use
+    bool local = false;
+    for (int i = NCLASS; i < 3 * NCLASS; ++i) local = local || n_entries[i];
+    if (local) {
+        std::lock_guard<std::mutex> lk(sv->mu);
+        bt->reserve = std::min(BATCH_SCRATCH_MAX, (sv->cfg.mem_budget - std::min(sv->cfg.mem_budget, sv->mem_used)) / 2);
+        sv->mem_used += bt->reserve;
+    }
     st = batch_root_entries(dg, G2, d_eptr, d_off, ws);
     if (st == PVT_OK)
         st = batch_count(dg, G2, d_work, (int)work.size(), eptr.data(), n_entries.data(), sv->binom, BINOM_W,
-                         sv->num_sms, d_ctl, ws);
+                         sv->num_sms, bt->reserve, d_ctl, ws);
     // ---- 5. results to pinned host memory, completion event
     for (int g = 0; g < G2; ++g) {
         Request &r = *ok[g];
@@ -392,6 +406,11 @@ void run_group(pvt_server *sv, std::vector<ReqPtr> &group)
         for (auto &r : ok) fail_request(sv, r, PVT_ECUDA, "server: batched walk launch failed");
         cudaEventDestroy(bt->done);
         for (void *q : bt->dallocs) cudaFree(q);
+        {
+            std::lock_guard<std::mutex> lk(sv->mu);
+            sv->mem_used -= bt->reserve;
+        }
+        sv->cv_work.notify_all();
         sv->pinned.put(bt->hctl, bt->hctl_cls);
         delete bt;
         return;
@@ -529,6 +548,7 @@ void complete_batch(pvt_server *sv, Batch *bt)
         sv->mem_used -= r->reserve;
         sv->inflight -= 1;
     }
+    sv->mem_used -= bt->reserve;
     sv->pinned.put(bt->hctl, bt->hctl_cls);
     cudaEventDestroy(bt->done);
     delete bt;

@@ -7,9 +7,9 @@ template pvt_status launch_local<1, MODE_EDGE>(pvt_dag *, const CountArgs &, int
 template pvt_status launch_local<2, MODE_EDGE>(pvt_dag *, const CountArgs &, int, cudaStream_t);
 template pvt_status launch_local_batch<1, MODE_EDGE>(const BatchGraph *, const uint64_t *, unsigned, unsigned *,
                                                      const unsigned long long *, int, unsigned *,
-                                                     unsigned long long *, int, cudaStream_t);
+                                                     unsigned long long *, int, size_t, cudaStream_t);
 template pvt_status launch_local_batch<2, MODE_EDGE>(const BatchGraph *, const uint64_t *, unsigned, unsigned *,
                                                      const unsigned long long *, int, unsigned *,
-                                                     unsigned long long *, int, cudaStream_t);
+                                                     unsigned long long *, int, size_t, cudaStream_t);
 
 }  // namespace pvt

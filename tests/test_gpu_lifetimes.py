@@ -269,6 +269,27 @@ def test_a_direct_query_keeps_to_the_budget(pvt, kind):
     assert np.array_equal(got.reshape(-1), want.cpu().numpy().reshape(-1))
 
 
+def test_a_batch_keeps_to_the_budget(pvt):
+    """Batched per-edge counts of dense graphs take their tables out of what the
+    budget has left, and fewer warps walk where that is little."""
+    qs = [graphs.gnp(110 + i, 0.5, 60 + i) for i in range(8)] + [graphs.gnp(60 + i, 0.5, 70 + i) for i in range(8)]
+    want = []
+    for rp, col in qs:
+        dag = gpu_dag(pvt, rp, col)
+        want.append(dag.count_local_edge(kmax=4).cpu().numpy().reshape(-1))
+        dag.free()
+    for budget in (16 << 20, 64 << 20, 4 << 30):
+        with limited_pool(max(budget, 32 << 20)) as used:
+            with pvt.Server(mem_budget=budget, direct_edges=-1) as sv:
+                tickets = [sv.submit(rp, col, "edge", kmax=4) for rp, col in qs]
+                got = []
+                for t in tickets:
+                    assert sv.wait(t, 60000)
+                    got.append(sv.result(t)[0].view(np.int64).reshape(-1))
+            assert used(RESERVED_MEM_HIGH) <= max(budget, 32 << 20)
+        assert all(np.array_equal(a, b) for a, b in zip(got, want))
+
+
 @pytest.mark.parametrize("streams", [1, 2])
 def test_free_waits_for_the_copies_of_the_core_numbers(pvt, streams):
     """pvt_dag_cores only enqueues its copy.  A dag freed while such copies wait
