@@ -65,7 +65,8 @@ typedef struct pvt_dag pvt_dag;
  *   row_ptr,col  device CSR as above.  It is borrowed, not copied: it must
  *                stay valid and unchanged until pvt_dag_free (per-edge counts
  *                read it again).
- *   flags        0, PVT_VALIDATE (else the CSR is trusted), PVT_PROFILE
+ *   flags        0, PVT_VALIDATE (else the CSR is trusted; one whose out-lists
+ *                do not add up to m entries is refused), PVT_PROFILE
  *   dag_out      receives the new pvt_dag (host pointer to a pointer)
  *   alpha_out    receives the largest out-degree (host; may be NULL)
  * Errors: PVT_EINVAL, PVT_ENOTSIMPLE, PVT_ENOMEM, PVT_ECUDA, PVT_ETIMEOUT.

@@ -1195,11 +1195,17 @@ __global__ void __launch_bounds__(256) k_outdeg(int64_t n, const int64_t *__rest
         if (sh[i]) atomicAdd(&st->deg_cnt[i], sh[i]);
 }
 
-// Out-lists in CSR order (ascending id), compacted with a warp ballot.
+// Out-lists in CSR order (ascending id), compacted with a warp ballot.  Every
+// edge of a symmetric CSR gives one entry, m in all; where the count of another
+// CSR differs, nothing is written.
 __global__ void k_fill(int64_t n, const int64_t *__restrict__ rp, const uint32_t *__restrict__ col,
                        const uint32_t *__restrict__ rnd, const int64_t *__restrict__ orow,
-                       uint32_t *ocol)
+                       uint32_t *ocol, int64_t m, unsigned *err)
 {
+    if (orow[n] != m) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(err, DERR_NOTSIMPLE);
+        return;
+    }
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1593,7 +1599,7 @@ pvt_status orient_build(pvt_dag *g, uint32_t flags, cudaStream_t s)
         k_outdeg<<<og, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, odeg, cst);
         PVT_CK(cudaGetLastError());
         if ((st = exclusive_scan_u32_i64(odeg, g->orow, n, s)) != PVT_OK) return st;
-        k_fill<<<og, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, g->orow, g->ocol);
+        k_fill<<<og, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, g->orow, g->ocol, g->m, g->d_err);
         k_deg_slots<<<1, 1024, 0, s>>>(cst);
         k_deg_scatter<<<og, 256, 0, s>>>(n, odeg, cst->deg_cnt, g->roots);
         PVT_CK(cudaGetLastError());

@@ -290,6 +290,22 @@ def test_a_batch_keeps_to_the_budget(pvt):
         assert all(np.array_equal(a, b) for a, b in zip(got, want))
 
 
+@pytest.mark.parametrize("extra", ["into the core", "out of the core"])
+def test_an_asymmetric_csr_is_refused_before_its_out_lists_are_written(pvt, extra):
+    """K_40 and 20 more vertices with 400 arcs one way.  Trusted without
+    validation, its out-lists would have more entries than nnz / 2 (arcs from
+    vertices that come before the core), or fewer."""
+    rows = [[u for u in range(40) if u != v] for v in range(40)] + [[] for _ in range(20)]
+    for v in range(40, 60):
+        for u in range(20):
+            (rows[v] if extra == "into the core" else rows[u]).append(u if extra == "into the core" else v)
+    rp = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64)
+    col = np.concatenate([np.asarray(r, np.uint32) for r in rows])
+    with pytest.raises(pvt.PivoterError) as e:
+        gpu_dag(pvt, rp, col, validate=False)
+    assert e.value.status == 2
+
+
 @pytest.mark.parametrize("streams", [1, 2])
 def test_free_waits_for_the_copies_of_the_core_numbers(pvt, streams):
     """pvt_dag_cores only enqueues its copy.  A dag freed while such copies wait
