@@ -218,10 +218,25 @@ static void res_to_dag(const DagRes &r, pvt_dag *g)
     g->binom_W = r.binom_W;
 }
 
+// The device's pool keeps freed scratch for the next call.  What a dag's
+// optional buffers held beyond POOL_KEEP (most dags stay below) goes back to
+// the device, where other allocators of the process find it.
+constexpr size_t POOL_KEEP = (size_t)2 << 30;
+static void give_back(int device)
+{
+    cudaMemPool_t pool;
+    uint64_t used = 0;
+    if (cudaDeviceGetMemPool(&pool, device) == cudaSuccess &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
+        cudaMemPoolTrimTo(pool, used + POOL_KEEP);
+}
+
 static void dag_release(pvt_dag *g)
 {
     if (!g) return;
     drop_graph(g);
+    size_t optional = g->cframes.n + g->cframes1.n;
+    for (const auto &b : g->lheavy) optional += b.n;
     // nothing of this dag is in flight once its side streams are idle and the
     // copies of its core numbers are made: every other entry point
     // synchronises the caller's stream before it returns
@@ -248,6 +263,7 @@ static void dag_release(pvt_dag *g)
     release(g->range_roots.p);
     release(g->range_pos.p);
     if (fs) cudaStreamSynchronize(fs);
+    if (optional * sizeof(uint32_t) > POOL_KEEP) give_back(g->device);
     DagRes r;
     r.device = g->device;
     r.d_err = g->d_err;

@@ -31,7 +31,7 @@ class PoolProps(ctypes.Structure):
                 ("usage", ctypes.c_ushort), ("reserved", ctypes.c_ubyte * 54)]
 
 
-RESERVED_MEM_HIGH, USED_MEM_CURRENT = 6, 7  # CU_MEMPOOL_ATTR_*
+RESERVED_MEM_CURRENT, RESERVED_MEM_HIGH, USED_MEM_CURRENT = 5, 6, 7  # CU_MEMPOOL_ATTR_*
 
 
 @contextlib.contextmanager
@@ -304,6 +304,29 @@ def test_an_asymmetric_csr_is_refused_before_its_out_lists_are_written(pvt, extr
     with pytest.raises(pvt.PivoterError) as e:
         gpu_dag(pvt, rp, col, validate=False)
     assert e.value.status == 2
+
+
+def test_large_frames_go_back_to_the_device(pvt):
+    """A dag whose frame buffer passed 2 GiB leaves at most that, beyond what is
+    in use, in the device's pool."""
+    import torch
+    cu = ctypes.CDLL("libcuda.so.1")
+    pool = ctypes.c_void_p()
+
+    def held(attr):
+        torch.cuda.synchronize()
+        x = ctypes.c_uint64()
+        assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
+        assert cu.cuMemPoolGetAttribute(pool, attr, ctypes.byref(x)) == 0
+        return x.value
+
+    rp, col = graphs.clique_minus_random(1000, 9, 57)
+    dag = gpu_dag(pvt, rp, col)
+    before = held(USED_MEM_CURRENT)
+    dag.count_global(kmax=4)
+    assert held(USED_MEM_CURRENT) - before > 2 << 30
+    dag.free()
+    assert held(RESERVED_MEM_CURRENT) - held(USED_MEM_CURRENT) <= 2 << 30
 
 
 @pytest.mark.parametrize("streams", [1, 2])
