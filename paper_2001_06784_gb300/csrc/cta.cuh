@@ -434,7 +434,7 @@ __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork
                             if (w == j) M[w] &= ~Rj;
                     }
                     top += before;
-                    small.close<true>(sh32, A, lane, h + 1, p, wc.nodes, wc.leaves, wc.words);
+                    small.close<true, false>(sh32, A, lane, h + 1, p, wc.nodes, wc.leaves, wc.words);
                     __syncwarp();
                     if (TOP && clock >= CTA_DONATE_EVERY) {
                         clock = 0;
@@ -490,7 +490,7 @@ __device__ __forceinline__ void cta_level(CtaQueue<NW> &Q, CtaWarp &CW, LaneWork
                 }
                 if (ps <= 2) {
                     const bool adjp = ps == 2 && ((rows[a * RS + (b >> 5)] >> (b & 31)) & 1u);
-                    close_small<true>(sh32, A, lane, ps, adjp, h, p + 1, wc.nodes, wc.leaves, wc.words);
+                    close_small<true, false>(sh32, A, lane, ps, adjp, h, p + 1, wc.nodes, wc.leaves, wc.words);
                 } else {
                     closed = false;
 #pragma unroll

@@ -194,10 +194,25 @@ constexpr uint32_t FRAME_NONE = 0u, FRAME_WIDE = 1u, FRAME_COMPACT = 2u;
 // Block-level (h, p) leaf histogram in shared memory for h < HIST_H, p < HIST_P
 // (where almost every leaf falls); other leaves go straight to the global one.
 constexpr int HIST_H = 32, HIST_P = 48;
+constexpr unsigned HIST_DRAIN = 1u << 18;
 
 // Walk statistics, the same on every lane of the warp.
 struct WalkCounters {
-    unsigned long long nodes = 0, leaves = 0, words = 0;
+    unsigned long long nodes = 0, leaves = 0, words = 0, drained = 0;
+    // Every HIST_DRAIN leaves of the warp it empties the block's histogram into
+    // the global one: with at most 16 warps a counter stays below 2^32.  (All
+    // lanes, at each wide node and after each one-word walk, whose tree has far
+    // fewer leaves than that.)
+    template <bool SHIST>
+    __device__ __forceinline__ void drain(unsigned *shist, const CountArgs &A, int lane)
+    {
+        if (!SHIST || leaves - drained < HIST_DRAIN) return;
+        drained = leaves;
+        for (int i = lane; i < HIST_H * HIST_P; i += 32) {
+            const unsigned x = atomicExch(&shist[i], 0u);
+            if (x) atomicAdd(&A.hist[(size_t)(i / HIST_P) * A.hstride + (i % HIST_P)], (unsigned long long)x);
+        }
+    }
     // add the warp's totals to stats[0..2] and, if cls >= 0, to stats[3 + cls]
     // (all lanes)
     __device__ __forceinline__ void flush(unsigned long long *stats, int cls, int lane)
@@ -223,6 +238,25 @@ __device__ __forceinline__ void tally_n(unsigned *shist, const CountArgs &A, int
     } else {
         atomicAdd(&A.hist[(size_t)h * A.hstride + p], (unsigned long long)n);
     }
+}
+
+// The same for the walks whose warps drain the block's histogram now and then
+// (WalkCounters::drain), so that no counter can wrap: nothing waits for its old
+// value.  A warp that walks alone is a chain of dependent instructions, and the
+// returned value was part of it.
+template <bool SHIST>
+__device__ __forceinline__ void tally_add(unsigned *shist, const CountArgs &A, int h, int p, unsigned n)
+{
+    if (SHIST && h < HIST_H && p < HIST_P) atomicAdd(&shist[h * HIST_P + p], n);
+    else atomicAdd(&A.hist[(size_t)h * A.hstride + p], (unsigned long long)n);
+}
+
+// Which of the two a walk takes: DRAINS, the second.
+template <bool SHIST, bool DRAINS>
+__device__ __forceinline__ void tally_of(unsigned *shist, const CountArgs &A, int h, int p, unsigned n)
+{
+    if (DRAINS) tally_add<SHIST>(shist, A, h, p, n);
+    else tally_n<SHIST>(shist, A, h, p, n);
 }
 
 // The block's 32-bit histogram into the global one (all threads of the block,
@@ -253,7 +287,7 @@ struct SmallCounts {
         else c2 += adjacent ? 1u : 0x10000u;
     }
     // all lanes; every lane passes the same (h, p)
-    template <bool SHIST, typename N>
+    template <bool SHIST, bool DRAINS, typename N>
     __device__ __forceinline__ void close(unsigned *shist, const CountArgs &A, int lane, int h, int p, N &nodes,
                                           N &leaves, N &words) const
     {
@@ -265,12 +299,12 @@ struct SmallCounts {
         leaves += n0 + n1 + adj + non + held;
         words += n1 + 2 * (adj + non);
         const unsigned n = lane == 0 ? n0 : lane == 1 ? n1 + non : lane == 2 ? adj : lane == 3 ? held : 0u;
-        if (n) tally_n<SHIST>(shist, A, lane == 3 ? h + 1 : h, lane == 3 ? p : p + lane, n);
+        if (n) tally_of<SHIST, DRAINS>(shist, A, lane == 3 ? h + 1 : h, lane == 3 ? p : p + lane, n);
     }
 };
 
 // The same for one label, every lane with the same arguments.
-template <bool SHIST, typename N>
+template <bool SHIST, bool DRAINS, typename N>
 __device__ __forceinline__ void close_small(unsigned *shist, const CountArgs &A, int lane, int cs, bool adjacent, int h,
                                             int p, N &nodes, N &leaves, N &words)
 {
@@ -279,8 +313,8 @@ __device__ __forceinline__ void close_small(unsigned *shist, const CountArgs &A,
     nodes += 1 + split + held;
     leaves += 1 + held;
     words += (unsigned)cs;
-    if (lane == 0) tally_n<SHIST>(shist, A, h, split ? p + 1 : p + cs, 1u);
-    if (lane == 1 && held) tally_n<SHIST>(shist, A, h + 1, p, 1u);
+    if (lane == 0) tally_of<SHIST, DRAINS>(shist, A, h, split ? p + 1 : p + cs, 1u);
+    if (lane == 1 && held) tally_of<SHIST, DRAINS>(shist, A, h + 1, p, 1u);
 }
 
 // Donated frames must carry enough work to pay for the queue round trip.
@@ -501,15 +535,17 @@ __device__ void compact_loop(WarpWork<NW> &Wk, unsigned *shist, const CountArgs 
                              Clock &clk)
 {
     auto tally = [&](int hh, int pp) {
-        if (lane == 0) tally_n<SHIST>(shist, A, hh, pp, 1u);
+        if (lane == 0) tally_add<SHIST>(shist, A, hh, pp, 1u);
     };
-    // this call's nodes, leaves and pivot words (every lane alike; at most a
-    // 32-member label's tree, so 32 bits hold them), added to wc on exit
-    unsigned cn = 0, cl = 0, cw = 0;
+    // this call's nodes, leaves and pivot words (every lane alike, and those of
+    // the labels a lane closed itself; at most a 32-member label's tree, so 32
+    // bits hold them), added to wc on exit
+    unsigned cn = 0, cl = 0, cw = 0, xn = 0, xl = 0, xw = 0;
     auto fold = [&]() {
-        wc.nodes += cn;
-        wc.leaves += cl;
-        wc.words += cw;
+        wc.nodes += cn + __reduce_add_sync(FULL, xn);
+        wc.leaves += cl + __reduce_add_sync(FULL, xl);
+        wc.words += cw + __reduce_add_sync(FULL, xw);
+        wc.drain<SHIST>(shist, A, lane);
     };
     int top = 0, bot = 0;
     for (;;) {
@@ -541,9 +577,19 @@ __device__ void compact_loop(WarpWork<NW> &Wk, unsigned *shist, const CountArgs 
                     const uint32_t child = inR ? (r1 & S1 & ~(R0 & ((1u << lane) - 1u))) : 0u;
                     const int cs = __popc(child);
                     const uint32_t ra = __shfl_sync(FULL, r1, (__ffs(child) - 1) & 31);
-                    SmallCounts small;
-                    if (inR && cs <= 2) small.add(cs, (ra >> ((31 - __clz(child)) & 31)) & 1u);
-                    small.close<SHIST>(shist, A, lane, h + 1, p, cn, cl, cw);
+                    // each lane closes its own (the cases of SmallCounts): sums over
+                    // the warp, or ballots, would lie on the walk's dependent chain
+                    // (99 roots of 65..128 members, heavy trees: 1049 ms with
+                    // SmallCounts, 781 with ballots, 738 like this)
+                    if (inR && cs <= 2) {
+                        const bool adj = cs == 2 && ((ra >> ((31 - __clz(child)) & 31)) & 1u);
+                        const bool non = cs == 2 && !adj, held = non && h + 2 <= A.kmax;
+                        xn += 1u + non + held;
+                        xl += 1u + held;
+                        xw += (unsigned)cs;
+                        tally_add<SHIST>(shist, A, h + 1, non ? p + 1 : p + cs, 1u);
+                        if (held) tally_add<SHIST>(shist, A, h + 2, p, 1u);
+                    }
                     R = __ballot_sync(FULL, inR && cs > 2);
                 }
                 const int nR = __popc(R);
@@ -612,7 +658,7 @@ __device__ void compact_loop(WarpWork<NW> &Wk, unsigned *shist, const CountArgs 
                 const int ps = __popc(P1);
                 if (ps <= 2) {
                     const uint32_t ra = __shfl_sync(FULL, r1, (__ffs(P1) - 1) & 31);
-                    close_small<SHIST>(shist, A, lane, ps, (ra >> ((31 - __clz(P1)) & 31)) & 1u, h, p + 1, cn, cl, cw);
+                    close_small<SHIST, true>(shist, A, lane, ps, (ra >> ((31 - __clz(P1)) & 31)) & 1u, h, p + 1, cn, cl, cw);
                 } else {
                     closed = false;
                     S1 = P1;
@@ -941,6 +987,7 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A,
     uint16_t link = 0;
     if (MODE != MODE_GLOBAL && lane == 0) Wk.path[0] = (uint16_t)d;
     for (;;) {
+        wc.drain<SHIST>(shist, A, lane);
         const int depth = h + p - 1;
         if (MODE != MODE_GLOBAL && depth > 0) {
             if (lane == 0) Wk.path[depth] = link;
@@ -957,7 +1004,7 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A,
         } else if ((wc.nodes++, clk.nodes++, s == 0)) {
             wc.leaves++;
             if (MODE == MODE_GLOBAL) {
-                if (lane == 0) tally_n<SHIST>(shist, A, h, p, 1u);
+                if (lane == 0) tally_add<SHIST>(shist, A, h, p, 1u);
             } else {
                 local_leaf<NW, MODE>(Wk, A, lane, r, rbeg, d, h, p, depth, nullptr);
             }
@@ -990,7 +1037,7 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A,
                 // S is a clique: one leaf with |S| more pivot links
                 wc.leaves++;
                 if (MODE == MODE_GLOBAL) {
-                    if (lane == 0) tally_n<SHIST>(shist, A, h, p + s, 1u);
+                    if (lane == 0) tally_add<SHIST>(shist, A, h, p + s, 1u);
                 } else {
                     local_leaf<NW, MODE>(Wk, A, lane, r, rbeg, d, h, p + s, depth, S);
                 }
@@ -1111,7 +1158,7 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A,
                         }
                     }
                     top += before;
-                    if (MODE == MODE_GLOBAL) small.close<SHIST>(shist, A, lane, h + 1, p, wc.nodes, wc.leaves, wc.words);
+                    if (MODE == MODE_GLOBAL) small.close<SHIST, true>(shist, A, lane, h + 1, p, wc.nodes, wc.leaves, wc.words);
                     __syncwarp();  // pushed frames visible to every lane
                     if (SPLIT && (int)(clk.nodes - clk.next) >= 0) {
                         clk.next = clk.nodes + clk.every;
@@ -1143,7 +1190,7 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A,
                 }
                 if (MODE == MODE_GLOBAL && ps <= 2) {
                     const bool adj = ps == 2 && ((Wk.adj[a * RS + (b >> 5)] >> (b & 31)) & 1u);
-                    close_small<SHIST>(shist, A, lane, ps, adj, h, p + 1, wc.nodes, wc.leaves, wc.words);
+                    close_small<SHIST, true>(shist, A, lane, ps, adj, h, p + 1, wc.nodes, wc.leaves, wc.words);
                 } else {
                     closed = false;
 #pragma unroll
