@@ -1241,14 +1241,12 @@ __device__ __forceinline__ void bind_warp(WarpWork<NW> &Wk, unsigned char *local
 // Lane 0 of a split launch: the next item -- 2 with v = a fresh item index
 // below nitems, 1 with v = the ticket of a donated frame, 3 when no work is
 // left (or an error or a timeout ended the launch).
-// A warp that may not wait leaves when no published frame is without a taker.
-__device__ __forceinline__ int queue_take(const CountArgs &A, unsigned nitems, unsigned &v, bool may_wait = true)
+__device__ __forceinline__ int queue_take(const CountArgs &A, unsigned nitems, unsigned &v)
 {
     if (vload(A.qctl + Q_ROOT) < nitems) {
         const unsigned rr = atomicAdd(A.qctl + Q_ROOT, 1u);
         if (rr < nitems) { v = rr; return 2; }
     }
-    if (!may_wait && vload64(A.qctl + Q_HEAD) >= vload64(A.qctl + Q_TAIL)) return 3;
     // a ticket for the next donated frame; wait on its own slot
     int kind = 0;
     const unsigned t = (unsigned)atomicAdd(qword(A.qctl + Q_HEAD), 1ull);
@@ -1304,14 +1302,13 @@ __global__ void __launch_bounds__(32 * warps_per_block<NW>())
     unsigned qi = 0, qend = 0;
     if (SPLIT) {
         // heavy roots and donated subtree frames from one device work queue.
-        // Once the roots are out, the second half of the blocks leaves instead
-        // of waiting for donations, so that the next class's kernel can start
-        // on the SMs (waiting was 28 % of the warps' time in the 129..256 class
-        // of the 10.8M-edge graph: donations, not takers, are what is scarce)
-        const bool may_wait = blockIdx.x < (gridDim.x + 1) / 2;
+        // Every warp waits to the end: a class's last roots may hold most of its
+        // tree.  (Half of the blocks left once the roots were out, so that the
+        // next class could start: 7.4 -> 7.0 ms of the 10.8M-edge graph's count,
+        // but 2.9 -> 5.2 s where dense groups of 90 to 120 vertices were the work.)
         for (;;) {
             unsigned v = 0;
-            int kind = lane == 0 ? queue_take(A, A.nroots, v, may_wait) : 0;
+            int kind = lane == 0 ? queue_take(A, A.nroots, v) : 0;
             kind = __shfl_sync(FULL, kind, 0);
             v = __shfl_sync(FULL, v, 0);
             if (kind == 3) break;
