@@ -299,19 +299,33 @@ static pvt_status launch_frames(pvt_dag *g, const CountArgs &base, cudaStream_t 
     return PVT_OK;
 }
 
-// Frames the wide walks may emit: an allowance per root by class (a wider
-// root meets many more small labels), at most 2^26 (9.7 GB).  The frame walk
-// takes 3 to 4 ns of the GPU per frame, the wide kernels' few warps about
-// ten times that for a frame walked in place: on a 12M-edge graph of
-// degeneracy 280 (k <= 4, 34M frames) a buffer of 2^22 frames cost 204 ms
-// in all, one that holds them 55 ms.
+// Frames the wide walks may emit: 2^19 (75 MB), and an allowance per root by
+// class (a wider root meets many more small labels), at most 2^26 (9.7 GB).
+// The frame walk takes 3 to 4 ns of the GPU per frame, the wide kernels' few
+// warps about ten times that for a frame walked in place: on a 12M-edge graph
+// of degeneracy 280 (k <= 4, 34M frames) a buffer of 2^22 frames cost 204 ms in
+// all, one that holds them 55 ms.  A few dense roots emit much: 373 roots in
+// four groups of 90 to 120 vertices and six of 40 to 60 (density 0.8 and 0.95,
+// k <= 8) met 228,000 labels, 345 ms with room for 76,000 of them, 7.7 ms with
+// room for all.
 constexpr unsigned FRAME_CAP_MIN = 1u << 16, FRAME_CAP_MAX = 1u << 26;
+constexpr int64_t FRAMES_BASE = 1 << 19, FRAMES_PER_ROOT[NCLASS] = {0, 0, 64, 64, 1024, 8192, 32768};
 static unsigned frame_cap(const pvt_dag *g)
 {
-    constexpr int64_t per_root[NCLASS] = {0, 0, 16, 64, 1024, 8192, 32768};
-    int64_t want = 1 << 16;
-    for (int c = 2; c < NCLASS; ++c) want += per_root[c] * g->wcnt[c];
+    int64_t want = FRAMES_BASE;
+    for (int c = 2; c < NCLASS; ++c) want += FRAMES_PER_ROOT[c] * g->wcnt[c];
     return (unsigned)(std::min<int64_t>(want, FRAME_CAP_MAX) / EMIT_RESERVE * EMIT_RESERVE);
+}
+
+// Slots of such a buffer that class c may fill: all but the allowances of the
+// narrower classes (at most three quarters of it).  The widest class, which
+// meets labels by the billion on a dense graph, would otherwise leave the
+// narrower ones, whose labels mostly fit, to walk theirs in place.
+static unsigned class_cap(const pvt_dag *g, unsigned cap, int c)
+{
+    int64_t narrower = 0;
+    for (int q = 2; q < c; ++q) narrower += FRAMES_PER_ROOT[q] * g->wcnt[q];
+    return (cap - (unsigned)std::min<int64_t>(narrower, cap / 4 * 3)) / EMIT_RESERVE * EMIT_RESERVE;
 }
 
 // The walk of a class above 32 with a warp per root.  Global counts take the
@@ -431,7 +445,7 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
         frames = st == PVT_OK && cap > 0;
         A.emit = frames ? g->cframes.p : nullptr;
         A.emit_count = reinterpret_cast<unsigned long long *>(g->d_q + 8);  // words 8..9
-        A.emit_cap = frames ? cap : 0;
+        A.emit_cap = A.emit_all = frames ? cap : 0;
     }
     // the gather's pass: as many roots as its frames find room for
     int64_t pass1 = std::min(g->wcnt[1], GATHER1_MAX);
@@ -467,6 +481,7 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
         // The <= 32 class needs none and runs beside them.
         cudaStream_t cs = serial ? s : g->side[MODE == MODE_GLOBAL && c >= 2 ? NCLASS - 1 : c];
         if (!serial) PVT_CK(cudaStreamWaitEvent(cs, g->ev_fork, 0));
+        if (c >= 2) A.emit_cap = class_cap(g, A.emit_all, c);
         st = launch_one<MODE>(g, A, c, (unsigned)pass1, slots1, cs);
         if (!serial) PVT_CK(cudaEventRecord(g->ev_join[c], cs));
     }
@@ -478,6 +493,7 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
             for (int c = NCLASS - 1; c >= (gather1 ? 1 : 2); --c)
                 if (g->wcnt[c]) PVT_CK(cudaStreamWaitEvent(s, g->ev_join[c], 0));
         A.emit1_cap = slots1;
+        A.emit_cap = A.emit_all;
         if ((st = launch_frames(g, A, s)) != PVT_OK) return st;
     }
     // the roots beyond the first pass of the gather

@@ -163,7 +163,8 @@ struct CountArgs {
     uint32_t *emit;             // [emit_cap][FRAME_WORDS]
     unsigned long long *emit_count;  // slots reserved so far (passes emit_cap once the buffer is
                                      // full; slots without a subtree are marked FRAME_NONE)
-    unsigned emit_cap;               // a multiple of EMIT_RESERVE
+    unsigned emit_cap;               // slots the launch may fill, a multiple of EMIT_RESERVE
+    unsigned emit_all;               // slots there are
     // two-phase <= 32 class: the frames its gather emits (emit1_count of
     // emit1_cap slots reserved, empty ones marked kind 0; null: none)
     uint32_t *emit1;
@@ -725,8 +726,9 @@ constexpr unsigned EMIT_RESERVE = 16;
 struct Emitter {
     unsigned long long met = 0;     // compacted subtrees met, emitted or walked in place
     unsigned slot = 0, end = 0;     // reserved slots
-    bool full = false;              // the buffer is full
-    // the next slot, or nullptr once the buffer is full (all lanes)
+    bool full = false;              // no more slots
+    // the next slot, or nullptr once the launch's share of the buffer is full
+    // (all lanes; the group that found it full holds no subtrees)
     __device__ __forceinline__ uint32_t *next(const CountArgs &A, int lane)
     {
         if (slot == end) {
@@ -736,6 +738,8 @@ struct Emitter {
             b = __shfl_sync(FULL, b, 0);
             if (b + EMIT_RESERVE > (unsigned long long)A.emit_cap) {
                 full = true;
+                if (b + EMIT_RESERVE <= (unsigned long long)A.emit_all && lane < (int)EMIT_RESERVE)
+                    A.emit[(size_t)(b + lane) * FRAME_WORDS] = FRAME_NONE;
                 return nullptr;
             }
             slot = (unsigned)b;
@@ -1075,7 +1079,7 @@ __device__ void walk_root(WarpWork<NW> &Wk, unsigned *shist, const CountArgs &A,
                     int before = 0;
                     const uint32_t low = (1u << lane) - 1u;
                     SmallCounts small;
-                    const bool emits = MODE == MODE_GLOBAL && NW > 1 && A.emit != nullptr;
+                    const bool emits = MODE == MODE_GLOBAL && NW > 1 && A.emit != nullptr && !em.full;
                     uint32_t Rl = 0;      // word `lane` of R
                     uint32_t emitl = 0;   // members of word `lane` whose labels are emitted
                     uint32_t M[NW];
