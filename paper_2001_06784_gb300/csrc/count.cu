@@ -472,14 +472,21 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
     int used = 0;
     for (int c = 1; c < NCLASS; ++c) used += g->wcnt[c] > 0;
     const bool serial = g->serial || g->policy.serial || used <= 1;
+    // The wide classes of a two-phase count follow one another, widest first,
+    // where each fills the GPU and shares the subtrees of its last roots: side by
+    // side they would only take shared memory from one another (counts of two
+    // graphs with 2,500 to 37,000 roots in each of three classes: 4.2 ms in one
+    // stream, 5.0 on a stream each; 7.4 on either).  Else they overlap: a class
+    // of few roots, or of roots that one warp walks to the end, leaves the GPU
+    // idle (three classes of 140 to 280 roots 3.1 -> 2.4 ms, without splitting
+    // 4.9 -> 3.0; the plain form of the 10.8M-edge graph 76 -> 65 ms).  The <= 32
+    // class, which needs no shared memory to speak of, runs beside them.
+    bool one_stream = A.emit != nullptr;
+    for (int c = 2; c < NCLASS; ++c) one_stream = one_stream && (g->wcnt[c] == 0 || g->fills[c]);
     if (!serial) PVT_CK(cudaEventRecord(g->ev_fork, s));
     for (int c = NCLASS - 1; c >= 1 && st == PVT_OK; --c) {
         if (g->wcnt[c] == 0) continue;
-        // a global count's wide classes follow one another, widest first: each
-        // fills the GPU, and side by side they only take shared memory from one
-        // another (count of the 10.8M-edge graph 7.0 ms, in one stream 6.2).
-        // The <= 32 class needs none and runs beside them.
-        cudaStream_t cs = serial ? s : g->side[MODE == MODE_GLOBAL && c >= 2 ? NCLASS - 1 : c];
+        cudaStream_t cs = serial ? s : g->side[one_stream && c >= 2 ? NCLASS - 1 : c];
         if (!serial) PVT_CK(cudaStreamWaitEvent(cs, g->ev_fork, 0));
         if (c >= 2) A.emit_cap = class_cap(g, A.emit_all, c);
         st = launch_one<MODE>(g, A, c, (unsigned)pass1, slots1, cs);
