@@ -220,15 +220,16 @@ static void res_to_dag(const DagRes &r, pvt_dag *g)
 
 // The device's pool keeps freed scratch for the next call.  What a dag's
 // optional buffers held beyond POOL_KEEP (most dags stay below) goes back to
-// the device, where other allocators of the process find it.
-constexpr size_t POOL_KEEP = (size_t)2 << 30;
+// the device, where other allocators of the process find it.  (The pool lets
+// go of whole chunks: it may keep up to POOL_CHUNK more than it is told to.)
+constexpr size_t POOL_KEEP = (size_t)2 << 30, POOL_CHUNK = (size_t)64 << 20;
 static void give_back(int device)
 {
     cudaMemPool_t pool;
     uint64_t used = 0;
     if (cudaDeviceGetMemPool(&pool, device) == cudaSuccess &&
         cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
-        cudaMemPoolTrimTo(pool, used + POOL_KEEP);
+        cudaMemPoolTrimTo(pool, used + POOL_KEEP - POOL_CHUNK);
 }
 
 static void dag_release(pvt_dag *g)
