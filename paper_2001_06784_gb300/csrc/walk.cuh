@@ -195,7 +195,7 @@ constexpr uint32_t FRAME_NONE = 0u, FRAME_WIDE = 1u, FRAME_COMPACT = 2u;
 // Block-level (h, p) leaf histogram in shared memory for h < HIST_H, p < HIST_P
 // (where almost every leaf falls); other leaves go straight to the global one.
 constexpr int HIST_H = 32, HIST_P = 48;
-constexpr unsigned HIST_DRAIN = 1u << 18;
+constexpr unsigned HIST_DRAIN = 1u << 16;
 
 // Walk statistics, the same on every lane of the warp.
 struct WalkCounters {

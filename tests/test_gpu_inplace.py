@@ -9,7 +9,7 @@ from tests.test_gpu_parity import gpu_dag
 
 pytestmark = pytest.mark.gpu
 
-DRAIN = 1 << 18  # leaves of a warp (HIST_DRAIN)
+DRAIN = 1 << 16  # leaves of a warp (HIST_DRAIN)
 
 
 def test_walks_past_a_drain():
