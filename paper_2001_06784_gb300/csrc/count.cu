@@ -473,8 +473,8 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
     for (int c = 1; c < NCLASS; ++c) used += g->wcnt[c] > 0;
     const bool serial = g->serial || g->policy.serial || used <= 1;
     // The wide classes of a two-phase count follow one another, widest first,
-    // where each fills the GPU and shares the subtrees of its last roots: side by
-    // side they would only take shared memory from one another (counts of two
+    // where each fills (half of) the GPU and shares the subtrees of its last roots:
+    // side by side they would only take shared memory from one another (counts of two
     // graphs with 2,500 to 37,000 roots in each of three classes: 4.2 ms in one
     // stream, 5.0 on a stream each; 7.4 on either).  Else they overlap: a class
     // of few roots, or of roots that one warp walks to the end, leaves the GPU

@@ -99,7 +99,7 @@ struct pvt_dag {
     // with less of them more is walked in place (pvt_dag_set_scratch_limit).
     size_t scratch = 0, scratch_limit = ~(size_t)0;
     bool sizing = false;           // the launch functions only size their buffers
-    bool fills[pvt::NCLASS] = {};  // (from sizing) the class's launch fills the GPU and shares its roots' subtrees
+    bool fills[pvt::NCLASS] = {};  // (from sizing) the class's launch fills at least half of the GPU and shares its roots' subtrees
     cudaEvent_t ev_t0[pvt::NPHASE] = {}, ev_t1[pvt::NPHASE] = {};
     bool phase_used[pvt::NPHASE] = {};
     pvt::DevBuf<uint32_t> gstack[pvt::NCLASS];  // DFS stacks of the wide classes (global memory)

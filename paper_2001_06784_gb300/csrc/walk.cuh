@@ -1492,7 +1492,7 @@ pvt_status launch_class(pvt_dag *g, const CountArgs &base, int cls, cudaStream_t
         if ((st = grow(g, g->etab[cls], (size_t)grid * WPB * D * D, s)) != PVT_OK) return st;
         A.eidtab = g->etab[cls].p;
     }
-    g->fills[cls] = split && grid == (unsigned)(g->num_sms * per_sm);
+    g->fills[cls] = split && 2 * grid >= (unsigned)(g->num_sms * per_sm);
     if (g->sizing) return PVT_OK;
     if (split) {
         PVT_CK(cudaMemsetAsync(g->qready[cls].p, 0, (size_t)SPLIT_QCAP * 2 * sizeof(uint32_t), s));

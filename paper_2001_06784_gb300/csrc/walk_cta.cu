@@ -30,7 +30,7 @@ static pvt_status launch_cta_nw(pvt_dag *g, CountArgs A, int cls, int dmax, cuda
         return PVT_ECUDA;
     }
     const unsigned blocks = std::max(1u, std::min<unsigned>((unsigned)(g->num_sms * per_sm), A.nroots));
-    g->fills[cls] = blocks == (unsigned)(g->num_sms * per_sm);
+    g->fills[cls] = 2 * blocks >= (unsigned)(g->num_sms * per_sm);
     pvt_status st =
         grow(g, g->gstack[cls], (size_t)blocks * warps * Lay::stack_words(dmax) + (size_t)blocks * Lay::gather_words(dmax), s);
     if (st != PVT_OK || g->sizing) return st;
