@@ -498,14 +498,30 @@ __global__ void __launch_bounds__(1024, 1) k_peel(int64_t n, const int64_t *__re
 constexpr unsigned CORE_CLAMP = MAX_ALPHA + 1;  // estimates are clamped here: a larger core is refused anyway
 constexpr unsigned CORE_ROUNDS_MAX = 192;       // then the level-wise peel (an entry's tag could hold 1023)
 constexpr unsigned CORE_FULL = 3;               // the last round that visits every vertex
-// A round whose largest changed estimate is at most CORE_BAIL_CORE, the first
-// one or one from CORE_BAIL_ROUND on, has only low levels left (meshes, road
-// networks, paths): the level-wise peel needs few levels there and follows a
-// chain in one cascade.  So does a round of at most CORE_THIN vertices from
-// round CORE_THIN_ROUND on (long chains at a higher level; the power-law
-// graphs measured end within 62 rounds, the 128M-edge one of degeneracy 733
-// within 86).
-constexpr unsigned CORE_BAIL_CORE = 6, CORE_BAIL_ROUND = 24, CORE_THIN = 64, CORE_THIN_ROUND = 96;
+// Graphs that need many rounds for few levels keep the level-wise peel, which
+// follows a chain of removals in one cascade.  They show early:
+//   * by the largest estimate that still changes.  At most CORE_BAIL_CORE in the
+//     first round: meshes, road networks, paths.  At most CORE_LOW after the
+//     full rounds (CORE_LOW_SMALL below CORE_LOW_N vertices, where a level of
+//     the peel costs less): trees and sparse random graphs.
+//   * by the vertices that a round still visits: above a tenth of all at round
+//     8, or a hundredth at round 16 (24 on a small graph).  The power-law graphs
+//     measured visit at most 3.4 % and 0.7 %, random graphs above the low cores
+//     0.9 %; chains that cross the graph, as in geometric graphs and bands, 10 %
+//     and more, 1.3 % and more.
+// Orientations, level-wise peel alone -> with these rules: a mesh of 1M vertices
+// 6.69 -> 6.79 ms, a random tree of 1M 1.10 -> 1.30, random graphs of 1M of
+// average degree 5.1, 8.3 and 9.9 1.62 -> 1.86, 1.81 -> 1.54 and 1.89 -> 1.66,
+// geometric graphs of 1M of average degree 8 and 20 2.15 -> 1.34 and 3.26 ->
+// 4.01, a band of 6,000 3.61 -> 3.86.  (Given up at round 24, 96 or 192 only, and
+// oriented on meaningless keys first, the tree took 1.86, the first random
+// graph 2.48 and the second geometric one 6.08 ms.)
+// A round of at most CORE_THIN vertices from round CORE_THIN_ROUND on is left to
+// the peel too (one long chain beside a graph that is done; the power-law
+// graphs measured end within 86 rounds).
+constexpr unsigned CORE_BAIL_CORE = 6, CORE_LOW = 8, CORE_LOW_SMALL = 10;
+constexpr int64_t CORE_LOW_N = 1 << 18, CORE_RULES_N = 1 << 15;
+constexpr unsigned CORE_THIN = 64, CORE_THIN_ROUND = 96;
 constexpr int CORE_THREADS = 1024;
 // Graphs of at most this many vertices and row entries stay in one block (300
 // vertices: 87 -> 75 us; 2,000 vertices with 41,000 entries: 151 us in one
@@ -725,8 +741,16 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_cores(int64_t n, const int6
         if (r > 1) {
             const unsigned most = *(volatile unsigned *)&mosts[(r - 1) % 3];
             if (most == 0) break;  // nothing changed
-            if (((r == 2 || r >= CORE_BAIL_ROUND) && most <= CORE_BAIL_CORE) ||
-                (r >= CORE_THIN_ROUND && n_small + n_big <= CORE_THIN) || r > CORE_ROUNDS_MAX) {
+            const int64_t visits = (int64_t)n_small + n_big;
+            bool bail = (r == 2 && most <= CORE_BAIL_CORE) || (r >= CORE_THIN_ROUND && visits <= CORE_THIN) ||
+                        r > CORE_ROUNDS_MAX;
+            if (!SMALL) {
+                if (n >= CORE_RULES_N)
+                    bail = bail || (r == CORE_FULL + 1 && most <= (n < CORE_LOW_N ? CORE_LOW_SMALL : CORE_LOW)) ||
+                           (r == 8 && visits * 10 > n) || (r == 16 && visits * 100 > n);
+                bail = bail || (r == 24 && visits * 100 > n);
+            }
+            if (bail) {
                 if (tid == 0) st->bail = 1;
                 return;
             }
@@ -1168,6 +1192,7 @@ __global__ void __launch_bounds__(256) k_outdeg(int64_t n, const int64_t *__rest
                                                 const uint32_t *__restrict__ col, const uint32_t *__restrict__ rnd,
                                                 uint32_t *odeg, CoreState *st)
 {
+    if (st->bail) return;  // the keys mean nothing yet
     __shared__ unsigned sh[CORE_CLAMP + 1];
     for (int i = threadIdx.x; i <= (int)CORE_CLAMP; i += blockDim.x) sh[i] = 0;
     __syncthreads();
@@ -1200,8 +1225,9 @@ __global__ void __launch_bounds__(256) k_outdeg(int64_t n, const int64_t *__rest
 // CSR differs, nothing is written.
 __global__ void k_fill(int64_t n, const int64_t *__restrict__ rp, const uint32_t *__restrict__ col,
                        const uint32_t *__restrict__ rnd, const int64_t *__restrict__ orow,
-                       uint32_t *ocol, int64_t m, unsigned *err)
+                       uint32_t *ocol, int64_t m, const CoreState *st, unsigned *err)
 {
+    if (st->bail) return;
     if (orow[n] != m) {
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(err, DERR_NOTSIMPLE);
         return;
@@ -1244,6 +1270,7 @@ __global__ void __launch_bounds__(1024) k_deg_slots(CoreState *st)
 {
     __shared__ unsigned s_warp[32], s_base;
     __shared__ unsigned s_cls[NCLASS + 1];
+    if (st->bail) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (threadIdx.x <= NCLASS) s_cls[threadIdx.x] = 0;
     if (threadIdx.x == 0) s_base = 0;
@@ -1283,9 +1310,10 @@ __global__ void __launch_bounds__(1024) k_deg_slots(CoreState *st)
 // Scatter roots so that out-degrees descend within the array (slot[d] holds
 // the next free position for out-degree d); lanes with equal out-degrees
 // share one atomic.
-__global__ void k_deg_scatter(int64_t n, const uint32_t *__restrict__ odeg, unsigned *slot,
-                              uint32_t *roots)
+__global__ void k_deg_scatter(int64_t n, const uint32_t *__restrict__ odeg, CoreState *st, uint32_t *roots)
 {
+    if (st->bail) return;
+    unsigned *slot = st->deg_cnt;
     const int lane = threadIdx.x & 31;
     for (int64_t base = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; base < n;
          base += (int64_t)gridDim.x * blockDim.x) {
@@ -1599,9 +1627,9 @@ pvt_status orient_build(pvt_dag *g, uint32_t flags, cudaStream_t s)
         k_outdeg<<<og, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, odeg, cst);
         PVT_CK(cudaGetLastError());
         if ((st = exclusive_scan_u32_i64(odeg, g->orow, n, s)) != PVT_OK) return st;
-        k_fill<<<og, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, g->orow, g->ocol, g->m, g->d_err);
+        k_fill<<<og, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, g->orow, g->ocol, g->m, cst, g->d_err);
         k_deg_slots<<<1, 1024, 0, s>>>(cst);
-        k_deg_scatter<<<og, 256, 0, s>>>(n, odeg, cst->deg_cnt, g->roots);
+        k_deg_scatter<<<og, 256, 0, s>>>(n, odeg, cst, g->roots);
         PVT_CK(cudaGetLastError());
         phase_end(g, 1, s);
         g->stats.launches += n <= SCAN_ONE_BLOCK ? 5 : 7;
