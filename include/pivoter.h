@@ -56,7 +56,8 @@ typedef struct pvt_dag pvt_dag;
 
 /*
  * Orient the graph along a degeneracy order (Lemma degen, Sec. 3.2; Alg. 1
- * step 1): k-core peeling on the device, then the out-neighbourhoods N+(v)
+ * step 1): core numbers and a degeneracy order on the device (by rounds over
+ * all levels, or by peeling level by level), then the out-neighbourhoods N+(v)
  * as a CSR over the DAG, every out-degree at most the degeneracy alpha.
  * alpha_out and pvt_dag_info report alpha = the degeneracy (the top core
  * level), which bounds every out-degree and does not depend on how removals
@@ -84,7 +85,7 @@ pvt_status pvt_dag_info(const pvt_dag *dag, int64_t *n, int64_t *m, int32_t *alp
                         int32_t *min_words);
 
 /*
- * Core numbers found by the peel (Sec. 3.2: the degeneracy order removes a
+ * Core numbers found by the orientation (Sec. 3.2: the degeneracy order removes a
  * vertex of smallest residual degree; the core number of v is the largest k
  * such that v lies in a subgraph of minimum degree k).  Unlike the removal
  * order, core numbers do not depend on how ties are broken.
@@ -193,7 +194,8 @@ pvt_status pvt_local_distribution(const uint64_t *table, int64_t rows, int32_t K
  * internal node, the AND + population-count word pairs of pivot selection
  * over rows restricted to the label's own members -- a property of the tree,
  * whichever row width a kernel walks it in.  ms[] holds device
- * time per phase when profiling is on (else zeros): [0] peel, [1] orient
+ * time per phase when profiling is on (else zeros): [0] core
+ * numbers and order (the last form taken), [1] orient
  * (DAG CSR and root classes), [2..7] the walk kernels of out-degree classes
  * <=32, <=64, <=128, <=256, <=512, <=1024, [8] combine/finish, [9] the
  * frame walk (policy.frames).  Phases of different classes overlap in time.
@@ -204,13 +206,15 @@ typedef struct pvt_stats {
     uint64_t pivot_words;
     uint64_t launches;      /* kernels launched by the call */
     uint64_t roots[7];      /* roots per out-degree class (0, <=32, ..., <=1024) */
-    uint64_t class_words[7];/* pivot_words of the class kernels (walk of labels > 32
-                               members only when frames are on) */
-    uint64_t frame_words;   /* pivot_words of the frame walk (policy.frames) */
+    uint64_t class_words[7];/* pivot_words by class: of the class kernels (labels > 32
+                               members only when frames are on) and, for the
+                               <= 32 class, of its roots wherever they are walked */
+    uint64_t frame_words;   /* pivot_words of the frame walk (policy.frames), those of
+                               <= 32 class roots left out */
     uint64_t frames;        /* frames the wide walks emitted (above the buffer:
                                walked in place) */
     float ms[10];
-    uint32_t peel_rounds;   /* orient: grid-wide barriers of the peel */
+    uint32_t peel_rounds;   /* orient: grid-wide barriers of the core rounds and the peel */
     uint32_t peel_levels;   /* orient: distinct core levels visited */
 } pvt_stats;
 
@@ -280,9 +284,9 @@ pvt_status pvt_measure_popc_rate(double *pairs_per_s, void *stream);
  *               its small labels itself.  Persistent form only.
  *   graph       1: pvt_count_global records its launch sequence as a CUDA
  *               graph at the first call with a given (kmax, W, C) and
- *               replays it at later calls with the same three (the dag's
- *               buffers are fixed after orientation); 0 (default): launch
- *               directly.  Replayed calls report no phase times.
+ *               replays it at later calls with the same three, unless a
+ *               buffer it uses has moved or changed its size since (then it
+ *               is recorded anew); 0 (default): launch directly.  Replayed calls report no phase times.
  *   wait_limit_us  0 (default): the bounded device-side waits of the walk
  *               (an idle warp waiting for a donated frame, a donor waiting
  *               for a free ring slot) give up after 120 s without progress

@@ -8,12 +8,12 @@
 // walk that root's SCT (Alg. 1) over the one shared copy.  The warps share
 // the root's subtrees through a small queue in shared memory: a warp whose
 // subtree is done takes the next pending one, and busy warps hand over
-// their oldest pending subtree (the largest) while a warp of the block has
-// none.  Labels of at most 32 members leave the wide walk: they are
-// relabelled to one-word rows (relabel_rows in walk.cuh) into
-// a free lane of the warp's lane batch and walked one subtree per lane
-// (lanes.cuh), so the many small subtrees below a dense root never leave the
-// SM.  A warp runs its lanes whenever it has no wide work or no free lane.
+// their oldest pending subtrees (the largest), two for each warp of the block
+// that has none.  Labels of at most 32 members leave the wide walk, relabelled
+// to one-word rows (relabel_rows in walk.cuh): as frames of the frame walk
+// while the launch's share of its buffer has room, else into a free lane of a
+// warp's lane batch, walked one subtree per lane (lanes.cuh) without leaving
+// the SM.  A warp runs its lanes whenever it has no wide work or no free lane.
 // The tree, its statistics and the (h, p) histogram are those of walk.cuh.
 #pragma once
 

@@ -27,7 +27,7 @@
 // table takes 2 to 8 KB of shared memory per warp).  Start -> now, whole
 // calls: per-vertex, 500k vertices, 8.25M edges, k <= 40: 23.6 -> 3.9 ms;
 // 90k vertices, k <= 5: 4.3 -> 0.85 ms; per-edge, 2M edges, k <= 12: 5.3 ->
-// 2.4 ms; 56k edges, k <= 22: 0.56 -> 0.39 ms.
+// 2.4 ms; 56k edges, k <= 22: 0.56 -> 0.23 ms.
 #pragma once
 
 #include "walk.cuh"

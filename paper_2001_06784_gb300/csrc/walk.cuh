@@ -836,7 +836,7 @@ __device__ __forceinline__ void gather_rows(Work &Wk, const CountArgs &A, int la
     // With the narrower rows of launch_wide, the rolled word loops and the
     // labels emitted where they are formed, the wide walks of the 10.8M-edge
     // graph went from 0.62 / 1.10 / 2.28 ms (33..64, 65..128, 129..256) to
-    // 0.50 / 0.86 / 1.08 ms.
+    // 0.50 / 0.83 / 1.78 ms.
     constexpr int FSH = 32 - Work::FILTER_LOG;
     for (int t = lane; t < (1 << Work::FILTER_LOG) / 32; t += 32) Wk.filter[t] = 0;
     __syncwarp();
@@ -1309,7 +1309,8 @@ __global__ void __launch_bounds__(32 * warps_per_block<NW>())
         // Every warp waits to the end: a class's last roots may hold most of its
         // tree.  (Half of the blocks left once the roots were out, so that the
         // next class could start: 7.4 -> 7.0 ms of the 10.8M-edge graph's count,
-        // but 2.9 -> 5.2 s where dense groups of 90 to 120 vertices were the work.)
+        // but 346 -> 481 ms where four dense groups of 90 to 120 vertices were
+        // nearly all of the work.)
         for (;;) {
             unsigned v = 0;
             int kind = lane == 0 ? queue_take(A, A.nroots, v) : 0;
