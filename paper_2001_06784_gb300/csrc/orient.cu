@@ -1190,9 +1190,9 @@ __device__ __forceinline__ bool key_less(uint32_t ra, uint32_t a, uint32_t rb, u
 // small values).
 __global__ void __launch_bounds__(256) k_outdeg(int64_t n, const int64_t *__restrict__ rp,
                                                 const uint32_t *__restrict__ col, const uint32_t *__restrict__ rnd,
-                                                uint32_t *odeg, CoreState *st)
+                                                uint32_t *odeg, CoreState *st, const unsigned *bail)
 {
-    if (st->bail) return;  // the keys mean nothing yet
+    if (bail && *bail) return;  // the keys mean nothing yet
     __shared__ unsigned sh[CORE_CLAMP + 1];
     for (int i = threadIdx.x; i <= (int)CORE_CLAMP; i += blockDim.x) sh[i] = 0;
     __syncthreads();
@@ -1225,13 +1225,10 @@ __global__ void __launch_bounds__(256) k_outdeg(int64_t n, const int64_t *__rest
 // CSR differs, nothing is written.
 __global__ void k_fill(int64_t n, const int64_t *__restrict__ rp, const uint32_t *__restrict__ col,
                        const uint32_t *__restrict__ rnd, const int64_t *__restrict__ orow,
-                       uint32_t *ocol, int64_t m, const CoreState *st, unsigned *err)
+                       uint32_t *ocol, int64_t m, const unsigned *bail, unsigned *err)
 {
-    if (st->bail) return;
-    if (orow[n] != m) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(err, DERR_NOTSIMPLE);
-        return;
-    }
+    if (bail && *bail) return;
+    const bool fits = orow[n] == m;  // (nothing waits for it before the first write)
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1247,10 +1244,11 @@ __global__ void k_fill(int64_t n, const int64_t *__restrict__ rp, const uint32_t
                 keep = key_less(rv, (uint32_t)v, rnd[u], u);
             }
             unsigned b = __ballot_sync(FULL, keep);
-            if (keep) ocol[out + __popc(b & ((1u << lane) - 1u))] = u;
+            if (keep && fits) ocol[out + __popc(b & ((1u << lane) - 1u))] = u;
             out += __popc(b);
         }
     }
+    if (!fits && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(err, DERR_NOTSIMPLE);
 }
 
 // Class of an out-degree: 0 for d = 0, else 1 + ceil(log2(ceil(d / 32))).
@@ -1266,11 +1264,11 @@ __host__ __device__ inline int degree_class(uint32_t d)
 // Counting sort of the roots by descending out-degree, in one block: each
 // out-degree's count becomes its first position (larger ones first), and the
 // classes' sizes are summed.
-__global__ void __launch_bounds__(1024) k_deg_slots(CoreState *st)
+__global__ void __launch_bounds__(1024) k_deg_slots(CoreState *st, const unsigned *bail)
 {
     __shared__ unsigned s_warp[32], s_base;
     __shared__ unsigned s_cls[NCLASS + 1];
-    if (st->bail) return;
+    if (bail && *bail) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (threadIdx.x <= NCLASS) s_cls[threadIdx.x] = 0;
     if (threadIdx.x == 0) s_base = 0;
@@ -1310,10 +1308,10 @@ __global__ void __launch_bounds__(1024) k_deg_slots(CoreState *st)
 // Scatter roots so that out-degrees descend within the array (slot[d] holds
 // the next free position for out-degree d); lanes with equal out-degrees
 // share one atomic.
-__global__ void k_deg_scatter(int64_t n, const uint32_t *__restrict__ odeg, CoreState *st, uint32_t *roots)
+__global__ void k_deg_scatter(int64_t n, const uint32_t *__restrict__ odeg, unsigned *slot,
+                              uint32_t *roots, const unsigned *bail)
 {
-    if (st->bail) return;
-    unsigned *slot = st->deg_cnt;
+    if (bail && *bail) return;
     const int lane = threadIdx.x & 31;
     for (int64_t base = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; base < n;
          base += (int64_t)gridDim.x * blockDim.x) {
@@ -1585,6 +1583,9 @@ pvt_status orient_build(pvt_dag *g, uint32_t flags, cudaStream_t s)
     CoreState *hst = reinterpret_cast<CoreState *>(reinterpret_cast<char *>(g->h_stats) + PIN_ORIENT);
     // small graphs: no more blocks than warps have vertices
     const int og = (int)std::max<int64_t>(1, std::min<int64_t>(grid, (n + 7) / 8));
+    // where the core rounds may give up, the kernels after them look whether they
+    // did; on a small graph they cost less than the look (1 us each)
+    const unsigned *bail = n >= CORE_RULES_N ? &cst->bail : nullptr;
     pvt_status st = PVT_OK;
     for (int form = 0;; ++form) {
         // core numbers and removal order: by rounds, else (once, if those
@@ -1624,12 +1625,12 @@ pvt_status orient_build(pvt_dag *g, uint32_t flags, cudaStream_t s)
         phase_end(g, 0, s);
         phase_begin(g, 1, s);
         // orientation; roots by descending out-degree, grouped into classes
-        k_outdeg<<<og, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, odeg, cst);
+        k_outdeg<<<og, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, odeg, cst, bail);
         PVT_CK(cudaGetLastError());
         if ((st = exclusive_scan_u32_i64(odeg, g->orow, n, s)) != PVT_OK) return st;
-        k_fill<<<og, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, g->orow, g->ocol, g->m, cst, g->d_err);
-        k_deg_slots<<<1, 1024, 0, s>>>(cst);
-        k_deg_scatter<<<og, 256, 0, s>>>(n, odeg, cst, g->roots);
+        k_fill<<<og, 256, 0, s>>>(n, g->row_ptr, g->col, g->rnd, g->orow, g->ocol, g->m, bail, g->d_err);
+        k_deg_slots<<<1, 1024, 0, s>>>(cst, bail);
+        k_deg_scatter<<<og, 256, 0, s>>>(n, odeg, cst->deg_cnt, g->roots, bail);
         PVT_CK(cudaGetLastError());
         phase_end(g, 1, s);
         g->stats.launches += n <= SCAN_ONE_BLOCK ? 5 : 7;
