@@ -23,8 +23,10 @@
 // rows, and a second launch walks each in parts that deal out the hold
 // children along the root's pivot chain, so one such root does not occupy one
 // warp after all others have finished.
-// What bounds it: issue slots and load latency at 16 to 32 warps per SM (the
-// table takes 2 to 8 KB of shared memory per warp).  Start -> now, whole
+// What bounds it: load latency in the gathers (the one-word one issues on 61 %
+// of the slots), dependent instructions and instruction fetch in the parts of
+// dense roots, at 11 to 32 warps per SM (the table takes 2 to 8 KB of shared
+// memory per warp).  Start -> now, whole
 // calls: per-vertex, 500k vertices, 8.25M edges, k <= 40: 23.6 -> 3.9 ms;
 // 90k vertices, k <= 5: 4.3 -> 0.85 ms; per-edge, 2M edges, k <= 12: 5.3 ->
 // 2.4 ms; 56k edges, k <= 22: 0.56 -> 0.23 ms.

@@ -499,29 +499,32 @@ constexpr unsigned CORE_CLAMP = MAX_ALPHA + 1;  // estimates are clamped here: a
 constexpr unsigned CORE_ROUNDS_MAX = 192;       // then the level-wise peel (an entry's tag could hold 1023)
 constexpr unsigned CORE_FULL = 3;               // the last round that visits every vertex
 // Graphs that need many rounds for few levels keep the level-wise peel, which
-// follows a chain of removals in one cascade.  They show early:
-//   * by the largest estimate that still changes.  At most CORE_BAIL_CORE in the
-//     first round: meshes, road networks, paths.  At most CORE_LOW after the
-//     full rounds (CORE_LOW_SMALL below CORE_LOW_N vertices, where a level of
-//     the peel costs less): trees and sparse random graphs.
-//   * by the vertices that a round still visits: above a tenth of all at round
-//     8, or a hundredth at round 16 (24 on a small graph).  The power-law graphs
-//     measured visit at most 3.4 % and 0.7 %, random graphs above the low cores
-//     0.9 %; chains that cross the graph, as in geometric graphs and bands, 10 %
-//     and more, 1.3 % and more.
-// Orientations, level-wise peel alone -> with these rules: a mesh of 1M vertices
-// 6.69 -> 6.79 ms, a random tree of 1M 1.10 -> 1.30, random graphs of 1M of
-// average degree 5.1, 8.3 and 9.9 1.62 -> 1.86, 1.81 -> 1.54 and 1.89 -> 1.66,
-// geometric graphs of 1M of average degree 8 and 20 2.15 -> 1.34 and 3.26 ->
-// 4.01, a band of 6,000 3.61 -> 3.86.  (Given up at round 24, 96 or 192 only, and
-// oriented on meaningless keys first, the tree took 1.86, the first random
-// graph 2.48 and the second geometric one 6.08 ms.)
+// follows a chain of removals in one cascade.  They are told by what a round
+// still does:
+//   * the first changes no estimate above CORE_BAIL_CORE: meshes, road networks;
+//   * at round 20 (CORE_RULES_N vertices and more) 1/64 of all vertices are
+//     visited, or, on a graph below CORE_LOW_N, nothing above CORE_BAIL_CORE
+//     changes; at round 32 (CORE_CHAIN_N and more) 1/40 of all are visited.
+// Of 311 random and power-law graphs of 1,000 to 400,000 vertices, average degree
+// 4 to 60, all but 41 are done by round 32, most of the random ones after a last
+// round or two that visit up to half of the vertices; an earlier look took those
+// for chains (36,000 vertices, degree 26: 386 -> 692 us).  None that either look
+// would still meet has as many vertices left; geometric graphs and bands have 2
+// to 9 %.  Orientations, level-wise peel alone -> with these rules:
+// a mesh of 1M vertices 6.69 -> 6.74 ms, a random tree 1.10 -> 0.99, random graphs
+// of average degree 5.1, 8.3 and 9.9 1.62 -> 1.51, 1.81 -> 1.52 and 1.89 -> 1.68,
+// one of 100,000 vertices and degree 5.1 0.49 -> 0.83, geometric graphs of 1M of
+// degree 8 and 20 2.15 -> 1.35 and 3.26 -> 4.48, a band of 6,000 vertices 3.61 ->
+// 3.95.  (Given up at round 24 where nothing above CORE_BAIL_CORE changed, else at
+// 96 or 192, and oriented on meaningless keys first, the tree took 1.86, the
+// random graphs 2.48, 2.72 and 0.93, the geometric ones 3.25 and 6.08, the band
+// 5.91 ms.)
 // A round of at most CORE_THIN vertices from round CORE_THIN_ROUND on is left to
 // the peel too (one long chain beside a graph that is done; the power-law
-// graphs measured end within 86 rounds).
-constexpr unsigned CORE_BAIL_CORE = 6, CORE_LOW = 8, CORE_LOW_SMALL = 10;
-constexpr int64_t CORE_LOW_N = 1 << 18, CORE_RULES_N = 1 << 15;
-constexpr unsigned CORE_THIN = 64, CORE_THIN_ROUND = 96;
+// graphs measured end within 86 rounds, a random one at a core threshold in 102).
+constexpr unsigned CORE_BAIL_CORE = 6;
+constexpr int64_t CORE_CHAIN_N = 1 << 12, CORE_RULES_N = 1 << 15, CORE_LOW_N = 1 << 18;
+constexpr unsigned CORE_THIN = 64, CORE_THIN_ROUND = 112;
 constexpr int CORE_THREADS = 1024;
 // Graphs of at most this many vertices and row entries stay in one block (300
 // vertices: 87 -> 75 us; 2,000 vertices with 41,000 entries: 151 us in one
@@ -744,12 +747,9 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_cores(int64_t n, const int6
             const int64_t visits = (int64_t)n_small + n_big;
             bool bail = (r == 2 && most <= CORE_BAIL_CORE) || (r >= CORE_THIN_ROUND && visits <= CORE_THIN) ||
                         r > CORE_ROUNDS_MAX;
-            if (!SMALL) {
-                if (n >= CORE_RULES_N)
-                    bail = bail || (r == CORE_FULL + 1 && most <= (n < CORE_LOW_N ? CORE_LOW_SMALL : CORE_LOW)) ||
-                           (r == 8 && visits * 10 > n) || (r == 16 && visits * 100 > n);
-                bail = bail || (r == 24 && visits * 100 > n);
-            }
+            if (!SMALL && r == 20 && n >= CORE_RULES_N)
+                bail = bail || visits * 64 > n || (n < CORE_LOW_N && most <= CORE_BAIL_CORE);
+            if (!SMALL && r == 32 && n >= CORE_CHAIN_N) bail = bail || visits * 40 > n;
             if (bail) {
                 if (tid == 0) st->bail = 1;
                 return;
@@ -1585,7 +1585,7 @@ pvt_status orient_build(pvt_dag *g, uint32_t flags, cudaStream_t s)
     const int og = (int)std::max<int64_t>(1, std::min<int64_t>(grid, (n + 7) / 8));
     // where the core rounds may give up, the kernels after them look whether they
     // did; on a small graph they cost less than the look (1 us each)
-    const unsigned *bail = n >= CORE_RULES_N ? &cst->bail : nullptr;
+    const unsigned *bail = n >= CORE_CHAIN_N ? &cst->bail : nullptr;
     pvt_status st = PVT_OK;
     for (int form = 0;; ++form) {
         // core numbers and removal order: by rounds, else (once, if those

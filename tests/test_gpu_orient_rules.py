@@ -27,14 +27,15 @@ def grid3(a):
 
 
 GRAPHS = {
-    # after the full rounds: below and above the size at which a random graph of
-    # low cores stays with the rounds, and the core just above them
+    # random graphs of low cores around the sizes from which round 20 is looked at,
+    # and up to which a low core is enough to leave the rounds there
     "sparse 40k": lambda: graphgen.generate(40_000, er_avg_deg=9.0, seed=1),
     "sparse 300k": lambda: graphgen.generate(300_000, er_avg_deg=5.2, seed=2),
     "less sparse 300k": lambda: graphgen.generate(300_000, er_avg_deg=9.9, seed=3),
     "sparse 32k": lambda: graphgen.generate(32_767, er_avg_deg=5.2, seed=4),
-    # many vertices at rounds 8, 16 and 24: bands of both sizes, a lattice
+    # many vertices at rounds 20 and 32: bands of three sizes; a lattice
     "band 40k": lambda: band(40_000, 9),
+    "band 6k": lambda: band(6_000, 12),
     "band 2k": lambda: band(2_000, 20),
     "bands and a clique": lambda: disjoint(*[band(400, 8) for _ in range(100)], band(40, 39)),
     "lattice": lambda: grid3(33),
