@@ -460,8 +460,8 @@ void pvt_server_destroy(pvt_server *sv);
 
 /* Release a pvt_dag and all its device memory (NULL is ignored).  The memory
  * goes to the device's stream-ordered pool, which the library keeps for later
- * calls (process-wide); where the dag's optional buffers held more than 2 GiB,
- * the pool is cut to 2 GiB beyond what is in use. */
+ * calls (process-wide); where the dag's optional buffers held more than 6 GiB,
+ * the pool is cut to 6 GiB beyond what is in use. */
 void pvt_dag_free(pvt_dag *dag);
 
 /* Message for the last failed call on this thread ("" if none). */

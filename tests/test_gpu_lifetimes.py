@@ -307,7 +307,7 @@ def test_an_asymmetric_csr_is_refused_before_its_out_lists_are_written(pvt, extr
 
 
 def test_large_frames_go_back_to_the_device(pvt):
-    """A dag whose frame buffer passed 2 GiB leaves at most that, beyond what is
+    """A dag whose frame buffer passed 6 GiB leaves at most that, beyond what is
     in use, in the device's pool."""
     import torch
     cu = ctypes.CDLL("libcuda.so.1")
@@ -320,13 +320,13 @@ def test_large_frames_go_back_to_the_device(pvt):
         assert cu.cuMemPoolGetAttribute(pool, attr, ctypes.byref(x)) == 0
         return x.value
 
-    rp, col = graphs.clique_minus_random(1000, 9, 57)
+    rp, col = disjoint(*[graphs.clique_minus_random(1000, 9, 57 + i) for i in range(4)])
     dag = gpu_dag(pvt, rp, col)
     before = held(USED_MEM_CURRENT)
     dag.count_global(kmax=4)
-    assert held(USED_MEM_CURRENT) - before > 2 << 30
+    assert held(USED_MEM_CURRENT) - before > 6 << 30
     dag.free()
-    assert held(RESERVED_MEM_CURRENT) - held(USED_MEM_CURRENT) <= 2 << 30
+    assert held(RESERVED_MEM_CURRENT) - held(USED_MEM_CURRENT) <= 6 << 30
 
 
 @pytest.mark.parametrize("streams", [1, 2])
