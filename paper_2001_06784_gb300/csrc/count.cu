@@ -443,17 +443,8 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
     bool gather1 = two_phase && g->policy.lanes && g->wcnt[1] >= GATHER1_MIN;
     // (a sequence being recorded finds every buffer as its direct call left it)
     if ((st = size_all<MODE>(g, A0, frames || gather1, s)) != PVT_OK) return st;
-    if (frames) {
-        unsigned cap = g->capturing ? (unsigned)(g->cframes.n / FRAME_WORDS) : frame_cap(g);
-        if (!g->capturing) st = grow_least(g, g->cframes, cap, FRAME_CAP_MIN, FRAME_WORDS, s);
-        if (st != PVT_OK && st != PVT_ENOMEM) return st;
-        cap = cap / EMIT_RESERVE * EMIT_RESERVE;
-        frames = st == PVT_OK && cap > 0;
-        A.emit = frames ? g->cframes.p : nullptr;
-        A.emit_count = reinterpret_cast<unsigned long long *>(g->d_q + 8);  // words 8..9
-        A.emit_cap = A.emit_all = frames ? cap : 0;
-    }
-    // the gather's pass: as many roots as its frames find room for
+    // the gather's pass: as many roots as its frames find room for, in at most
+    // half of what the dag's limit leaves
     int64_t pass1 = std::min(g->wcnt[1], GATHER1_MAX);
     unsigned slots1 = 0;
     for (; gather1; pass1 /= 4) {
@@ -462,7 +453,7 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
             slots1 = gather1_slots(g, (unsigned)pass1);
             const size_t words = (size_t)slots1 * FRAME_WORDS;
             if (words <= g->cframes1.n) break;
-            if (g->capturing || words > optional_words(g, g->cframes1)) continue;
+            if (g->capturing || words > optional_words(g, g->cframes1) / 2) continue;
             st = grow_own(g, g->cframes1, words, s);
             if (st == PVT_OK) break;
             if (st != PVT_ENOMEM) return st;
@@ -472,6 +463,17 @@ static pvt_status launch_all(pvt_dag *g, const CountArgs &A0, cudaStream_t s)
     if (!gather1) slots1 = 0;
     A.emit1 = gather1 ? g->cframes1.p : nullptr;
     A.emit1_count = g->d_q + 10;
+    if (frames) {
+        unsigned cap = g->capturing ? (unsigned)(g->cframes.n / FRAME_WORDS) : frame_cap(g);
+        if (!g->capturing) st = grow_least(g, g->cframes, cap, FRAME_CAP_MIN, FRAME_WORDS, s);
+        if (st != PVT_OK && st != PVT_ENOMEM) return st;
+        cap = cap / EMIT_RESERVE * EMIT_RESERVE;
+        frames = st == PVT_OK && cap > 0;
+        A.emit = frames ? g->cframes.p : nullptr;
+        A.emit_count = reinterpret_cast<unsigned long long *>(g->d_q + 8);  // words 8..9
+        A.emit_cap = A.emit_all = frames ? cap : 0;
+        st = PVT_OK;
+    }
     // classes on side streams (or all on s, one after another, when the
     // autotuner times them); classes without roots launch nothing, and a
     // single class needs no stream of its own

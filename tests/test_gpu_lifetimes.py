@@ -192,15 +192,18 @@ def test_counts_within_a_scratch_limit(pvt, what):
     if want.dim() == 2:
         assert pvt.to_ints(want) == ref["C"]
     tree = [dag.stats()[k] for k in ("sct_nodes", "sct_leaves", "pivot_words", "roots")]
-    launches = set()
-    for mb in (1, 48, 64, 72, 80, 88, 96, 104, 112, 120, 128, 160, 256, 0):
+    launches = {}
+    for mb in [1, *range(48, 321, 8), 0]:
         dag.set_scratch_limit(mb << 20)
         assert torch.equal(COUNTS[what](dag, 4), want), mb
         st = dag.stats()
         if what in ("global", "vertex", "edge"):
             assert [st[k] for k in ("sct_nodes", "sct_leaves", "pivot_words", "roots")] == tree, mb
-        launches.add(st["launches"])
-    assert what == "range" or len(launches) >= 2  # more than one route was taken
+        launches[mb] = st["launches"]
+    if what == "global":
+        assert max(launches.values()) > launches[0]  # the gather went in passes
+    if what != "range":  # (whose last call is the combine)
+        assert min(launches.values()) < launches[0]  # something optional was left out
     dag.free()
 
 
